@@ -285,6 +285,12 @@ struct nb_ctx {
   int64_t *scal = nullptr;      // [0] t_next ticks, [1] n_act
   double *part = nullptr;       // force partial sums
   size_t part_cap = 0;
+  // partial sums of the pair-symmetric force of all particles (allocated at
+  // its first use; sym_off: no room for them, the one-sided kernel runs)
+  float2 *sym_i = nullptr, *sym_j = nullptr;
+  unsigned char *sym_rec = nullptr;
+  size_t sym_i_cap = 0, sym_j_cap = 0;
+  bool sym_off = false;
   double *red = nullptr;        // energy scratch
   int *err = nullptr;           // device error word
   unsigned long long *clamped = nullptr;
@@ -478,6 +484,90 @@ nb_status ensure_part(nb_ctx *c, size_t bytes) {
   return NB_OK;
 }
 
+// Smallest n of the pair-symmetric force.  Below it the ring has too few
+// tiles per CTA: N = 12,000 0.205 ms against 0.193 one-sided (split
+// precision, jerk), N = 16,384 0.261 against 0.308.
+constexpr int64_t kSymMin = 16384;
+
+// The split and scratch of the pair-symmetric force of all particles; false
+// when this context does not take it: too few particles, or no room for
+// its partial sums (at most 1/16 of the device's memory).
+bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
+  if (c->sym_off || c->n < kSymMin) return false;
+  const int prec = c->cfg.precision, mask = eps_masks(c->cfg.eps);
+  SymSplit S;
+  if (!sym_split(c->n_jt, sym_block_i(prec, mask, jrk), c->num_sms, &S)) return false;
+  const size_t ib = sym_ipart_bytes(S, jrk), jb = sym_jpart_bytes(S, jrk);
+  const size_t rb = sym_record_bytes(c->n_jt, prec);
+  if (ib > c->sym_i_cap || jb > c->sym_j_cap) {
+    size_t avail = 0, total = 0;
+    bool ok = cudaMemGetInfo(&avail, &total) == cudaSuccess && ib + jb + rb <= total / 16 &&
+              ib + jb + rb <= avail / 2;
+    const char *cap = std::getenv("NB_TEST_MAX_BYTES");
+    if (cap && jb > static_cast<size_t>(std::strtoull(cap, nullptr, 10))) ok = false;
+    // grows once: from the acceleration's sums to the jerk's
+    float2 *ni = nullptr, *nj = nullptr;
+    if (ok && !c->sym_rec) ok = cudaMalloc(reinterpret_cast<void **>(&c->sym_rec), rb) == cudaSuccess;
+    if (ok) ok = cudaMalloc(reinterpret_cast<void **>(&ni), ib) == cudaSuccess &&
+                 cudaMalloc(reinterpret_cast<void **>(&nj), jb) == cudaSuccess;
+    if (ok) ok = sym_prepare(prec, mask, true) == cudaSuccess &&
+                 sym_prepare(prec, mask, false) == cudaSuccess;
+    if (!ok) {
+      cudaGetLastError();  // the refused allocation is not this call's error
+      if (ni) cudaFree(ni);
+      if (nj) cudaFree(nj);
+      // scratch that is there still serves the acceleration
+      if (!c->sym_j) c->sym_off = true;
+      return false;
+    }
+    if (c->sym_j) {
+      cudaStreamSynchronize(c->stream);
+      cudaFree(c->sym_i);
+      cudaFree(c->sym_j);
+      if (c->sym_graph) {  // holds the old scratch
+        cudaGraphExecDestroy(c->sym_graph);
+        c->sym_graph = nullptr;
+      }
+    }
+    c->sym_i = ni;
+    c->sym_j = nj;
+    c->sym_i_cap = ib;
+    c->sym_j_cap = jb;
+  }
+  A->jhi = c->jhi;
+  A->jlo = c->jlo;
+  A->jvel = c->jvel;
+  A->jrel = c->jrel;
+  A->tinfo = c->tinfo;
+  A->n_jt = c->n_jt;
+  A->n = c->n;
+  A->eps2 = eps2_f32(c->cfg.eps);
+  A->G = c->cfg.G;
+  A->recs = c->sym_rec;
+  A->ipart = c->sym_i;
+  A->jpart = c->sym_j;
+  A->err = c->err;
+  A->split = S;
+  return true;
+}
+
+// Shared steps move every particle in every step: their force is the
+// pair-symmetric one.  Block steps keep the one-sided kernel, whose sums do
+// not depend on which other particles are due.
+bool sym_hermite(nb_ctx *c, SymArgs *A) {
+  return !c->cfg.block_steps && c->sh.p == 1 && sym_ready(c, true, A);
+}
+
+nb_status queue_sym(nb_ctx *c, SymArgs &A, double *d_acc, double *d_jerk) {
+  A.acc = d_acc;
+  A.jerk = d_jerk;
+  int nl = 0;
+  NB_CUDA(launch_sym_force(c->cfg.precision, eps_masks(c->cfg.eps), A, c->stream, &nl));
+  c->launches += nl;
+  c->interactions += c->n * c->n;
+  return NB_OK;
+}
+
 // Queue one force evaluation of n_i i-particles (d_idx may be null for the
 // identity list) into d_acc / d_jerk.
 nb_status queue_force(nb_ctx *c, const int32_t *d_idx, int64_t n_i, double *d_acc,
@@ -588,6 +678,9 @@ void nb_destroy(nb_ctx *c) {
   cudaStreamSynchronize(c->stream);
   for (void *p : c->allocs)
     if (p) cudaFree(p);
+  if (c->sym_rec) cudaFree(c->sym_rec);
+  if (c->sym_i) cudaFree(c->sym_i);
+  if (c->sym_j) cudaFree(c->sym_j);
   if (c->h_scal) cudaFreeHost(c->h_scal);
   if (c->h_energy) cudaFreeHost(c->h_energy);
   if (c->h_sh_off) cudaFreeHost(c->h_sh_off);
@@ -705,7 +798,11 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x,
   TRYC(launch_pad_records(n, c->n_pad, c->jhi, c->jlo, c->jvel, st));
   c->launches += 1;
   TRY(queue_predict(c, 0));
-  TRY(queue_force(c, nullptr, n, c->a, c->jk));
+  SymArgs SA;
+  if (sym_hermite(c, &SA))
+    TRY(queue_sym(c, SA, c->a, c->jk));
+  else
+    TRY(queue_force(c, nullptr, n, c->a, c->jk));
   TRYC(launch_init_levels(n, c->a, c->jk, cfg->eta_start, cfg->lev_min, cfg->lev_max,
                           cfg->block_steps, cfg->lev_shared, c->lev, c->t_tick, st));
   c->launches += 1;
@@ -779,6 +876,37 @@ nb_status nb_predict(nb_ctx *c, double t) {
   return NB_OK;
 }
 
+}  // extern "C"
+
+namespace {
+
+// Force of the active list (a shard: its slice of it) into a1, j1.  With
+// rows, the caller reads them: they are then the one-sided kernel's, the
+// same values that an index list gives.  Without, a step of all particles
+// takes the pair-symmetric kernel (no forced shape, table or grid).
+nb_status force_active(nb_ctx *c, int64_t n_idx, bool rows) {
+  if (!c->have_block) return fail(NB_ERR_STATE, "no active list: call nb_next_block first");
+  if (n_idx >= 0 && n_idx != c->n_act)
+    return fail(NB_ERR_INVALID_ARG, "n_idx %lld != active count %lld", (long long)n_idx,
+                (long long)c->n_act);
+  if (c->t_pred != c->t_block)
+    return fail(NB_ERR_STATE, "prediction time differs from the block time");
+  const int64_t lo = c->own_lo, cnt = c->own_hi - c->own_lo;
+  SymArgs A;
+  nb_status s;
+  if (!rows && c->n_act == c->n && c->variant_override < 0 && c->table_count == 0 &&
+      c->grid_cap == 0 && sym_hermite(c, &A))
+    s = queue_sym(c, A, c->a1, c->j1);
+  else
+    s = queue_force(c, c->act + lo, cnt, c->a1 + 3 * lo, c->j1 + 3 * lo);
+  if (s == NB_OK) c->force_done = true;
+  return s;
+}
+
+}  // namespace
+
+extern "C" {
+
 nb_status nb_force_jerk_dev(nb_ctx *c, const int32_t *d_idx, int64_t n_idx, double *d_acc,
                             double *d_jerk) {
   Range r("nb_force_jerk");
@@ -786,23 +914,15 @@ nb_status nb_force_jerk_dev(nb_ctx *c, const int32_t *d_idx, int64_t n_idx, doub
   if (s != NB_OK) return s;
   if (c->t_pred < 0) return fail(NB_ERR_STATE, "nb_predict must come first");
   if (d_idx == nullptr) {
-    if (!c->have_block) return fail(NB_ERR_STATE, "no active list: call nb_next_block first");
-    if (n_idx >= 0 && n_idx != c->n_act)
-      return fail(NB_ERR_INVALID_ARG, "n_idx %lld != active count %lld", (long long)n_idx,
-                  (long long)c->n_act);
-    if (c->t_pred != c->t_block)
-      return fail(NB_ERR_STATE, "prediction time differs from the block time");
-    // a shard evaluates its own slice of the active list
-    const int64_t lo = c->own_lo, cnt = c->own_hi - c->own_lo;
-    s = queue_force(c, c->act + lo, cnt, c->a1 + 3 * lo, c->j1 + 3 * lo);
+    s = force_active(c, n_idx, d_acc || d_jerk);
     if (s != NB_OK) return s;
+    const int64_t lo = c->own_lo, cnt = c->own_hi - c->own_lo;
     if (d_acc && cnt)
       NB_CUDA(cudaMemcpyAsync(d_acc, c->a1 + 3 * lo, 3 * cnt * sizeof(double),
                               cudaMemcpyDeviceToDevice, c->stream));
     if (d_jerk && cnt)
       NB_CUDA(cudaMemcpyAsync(d_jerk, c->j1 + 3 * lo, 3 * cnt * sizeof(double),
                               cudaMemcpyDeviceToDevice, c->stream));
-    c->force_done = true;
     return NB_OK;
   }
   if (n_idx < 0) return fail(NB_ERR_INVALID_ARG, "negative n_idx");
@@ -826,7 +946,7 @@ nb_status nb_force_jerk(nb_ctx *c, const int32_t *idx, int64_t n_idx, double *ac
   const double *src_a = nullptr, *src_j = nullptr;
   int64_t cnt = 0;
   if (idx == nullptr) {
-    s = nb_force_jerk_dev(c, nullptr, n_idx, nullptr, nullptr);
+    s = force_active(c, n_idx, acc || jerk);
     if (s != NB_OK) return s;
     src_a = c->a1 + 3 * c->own_lo;
     src_j = c->j1 + 3 * c->own_lo;
@@ -925,19 +1045,23 @@ namespace {
 constexpr int kGraphSteps = 32;  // block steps per graph replay
 
 // Force shapes of the device-resident steps: the built-in choice per
-// active-count bucket (the same shapes nb_step runs).
+// active-count bucket (the same shapes nb_step runs).  Where the context
+// takes the pair-symmetric kernel for steps of all particles, the buckets
+// end below n.
 struct Bucket {
   int64_t lo, hi;
   int v;
 };
 
-int step_buckets(const nb_ctx *c, Bucket *b) {
+int step_buckets(nb_ctx *c, Bucket *b) {
+  SymArgs unused;
+  const int64_t top = sym_hermite(c, &unused) ? c->n : INT64_MAX;
   const ShapeBuckets sb = shape_buckets(c->cfg.precision, eps_masks(c->cfg.eps), c->n_jt,
                                         c->num_sms);
   // buckets no active count can reach (or empty ones) are left out
   int k = 0;
   for (int q = 0; q < sb.nbk; ++q) {
-    const int64_t hi = q + 1 < sb.nbk ? sb.lo[q + 1] : INT64_MAX;
+    const int64_t hi = q + 1 < sb.nbk ? std::min(sb.lo[q + 1], top) : top;
     if (sb.lo[q] <= c->n && sb.lo[q] < hi) b[k++] = {sb.lo[q], hi, sb.v[q]};
   }
   return k;
@@ -971,6 +1095,13 @@ nb_status queue_device_blocks(nb_ctx *c, cudaStream_t s, int64_t *launches) {
   Bucket b[3];
   const int nbk = step_buckets(c, b);
   const int prec = c->cfg.precision;
+  SymArgs SA;
+  const bool sym = sym_hermite(c, &SA);
+  if (sym) {
+    SA.acc = c->a1;
+    SA.jerk = c->j1;
+    SA.ctl = c->scal;
+  }
   for (int step = 0; step < kGraphSteps; ++step) {
     int nl = 0;
     NB_CUDA(launch_next_block(c->n, c->t_tick, c->lev, c->act, c->blk, c->scal, s, &nl));
@@ -985,6 +1116,7 @@ nb_status queue_device_blocks(nb_ctx *c, cudaStream_t s, int64_t *launches) {
       const int grid = c->num_sms * ctas_per_sm(b[k].v);
       NB_CUDA(launch_force_dev(b[k].v, device_force_args(c, b[k]), grid, c->n, s, &nl));
     }
+    if (sym) NB_CUDA(launch_sym_force(prec, eps_masks(c->cfg.eps), SA, s, &nl));
     NB_CUDA(launch_correct(c->n, c->act, 0, c->x, c->v, c->a, c->jk, c->t_tick, c->lev, c->a1,
                            c->j1, c->cfg.eta, c->cfg.lev_min, c->cfg.lev_max,
                            c->cfg.block_steps, c->clamped, c->ext, s, c->scal));
@@ -1023,6 +1155,14 @@ nb_status queue_fused_blocks(nb_ctx *c, cudaStream_t s, int64_t *launches) {
   B.rel_lo = INT64_MAX;
   for (int k = 0; k < nbk; ++k)
     if (variant_at(b[k].v).rel && b[k].lo < B.rel_lo) B.rel_lo = b[k].lo;
+  SymArgs SA;
+  const bool sym = sym_hermite(c, &SA);
+  if (sym) {
+    SA.acc = c->a1;
+    SA.jerk = c->j1;
+    SA.ctl = c->scal;
+    B.rel_lo = std::min(B.rel_lo, c->n);
+  }
   B.act = c->act;
   B.ctl = c->scal;
   B.status = c->lb_status;
@@ -1034,6 +1174,7 @@ nb_status queue_fused_blocks(nb_ctx *c, cudaStream_t s, int64_t *launches) {
   EndArgs E;
   E.n = c->n;
   E.n_jt = c->n_jt;
+  E.sym_all = sym ? 1 : 0;
   E.nbk = nbk;
   for (int k = 0; k < nbk; ++k) {
     E.lo[k] = b[k].lo;
@@ -1085,6 +1226,8 @@ nb_status queue_fused_blocks(nb_ctx *c, cudaStream_t s, int64_t *launches) {
       if (e == cudaSuccess) e = cudaEventRecord(join[k], bs[k]);
       if (e == cudaSuccess) e = cudaStreamWaitEvent(s, join[k], 0);
     }
+    if (sym && e == cudaSuccess)
+      e = launch_sym_force(c->cfg.precision, eps_masks(c->cfg.eps), SA, s, &nl);
     if (e == cudaSuccess) e = launch_block_end(E, end_grid, s);
     *launches += 2 + nl;
   }
@@ -1130,9 +1273,20 @@ struct SymArrays {
   const double *m;
 };
 
-// Acceleration of every particle into S.a (acceleration-only kernel of the
-// built-in shape for n, or its acceleration-only counterpart).
-nb_status queue_acc_all(nb_ctx *c, const SymArrays &S, cudaStream_t s, int64_t *launches) {
+// Acceleration of every particle into S.a: the pair-symmetric kernel, or
+// the acceleration-only kernel of the built-in shape for n (or its
+// acceleration-only counterpart).
+nb_status queue_acc_all(nb_ctx *c, const SymArrays &S, cudaStream_t s, int64_t *launches,
+                        bool stepping) {
+  SymArgs SA;
+  if (stepping && sym_ready(c, false, &SA)) {
+    SA.acc = S.a;
+    SA.jerk = nullptr;
+    int nl = 0;
+    NB_CUDA(launch_sym_force(c->cfg.precision, eps_masks(c->cfg.eps), SA, s, &nl));
+    *launches += nl;
+    return NB_OK;
+  }
   const int v = acc_shape(choose_variant(c->cfg.precision, eps_masks(c->cfg.eps), c->n,
                                          c->n_jt, c->num_sms));
   if (!has_acc_only(v)) return fail(NB_ERR_STATE, "force shape %d has no acceleration-only kernel", v);
@@ -1175,7 +1329,7 @@ nb_status queue_symplectic_step(nb_ctx *c, const SymArrays &A, cudaStream_t s, c
   for (int k = 0; k < S; ++k) {
     const double h = 0.5 * dt * ((k > 0 ? w[k - 1] : 0.0) + w[k]);
     nb_status st = queue_kick_drift(c, A, s, h, w[k] * dt, true, launches);
-    if (st == NB_OK) st = queue_acc_all(c, A, s, launches);
+    if (st == NB_OK) st = queue_acc_all(c, A, s, launches, true);
     if (st != NB_OK) return st;
   }
   return queue_kick_drift(c, A, s, 0.5 * dt * w[S - 1], 0.0, false, launches);
@@ -1474,7 +1628,8 @@ extern "C" nb_status nb_symplectic(nb_ctx *c, int32_t order, double dt, int64_t 
   // step's graph
   int64_t nl = 0;
   s = queue_kick_drift(c, A, c->stream, 0.0, 0.0, true, &nl);
-  if (s == NB_OK) s = queue_acc_all(c, A, c->stream, &nl);
+  // with nsteps = 0 the call only refreshes A(x), with the sums nb_init makes
+  if (s == NB_OK) s = queue_acc_all(c, A, c->stream, &nl, nsteps > 0);
   if (s != NB_OK) return s;
   c->launches += nl;
   c->interactions += c->n * c->n;

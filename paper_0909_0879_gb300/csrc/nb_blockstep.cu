@@ -404,14 +404,18 @@ __global__ void __launch_bounds__(kEndThreads) block_end_kernel(const EndArgs E)
   int b = -1;
   for (int q = 0; q < E.nbk; ++q)
     if (n_act >= E.lo[q] && n_act < E.hi[q]) b = q;
-  if (b < 0) return;
-  // the split the force launch of this bucket derived from the same count
-  const int BI = E.bi[b];
+  const bool whole = b < 0 && E.sym_all && n_act == E.n;
+  if (b < 0 && !whole) return;
+  // the split the force launch of this bucket derived from the same count;
+  // one CTA for everything (no split i-block) where the pair-symmetric
+  // kernel's fix-up has written the sums
+  const int BI = whole ? E.bi[0] : E.bi[b];
   const uint64_t U = dev::udiv(static_cast<uint64_t>(n_act + BI - 1), BI) *
                      static_cast<uint64_t>(E.n_jt);
-  const uint64_t mu = static_cast<uint64_t>(E.mu[b]);
+  const uint64_t mu = static_cast<uint64_t>(whole ? 1 : E.mu[b]);
   const uint64_t pm = (U + mu - 1) / mu;
-  const int P = static_cast<int>(pm < static_cast<uint64_t>(E.pmax[b]) ? pm : E.pmax[b]);
+  const int pmax = whole ? 1 : E.pmax[b];
+  const int P = static_cast<int>(pm < static_cast<uint64_t>(pmax) ? pm : pmax);
   // short lists: one entry per warp per round (the fix-ups in parallel);
   // long lists: four, so that the corrector warp runs 32 lanes
   if (n_act <= static_cast<int64_t>(kEndWarps) * gridDim.x) {

@@ -195,6 +195,49 @@ __device__ __forceinline__ void tile_frame(int64_t tile, int64_t j, bool real, f
   }
 }
 
+// Error-free addition of x into the unevaluated sum hi + lo (two-sum).
+__device__ __forceinline__ void ds_add(float &hi, float &lo, float x) {
+  const float s = hi + x;
+  const float bp = s - hi;
+  const float e = (hi - (s - bp)) + (x - bp);
+  hi = s;
+  lo += e;
+}
+
+// Split-precision accumulators of IPT i-particles: acceleration and jerk,
+// high and low words.  In registers, or (SMEM) in shared memory at a
+// per-thread slot so that wide IPT shapes keep registers for the pair
+// arithmetic; the slots are touched only at folds.
+template <int IPT, int NT, bool SMEM>
+struct DsAcc;
+template <int IPT, int NT>
+struct DsAcc<IPT, NT, false> {
+  float ah[IPT][3], al[IPT][3], jh[IPT][3], jl[IPT][3];
+  __device__ __forceinline__ void init(float *, int) {
+#pragma unroll
+    for (int q = 0; q < IPT; ++q)
+#pragma unroll
+      for (int c = 0; c < 3; ++c) ah[q][c] = al[q][c] = jh[q][c] = jl[q][c] = 0.f;
+  }
+  __device__ __forceinline__ float &AH(int q, int c) { return ah[q][c]; }
+  __device__ __forceinline__ float &AL(int q, int c) { return al[q][c]; }
+  __device__ __forceinline__ float &JH(int q, int c) { return jh[q][c]; }
+  __device__ __forceinline__ float &JL(int q, int c) { return jl[q][c]; }
+};
+template <int IPT, int NT>
+struct DsAcc<IPT, NT, true> {
+  float *b;
+  __device__ __forceinline__ void init(float *smem, int tid) {
+    b = smem + tid;
+#pragma unroll
+    for (int k = 0; k < 12 * IPT; ++k) b[k * NT] = 0.f;
+  }
+  __device__ __forceinline__ float &AH(int q, int c) { return b[(12 * q + c) * NT]; }
+  __device__ __forceinline__ float &AL(int q, int c) { return b[(12 * q + 3 + c) * NT]; }
+  __device__ __forceinline__ float &JH(int q, int c) { return b[(12 * q + 6 + c) * NT]; }
+  __device__ __forceinline__ float &JL(int q, int c) { return b[(12 * q + 9 + c) * NT]; }
+};
+
 // Unsigned division and remainder, in 32 bits when both operands fit (a
 // 64-bit division is a long instruction sequence; the result is the same).
 __host__ __device__ __forceinline__ uint64_t udiv(uint64_t a, uint64_t b) {

@@ -36,6 +36,7 @@
 //  * FP64 only where a value leaves the kernel (the FP64 pipe of this part
 //    retires one warp instruction per ~68 cycles per scheduler).
 #include "nb_device.cuh"
+#include "nb_pipe.cuh"
 
 #include <algorithm>
 #include <mutex>
@@ -50,104 +51,11 @@ namespace {
 // split-precision accumulators.
 constexpr int kFoldChunk = 32;
 
-__device__ __forceinline__ uint32_t smem_u32(const void *p) {
-  return static_cast<uint32_t>(__cvta_generic_to_shared(p));
-}
-
-__device__ __forceinline__ void mbar_init(uint64_t *bar, uint32_t count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_u32(bar)),
-               "r"(count)
-               : "memory");
-}
-
-__device__ __forceinline__ void mbar_fence_init() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-
-__device__ __forceinline__ void mbar_expect_tx(uint64_t *bar, uint32_t bytes) {
-  asm volatile(
-      "mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(
-          smem_u32(bar)),
-      "r"(bytes)
-      : "memory");
-}
-
-// 1-D bulk copy global -> shared through the TMA engine; completion is
-// signalled on the mbarrier as transaction bytes.  dst, src 16-byte aligned
-// and bytes a multiple of 16 (always kJT * 16 here).
-__device__ __forceinline__ void bulk_g2s(void *dst, const void *src,
-                                         uint32_t bytes, uint64_t *bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes "
-      "[%0], [%1], %2, [%3];" ::"r"(smem_u32(dst)),
-      "l"(src), "r"(bytes), "r"(smem_u32(bar))
-      : "memory");
-}
-
-__device__ __forceinline__ bool mbar_try_wait(uint64_t *bar, uint32_t phase) {
-  uint32_t ok;
-  asm volatile(
-      "{\n\t.reg .pred p;\n\t"
-      "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
-      "selp.u32 %0, 1, 0, p;\n\t}\n"
-      : "=r"(ok)
-      : "r"(smem_u32(bar)), "r"(phase)
-      : "memory");
-  return ok != 0;
-}
-
-// Bounded wait: false after kWaitLimit unsuccessful polls.
-__device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t phase) {
-  for (uint32_t it = 0; it < kWaitLimit; ++it)
-    if (mbar_try_wait(bar, phase)) return true;
-  return false;
-}
-
-// Error-free addition of x into the unevaluated sum hi + lo (two-sum).
-__device__ __forceinline__ void ds_add(float &hi, float &lo, float x) {
-  const float s = hi + x;
-  const float bp = s - hi;
-  const float e = (hi - (s - bp)) + (x - bp);
-  hi = s;
-  lo += e;
-}
-
 using dev::VOps;
+using namespace pipe;
 
-// Split-precision accumulators of IPT i-particles: acceleration and jerk,
-// high and low words.  In registers, or (SMEM) in shared memory at a
-// per-thread slot so that wide IPT shapes keep registers for the pair
-// arithmetic; the slots are touched only at folds.
-template <int IPT, int NT, bool SMEM>
-struct DsAcc;
-template <int IPT, int NT>
-struct DsAcc<IPT, NT, false> {
-  float ah[IPT][3], al[IPT][3], jh[IPT][3], jl[IPT][3];
-  __device__ __forceinline__ void init(float *, int) {
-#pragma unroll
-    for (int q = 0; q < IPT; ++q)
-#pragma unroll
-      for (int c = 0; c < 3; ++c) ah[q][c] = al[q][c] = jh[q][c] = jl[q][c] = 0.f;
-  }
-  __device__ __forceinline__ float &AH(int q, int c) { return ah[q][c]; }
-  __device__ __forceinline__ float &AL(int q, int c) { return al[q][c]; }
-  __device__ __forceinline__ float &JH(int q, int c) { return jh[q][c]; }
-  __device__ __forceinline__ float &JL(int q, int c) { return jl[q][c]; }
-};
-template <int IPT, int NT>
-struct DsAcc<IPT, NT, true> {
-  float *b;
-  __device__ __forceinline__ void init(float *smem, int tid) {
-    b = smem + tid;
-#pragma unroll
-    for (int k = 0; k < 12 * IPT; ++k) b[k * NT] = 0.f;
-  }
-  __device__ __forceinline__ float &AH(int q, int c) { return b[(12 * q + c) * NT]; }
-  __device__ __forceinline__ float &AL(int q, int c) { return b[(12 * q + 3 + c) * NT]; }
-  __device__ __forceinline__ float &JH(int q, int c) { return b[(12 * q + 6 + c) * NT]; }
-  __device__ __forceinline__ float &JL(int q, int c) { return b[(12 * q + 9 + c) * NT]; }
-};
-
+using dev::ds_add;
+using dev::DsAcc;
 using dev::owner_of;
 
 // JRK = 0: acceleration only (no velocity records, no jerk sums).

@@ -161,6 +161,43 @@ cudaError_t launch_force(int v, const ForceArgs &A, int grid, cudaStream_t s,
 cudaError_t launch_force_dev(int v, const ForceArgs &A, int grid, int64_t n_max,
                              cudaStream_t s, int *launches, bool with_fixup = true);
 
+// --- Pair-symmetric force of all particles on all (nb_symforce.cu) ---
+// Split of the block pairs over the CTAs.  i-blocks of tb tiles lie on a
+// ring of nb blocks; row ib takes the tiles of its own block and of the
+// blocks at ring distances 1, 2, ...: l1 tiles for rows below rows1, l2 for
+// the others.  The rows' tiles, in order, are cut into `ctas` equal ranges.
+struct SymSplit {
+  uint32_t tb, nb;
+  uint32_t rows1, l1, l2, u1;  // u1: units of the first rows1 rows
+  uint32_t units, ctas;
+  uint32_t irows;   // rows a CTA's range can touch
+  uint32_t jslots;  // ring tiles from its first row's first tile on
+};
+struct SymArgs {
+  const float4 *jhi, *jlo, *jvel, *jrel, *tinfo;
+  int64_t n_jt, n;
+  float eps2;
+  double G;
+  double *acc, *jerk;    // (n, 3); jerk null: acceleration only
+  unsigned char *recs;   // the records in pairs (scratch)
+  float2 *ipart, *jpart; // partial sums (hi, lo pairs; scratch)
+  int *err;
+  SymSplit split;
+  // Device-resident mode: a launch does nothing unless ctl[kCtlNact] == n.
+  const int64_t *ctl = nullptr;
+};
+// i-particles per block of the kernel for this precision / masking / output.
+int sym_block_i(int prec, int mask, bool jrk);
+// False when n_jt tiles are too few (or too many) for a ring of such blocks.
+bool sym_split(int64_t n_jt, int bi, int ctas, SymSplit *out);
+size_t sym_record_bytes(int64_t n_jt, int prec);
+size_t sym_ipart_bytes(const SymSplit &S, bool jrk);
+size_t sym_jpart_bytes(const SymSplit &S, bool jrk);
+// Shared-memory attribute of the kernel; before its first launch or capture.
+cudaError_t sym_prepare(int prec, int mask, bool jrk);
+cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
+                             int *launches);
+
 // --- Hermite and bookkeeping kernels (nb_hermite.cu) ---
 // With ctl set, t_next is read from ctl[kCtlTnext] (negative: no-op).
 cudaError_t launch_predict(int64_t n, int64_t t_next, const double *x,
@@ -249,6 +286,7 @@ struct EndArgs {
   int64_t lo[3], hi[3];              // active-count range of each bucket
   int bi[3], pmax[3];                // i-block size and persistent grid
   int mu[3];                         // minimum j-tiles per CTA (min_units)
+  int sym_all;                       // steps of all n particles: force already whole in a1, j1
   const float2 *part;                // partial sums of split i-blocks (hi, lo pairs)
   double G;
   double *a1, *j1;

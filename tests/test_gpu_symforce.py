@@ -1,0 +1,122 @@
+"""The pair-symmetric force of all particles (contexts with shared steps,
+symplectic steps) against the FP64 oracle and the one-sided kernel, at the
+edges of its block ring; bars as for the one-sided kernel (FP32 pair
+arithmetic: condition-relative and norm-wise, 1e-6 / 1e-5 in split
+precision)."""
+import os
+
+import numpy as np
+import pytest
+
+from paper_0909_0879_gb300 import ics
+
+pytestmark = pytest.mark.gpu
+
+TOL = {"ds": (1e-6, 1e-5), "fp32": (1e-3, 1e-3)}
+MIN_N = 16384  # smallest n of the pair-symmetric kernel
+
+
+@pytest.fixture(scope="module")
+def nb():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0909_0879_gb300 import _lib
+
+    _lib.load()
+    return _lib
+
+
+def _system(nb, n, sort, seed=31):
+    m, x, v = ics.plummer(n, seed, masses=ics.salpeter_masses(n, seed))
+    if sort:
+        p = nb.spatial_order(x, 256)
+        m, x, v = m[p], x[p], v[p]
+    return m, x, v
+
+
+# 16 whole blocks (even ring), one particle more (17 blocks, the last one
+# with one particle), a last block of two tiles, an odd ring of whole
+# blocks; in spatial order most tiles take the far field
+@pytest.mark.parametrize("n", [MIN_N, MIN_N + 1, 17 * 1024 + 300, 21 * 1024])
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+@pytest.mark.parametrize("eps", [1e-3, 0.0])
+@pytest.mark.parametrize("sort", [False, True])
+def test_matches_oracle_and_one_sided(nb, oracle_mod, n, prec, eps, sort):
+    m, x, v = _system(nb, n, sort)
+    with nb.NBody(m, x, v, eps=eps, precision=prec, block_steps=False, lev_shared=10) as s:
+        got = s.get_state(want=("a", "jerk"))
+    with nb.NBody(m, x, v, eps=eps, precision=prec) as s:
+        one = s.get_state(want=("a", "jerk"))  # block steps: one-sided
+        s.set_symplectic_layout("as_given")
+        s.symplectic(2, 0.0, 1)  # the acceleration-only kernel, x unchanged
+        acc = s.get_state(want=("a", "x"))
+    assert np.array_equal(acc["x"], x)
+    idx = np.unique(np.concatenate([np.arange(64), np.arange(n - 64, n),
+                                    np.random.default_rng(n).integers(0, n, 900)])).astype(np.int32)
+    ra, rj = oracle_mod.force_jerk(m, x, v, eps, idx=idx)
+    ca, cj = oracle_mod.force_jerk_abs(m, x, v, eps, idx=idx)
+    ta, tj = TOL[prec]
+    for a in (got["a"], acc["a"]):
+        assert np.max(np.linalg.norm(a[idx] - ra, axis=1) / ca) <= ta
+        assert np.linalg.norm(a[idx] - ra) <= ta * np.linalg.norm(ra)
+        assert np.linalg.norm(a - one["a"]) <= 2 * ta * np.linalg.norm(one["a"])
+    assert np.max(np.linalg.norm(got["jerk"][idx] - rj, axis=1) / cj) <= tj
+    assert np.linalg.norm(got["jerk"] - one["jerk"]) <= 2 * tj * np.linalg.norm(one["jerk"])
+    # it is the pair-symmetric kernel that ran, not the one-sided one
+    assert not np.array_equal(got["a"], one["a"])
+
+
+@pytest.mark.parametrize("prec,eps", [("ds", 1e-3), ("fp32", 1e-3), ("ds", 0.0)])
+def test_step_loop_and_device_steps_agree_bitwise(nb, prec, eps):
+    """nb_step, the fused and the general device-resident steps take the same
+    kernel for steps of all particles, with the same bits, run after run."""
+    n = MIN_N + 1
+    m, x, v = _system(nb, n, True)
+    kw = dict(eps=eps, precision=prec, block_steps=False, lev_shared=10)
+    res = []
+    for mode in ("step", "step", "auto", "general"):
+        with nb.NBody(m, x, v, **kw) as s:
+            if mode == "step":
+                for _ in range(3):
+                    s.step()
+            else:
+                s.set_block_mode(mode)
+                assert s.run_blocks(3 * 2.0**-10)[0] == 3
+            res.append(s.get_state())
+    for st in res[1:]:
+        for k in st:
+            assert np.array_equal(st[k], res[0][k]), k
+
+
+def test_one_sided_where_rows_or_shapes_are_asked_for_and_without_scratch(nb):
+    """Rows of the active list handed to the caller are those an index list
+    gives; a forced shape is the shape that runs; without room for the
+    partial sums the one-sided kernel runs and the call succeeds."""
+    n = MIN_N
+    m, x, v = _system(nb, n, False)
+    kw = dict(eps=1e-3, block_steps=False, lev_shared=10)
+    with nb.NBody(m, x, v, **kw) as s:
+        t, na = s.next_block()
+        s.predict(t)
+        a, j = s.force_jerk()
+        ai, ji = s.force_jerk(np.arange(n))
+        assert np.array_equal(a, ai) and np.array_equal(j, ji)
+        s.correct(t)
+        rows = s.get_state(want=("a",))["a"]
+        assert np.array_equal(rows, a)
+    with nb.NBody(m, x, v, **kw) as s:
+        s.set_force_variant(26)
+        s.step()
+        forced = s.get_state(want=("a",))["a"]
+        assert np.array_equal(forced, a) or np.linalg.norm(forced - a) <= 2e-6 * np.linalg.norm(a)
+    os.environ["NB_TEST_MAX_BYTES"] = str(32 << 20)
+    try:
+        with nb.NBody(m, x, v, **kw) as s, nb.NBody(m, x, v, eps=1e-3) as o:
+            assert np.array_equal(s.get_state(want=("a",))["a"], o.get_state(want=("a",))["a"])
+            s.step()
+            o.symplectic(2, 2.0**-10, 1)
+            assert np.isfinite(s.get_state(want=("x",))["x"]).all()
+    finally:
+        del os.environ["NB_TEST_MAX_BYTES"]
