@@ -292,6 +292,7 @@ struct nb_ctx {
   size_t sym_i_cap = 0, sym_j_cap = 0;
   bool sym_off = false;
   double *red = nullptr;        // energy scratch
+  unsigned char *en_rec = nullptr;  // records of the split-precision energy
   int *err = nullptr;           // device error word
   unsigned long long *clamped = nullptr;
   int32_t *qidx = nullptr;      // staged host index lists
@@ -399,6 +400,17 @@ nb_status dev_alloc_t(nb_ctx *c, T **p, size_t count) {
   return dev_alloc(c, reinterpret_cast<void **>(p), count * sizeof(T));
 }
 
+// Optional scratch: false (and no error) where there is no room, and the
+// caller takes a path without it.
+bool scratch_alloc(void **p, size_t bytes) {
+  const char *cap = std::getenv("NB_TEST_MAX_BYTES");
+  if (cap && bytes > static_cast<size_t>(std::strtoull(cap, nullptr, 10))) return false;
+  if (cudaMalloc(p, bytes) == cudaSuccess) return true;
+  cudaGetLastError();
+  *p = nullptr;
+  return false;
+}
+
 // Wait for the stream with a host watchdog, then read the device error word
 // and the small scalars into pinned memory.
 nb_status sync_ctx(nb_ctx *c) {
@@ -503,17 +515,15 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
     size_t avail = 0, total = 0;
     bool ok = cudaMemGetInfo(&avail, &total) == cudaSuccess && ib + jb + rb <= total / 16 &&
               ib + jb + rb <= avail / 2;
-    const char *cap = std::getenv("NB_TEST_MAX_BYTES");
-    if (cap && jb > static_cast<size_t>(std::strtoull(cap, nullptr, 10))) ok = false;
     // grows once: from the acceleration's sums to the jerk's
     float2 *ni = nullptr, *nj = nullptr;
-    if (ok && !c->sym_rec) ok = cudaMalloc(reinterpret_cast<void **>(&c->sym_rec), rb) == cudaSuccess;
-    if (ok) ok = cudaMalloc(reinterpret_cast<void **>(&ni), ib) == cudaSuccess &&
-                 cudaMalloc(reinterpret_cast<void **>(&nj), jb) == cudaSuccess;
+    if (ok && !c->sym_rec) ok = scratch_alloc(reinterpret_cast<void **>(&c->sym_rec), rb);
+    if (ok) ok = scratch_alloc(reinterpret_cast<void **>(&ni), ib) &&
+                 scratch_alloc(reinterpret_cast<void **>(&nj), jb);
     if (ok) ok = sym_prepare(prec, mask, true) == cudaSuccess &&
                  sym_prepare(prec, mask, false) == cudaSuccess;
     if (!ok) {
-      cudaGetLastError();  // the refused allocation is not this call's error
+      cudaGetLastError();  // a refused query is not this call's error
       if (ni) cudaFree(ni);
       if (nj) cudaFree(nj);
       // scratch that is there still serves the acceleration
@@ -678,6 +688,7 @@ void nb_destroy(nb_ctx *c) {
   cudaStreamSynchronize(c->stream);
   for (void *p : c->allocs)
     if (p) cudaFree(p);
+  if (c->en_rec) cudaFree(c->en_rec);
   if (c->sym_rec) cudaFree(c->sym_rec);
   if (c->sym_i) cudaFree(c->sym_i);
   if (c->sym_j) cudaFree(c->sym_j);
@@ -1797,8 +1808,11 @@ nb_status nb_energy(nb_ctx *c, double *kin, double *pot, double *tot) {
   if (s != NB_OK) return s;
   int nl = 0;
   double *d_out = c->red + energy_scratch_doubles(c->n) - 3;
-  NB_CUDA(launch_energy(c->n, c->m, c->x, c->v, c->cfg.G, c->cfg.eps, c->ext, c->red, d_out,
-                        c->stream, &nl));
+  const size_t rb = energy_record_bytes(c->n);
+  // without room for the records: the FP64 pair sum
+  if (rb && !c->en_rec) scratch_alloc(reinterpret_cast<void **>(&c->en_rec), rb);
+  NB_CUDA(launch_energy(c->n, c->m, c->x, c->v, c->cfg.G, c->cfg.eps, c->ext, c->red,
+                        rb ? c->en_rec : nullptr, c->num_sms, d_out, c->stream, &nl));
   c->launches += nl;
   NB_CUDA(cudaMemcpyAsync(c->h_energy, d_out, 3 * sizeof(double), cudaMemcpyDeviceToHost,
                           c->stream));

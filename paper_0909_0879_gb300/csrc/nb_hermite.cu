@@ -2,7 +2,7 @@
 // of the j-records (split precision on the FP32 pipe), FP64 corrector
 // with the Aarseth step criterion and power-of-two block quantisation,
 // block scheduling (minimum next time and ordered compaction of the active
-// list), and the FP64 energy diagnostic.
+// list).
 //
 // Sources: predictor / corrector after Makino & Aarseth (1992); time-step
 // criterion Aarseth (1985), cited in the paper's Sec. 2; individual (block)
@@ -258,101 +258,6 @@ __global__ void due_scatter_kernel(int64_t n, const int64_t *__restrict__ t_tick
   }
 }
 
-// ---- energy ---------------------------------------------------------------
-
-constexpr int kEnThreads = 256;
-
-// Fixed-order block reduction of one double per thread.
-__device__ __forceinline__ double block_sum(double v, double *sh) {
-  sh[threadIdx.x] = v;
-  __syncthreads();
-  for (int s = blockDim.x / 2; s > 0; s >>= 1) {
-    if (threadIdx.x < s) sh[threadIdx.x] += sh[threadIdx.x + s];
-    __syncthreads();
-  }
-  const double r = sh[0];
-  __syncthreads();
-  return r;
-}
-
-__global__ void kinetic_kernel(int64_t n, const double *__restrict__ m,
-                               const double *__restrict__ v, double *__restrict__ part) {
-  __shared__ double sh[kEnThreads];
-  double s = 0.0;
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) {
-    const double vx = v[3 * i], vy = v[3 * i + 1], vz = v[3 * i + 2];
-    s = 0.5 * m[i] * (vx * vx + vy * vy + vz * vz);
-  }
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-// w_i = m_i sum_{j > i} m_j / sqrt(r^2 + eps^2), FP64, j staged in tiles
-// from the CTA's own diagonal tile on (each pair once); the block's sum of
-// w_i goes to part[blockIdx.x].
-__global__ void potential_kernel(int64_t n, const double *__restrict__ m,
-                                 const double *__restrict__ x, double eps2,
-                                 double *__restrict__ part) {
-  __shared__ double sx[kEnThreads], sy[kEnThreads], sz[kEnThreads], sm[kEnThreads];
-  __shared__ double sh[kEnThreads];
-  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * blockDim.x;
-  const int64_t i = i0 + threadIdx.x;
-  const bool valid = i < n;
-  const double xi = valid ? x[3 * i] : 0.0;
-  const double yi = valid ? x[3 * i + 1] : 0.0;
-  const double zi = valid ? x[3 * i + 2] : 0.0;
-  double w = 0.0;
-  for (int64_t j0 = i0; j0 < n; j0 += kEnThreads) {
-    const int64_t jl = j0 + threadIdx.x;
-    if (jl < n) {
-      sx[threadIdx.x] = x[3 * jl];
-      sy[threadIdx.x] = x[3 * jl + 1];
-      sz[threadIdx.x] = x[3 * jl + 2];
-      sm[threadIdx.x] = m[jl];
-    }
-    __syncthreads();
-    const int cnt = (n - j0) < kEnThreads ? static_cast<int>(n - j0) : kEnThreads;
-    // on the diagonal tile only j > i counts
-    const int t0 = (j0 == i0) ? static_cast<int>(threadIdx.x) + 1 : 0;
-    for (int t = t0; t < cnt; ++t) {
-      const double dx = sx[t] - xi, dy = sy[t] - yi, dz = sz[t] - zi;
-      const double s2 = dx * dx + dy * dy + dz * dz + eps2;
-      w += sm[t] * rsqrt(s2);
-    }
-    __syncthreads();
-  }
-  const double wi = valid ? m[i] * w : 0.0;
-  const double s = block_sum(wi, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-// One CTA sums part[0..cnt) in a fixed order and writes out[slot].
-// e_i = m_i Phi_ext(x_i); the block's sum goes to part[blockIdx.x].
-__global__ void ext_potential_kernel(int64_t n, const ExtField E, const double *__restrict__ m,
-                                     const double *__restrict__ x, double *__restrict__ part) {
-  __shared__ double sh[kEnThreads];
-  double s = 0.0;
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (i < n) {
-    const double xv[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
-    double av[3] = {0.0, 0.0, 0.0}, phi = 0.0;
-    dev::ext_field(E, xv, nullptr, av, nullptr, &phi);
-    s = m[i] * phi;
-  }
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) part[blockIdx.x] = s;
-}
-
-__global__ void final_sum_kernel(int64_t cnt, const double *__restrict__ part, double scale,
-                                 double *__restrict__ out, int slot) {
-  __shared__ double sh[kEnThreads];
-  double s = 0.0;
-  for (int64_t b = threadIdx.x; b < cnt; b += blockDim.x) s += part[b];
-  s = block_sum(s, sh);
-  if (threadIdx.x == 0) out[slot] = scale * s;
-}
-
 }  // namespace
 
 cudaError_t launch_predict(int64_t n, int64_t t_next, const double *x, const double *v,
@@ -434,25 +339,6 @@ cudaError_t launch_next_block(int64_t n, const int64_t *t_tick, const int32_t *l
   due_scatter_kernel<<<static_cast<unsigned>(nblk), kSchedThreads, 0, s>>>(
       n, t_tick, lev, d_scal, blk_count, act);
   if (launches) *launches += 4;
-  return cudaGetLastError();
-}
-
-int64_t energy_scratch_doubles(int64_t n) { return 3 * ((n + kEnThreads - 1) / kEnThreads) + 3; }
-
-cudaError_t launch_energy(int64_t n, const double *m, const double *x, const double *v,
-                          double G, double eps, const ExtField &E, double *red, double *d_out,
-                          cudaStream_t s, int *launches) {
-  const int64_t nb = (n + kEnThreads - 1) / kEnThreads;
-  double *pk = red;
-  double *pw = red + nb;
-  double *pe = red + 2 * nb;
-  kinetic_kernel<<<static_cast<unsigned>(nb), kEnThreads, 0, s>>>(n, m, v, pk);
-  potential_kernel<<<static_cast<unsigned>(nb), kEnThreads, 0, s>>>(n, m, x, eps * eps, pw);
-  if (E.on) ext_potential_kernel<<<static_cast<unsigned>(nb), kEnThreads, 0, s>>>(n, E, m, x, pe);
-  final_sum_kernel<<<1, kEnThreads, 0, s>>>(nb, pk, 1.0, d_out, 0);
-  final_sum_kernel<<<1, kEnThreads, 0, s>>>(nb, pw, -G, d_out, 1);
-  final_sum_kernel<<<1, kEnThreads, 0, s>>>(E.on ? nb : 0, pe, 1.0, d_out, 2);
-  if (launches) *launches += E.on ? 6 : 5;
   return cudaGetLastError();
 }
 

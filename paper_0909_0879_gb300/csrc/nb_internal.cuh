@@ -240,12 +240,19 @@ cudaError_t launch_next_block(int64_t n, const int64_t *t_tick,
                               int32_t *blk_count, int64_t *d_scal,
                               cudaStream_t s, int *launches);
 int64_t next_block_scratch_ints(int64_t n);
-// Kinetic and softened potential energy in FP64 into d_out[0..1], and the
-// external field's potential energy sum_i m_i Phi(x_i) into d_out[2] (0
-// when E.on is 0).
+
+// --- Energy (nb_energy.cu) ---
+constexpr int64_t kEnMaxCtas = 1024;
+// Kinetic and softened potential energy into d_out[0..1], and the external
+// field's potential energy sum_i m_i Phi(x_i) into d_out[2] (0 when E.on
+// is 0).  recs: energy_record_bytes(n) of scratch, or null for the FP64
+// pair sum.
 cudaError_t launch_energy(int64_t n, const double *m, const double *x,
                           const double *v, double G, double eps, const ExtField &E,
-                          double *red, double *d_out, cudaStream_t s, int *launches);
+                          double *red, unsigned char *recs, int num_sms, double *d_out,
+                          cudaStream_t s, int *launches);
+// 0: n takes the FP64 pair sum.
+size_t energy_record_bytes(int64_t n);
 int64_t energy_scratch_doubles(int64_t n);
 
 // --- Fused device-resident block steps (nb_blockstep.cu) ---

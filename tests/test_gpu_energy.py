@@ -1,0 +1,107 @@
+"""The energy of a state against a sum in extended precision, around the size
+where the split-precision pair sum takes over from the FP64 one (n = 1,024)
+and at ragged sizes.  Bar: 2e-15 of the pair energy; a term carries 2^-46 =
+1.4e-14 at most, independent from pair to pair, so that n >= 1,024 particles
+(5e5 pairs) leave less than an ulp, and the FP64 sums a few."""
+import math
+import os
+
+import numpy as np
+import pytest
+
+from paper_0909_0879_gb300 import ics
+
+pytestmark = pytest.mark.gpu
+
+BAR = 2e-15
+
+
+@pytest.fixture(scope="module")
+def nb():
+    import torch
+
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_0909_0879_gb300 import _lib
+
+    _lib.load()
+    return _lib
+
+
+def _reference(m, x, v, eps):
+    """Kinetic and pair energy: FP64 terms, exact sums (each term's own
+    rounding is 1e-16 and averages over the pairs)."""
+    w = []
+    for i in range(len(m) - 1):
+        d = x[i + 1:] - x[i]
+        r2 = d[:, 0] * d[:, 0] + d[:, 1] * d[:, 1] + d[:, 2] * d[:, 2] + eps * eps
+        w.append(m[i] * math.fsum(m[i + 1:] / np.sqrt(r2)))
+    return math.fsum((0.5 * m[:, None] * v * v).ravel()), -math.fsum(w)
+
+
+def _system(n, kind):
+    m, x, v = ics.plummer(n, 71, masses=ics.salpeter_masses(n, 72))
+    if kind == "offset":  # a small cluster far from the origin
+        x = 0.01 * x + np.array([8.5, -3.0, 0.25])
+    if kind == "binaries":  # hard binaries that hold most of the energy
+        for k in range(0, 12, 2):
+            x[k + 1] = x[k] + 1e-6 * (1 + k) * np.array([0.3, 0.5, -0.7])
+    if kind == "massless":
+        m[1::3] = 0.0
+        x[4] = x[3] + 1e-17
+    return m, x, v
+
+
+@pytest.mark.parametrize("n", [1023, 1024, 1025, 1279, 3000])
+@pytest.mark.parametrize("eps", [0.0, 1e-4])
+@pytest.mark.parametrize("kind", ["plain", "offset", "binaries", "massless"])
+def test_energy_against_exact_sum(nb, n, eps, kind):
+    m, x, v = _system(n, kind)
+    if eps == 0.0 and kind == "massless":
+        pytest.skip("a coincident pair")
+    k_ref, w_ref = _reference(m, x, v, eps)
+    with nb.NBody(m, x, v, eps=eps) as s:
+        k, w, e = s.energy()
+    assert abs(k / k_ref - 1.0) <= BAR
+    assert abs(w / w_ref - 1.0) <= BAR
+    assert e == k + w
+
+
+@pytest.mark.parametrize("scale", [1e-30, 1e30])
+def test_energy_in_other_units(nb, scale):
+    """Lengths and masses far from 1: the sum is scaled by powers of two."""
+    n = 1100
+    m, x, v = _system(n, "plain")
+    k0, w0 = _reference(m, x, v, 1e-3)
+    with nb.NBody(m, x, v, eps=1e-3) as s:
+        st = s.get_state()
+        st["x"] = x * 2.0**60 if scale > 1 else x * 2.0**-60
+        # the context keeps its own softening, so the reference does too
+        s.set_state(st)
+        k, w, _ = s.energy()
+    k_ref, w_ref = _reference(m, st["x"], v, 1e-3)
+    assert abs(k / k0 - 1.0) <= BAR
+    # (2^-60: every distance far below the softening, hardly any of the
+    # roundings are independent)
+    assert abs(w / w_ref - 1.0) <= (BAR if scale > 1 else 1e-14)
+
+
+def test_energy_of_coincident_particles_and_without_scratch(nb):
+    n = 1200
+    m, x, v = _system(n, "plain")
+    with nb.NBody(m, x, v, eps=0.0) as s:
+        st = s.get_state()
+        w0 = s.energy()[1]
+        st["x"][700] = st["x"][20]
+        s.set_state(st)
+        with pytest.raises(nb.NBodyError) as e:
+            s.energy()
+        assert e.value.status == nb.NB_ERR_NUMERIC
+    with nb.NBody(m, x, v, eps=0.0) as s:
+        os.environ["NB_TEST_MAX_BYTES"] = "1000"
+        try:
+            w1 = s.energy()[1]  # the FP64 sum
+        finally:
+            del os.environ["NB_TEST_MAX_BYTES"]
+        w2 = s.energy()[1]
+    assert abs(w1 / w0 - 1.0) <= BAR and w2 == w0
