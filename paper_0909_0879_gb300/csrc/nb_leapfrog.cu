@@ -8,19 +8,19 @@
 // tidal tensor T(d) = I / s^3 - 3 d d^T / s^5 (symmetric, even in d):
 //   dL/dx_k = G sum_{j != k} T(x_j - x_k) (m_k g_j - m_j g_k)
 //   dL/dm_k = G sum_{i != k} g_i . (x_k - x_i) / s_ik^3
-// Both sums are i-parallel: each CTA holds 32 i-particles, 8 threads per
-// particle split the j-range and meet by a warp-shuffle butterfly, so the
-// results do not depend on launch order.  j-tiles are staged in shared
-// memory by the CTA's threads.  The i == j term is exactly zero for eps > 0
-// and masked for eps == 0.
+// Both sums are i-parallel: several lanes split a particle's j-range and meet
+// by a warp-shuffle butterfly, so the results do not depend on launch order.
+// The i == j term is exactly zero for eps > 0 and masked for eps == 0.
 //
 // Reverse of one KDK step (x, v) -> (x', v'):
 //   v_h = v + A(x) dt/2, x' = x + v_h dt, v' = v_h + A(x') dt/2
 //   lv_h = lv'; (lx', lm) += vjp_A(x'; lv' dt/2); lv_h += lx' dt;
 //   (lx, lm) += vjp_A(x; lv_h dt/2); lx = lx', lv = lv_h
-// The forward pass stores (x, v) every `ckpt_every` steps; the reverse pass
-// re-runs each segment from its checkpoint, keeping the segment's positions,
-// then walks it backwards.
+// The first kick of a step and the second kick of the step before it meet at
+// the same x and lv, so a reverse pass takes one vjp_A(x; lv dt) there: n + 1
+// of them for n steps.  The forward pass stores (x, v) every `ckpt_every`
+// steps; the reverse pass re-runs each segment from its checkpoint, keeping
+// the segment's positions, then walks it backwards.
 #include "../../include/nbody.h"
 #include "nb_internal.cuh"
 
@@ -30,53 +30,193 @@
 namespace nbi {
 namespace {
 
-constexpr int kLfT = 256;              // threads per CTA
-constexpr int kLfTpi = 8;              // threads per i-particle
-constexpr int kLfI = kLfT / kLfTpi;    // i-particles per CTA
-constexpr int kLfJT = 256;             // j-records per shared tile
+constexpr int kLfT = 256;              // threads per CTA, wide shape
+constexpr int kLfJT = 256;             // j-records per shared tile, wide shape
+
+// Small and middle N.  A particle's sum runs over eight chains of every
+// eighth record.  A group of four warps holds 32 particles, one per lane;
+// each warp takes two chains, side by side in packed FP32x2 instructions, so
+// that a pair of records is one shared-memory broadcast.  The elementwise
+// work around a force (kicks, drift, checkpoint) is done by the CTA that holds
+// the particles, so a step is one launch.  Records come in tiles by
+// asynchronous copies, the next tile while the current one is summed, stored
+// in pairs so that a packed instruction takes two of them without a move.
+// Measured per evaluation, N = 1,000 / 4,096 / 16,000 / 60,000: 6.5 / 16.7 / 132
+// / 1,612 us (eight threads per particle, synchronous tile loads: 8.3 / 21.3 /
+// 162 / 1,784, and a second launch for the step).  At N = 4,096 the eight
+// chains leave one warp per scheduler, whose latencies set the time.  Lanes
+// that split a particle's records, with one, two or four particles per lane,
+// give 18.7 / 16.7 / - us at N = 4,096 and 1,860 / 1,786 / 1,763 at 60,000;
+// programmatic dependent launch stacks waiting CTAs on some SMs (22 us).
+constexpr int kLfTile = 512;
+constexpr int kLfVjpTile = 1024;
+constexpr int kLfAccWarps = 4;  // warps of a group of 32 particles
+constexpr int kLfVjpTpi = 64;   // threads of a particle pair: vector-Jacobian product
+constexpr int kLfMaxThreads = 512, kLfVjpMaxThreads = 1024;
+
+__device__ __forceinline__ float2 dup(float s) { return make_float2(s, s); }
 
 template <int MASK>
-__global__ void __launch_bounds__(kLfT) lf_acc_kernel(int64_t n, const float *__restrict__ x,
-                                                      const float *__restrict__ m, float eps2,
-                                                      float G, float *__restrict__ acc) {
-  __shared__ float4 sj[kLfJT];
-  const int g = threadIdx.x / kLfTpi, r = threadIdx.x % kLfTpi;
-  const int64_t i = static_cast<int64_t>(blockIdx.x) * kLfI + g;
-  const int64_t ii = i < n ? i : 0;
-  const float xi = x[3 * ii], yi = x[3 * ii + 1], zi = x[3 * ii + 2];
-  float ax = 0.f, ay = 0.f, az = 0.f;
-  for (int64_t j0 = 0; j0 < n; j0 += kLfJT) {
-    const int64_t j = j0 + threadIdx.x;
-    sj[threadIdx.x] = j < n ? make_float4(x[3 * j], x[3 * j + 1], x[3 * j + 2], m[j])
-                            : make_float4(1.0e15f, 1.0e15f, 1.0e15f, 0.f);
-    __syncthreads();
-#pragma unroll 4
-    for (int t = r; t < kLfJT; t += kLfTpi) {
-      const float4 q = sj[t];
-      const float dx = q.x - xi, dy = q.y - yi, dz = q.z - zi;
-      const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
-      float rinv;
-      if (MASK)
-        rinv = s2 > 0.f ? rsqrtf(s2) : 0.f;
-      else
-        rinv = rsqrtf(s2);
-      const float f = (q.w * rinv) * (rinv * rinv);
-      ax = fmaf(f, dx, ax);
-      ay = fmaf(f, dy, ay);
-      az = fmaf(f, dz, az);
-    }
-    __syncthreads();
-  }
+__device__ __forceinline__ float2 lf_rsq2(float2 s2) {
+  float2 r;
+  r.x = MASK ? (s2.x > 0.f ? rsqrtf(s2.x) : 0.f) : rsqrtf(s2.x);
+  r.y = MASK ? (s2.y > 0.f ? rsqrtf(s2.y) : 0.f) : rsqrtf(s2.y);
+  return r;
+}
+
+// A rounded packed product that no following addition is fused with.
+__device__ __forceinline__ float2 mul2_alone(float2 a, float2 b) {
+  float2 c;
+  asm("{\n\t.reg .b64 a, b, c;\n\tmov.b64 a, {%2, %3};\n\tmov.b64 b, {%4, %5};\n\t"
+      "mul.rn.f32x2 c, a, b;\n\tmov.b64 {%0, %1}, c;\n\t}"
+      : "=f"(c.x), "=f"(c.y)
+      : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+  return c;
+}
+
+// Asynchronous copy of one float, completed by copies_wait().
+__device__ __forceinline__ void copy_float(float *dst, const float *src) {
+  asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(
+                   static_cast<uint32_t>(__cvta_generic_to_shared(dst))),
+               "l"(src)
+               : "memory");
+}
+__device__ __forceinline__ void copies_commit() {
+  asm volatile("cp.async.commit_group;" ::: "memory");
+}
+template <int LEFT>
+__device__ __forceinline__ void copies_wait() {
+  asm volatile("cp.async.wait_group %0;" ::"n"(LEFT) : "memory");
+}
+
+// Queue the copies of records (x, y, z, w) of a tile, w from m;
+// past the end: no mass, far away.
+__device__ __forceinline__ void stage_xm(float4 *t, int64_t j0, int64_t n, const float *x,
+                                         const float *m) {
+  for (int r = threadIdx.x; r < kLfVjpTile; r += blockDim.x) {
+    const int64_t j = j0 + r;
+    float *const d = reinterpret_cast<float *>(t + r);
+    if (j < n) {
 #pragma unroll
-  for (int off = 1; off < kLfTpi; off <<= 1) {
-    ax += __shfl_xor_sync(0xffffffffu, ax, off);
-    ay += __shfl_xor_sync(0xffffffffu, ay, off);
-    az += __shfl_xor_sync(0xffffffffu, az, off);
+      for (int c = 0; c < 3; ++c) copy_float(d + c, x + 3 * j + c);
+      copy_float(d + 3, m + j);
+    } else {
+      t[r] = make_float4(1.0e15f, 1.0e15f, 1.0e15f, 0.f);
+    }
   }
-  if (r == 0 && i < n) {
-    acc[3 * i] = G * ax;
-    acc[3 * i + 1] = G * ay;
-    acc[3 * i + 2] = G * az;
+}
+// The same in pairs: planes of (x0 x1 y0 y1) and (z0 z1 m0 m1), kLfTile / 2
+// each.
+__device__ __forceinline__ void stage_pairs(float4 *t, int64_t j0, int64_t n, const float *x,
+                                            const float *m) {
+  for (int r = threadIdx.x; r < kLfTile; r += blockDim.x) {
+    const int64_t j = j0 + r;
+    float *const xy = reinterpret_cast<float *>(t) + 4 * (r >> 1) + (r & 1);
+    float *const zm = xy + 2 * kLfTile;
+    if (j < n) {
+      copy_float(xy, x + 3 * j);
+      copy_float(xy + 2, x + 3 * j + 1);
+      copy_float(zm, x + 3 * j + 2);
+      copy_float(zm + 2, m + j);
+    } else {
+      xy[0] = xy[2] = zm[0] = 1.0e15f;
+      zm[2] = 0.f;
+    }
+  }
+}
+// The same for cotangents (zero past the end).
+__device__ __forceinline__ void stage_g(float4 *t, int64_t j0, int64_t n, const float *g) {
+  for (int r = threadIdx.x; r < kLfVjpTile; r += blockDim.x) {
+    const int64_t j = j0 + r;
+    float *const d = reinterpret_cast<float *>(t + r);
+    if (j < n) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) copy_float(d + c, g + 3 * j + c);
+    } else {
+      t[r] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  }
+}
+
+// What follows a force evaluation, per element: with close, the kick v += a
+// h that ends the previous step; then, when ck is set, the checkpoint (x, v)
+// of the step boundary; then, when x_out is set, this step's opening kick v +=
+// a h and the drift x_out = x + v dt.  acc (may be null) receives a.
+struct LfTail {
+  const float *v_in = nullptr;
+  float *v_out = nullptr;
+  float *x_out = nullptr;
+  float *acc = nullptr;
+  float *ck = nullptr;
+  int close = 0;
+  float h = 0.f, dt = 0.f;
+};
+
+template <int MASK>
+__global__ void __launch_bounds__(kLfMaxThreads)
+    lf_eval_kernel(int64_t n, int per_cta, const float *__restrict__ x,
+                   const float *__restrict__ m, float eps2, float G, const LfTail T) {
+  __shared__ float4 tiles[2][kLfTile];
+  __shared__ float part[kLfMaxThreads][3];
+  constexpr int kPairs = kLfTile / 2;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int r = wid % kLfAccWarps;  // the warp's chains
+  const int64_t i0 = static_cast<int64_t>(blockIdx.x) * per_cta;
+  const int64_t i = i0 + wid / kLfAccWarps * 32 + lane;
+  const int64_t ii = i < n ? i : 0;
+  const float2 nx = dup(-x[3 * ii]), ny = dup(-x[3 * ii + 1]), nz = dup(-x[3 * ii + 2]);
+  const float2 e2 = dup(eps2);
+  float2 px = dup(0.f), py = px, pz = px;
+  stage_pairs(tiles[0], 0, n, x, m);
+  copies_commit();
+  int b = 0;
+  for (int64_t j0 = 0; j0 < n; j0 += kLfTile, b ^= 1) {
+    if (j0 + kLfTile < n) stage_pairs(tiles[b ^ 1], j0 + kLfTile, n, x, m);
+    copies_commit();
+    copies_wait<1>();
+    __syncthreads();
+    const float4 *t = tiles[b];
+    auto pair = [&](int k) {
+      const float4 q = t[k], w = t[kPairs + k];
+      const float2 dx = __fadd2_rn(make_float2(q.x, q.y), nx);
+      const float2 dy = __fadd2_rn(make_float2(q.z, q.w), ny);
+      const float2 dz = __fadd2_rn(make_float2(w.x, w.y), nz);
+      const float2 s2 = __ffma2_rn(dx, dx, __ffma2_rn(dy, dy, __ffma2_rn(dz, dz, e2)));
+      const float2 ri = lf_rsq2<MASK>(s2);
+      const float2 f = __fmul2_rn(__fmul2_rn(make_float2(w.z, w.w), ri), __fmul2_rn(ri, ri));
+      px = __ffma2_rn(f, dx, px);
+      py = __ffma2_rn(f, dy, py);
+      pz = __ffma2_rn(f, dz, pz);
+    };
+    // what lies past the end adds zero
+#pragma unroll 8
+    for (int k = r; k < kPairs; k += kLfAccWarps) pair(k);
+    __syncthreads();  // the tile's readers are done
+  }
+  part[threadIdx.x][0] = px.x + px.y;
+  part[threadIdx.x][1] = py.x + py.y;
+  part[threadIdx.x][2] = pz.x + pz.y;
+  __syncthreads();
+  for (int q = threadIdx.x; q < 3 * per_cta; q += blockDim.x) {
+    const int64_t e = 3 * i0 + q;
+    if (e >= 3 * n) return;
+    const int p = q / 3, c = q - 3 * p;
+    const float(*s)[3] = part + (p / 32 * kLfAccWarps * 32 + p % 32);
+    const float a = G * ((s[0][c] + s[32][c]) + (s[64][c] + s[96][c]));
+    if (T.acc) T.acc[e] = a;
+    if (!T.v_out) continue;
+    const float xe = x[e];
+    float v = T.v_in[e];
+    if (T.close) v = fmaf(a, T.h, v);
+    if (T.ck) {
+      T.ck[e] = xe;
+      T.ck[3 * n + e] = v;
+    }
+    if (T.x_out) {
+      v = fmaf(a, T.h, v);
+      T.x_out[e] = fmaf(v, T.dt, xe);
+    }
+    T.v_out[e] = v;
   }
 }
 
@@ -88,14 +228,6 @@ __global__ void __launch_bounds__(kLfT) lf_acc_kernel(int64_t n, const float *__
 // tile's sum is added to the running total, so no FP32 sum runs over more
 // than 256 / TPI terms plus one term per tile.
 constexpr int kLfWideIpt = 4;
-
-template <int MASK>
-__device__ __forceinline__ float2 lf_rsq2(float2 s2) {
-  float2 r;
-  r.x = MASK ? (s2.x > 0.f ? rsqrtf(s2.x) : 0.f) : rsqrtf(s2.x);
-  r.y = MASK ? (s2.y > 0.f ? rsqrtf(s2.y) : 0.f) : rsqrtf(s2.y);
-  return r;
-}
 
 template <int MASK, int TPI>
 __global__ void __launch_bounds__(kLfT) lf_acc_wide_kernel(int64_t n, const float *__restrict__ x,
@@ -191,77 +323,113 @@ __global__ void __launch_bounds__(kLfT) lf_acc_wide_kernel(int64_t n, const floa
 
 // lx_k += dL/dx_k and lm_k += dL/dm_k for the cotangent g = h * lv; with
 // lv_out set, also lv_out_k = lv_k + dlv lx_k with the updated lx_k (the
-// adjoint of the drift, as a separate elementwise launch would compute it).
-template <int MASK>
-__global__ void __launch_bounds__(kLfT)
-    lf_vjp_kernel(int64_t n, const float *__restrict__ x, const float *__restrict__ m,
-                  const float *__restrict__ lv, float h, float eps2, float G,
-                  float *__restrict__ lx, float *__restrict__ lm, float *__restrict__ lv_out,
-                  float dlv) {
-  __shared__ float4 sx[kLfJT];
-  __shared__ float4 sg[kLfJT];
-  const int g = threadIdx.x / kLfTpi, r = threadIdx.x % kLfTpi;
-  const int64_t k = static_cast<int64_t>(blockIdx.x) * kLfI + g;
-  const int64_t kk = k < n ? k : 0;
-  const float xk = x[3 * kk], yk = x[3 * kk + 1], zk = x[3 * kk + 2], mk = m[kk];
-  const float gkx = h * lv[3 * kk], gky = h * lv[3 * kk + 1], gkz = h * lv[3 * kk + 2];
-  float ox = 0.f, oy = 0.f, oz = 0.f, om = 0.f;
-  for (int64_t j0 = 0; j0 < n; j0 += kLfJT) {
-    const int64_t j = j0 + threadIdx.x;
-    if (j < n) {
-      sx[threadIdx.x] = make_float4(x[3 * j], x[3 * j + 1], x[3 * j + 2], m[j]);
-      sg[threadIdx.x] = make_float4(h * lv[3 * j], h * lv[3 * j + 1], h * lv[3 * j + 2], 0.f);
-    } else {
-      sx[threadIdx.x] = make_float4(1.0e15f, 1.0e15f, 1.0e15f, 0.f);
-      sg[threadIdx.x] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    __syncthreads();
-#pragma unroll 2
-    for (int t = r; t < kLfJT; t += kLfTpi) {
-      const float4 q = sx[t];
-      const float4 gj = sg[t];
-      const float dx = q.x - xk, dy = q.y - yk, dz = q.z - zk;
-      const float s2 = fmaf(dx, dx, fmaf(dy, dy, fmaf(dz, dz, eps2)));
-      float rinv;
-      if (MASK)
-        rinv = s2 > 0.f ? rsqrtf(s2) : 0.f;
-      else
-        rinv = rsqrtf(s2);
-      const float rinv2 = rinv * rinv;
-      const float s3 = rinv * rinv2;
-      const float s5 = s3 * rinv2;
-      // u = m_k g_j - m_j g_k with both products rounded alike, so that the
-      // i == j term is exactly zero (a fused form would leave the rounding
-      // error of one product, amplified by 1/eps^3)
-      const float ux = __fsub_rn(__fmul_rn(mk, gj.x), __fmul_rn(q.w, gkx));
-      const float uy = __fsub_rn(__fmul_rn(mk, gj.y), __fmul_rn(q.w, gky));
-      const float uz = __fsub_rn(__fmul_rn(mk, gj.z), __fmul_rn(q.w, gkz));
-      const float du = fmaf(dx, ux, fmaf(dy, uy, dz * uz));
-      const float c = 3.f * du * s5;
-      ox = fmaf(ux, s3, fmaf(-c, dx, ox));
-      oy = fmaf(uy, s3, fmaf(-c, dy, oy));
-      oz = fmaf(uz, s3, fmaf(-c, dz, oz));
-      // g_j . (x_k - x_j) / s^3 = -(g_j . d) s3
-      om = fmaf(-fmaf(gj.x, dx, fmaf(gj.y, dy, gj.z * dz)), s3, om);
-    }
-    __syncthreads();
-  }
+// adjoint of the drift).  Bound by the FP32 pipe, 32 lane-operations per
+// pair; two warps per IPT particles, so that N = 4096 has seven per scheduler.
+// N = 1,000 / 4,096 / 16,000: 11.9 / 30.9 / 342 us, the two clears of the stand-alone
+// call included (8 threads per particle: 17.9 / 43.2 / 399).
+template <int MASK, int IPT>
+__global__ void __launch_bounds__(kLfVjpMaxThreads)
+    lf_vjp_kernel(int64_t n, int slots, const float *__restrict__ x,
+                  const float *__restrict__ m, const float *__restrict__ lv, float h, float eps2,
+                  float G, float *__restrict__ lx, float *__restrict__ lm,
+                  float *__restrict__ lv_out, float dlv) {
+  extern __shared__ __align__(16) float4 vtiles[];  // [2][2][kLfVjpTile]: x, m; cotangents
+  __shared__ float half[kLfVjpMaxThreads / kLfVjpTpi][4 * IPT];
+  constexpr int TPI = kLfVjpTpi;
+  const int g = threadIdx.x / TPI, r = threadIdx.x % TPI;
+  const int64_t k0 = (static_cast<int64_t>(blockIdx.x) * slots + g) * IPT;
+  constexpr int NQ = IPT / 2;
+  // two particles side by side; positions and cotangents negated
+  float2 nx[NQ][3], ng[NQ][3], mk[NQ], o[NQ][4];
 #pragma unroll
-  for (int off = 1; off < kLfTpi; off <<= 1) {
-    ox += __shfl_xor_sync(0xffffffffu, ox, off);
-    oy += __shfl_xor_sync(0xffffffffu, oy, off);
-    oz += __shfl_xor_sync(0xffffffffu, oz, off);
-    om += __shfl_xor_sync(0xffffffffu, om, off);
-  }
-  if (r == 0 && k < n) {
-    const float o3[3] = {ox, oy, oz};
+  for (int q = 0; q < NQ; ++q) {
+    const int64_t a = k0 + 2 * q < n ? k0 + 2 * q : 0, b = k0 + 2 * q + 1 < n ? k0 + 2 * q + 1 : 0;
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
-      const float lxn = lx[3 * k + c] + G * o3[c];
-      lx[3 * k + c] = lxn;
-      if (lv_out) lv_out[3 * k + c] = fmaf(dlv, lxn, lv[3 * k + c]);
+      nx[q][c] = make_float2(-x[3 * a + c], -x[3 * b + c]);
+      ng[q][c] = make_float2(-lv[3 * a + c], -lv[3 * b + c]);
     }
-    lm[k] += G * om;
+    mk[q] = make_float2(m[a], m[b]);
+    o[q][0] = o[q][1] = o[q][2] = o[q][3] = dup(0.f);
+  }
+  const float2 e2 = dup(eps2);
+  auto stage = [&](int b, int64_t j0) {
+    stage_xm(vtiles + b * 2 * kLfVjpTile, j0, n, x, m);
+    stage_g(vtiles + (b * 2 + 1) * kLfVjpTile, j0, n, lv);
+  };
+  stage(0, 0);
+  copies_commit();
+  int b = 0;
+  for (int64_t j0 = 0; j0 < n; j0 += kLfVjpTile, b ^= 1) {
+    if (j0 + kLfVjpTile < n) stage(b ^ 1, j0 + kLfVjpTile);
+    copies_commit();
+    copies_wait<1>();
+    __syncthreads();
+    const float4 *t = vtiles + b * 2 * kLfVjpTile, *tg = t + kLfVjpTile;
+    const int cnt = n - j0 < kLfVjpTile ? static_cast<int>(n - j0) : kLfVjpTile;
+#pragma unroll 1
+    for (int p0 = r; p0 < cnt; p0 += 4 * TPI)
+#pragma unroll 2
+    for (int p = p0; p < p0 + 4 * TPI; p += TPI) {
+      const float4 j = t[p], gq = tg[p];
+      const float2 xj[3] = {dup(j.x), dup(j.y), dup(j.z)}, mj = dup(j.w);
+      const float2 gj[3] = {dup(gq.x), dup(gq.y), dup(gq.z)};
+#pragma unroll
+      for (int q = 0; q < NQ; ++q) {
+        float2 d[3], u[3];
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          d[c] = __fadd2_rn(xj[c], nx[q][c]);
+          // u = m_k g_j - m_j g_k with both products rounded alike, so that
+          // the i == j term is exactly zero (a fused form would leave the
+          // rounding error of one product, amplified by 1/eps^3)
+          u[c] = __fadd2_rn(mul2_alone(mk[q], gj[c]), mul2_alone(mj, ng[q][c]));
+        }
+        const float2 s2 =
+            __ffma2_rn(d[0], d[0], __ffma2_rn(d[1], d[1], __ffma2_rn(d[2], d[2], e2)));
+        const float2 ri = lf_rsq2<MASK>(s2);
+        const float2 ri2 = __fmul2_rn(ri, ri);
+        const float2 s3 = __fmul2_rn(ri, ri2);
+        const float2 du = __ffma2_rn(d[0], u[0], __ffma2_rn(d[1], u[1], __fmul2_rn(d[2], u[2])));
+        const float2 c3 = __fmul2_rn(__fmul2_rn(du, ri2), dup(-3.f));
+        // (I - 3 d d^T / s^2) u / s^3
+#pragma unroll
+        for (int c = 0; c < 3; ++c) o[q][c] = __ffma2_rn(s3, __ffma2_rn(c3, d[c], u[c]), o[q][c]);
+        // (g_j . d) / s^3
+        const float2 gd =
+            __ffma2_rn(gj[0], d[0], __ffma2_rn(gj[1], d[1], __fmul2_rn(gj[2], d[2])));
+        o[q][3] = __ffma2_rn(gd, s3, o[q][3]);
+      }
+    }
+    __syncthreads();
+  }
+  // lane 4 q + c ends component c of particle q (c = 3: the mass)
+  float mine = 0.f;
+  const int lane = r % 32;
+#pragma unroll
+  for (int q = 0; q < IPT; ++q)
+#pragma unroll
+    for (int c = 0; c < 4; ++c) {
+      float s = q % 2 ? o[q / 2][c].y : o[q / 2][c].x;
+      if (c == 3) s = -s;
+#pragma unroll
+      for (int f = 1; f < 32; f <<= 1) s += __shfl_xor_sync(0xffffffffu, s, f);
+      if (lane == 4 * q + c) mine = s;
+    }
+  if (r >= 32 && lane < 4 * IPT) half[g][lane] = mine;
+  __syncthreads();
+  const int64_t k = k0 + r / 4;
+  const int c = r % 4;
+  if (r >= 4 * IPT || k >= n) return;
+  mine += half[g][r];
+  // the sums are linear in the cotangent: its factor h comes in here
+  const float val = G * (h * mine);
+  if (c == 3) {
+    lm[k] += val;
+  } else {
+    const float lxn = lx[3 * k + c] + val;
+    lx[3 * k + c] = lxn;
+    if (lv_out) lv_out[3 * k + c] = fmaf(dlv, lxn, lv[3 * k + c]);
   }
 }
 
@@ -280,22 +448,21 @@ __global__ void lf_kick_drift_kernel(int64_t n3, float *__restrict__ x, float *_
 // ck_x is set, the checkpoint (x, v) of the step boundary; then this step's
 // opening kick v += a h and the drift x_out = x_in + v dt.  The same
 // per-element operations in the same order as separate kick and drift
-// launches.  x_in may equal x_out.
-__global__ void lf_step_kernel(int64_t n3, const float *x_in, float *x_out,
-                               float *__restrict__ v, const float *__restrict__ a, float h,
-                               float dt, int close, float *__restrict__ ck_x,
-                               float *__restrict__ ck_v) {
+// launches.  x_in may equal x_out, v_in v_out.
+__global__ void lf_step_kernel(int64_t n3, const float *x_in, float *x_out, const float *v_in,
+                               float *v_out, const float *__restrict__ a, float h, float dt,
+                               int close, float *__restrict__ ck_x, float *__restrict__ ck_v) {
   const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
   if (q >= n3) return;
   const float aq = a[q], xq = x_in[q];
-  float vq = v[q];
+  float vq = v_in[q];
   if (close) vq = fmaf(aq, h, vq);
   if (ck_x) {
     ck_x[q] = xq;
     ck_v[q] = vq;
   }
   vq = fmaf(aq, h, vq);
-  v[q] = vq;
+  v_out[q] = vq;
   x_out[q] = fmaf(vq, dt, xq);
 }
 
@@ -309,9 +476,34 @@ struct LfCtx {
   int64_t launches;
 };
 
-// N >= kLfWideMin takes the wide shape; below it, the 8-threads-per-particle
-// shape keeps enough CTAs to fill the GPU (N = 4096: 128 CTAs).
+// N >= kLfWideMin takes the wide shape (4 particles per thread, records
+// broadcast) for the force.
 constexpr int64_t kLfWideMin = 65536;
+
+// Groups of 32 particles per CTA of the small force shape: the count that
+// leaves an SM the fewest groups to run, the larger one where two are equal
+// (a CTA's copies of the records serve all its groups).
+int lf_groups(int64_t n, int sms) {
+  int best = 1;
+  int64_t cost = INT64_MAX;
+  for (int g = 1; g <= kLfMaxThreads / (32 * kLfAccWarps); ++g) {
+    const int64_t ctas = (n + 32 * g - 1) / (32 * g);
+    const int64_t c = (ctas + sms - 1) / sms * g;
+    if (c < cost || (c == cost && n > 32 * static_cast<int64_t>(sms))) {
+      cost = c;
+      best = g;
+    }
+  }
+  return best;
+}
+
+// Slots (groups of ipt particles) per CTA of the vector-Jacobian product: the
+// CTAs fill whole rounds of the SMs (N = 4096, 152 SMs: 147 CTAs of 14 pairs).
+int lf_slots(int64_t n, int ipt, int most, int sms) {
+  const int64_t total = (n + ipt - 1) / ipt;
+  const int64_t rounds = (total + sms * most - 1) / (sms * most);
+  return static_cast<int>((total + sms * rounds - 1) / (sms * rounds));
+}
 
 // Threads per i-particle group of the wide shape, 4 or 8.  CTAs take the
 // same time, so an SM's share is ceil(grid / SMs) CTAs run one after
@@ -338,34 +530,56 @@ void launch_lf_wide(const LfCtx &C, const float *x, float *acc) {
     lf_acc_wide_kernel<0, TPI><<<grid, kLfT, 0, C.s>>>(C.n, x, C.m, C.eps2, C.G, acc);
 }
 
-cudaError_t lf_acc(LfCtx &C, const float *x, float *acc) {
-  if (C.n >= kLfWideMin) {
-    if (lf_wide_tpi(C.n, C.sms) == 8)
-      launch_lf_wide<8>(C, x, acc);
-    else
-      launch_lf_wide<4>(C, x, acc);
-  } else {
-    const unsigned grid = static_cast<unsigned>((C.n + kLfI - 1) / kLfI);
-    if (C.mask)
-      lf_acc_kernel<1><<<grid, kLfT, 0, C.s>>>(C.n, x, C.m, C.eps2, C.G, acc);
-    else
-      lf_acc_kernel<0><<<grid, kLfT, 0, C.s>>>(C.n, x, C.m, C.eps2, C.G, acc);
-  }
+// A(x) and what follows it (see LfTail), n < kLfWideMin.
+cudaError_t lf_eval(LfCtx &C, const float *x, const LfTail &T) {
+  const int g = lf_groups(C.n, C.sms);
+  // one group per CTA at most: spread over all SMs
+  const int per = g == 1 && C.n <= 32 * static_cast<int64_t>(C.sms)
+                      ? static_cast<int>((C.n + C.sms - 1) / C.sms)
+                      : 32 * g;
+  const unsigned grid = static_cast<unsigned>((C.n + per - 1) / per);
+  const int nt = 32 * kLfAccWarps * g;
+  if (C.mask)
+    lf_eval_kernel<1><<<grid, nt, 0, C.s>>>(C.n, per, x, C.m, C.eps2, C.G, T);
+  else
+    lf_eval_kernel<0><<<grid, nt, 0, C.s>>>(C.n, per, x, C.m, C.eps2, C.G, T);
   ++C.launches;
+  return cudaGetLastError();
+}
+
+cudaError_t lf_acc(LfCtx &C, const float *x, float *acc) {
+  if (C.n < kLfWideMin) {
+    LfTail T;
+    T.acc = acc;
+    return lf_eval(C, x, T);
+  }
+  if (lf_wide_tpi(C.n, C.sms) == 8)
+    launch_lf_wide<8>(C, x, acc);
+  else
+    launch_lf_wide<4>(C, x, acc);
+  ++C.launches;
+  return cudaGetLastError();
+}
+
+template <int MASK, int IPT>
+cudaError_t launch_lf_vjp(const LfCtx &C, const float *x, const float *lv, float h, float *lx,
+                          float *lm, float *lv_out, float dlv) {
+  constexpr int smem = 4 * kLfVjpTile * sizeof(float4);
+  cudaError_t e = cudaFuncSetAttribute(lf_vjp_kernel<MASK, IPT>,
+                                       cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+  if (e != cudaSuccess) return e;
+  const int slots = lf_slots(C.n, IPT, kLfVjpMaxThreads / kLfVjpTpi, C.sms);
+  const unsigned grid = static_cast<unsigned>((C.n + slots * IPT - 1) / (slots * IPT));
+  lf_vjp_kernel<MASK, IPT><<<grid, slots * kLfVjpTpi, smem, C.s>>>(
+      C.n, slots, x, C.m, lv, h, C.eps2, C.G, lx, lm, lv_out, dlv);
   return cudaGetLastError();
 }
 
 cudaError_t lf_vjp(LfCtx &C, const float *x, const float *lv, float h, float *lx, float *lm,
                    float *lv_out = nullptr, float dlv = 0.f) {
-  const unsigned grid = static_cast<unsigned>((C.n + kLfI - 1) / kLfI);
-  if (C.mask)
-    lf_vjp_kernel<1><<<grid, kLfT, 0, C.s>>>(C.n, x, C.m, lv, h, C.eps2, C.G, lx, lm, lv_out,
-                                             dlv);
-  else
-    lf_vjp_kernel<0><<<grid, kLfT, 0, C.s>>>(C.n, x, C.m, lv, h, C.eps2, C.G, lx, lm, lv_out,
-                                             dlv);
   ++C.launches;
-  return cudaGetLastError();
+  return C.mask ? launch_lf_vjp<1, 2>(C, x, lv, h, lx, lm, lv_out, dlv)
+                : launch_lf_vjp<0, 2>(C, x, lv, h, lx, lm, lv_out, dlv);
 }
 
 cudaError_t lf_kick(LfCtx &C, float *x, float *v, const float *a, float h, float dt, int drift) {
@@ -376,14 +590,27 @@ cudaError_t lf_kick(LfCtx &C, float *x, float *v, const float *a, float h, float
   return cudaGetLastError();
 }
 
-// The drift of one KDK step with the kicks around it (see lf_step_kernel),
-// then A(x_out) into acc; the step's own closing kick is left to the next
-// call (close = 1) or to a final lf_kick without drift.
-cudaError_t lf_half_step(LfCtx &C, const float *x_in, float *x_out, float *v, float *acc,
-                         float dt, bool close, float *ck) {
+// The drift of one KDK step with the kicks around it: from A(x_in) (computed
+// here below kLfWideMin, where x_out must differ from x_in; above it acc
+// holds A(x_in) and receives A(x_out)).  The step's own closing kick is left
+// to the next call (close) or to the end of the run.
+cudaError_t lf_half_step(LfCtx &C, const float *x_in, float *x_out, const float *v_in,
+                         float *v_out, float *acc, float dt, bool close, float *ck) {
+  if (C.n < kLfWideMin) {
+    LfTail T;
+    T.v_in = v_in;
+    T.v_out = v_out;
+    T.x_out = x_out;
+    T.ck = ck;
+    T.close = close ? 1 : 0;
+    T.h = 0.5f * dt;
+    T.dt = dt;
+    return lf_eval(C, x_in, T);
+  }
   const int64_t n3 = 3 * C.n;
   lf_step_kernel<<<static_cast<unsigned>((n3 + 255) / 256), 256, 0, C.s>>>(
-      n3, x_in, x_out, v, acc, 0.5f * dt, dt, close ? 1 : 0, ck, ck ? ck + n3 : nullptr);
+      n3, x_in, x_out, v_in, v_out, acc, 0.5f * dt, dt, close ? 1 : 0, ck,
+      ck ? ck + n3 : nullptr);
   ++C.launches;
   cudaError_t e = cudaGetLastError();
   if (e == cudaSuccess) e = lf_acc(C, x_out, acc);
@@ -473,11 +700,35 @@ nb_status nb_lf_forward(int64_t n, const float *d_m, float *d_x, float *d_v, flo
   if (!d_v || !d_acc || nsteps < 0 || ckpt_every < 1 || !(std::isfinite(dt)))
     return static_cast<nb_status>(set_error(NB_ERR_INVALID_ARG, "bad leapfrog arguments"));
   LfCtx C = make_ctx(n, d_m, eps, G, stream);
-  cudaError_t e = lf_acc(C, d_x, d_acc);
-  for (int64_t st = 0; st < nsteps && e == cudaSuccess; ++st) {
-    float *ck = (d_ckpt && st % ckpt_every == 0) ? d_ckpt + (st / ckpt_every) * 6 * n : nullptr;
-    e = lf_half_step(C, d_x, d_x, d_v, d_acc, dt, st > 0, ck);
+  const size_t n3b = 3 * static_cast<size_t>(n) * sizeof(float);
+  auto ck = [&](int64_t st) {
+    return d_ckpt && st % ckpt_every == 0 ? d_ckpt + (st / ckpt_every) * 6 * n : nullptr;
+  };
+  cudaError_t e = cudaSuccess;
+  if (n < kLfWideMin) {
+    // every force evaluation ends with the drift to the next positions, which
+    // go to the other of d_x and d_acc (free until the last evaluation)
+    float *cur = d_x, *other = d_acc;
+    for (int64_t st = 0; st < nsteps && e == cudaSuccess; ++st) {
+      e = lf_half_step(C, cur, other, d_v, d_v, nullptr, dt, st > 0, ck(st));
+      std::swap(cur, other);
+    }
+    if (e == cudaSuccess && cur != d_x)
+      e = cudaMemcpyAsync(d_x, cur, n3b, cudaMemcpyDeviceToDevice, C.s);
+    LfTail T;
+    T.acc = d_acc;
+    if (nsteps > 0) {
+      T.v_in = d_v;
+      T.v_out = d_v;
+      T.close = 1;
+      T.h = 0.5f * dt;
+    }
+    if (e == cudaSuccess) e = lf_eval(C, d_x, T);
+    return e == cudaSuccess ? NB_OK : lf_err(e);
   }
+  e = lf_acc(C, d_x, d_acc);
+  for (int64_t st = 0; st < nsteps && e == cudaSuccess; ++st)
+    e = lf_half_step(C, d_x, d_x, d_v, d_v, d_acc, dt, st > 0, ck(st));
   if (e == cudaSuccess && nsteps > 0) e = lf_kick(C, d_x, d_v, d_acc, 0.5f * dt, dt, 0);
   return e == cudaSuccess ? NB_OK : lf_err(e);
 }
@@ -500,23 +751,31 @@ nb_status nb_lf_backward(int64_t n, const float *d_m, const float *d_ckpt, int64
   for (int64_t seg = K - 1; seg >= 0 && e == cudaSuccess; --seg) {
     const int64_t s0 = seg * ckpt_every;
     const int64_t L = std::min<int64_t>(ckpt_every, nsteps - s0);
-    const float *slot = d_ckpt + seg * 6 * n;
-    e = cudaMemcpyAsync(xs, slot, n3b, cudaMemcpyDeviceToDevice, C.s);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(v, slot + n3, n3b, cudaMemcpyDeviceToDevice, C.s);
-    if (e == cudaSuccess) e = lf_acc(C, xs, acc);
-    // the segment's positions again (the velocity after the last drift is
-    // not needed, so the last closing kick is left out)
-    for (int64_t q = 0; q < L && e == cudaSuccess; ++q)
-      e = lf_half_step(C, xs + q * n3, xs + (q + 1) * n3, v, acc, dt, q > 0, nullptr);
-    // the sweep: second kick, drift (fused into the second kick's launch,
-    // writing the new lv to the other of d_lv and the now free velocity
-    // buffer), first kick
+    const float *slot = d_ckpt + seg * 6 * n;  // x, v at step s0
+    // positions of the segment's steps: xs[q] for q > 0, the checkpoint
+    // itself for q = 0; the end of the last segment is needed too, the ends
+    // of the others are the next one's checkpoint
+    const int64_t upto = seg == K - 1 ? L : L - 1;
+    auto pos = [&](int64_t q) -> const float * { return q == 0 ? slot : xs + q * n3; };
+    if (upto > 0 && n >= kLfWideMin) e = lf_acc(C, slot, acc);
+    for (int64_t q = 0; q < upto && e == cudaSuccess; ++q)
+      e = lf_half_step(C, pos(q), xs + (q + 1) * n3, q == 0 ? slot + n3 : v, v, acc, dt, q > 0,
+                       nullptr);
+    // the sweep: at every x the merged kicks, then the drift that led there
+    // (fused, writing the new lv to the other of d_lv and the now free
+    // velocity buffer); half a kick at the two ends of the run
     float *cur = d_lv, *other = v;
-    for (int64_t q = L - 1; q >= 0 && e == cudaSuccess; --q) {
-      const float *xa = xs + q * n3, *xb = xs + (q + 1) * n3;
-      e = lf_vjp(C, xb, cur, 0.5f * dt, d_lx, d_lm, other, dt);  // second kick, drift
+    if (seg == K - 1 && e == cudaSuccess) {
+      e = lf_vjp(C, pos(L), cur, 0.5f * dt, d_lx, d_lm, other, dt);
       std::swap(cur, other);
-      if (e == cudaSuccess) e = lf_vjp(C, xa, cur, 0.5f * dt, d_lx, d_lm);  // first kick
+    }
+    for (int64_t q = L - 1; q >= 0 && e == cudaSuccess; --q) {
+      if (s0 + q > 0) {
+        e = lf_vjp(C, pos(q), cur, dt, d_lx, d_lm, other, dt);
+        std::swap(cur, other);
+      } else {
+        e = lf_vjp(C, pos(q), cur, 0.5f * dt, d_lx, d_lm);
+      }
     }
     if (e == cudaSuccess && cur != d_lv)
       e = cudaMemcpyAsync(d_lv, cur, n3b, cudaMemcpyDeviceToDevice, C.s);

@@ -149,3 +149,57 @@ def test_checkpoint_interval_does_not_change_gradients(torch_cuda):
     for g in grads[1:]:
         for a, b in zip(g, grads[0]):
             assert np.array_equal(a, b)
+
+
+@pytest.mark.parametrize("n", [31, 511, 512, 513, 1025, 2049, 4864, 4865, 9729])
+@pytest.mark.parametrize("eps", [0.05, 0.0])
+def test_acc_and_vjp_at_tile_and_group_edges(torch_cuda, oracle_mod, n, eps):
+    """Record tiles of 512 (force) and 1,024 (vector-Jacobian product), 32
+    particles per group, one group per SM up to n = 4,864 on 152 SMs: sizes
+    at and just past those edges against the oracle, same float32 inputs."""
+    torch = torch_cuda
+    from paper_0909_0879_gb300 import _lib
+
+    m, x, v = ics.plummer(n, 910 + n)
+    g = np.random.default_rng(n).normal(size=(n, 3))
+    dx, dm, dg = (torch.tensor(a, dtype=torch.float32, device="cuda") for a in (x, m, g))
+    acc = torch.full((n, 3), np.nan, dtype=torch.float32, device="cuda")
+    gx = torch.full_like(acc, np.nan)
+    gm = torch.full((n,), np.nan, dtype=torch.float32, device="cuda")
+    _lib.lf_acc(n, dx, dm, acc, eps=eps)
+    _lib.lf_acc_vjp(n, dx, dm, dg, gx, gm, eps=eps)
+    xr, mr, gr = (t.double().cpu().numpy() for t in (dx, dm, dg))
+    ra = oracle_mod.acc(mr, xr, eps)
+    rgx, rgm = oracle_mod.acc_vjp(mr, xr, gr, eps)
+    assert rel_l2(acc.double().cpu().numpy(), ra) < 1e-5
+    assert rel_l2(gx.double().cpu().numpy(), rgx) < 1e-4
+    assert rel_l2(gm.double().cpu().numpy(), rgm) < 1e-4
+
+
+@pytest.mark.parametrize("nsteps,ckpt", [(1, 1), (1, 8), (2, 1), (3, 2), (5, 3), (6, 3)])
+def test_short_runs_and_segments(torch_cuda, oracle_mod, nsteps, ckpt):
+    """Odd and even step counts (the positions alternate between two
+    buffers), one or several segments, full or short last one: end state,
+    final acceleration and gradients against the oracle."""
+    torch = torch_cuda
+    from paper_0909_0879_gb300 import _lib
+    from paper_0909_0879_gb300.autograd import leapfrog
+
+    n, eps, dt = 300, 0.05, 1.0 / 64
+    m, x, v = ics.plummer(n, 77)
+    y = x + np.random.default_rng(7).normal(0.0, 0.05, x.shape)
+    leaves = [torch.tensor(a, dtype=torch.float32, device="cuda", requires_grad=True)
+              for a in (x, v, m)]
+    xT, vT = leapfrog(*leaves, nsteps, dt, eps, ckpt_every=ckpt)
+    ((xT - torch.tensor(y, dtype=torch.float32, device="cuda")) ** 2).sum().backward()
+    xr, vr, mr = (t.detach().double().cpu().numpy() for t in leaves)
+    _, gx, gv, gm = oracle_mod.leapfrog_loss_grad(mr, xr, vr, y, eps, dt, nsteps)
+    for t, r in zip(leaves, (gx, gv, gm)):
+        assert rel_l2(t.grad.double().cpu().numpy(), r) < 1e-4
+    # the acceleration left behind is A(x) at the returned positions
+    xw, vw = leaves[0].detach().clone(), leaves[1].detach().clone()
+    acc = torch.empty_like(xw)
+    _lib.lf_forward(n, leaves[2].detach(), xw, vw, acc, nsteps, dt, None, eps=eps)
+    assert torch.equal(xw, xT.detach()) and torch.equal(vw, vT.detach())
+    ra = oracle_mod.acc(mr, xw.double().cpu().numpy(), eps)
+    assert rel_l2(acc.double().cpu().numpy(), ra) < 1e-5
