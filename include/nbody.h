@@ -90,7 +90,12 @@ void nb_destroy(nb_ctx *ctx);
 /* Block scheduling (paper Sec. 2, individual time steps): t_next =
  * min_i (t_i + dt_i); the active list becomes every i with t_i + dt_i ==
  * t_next, in ascending index order (deterministic).  Returns t_next (time
- * units) and the number of active particles; synchronises the stream. */
+ * units) and the number of active particles.  Synchronises the stream, except
+ * in a context with shared steps (block_steps == 0) whose particles are all at
+ * one time and level, as nb_init, the steps of this library and an nb_set_state
+ * with such values leave them: there the answer is known on the host, the
+ * call (and nb_step) waits for nothing, and a device-side error of earlier work
+ * is reported by the next call that does. */
 nb_status nb_next_block(nb_ctx *ctx, double *t_next, int64_t *n_active);
 
 /* Predict every particle to time t (Hermite predictor, FP64):

@@ -82,10 +82,12 @@ bool finite_all(const double *p, int64_t cnt) {
 
 // Particles [b, e) of a state nb_set_state takes: the first particle with
 // a non-finite value (*nonfinite set) or an invalid level or tick, else e.
+// *uniform is cleared when a time or level differs from particle 0's.
 int64_t first_bad_particle(const double *x, const double *v, const double *a,
                            const double *jerk, const int64_t *t_tick, const int32_t *lev,
-                           int64_t b, int64_t e, bool *nonfinite) {
+                           int64_t b, int64_t e, bool *nonfinite, bool *uniform) {
   constexpr int64_t kBlk = 1024;
+  uint64_t differ = 0;
   for (int64_t i0 = b; i0 < e; i0 += kBlk) {
     const int64_t i1 = i0 + kBlk < e ? i0 + kBlk : e;
     const int64_t m = 3 * (i1 - i0);
@@ -100,12 +102,16 @@ int64_t first_bad_particle(const double *x, const double *v, const double *a,
         }
     }
     for (int64_t i = i0; i < i1; ++i)
+      differ |= static_cast<uint64_t>(t_tick[i] ^ t_tick[0]) |
+                static_cast<uint32_t>(lev[i] ^ lev[0]);
+    for (int64_t i = i0; i < i1; ++i)
       if (lev[i] < 0 || lev[i] > kTicksLog2 || t_tick[i] < 0 ||
           (t_tick[i] & ((int64_t(1) << (kTicksLog2 - lev[i])) - 1)) != 0) {
         *nonfinite = false;
         return i;
       }
   }
+  if (differ) *uniform = false;
   return e;
 }
 
@@ -114,22 +120,23 @@ int64_t first_bad_particle(const double *x, const double *v, const double *a,
 // particle in index order, or n.
 int64_t first_bad_particle_par(int64_t n, const double *x, const double *v, const double *a,
                                const double *jerk, const int64_t *t_tick, const int32_t *lev,
-                               bool *nonfinite) {
+                               bool *nonfinite, bool *uniform) {
   const unsigned hw = std::thread::hardware_concurrency();
   int T = hw ? static_cast<int>(hw) : 1;
   if (T > 16) T = 16;
   if (n < (int64_t(1) << 16) || T < 2)
-    return first_bad_particle(x, v, a, jerk, t_tick, lev, 0, n, nonfinite);
+    return first_bad_particle(x, v, a, jerk, t_tick, lev, 0, n, nonfinite, uniform);
   const int64_t chunk = (n + T - 1) / T;
   std::vector<int64_t> bad(T, n);
-  std::vector<char> nf(T, 0);
+  std::vector<char> nf(T, 0), uni(T, 1);
   std::vector<std::thread> th;
   int spawned = 0;
   auto run = [&](int k) {
     const int64_t b = k * chunk, e = b + chunk < n ? b + chunk : n;
     if (b >= e) return;
-    bool f = false;
-    const int64_t r = first_bad_particle(x, v, a, jerk, t_tick, lev, b, e, &f);
+    bool f = false, same = true;
+    const int64_t r = first_bad_particle(x, v, a, jerk, t_tick, lev, b, e, &f, &same);
+    uni[k] = same ? 1 : 0;
     if (r < e) {
       bad[k] = r;
       nf[k] = f ? 1 : 0;
@@ -145,6 +152,8 @@ int64_t first_bad_particle_par(int64_t n, const double *x, const double *v, cons
   }
   for (int k = spawned; k < T; ++k) run(k);
   for (auto &t : th) t.join();
+  for (int k = 0; k < T; ++k)
+    if (!uni[k]) *uniform = false;
   for (int k = 0; k < T; ++k)
     if (bad[k] < n) {
       *nonfinite = nf[k] != 0;
@@ -341,6 +350,13 @@ struct nb_ctx {
   double *lx = nullptr, *lv = nullptr, *la = nullptr, *lm = nullptr;
   int64_t *lperm = nullptr;
   bool fresh = true;             // every particle still at t = 0 from nb_init
+  // shared steps: every particle is at tick u_tick on level u_lev, so the next
+  // block is all of them one step on, known without asking the device;
+  // act_all: the active list on the device holds 0 .. n-1
+  bool uniform = false;
+  int64_t u_tick = 0;
+  int32_t u_lev = 0;
+  bool act_all = false;
   // nb_symplectic moved x and v: the Hermite fields (jerk, times, levels)
   // no longer belong to them until nb_set_state
   bool sym_moved = false;
@@ -579,9 +595,10 @@ nb_status queue_sym(nb_ctx *c, SymArgs &A, double *d_acc, double *d_jerk) {
 }
 
 // Queue one force evaluation of n_i i-particles (d_idx may be null for the
-// identity list) into d_acc / d_jerk.
+// identity list) into d_acc / d_jerk.  With end set, the sums of split
+// i-blocks are left to the block-end kernel, whose arguments it completes.
 nb_status queue_force(nb_ctx *c, const int32_t *d_idx, int64_t n_i, double *d_acc,
-                      double *d_jerk) {
+                      double *d_jerk, EndArgs *end = nullptr) {
   if (n_i == 0) return NB_OK;
   int cap = 0;
   const int v = pick_variant(c, n_i, &cap);
@@ -603,21 +620,22 @@ nb_status queue_force(nb_ctx *c, const int32_t *d_idx, int64_t n_i, double *d_ac
   A.jerk = d_jerk;
   A.part = reinterpret_cast<float2 *>(c->part);
   A.err = c->err;
+  if (end) {
+    end->h_bi = block_i(variant_at(v));
+    end->h_p = grid;
+    end->part = A.part;
+  }
   int nl = 0;
-  NB_CUDA(launch_force(v, A, grid, c->stream, &nl));
+  NB_CUDA(launch_force(v, A, grid, c->stream, &nl, end == nullptr));
   c->launches += nl;
   c->interactions += n_i * c->n;
   return NB_OK;
 }
 
 nb_status queue_predict(nb_ctx *c, int64_t tick) {
-  NB_CUDA(launch_predict(c->n, tick, c->x, c->v, c->a, c->jk, c->m, c->t_tick,
-                         c->cfg.precision, c->jhi, c->jlo, c->jvel, c->stream));
+  NB_CUDA(launch_predict(c->n, c->n_jt, tick, c->x, c->v, c->a, c->jk, c->m, c->t_tick,
+                         c->cfg.precision, c->jhi, c->jlo, c->jvel, c->jrel, c->tinfo, c->stream));
   c->launches += 1;
-  if (c->jrel) {
-    NB_CUDA(launch_tile_info(c->n, c->n_jt, c->jhi, c->jlo, c->jrel, c->tinfo, c->stream));
-    c->launches += 1;
-  }
   c->t_pred = tick;
   return NB_OK;
 }
@@ -835,6 +853,8 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x,
   }
   c->have_block = false;
   c->force_done = false;
+  c->uniform = !cfg->block_steps;
+  c->u_lev = cfg->lev_shared;
   *out = c;
   return NB_OK;
 #undef TRY
@@ -849,7 +869,28 @@ nb_status nb_next_block(nb_ctx *c, double *t_next, int64_t *n_active) {
     return fail(NB_ERR_STATE, "shard: nb_shard_import of the last block's records comes first");
   s = relayout_if_due(c);
   if (s != NB_OK) return s;
+  if (c->uniform) {
+    // nothing to look up and nothing to wait for
+    if (!c->act_all) {
+      NB_CUDA(launch_iota(c->n, c->act, c->stream));
+      c->launches += 1;
+      c->act_all = true;
+    }
+    c->t_block = c->u_tick + (int64_t(1) << (kTicksLog2 - c->u_lev));
+    c->n_act = c->n;
+    c->sh_off_valid = true;
+    c->own_lo = 0;
+    c->own_hi = c->n;
+    c->have_block = true;
+    c->fresh = false;
+    c->force_done = false;
+    c->n_blocks += 1;
+    if (t_next) *t_next = std::ldexp(static_cast<double>(c->t_block), -kTicksLog2);
+    if (n_active) *n_active = c->n_act;
+    return NB_OK;
+  }
   int nl = 0;
+  c->act_all = false;
   NB_CUDA(launch_next_block(c->n, c->t_tick, c->lev, c->act, c->blk, c->scal, c->stream, &nl));
   c->launches += nl;
   if (c->sh.p > 1) {
@@ -891,11 +932,42 @@ nb_status nb_predict(nb_ctx *c, double t) {
 
 namespace {
 
+// Arguments of the block-end kernel that every use shares.
+EndArgs end_args(const nb_ctx *c) {
+  EndArgs E;
+  E.n = c->n;
+  E.n_jt = c->n_jt;
+  E.sym_all = 0;
+  E.nbk = 0;
+  E.part = reinterpret_cast<const float2 *>(c->part);
+  E.G = c->cfg.G;
+  E.a1 = c->a1;
+  E.j1 = c->j1;
+  E.act = c->act;
+  E.x = c->x;
+  E.v = c->v;
+  E.a = c->a;
+  E.jk = c->jk;
+  E.t_tick = c->t_tick;
+  E.lev = c->lev;
+  E.eta = c->cfg.eta;
+  E.lev_min = c->cfg.lev_min;
+  E.lev_max = c->cfg.lev_max;
+  E.block_steps = c->cfg.block_steps;
+  E.n_clamped = c->clamped;
+  E.ctl = c->scal;
+  E.ext = c->ext;
+  E.sp4 = c->sp4;
+  E.sp2 = c->sp2;
+  return E;
+}
+
 // Force of the active list (a shard: its slice of it) into a1, j1.  With
 // rows, the caller reads them: they are then the one-sided kernel's, the
 // same values that an index list gives.  Without, a step of all particles
 // takes the pair-symmetric kernel (no forced shape, table or grid).
-nb_status force_active(nb_ctx *c, int64_t n_idx, bool rows) {
+// With end, the split i-blocks' sums are left to the block-end kernel.
+nb_status force_active(nb_ctx *c, int64_t n_idx, bool rows, EndArgs *end = nullptr) {
   if (!c->have_block) return fail(NB_ERR_STATE, "no active list: call nb_next_block first");
   if (n_idx >= 0 && n_idx != c->n_act)
     return fail(NB_ERR_INVALID_ARG, "n_idx %lld != active count %lld", (long long)n_idx,
@@ -909,7 +981,7 @@ nb_status force_active(nb_ctx *c, int64_t n_idx, bool rows) {
       c->grid_cap == 0 && sym_hermite(c, &A))
     s = queue_sym(c, A, c->a1, c->j1);
   else
-    s = queue_force(c, c->act + lo, cnt, c->a1 + 3 * lo, c->j1 + 3 * lo);
+    s = queue_force(c, c->act + lo, cnt, c->a1 + 3 * lo, c->j1 + 3 * lo, end);
   if (s == NB_OK) c->force_done = true;
   return s;
 }
@@ -1026,6 +1098,7 @@ nb_status nb_correct(nb_ctx *c, double t) {
   c->launches += 1;
   c->force_done = false;
   c->have_block = false;
+  c->u_tick = c->t_block;  // (of use only where every particle was due)
   if (c->sh.p > 1) {
     c->sh_corrected = true;
     c->sh_nact = c->n_act;
@@ -1040,10 +1113,33 @@ nb_status nb_step(nb_ctx *c, double *t_next, int64_t *n_active) {
   if (s != NB_OK) return s;
   s = nb_predict(c, tn);
   if (s != NB_OK) return s;
-  s = nb_force_jerk_dev(c, nullptr, na, nullptr, nullptr);
-  if (s != NB_OK) return s;
-  s = nb_correct(c, tn);
-  if (s != NB_OK) return s;
+  const int64_t short_list = static_cast<int64_t>(kEndThreads / 32) * 2 * c->num_sms;
+  if (c->sh.p > 1 || na > short_list) {
+    s = nb_force_jerk_dev(c, nullptr, na, nullptr, nullptr);
+    if (s != NB_OK) return s;
+    s = nb_correct(c, tn);
+    if (s != NB_OK) return s;
+  } else {
+    // short lists, up to one particle per warp of the block-end kernel: the
+    // fix-up of split i-blocks and the corrector in one launch, the arithmetic
+    // of nb_force_jerk_dev and nb_correct (N = 1024 shared steps: 29 -> 20 us
+    // per step; longer lists are 1 % slower that way)
+    EndArgs E = end_args(c);
+    E.ctl = nullptr;
+    E.sp4 = nullptr;  // rebuilt by nb_run_blocks
+    E.sp2 = nullptr;
+    E.t_next = c->t_block;
+    E.n_act = na;
+    s = force_active(c, na, false, &E);
+    if (s != NB_OK) return s;
+    Range r("nb_correct");
+    const int64_t ctas = (na + kEndThreads / 32 - 1) / (kEndThreads / 32);
+    NB_CUDA(launch_block_end(E, static_cast<int>(ctas), c->stream));
+    c->launches += 1;
+    c->force_done = false;
+    c->have_block = false;
+    c->u_tick = c->t_block;
+  }
   if (t_next) *t_next = tn;
   if (n_active) *n_active = na;
   return NB_OK;
@@ -1116,13 +1212,9 @@ nb_status queue_device_blocks(nb_ctx *c, cudaStream_t s, int64_t *launches) {
   for (int step = 0; step < kGraphSteps; ++step) {
     int nl = 0;
     NB_CUDA(launch_next_block(c->n, c->t_tick, c->lev, c->act, c->blk, c->scal, s, &nl));
-    NB_CUDA(launch_predict(c->n, 0, c->x, c->v, c->a, c->jk, c->m, c->t_tick, prec, c->jhi,
-                           c->jlo, c->jvel, s, c->scal));
+    NB_CUDA(launch_predict(c->n, c->n_jt, 0, c->x, c->v, c->a, c->jk, c->m, c->t_tick, prec,
+                           c->jhi, c->jlo, c->jvel, c->jrel, c->tinfo, s, c->scal));
     ++nl;
-    if (c->jrel) {
-      NB_CUDA(launch_tile_info(c->n, c->n_jt, c->jhi, c->jlo, c->jrel, c->tinfo, s, c->scal));
-      ++nl;
-    }
     for (int k = 0; k < nbk; ++k) {
       const int grid = c->num_sms * ctas_per_sm(b[k].v);
       NB_CUDA(launch_force_dev(b[k].v, device_force_args(c, b[k]), grid, c->n, s, &nl));
@@ -1182,9 +1274,7 @@ nb_status queue_fused_blocks(nb_ctx *c, cudaStream_t s, int64_t *launches) {
     B.lb_wait_limit = 256;
     B.lb_epoch_skew = uint64_t(1) << 24;
   }
-  EndArgs E;
-  E.n = c->n;
-  E.n_jt = c->n_jt;
+  EndArgs E = end_args(c);
   E.sym_all = sym ? 1 : 0;
   E.nbk = nbk;
   for (int k = 0; k < nbk; ++k) {
@@ -1194,26 +1284,6 @@ nb_status queue_fused_blocks(nb_ctx *c, cudaStream_t s, int64_t *launches) {
     E.pmax[k] = c->num_sms * ctas_per_sm(b[k].v);
     E.mu[k] = static_cast<int>(min_units(variant_at(b[k].v).tpi));
   }
-  E.part = reinterpret_cast<const float2 *>(c->part);
-  E.G = c->cfg.G;
-  E.a1 = c->a1;
-  E.j1 = c->j1;
-  E.act = c->act;
-  E.x = c->x;
-  E.v = c->v;
-  E.a = c->a;
-  E.jk = c->jk;
-  E.t_tick = c->t_tick;
-  E.lev = c->lev;
-  E.eta = c->cfg.eta;
-  E.lev_min = c->cfg.lev_min;
-  E.lev_max = c->cfg.lev_max;
-  E.block_steps = c->cfg.block_steps;
-  E.n_clamped = c->clamped;
-  E.ctl = c->scal;
-  E.ext = c->ext;
-  E.sp4 = c->sp4;
-  E.sp2 = c->sp2;
   const int end_grid = c->num_sms * 2;
   // The bucket launches are independent graph branches (fork after
   // block_begin, join before block_end), so the ones outside their range
@@ -1721,6 +1791,10 @@ extern "C" nb_status nb_run_blocks(nb_ctx *c, double t_end, int64_t max_blocks,
   }
   s = ensure_part(c, pb);
   if (s != NB_OK) return s;
+  // until the steps are done and counted the particles' time is not known
+  const bool uniform = c->uniform;
+  c->uniform = false;
+  c->act_all = false;
   if (c->block_mode == 0) {
     // per-level counts and the level-structure check for the fused steps
     NB_CUDA(cudaMemsetAsync(c->scal + kCtlTicket, 0,
@@ -1777,6 +1851,8 @@ extern "C" nb_status nb_run_blocks(nb_ctx *c, double t_end, int64_t max_blocks,
   c->have_block = false;
   c->force_done = false;
   c->t_pred = -1;
+  c->uniform = uniform;
+  if (done > 0) c->u_tick = c->h_scal[kCtlLastT];
   c->last_fused = fused ? 1 : 0;
   if (blocks_done) *blocks_done = done;
   if (t_last) *t_last = std::ldexp(static_cast<double>(c->h_scal[kCtlLastT]), -kTicksLog2);
@@ -1882,8 +1958,8 @@ nb_status nb_set_state(nb_ctx *c, const double *x, const double *v, const double
   const int64_t n = c->n;
   // one pass over the six arrays on the host's cores before any copy, so a
   // rejected state leaves the context's state as it was
-  bool nonfinite = false;
-  const int64_t bad = first_bad_particle_par(n, x, v, a, jerk, t_tick, lev, &nonfinite);
+  bool nonfinite = false, uniform = true;
+  const int64_t bad = first_bad_particle_par(n, x, v, a, jerk, t_tick, lev, &nonfinite, &uniform);
   if (bad < n) {
     if (nonfinite) return fail(NB_ERR_INVALID_ARG, "non-finite state (particle %lld)",
                                (long long)bad);
@@ -1924,6 +2000,9 @@ nb_status nb_set_state(nb_ctx *c, const double *x, const double *v, const double
   c->fresh = false;
   c->sh_corrected = false;
   c->sh_off_valid = false;
+  c->uniform = uniform && !c->cfg.block_steps && c->sh.p == 1;
+  c->u_tick = t_tick[0];
+  c->u_lev = lev[0];
   return sync_ctx(c);
 }
 
@@ -2111,6 +2190,7 @@ nb_status nb_shard_set(nb_ctx *c, int32_t nranks, int32_t rank, const int64_t *b
       return fail(NB_ERR_CUDA, "pinned host buffer for the shard offsets");
     }
   }
+  c->uniform = false;  // slices of the list come from the device
   c->sh.p = nranks;
   c->sh_rank = nranks > 1 ? rank : 0;
   for (int r = 0; r <= kMaxShards; ++r) c->sh.b[r] = 0;

@@ -383,39 +383,44 @@ __device__ __forceinline__ void end_round(const EndArgs &E, int64_t k0, int64_t 
     const unsigned mask = nv >= 10 ? 0x3fffffffu : ((1u << (3 * nv)) - 1u);
     dev::correct_vals3(cq, mask, lane - cq, ci, st, an, jn, t_next, E.x, E.v, E.a, E.jk,
                        E.t_tick, E.lev, E.eta, E.lev_min, E.lev_max, E.block_steps,
-                       E.n_clamped, E.ctl + kCtlLevCnt, &E.ext, E.sp4, E.sp2);
+                       E.n_clamped, E.ctl ? E.ctl + kCtlLevCnt : nullptr, &E.ext, E.sp4, E.sp2);
   }
   __syncthreads();
 }
 
 __global__ void __launch_bounds__(kEndThreads) block_end_kernel(const EndArgs E) {
   __shared__ EndStage sg;
-  const int64_t t_next = E.ctl[kCtlTnext];
-  if (t_next < 0) return;
-  const int64_t n_act = E.ctl[kCtlNact];
-  if (blockIdx.x == 0 && threadIdx.x == 0) {
-    // reductions without a return value: the thread does not wait for a
-    // round trip before its CTA's corrector work
-    atomicAdd(reinterpret_cast<unsigned long long *>(E.ctl + kCtlBlocks), 1ull);
-    atomicAdd(reinterpret_cast<unsigned long long *>(E.ctl + kCtlInter),
-              static_cast<unsigned long long>(n_act * E.n));
-    E.ctl[kCtlLastT] = t_next;
+  int64_t t_next = E.t_next, n_act = E.n_act;
+  int BI = E.h_bi, P = E.h_p;
+  uint64_t U = dev::udiv(static_cast<uint64_t>(n_act + BI - 1), BI) *
+               static_cast<uint64_t>(E.n_jt);
+  if (E.ctl) {
+    t_next = E.ctl[kCtlTnext];
+    if (t_next < 0) return;
+    n_act = E.ctl[kCtlNact];
+    if (blockIdx.x == 0 && threadIdx.x == 0) {
+      // reductions without a return value: the thread does not wait for a
+      // round trip before its CTA's corrector work
+      atomicAdd(reinterpret_cast<unsigned long long *>(E.ctl + kCtlBlocks), 1ull);
+      atomicAdd(reinterpret_cast<unsigned long long *>(E.ctl + kCtlInter),
+                static_cast<unsigned long long>(n_act * E.n));
+      E.ctl[kCtlLastT] = t_next;
+    }
+    int b = -1;
+    for (int q = 0; q < E.nbk; ++q)
+      if (n_act >= E.lo[q] && n_act < E.hi[q]) b = q;
+    const bool whole = b < 0 && E.sym_all && n_act == E.n;
+    if (b < 0 && !whole) return;
+    // the split the force launch of this bucket derived from the same count;
+    // one CTA for everything (no split i-block) where the pair-symmetric
+    // kernel's fix-up has written the sums
+    BI = whole ? E.bi[0] : E.bi[b];
+    U = dev::udiv(static_cast<uint64_t>(n_act + BI - 1), BI) * static_cast<uint64_t>(E.n_jt);
+    const uint64_t mu = static_cast<uint64_t>(whole ? 1 : E.mu[b]);
+    const uint64_t pm = (U + mu - 1) / mu;
+    const int pmax = whole ? 1 : E.pmax[b];
+    P = static_cast<int>(pm < static_cast<uint64_t>(pmax) ? pm : pmax);
   }
-  int b = -1;
-  for (int q = 0; q < E.nbk; ++q)
-    if (n_act >= E.lo[q] && n_act < E.hi[q]) b = q;
-  const bool whole = b < 0 && E.sym_all && n_act == E.n;
-  if (b < 0 && !whole) return;
-  // the split the force launch of this bucket derived from the same count;
-  // one CTA for everything (no split i-block) where the pair-symmetric
-  // kernel's fix-up has written the sums
-  const int BI = whole ? E.bi[0] : E.bi[b];
-  const uint64_t U = dev::udiv(static_cast<uint64_t>(n_act + BI - 1), BI) *
-                     static_cast<uint64_t>(E.n_jt);
-  const uint64_t mu = static_cast<uint64_t>(whole ? 1 : E.mu[b]);
-  const uint64_t pm = (U + mu - 1) / mu;
-  const int pmax = whole ? 1 : E.pmax[b];
-  const int P = static_cast<int>(pm < static_cast<uint64_t>(pmax) ? pm : pmax);
   // short lists: one entry per warp per round (the fix-ups in parallel);
   // long lists: four, so that the corrector warp runs 32 lanes
   if (n_act <= static_cast<int64_t>(kEndWarps) * gridDim.x) {

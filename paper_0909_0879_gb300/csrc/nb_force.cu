@@ -673,7 +673,7 @@ bool has_acc_only(int v) { return kTable[v].acc_fn != nullptr; }
 int acc_shape(int v) { return v == 14 ? 29 : v; }
 
 cudaError_t launch_force(int v, const ForceArgs &A, int grid, cudaStream_t s,
-                         int *launches) {
+                         int *launches, bool with_fixup) {
   const Entry &E = kTable[v];
   const KernelFn fn = A.jerk ? E.fn : E.acc_fn;
   if (!fn) return cudaErrorInvalidValue;
@@ -696,7 +696,7 @@ cudaError_t launch_force(int v, const ForceArgs &A, int grid, cudaStream_t s,
   if (e != cudaSuccess) return e;
   int nl = 1;
   // Split i-blocks exist unless every CTA range is whole i-blocks.
-  if (!(U % static_cast<uint64_t>(grid) == 0 &&
+  if (with_fixup && !(U % static_cast<uint64_t>(grid) == 0 &&
         (U / grid) % static_cast<uint64_t>(A.n_jt) == 0)) {
     const int tb = 256;  // 8 warps, one i-particle each
     const int64_t nb = (A.n_i + 7) / 8;

@@ -18,24 +18,28 @@ namespace {
 
 using dev::kTick;
 
-__global__ void predict_kernel(int64_t n, int64_t t_next, const double *__restrict__ x,
-                               const double *__restrict__ v, const double *__restrict__ a,
-                               const double *__restrict__ jk, const double *__restrict__ m,
-                               const int64_t *__restrict__ t_tick, int prec,
-                               float4 *__restrict__ jhi, float4 *__restrict__ jlo,
-                               float4 *__restrict__ jvel, const int64_t *ctl) {
+// One CTA per tile of kJT records, thread t on record j = tile * kJT + t.
+__global__ void __launch_bounds__(kJT)
+    predict_kernel(int64_t n, int64_t t_next, const double *__restrict__ x,
+                   const double *__restrict__ v, const double *__restrict__ a,
+                   const double *__restrict__ jk, const double *__restrict__ m,
+                   const int64_t *__restrict__ t_tick, int prec, float4 *__restrict__ jhi,
+                   float4 *__restrict__ jlo, float4 *__restrict__ jvel,
+                   float4 *__restrict__ jrel, float4 *__restrict__ tinfo, const int64_t *ctl) {
   if (ctl) {
     t_next = ctl[kCtlTnext];
     if (t_next < 0) return;
   }
-  for (int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x; i < n;
-       i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-    const float dt = static_cast<float>(t_next - t_tick[i]) * static_cast<float>(kTick);
+  const int64_t j = static_cast<int64_t>(blockIdx.x) * kJT + threadIdx.x;
+  const bool real = j < n;
+  float4 h = make_float4(0.f, 0.f, 0.f, 0.f), l = h;
+  if (real) {
+    const float dt = static_cast<float>(t_next - t_tick[j]) * static_cast<float>(kTick);
     float xh[3], xl[3], vp[3];
-    dev::predict_ds(x, v, a, jk, i, dt, xh, xl, vp);
-    float4 lo;
-    dev::store_records_ds(i, xh, xl, vp, m[i], prec, jhi, jlo, jvel, &lo);
+    dev::predict_ds(x, v, a, jk, j, dt, xh, xl, vp);
+    h = dev::store_records_ds(j, xh, xl, vp, m[j], prec, jhi, jlo, jvel, &l);
   }
+  if (jrel) dev::tile_frame(blockIdx.x, j, real, h, l, jrel, tinfo);
 }
 
 // Padding records: zero mass far away, so they add exactly zero to every sum.
@@ -49,17 +53,9 @@ __global__ void pad_kernel(int64_t n, int64_t n_pad, float4 *jhi, float4 *jlo,
   jvel[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// One CTA per tile of kJT records.
-__global__ void __launch_bounds__(kJT)
-    tile_info_kernel(int64_t n, const float4 *__restrict__ jhi, const float4 *__restrict__ jlo,
-                     float4 *__restrict__ jrel, float4 *__restrict__ tinfo,
-                     const int64_t *ctl) {
-  if (ctl && ctl[kCtlTnext] < 0) return;
-  const int64_t j = static_cast<int64_t>(blockIdx.x) * kJT + threadIdx.x;
-  const bool real = j < n;
-  const float4 h = jhi[j];
-  const float4 l = real ? jlo[j] : make_float4(0.f, 0.f, 0.f, 0.f);
-  dev::tile_frame(blockIdx.x, j, real, h, l, jrel, tinfo);
+__global__ void iota_kernel(int64_t n, int32_t *__restrict__ act) {
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+  if (i < n) act[i] = static_cast<int32_t>(i);
 }
 
 __global__ void correct_kernel(int64_t n_act, const int32_t *__restrict__ act, int64_t t_next,
@@ -260,21 +256,18 @@ __global__ void due_scatter_kernel(int64_t n, const int64_t *__restrict__ t_tick
 
 }  // namespace
 
-cudaError_t launch_predict(int64_t n, int64_t t_next, const double *x, const double *v,
-                           const double *a, const double *jk, const double *m,
+cudaError_t launch_predict(int64_t n, int64_t n_jt, int64_t t_next, const double *x,
+                           const double *v, const double *a, const double *jk, const double *m,
                            const int64_t *t_tick, int prec, float4 *jhi, float4 *jlo,
-                           float4 *jvel, cudaStream_t s, const int64_t *ctl) {
-  const int tb = 256;
-  int64_t nb = (n + tb - 1) / tb;
-  if (nb > 65535 * 16) nb = 65535 * 16;
-  predict_kernel<<<static_cast<unsigned>(nb), tb, 0, s>>>(n, t_next, x, v, a, jk, m, t_tick,
-                                                          prec, jhi, jlo, jvel, ctl);
+                           float4 *jvel, float4 *jrel, float4 *tinfo, cudaStream_t s,
+                           const int64_t *ctl) {
+  predict_kernel<<<static_cast<unsigned>(n_jt), kJT, 0, s>>>(
+      n, t_next, x, v, a, jk, m, t_tick, prec, jhi, jlo, jvel, jrel, tinfo, ctl);
   return cudaGetLastError();
 }
 
-cudaError_t launch_tile_info(int64_t n, int64_t n_jt, const float4 *jhi, const float4 *jlo,
-                             float4 *jrel, float4 *tinfo, cudaStream_t s, const int64_t *ctl) {
-  tile_info_kernel<<<static_cast<unsigned>(n_jt), kJT, 0, s>>>(n, jhi, jlo, jrel, tinfo, ctl);
+cudaError_t launch_iota(int64_t n, int32_t *act, cudaStream_t s) {
+  iota_kernel<<<static_cast<unsigned>((n + 255) / 256), 256, 0, s>>>(n, act);
   return cudaGetLastError();
 }
 

@@ -152,8 +152,10 @@ int acc_shape(int v);
 // With A.jerk null the acceleration-only kernel runs (cudaErrorInvalidValue
 // when the variant has none).  Returns the number of kernel launches
 // through *launches.
+// Without with_fixup the split i-blocks' partial sums are left in A.part for
+// the block-end kernel (with the jerk only).
 cudaError_t launch_force(int v, const ForceArgs &A, int grid, cudaStream_t s,
-                         int *launches);
+                         int *launches, bool with_fixup = true);
 // Device-resident form: A.ctl, A.lo, A.hi set; `grid` is the largest
 // persistent grid of the variant and n_max bounds the active count.
 // Without with_fixup the split i-blocks' partial sums are left in A.part
@@ -199,20 +201,19 @@ cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t 
                              int *launches);
 
 // --- Hermite and bookkeeping kernels (nb_hermite.cu) ---
-// With ctl set, t_next is read from ctl[kCtlTnext] (negative: no-op).
-cudaError_t launch_predict(int64_t n, int64_t t_next, const double *x,
+// The j-records of every particle at t_next and, with jrel set, per
+// 256-record tile its bounding box, origin O_t (FP32 box centre), radius R_t
+// and every record's position relative to O_t.  With ctl set, t_next is read
+// from ctl[kCtlTnext] (negative: no-op).
+cudaError_t launch_predict(int64_t n, int64_t n_jt, int64_t t_next, const double *x,
                            const double *v, const double *a, const double *jk,
                            const double *m, const int64_t *t_tick, int prec,
-                           float4 *jhi, float4 *jlo, float4 *jvel,
+                           float4 *jhi, float4 *jlo, float4 *jvel, float4 *jrel, float4 *tinfo,
                            cudaStream_t s, const int64_t *ctl = nullptr);
 cudaError_t launch_pad_records(int64_t n, int64_t n_pad, float4 *jhi,
                                float4 *jlo, float4 *jvel, cudaStream_t s);
-// Per 256-record tile: bounding box, origin O_t (FP32 box centre), radius
-// R_t, and every record's position relative to O_t.  With ctl set, a
-// negative ctl[kCtlTnext] makes it a no-op.
-cudaError_t launch_tile_info(int64_t n, int64_t n_jt, const float4 *jhi,
-                             const float4 *jlo, float4 *jrel, float4 *tinfo,
-                             cudaStream_t s, const int64_t *ctl = nullptr);
+// act[i] = i.
+cudaError_t launch_iota(int64_t n, int32_t *act, cudaStream_t s);
 // With ctl set, n_act and t_next come from ctl (n_act is then a bound).
 cudaError_t launch_correct(int64_t n_act, const int32_t *act, int64_t t_next,
                            double *x, double *v, double *a, double *jk,
@@ -294,6 +295,11 @@ struct EndArgs {
   int bi[3], pmax[3];                // i-block size and persistent grid
   int mu[3];                         // minimum j-tiles per CTA (min_units)
   int sym_all;                       // steps of all n particles: force already whole in a1, j1
+  // Host-driven step (ctl null): its time, active count and, when the force
+  // launch left split i-blocks, that launch's i-block size and CTAs (P = 1:
+  // the force is whole in a1, j1).
+  int64_t t_next = 0, n_act = 0;
+  int h_bi = 1, h_p = 1;
   const float2 *part;                // partial sums of split i-blocks (hi, lo pairs)
   double G;
   double *a1, *j1;

@@ -539,3 +539,39 @@ def test_fused_steps_rebuild_the_predictor_split_after_set_state(nb):
     assert d_a == d_b
     for k in want:
         assert np.array_equal(got[k], want[k]), k
+
+
+@pytest.mark.parametrize("n", [1000, 2432, 2433])
+def test_shared_steps_without_a_look_at_the_schedule(nb, n):
+    """A context with shared steps knows its next block; the same state told
+    apart (one particle on another level, then set back) is scheduled on the
+    device, as block steps are.  nb_step loops over both agree bit for bit with
+    the separate calls, and a resumed state goes on from its own time."""
+    m, x, v = ics.plummer(n, 93, masses=ics.salpeter_masses(n, 93))
+    kw = dict(eps=1e-3, block_steps=False, lev_shared=9)
+    with nb.NBody(m, x, v, **kw) as a, nb.NBody(m, x, v, **kw) as b:
+        for k in range(3):
+            t, na = a.step()
+            assert (t, na) == ((k + 1) * 2.0**-9, n)
+            t, na = b.next_block()
+            assert na == n and np.array_equal(b.active(), np.arange(n))
+            b.predict(t)
+            b.force_jerk_dev(None, na, None, None)
+            b.correct(t)
+        sa, sb = a.get_state(), b.get_state()
+        for k in sa:
+            assert np.array_equal(sa[k], sb[k]), k
+        odd = {k: u.copy() for k, u in sa.items()}
+        odd["lev"][0] = 10
+        odd["lev"][1:] = 9
+        b.set_state(odd)
+        t, na = b.next_block()
+        assert na == 1 and t == 3 * 2.0**-9 + 2.0**-10
+        b.set_state(sa)
+        ta, tb = a.run_blocks(5 * 2.0**-9)[1], b.step()[0]
+        assert ta == 5 * 2.0**-9 and tb == 4 * 2.0**-9
+        b.step()
+        sa, sb = a.get_state(), b.get_state()
+        for k in sa:
+            assert np.array_equal(sa[k], sb[k]), k
+        assert a.step()[0] == 6 * 2.0**-9
