@@ -300,6 +300,8 @@ struct nb_ctx {
   unsigned char *sym_rec = nullptr;
   size_t sym_i_cap = 0, sym_j_cap = 0;
   bool sym_off = false;
+  bool eq_mass = false;  // every mass is m_eq
+  double m_eq = 0.0;
   double *red = nullptr;        // energy scratch
   unsigned char *en_rec = nullptr;  // records of the split-precision energy
   int *err = nullptr;           // device error word
@@ -536,8 +538,8 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
     if (ok && !c->sym_rec) ok = scratch_alloc(reinterpret_cast<void **>(&c->sym_rec), rb);
     if (ok) ok = scratch_alloc(reinterpret_cast<void **>(&ni), ib) &&
                  scratch_alloc(reinterpret_cast<void **>(&nj), jb);
-    if (ok) ok = sym_prepare(prec, mask, true) == cudaSuccess &&
-                 sym_prepare(prec, mask, false) == cudaSuccess;
+    if (ok) ok = sym_prepare(prec, mask, true, c->eq_mass) == cudaSuccess &&
+                 sym_prepare(prec, mask, false, c->eq_mass) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();  // a refused query is not this call's error
       if (ni) cudaFree(ni);
@@ -569,6 +571,8 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
   A->n = c->n;
   A->eps2 = eps2_f32(c->cfg.eps);
   A->G = c->cfg.G;
+  A->eq = c->eq_mass ? 1 : 0;
+  A->m_eq = static_cast<float>(c->m_eq);
   A->recs = c->sym_rec;
   A->ipart = c->sym_i;
   A->jpart = c->sym_j;
@@ -738,6 +742,8 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x,
   if (!c) return fail(NB_ERR_OOM, "host memory for the context");
   c->cfg = *cfg;
   c->n = n;
+  c->m_eq = m[0];
+  c->eq_mass = std::all_of(m, m + n, [&](double q) { return q == m[0]; });
   c->n_jt = (n + kJT - 1) / kJT;
   c->n_pad = c->n_jt * kJT;
   c->stream = static_cast<cudaStream_t>(cfg->stream);

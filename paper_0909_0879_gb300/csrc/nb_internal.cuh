@@ -181,6 +181,8 @@ struct SymArgs {
   float eps2;
   double G;
   double *acc, *jerk;    // (n, 3); jerk null: acceleration only
+  int eq = 0;            // every mass is m_eq (as the records hold it)
+  float m_eq = 0.f;
   unsigned char *recs;   // the records in pairs (scratch)
   float2 *ipart, *jpart; // partial sums (hi, lo pairs; scratch)
   int *err;
@@ -196,7 +198,7 @@ size_t sym_record_bytes(int64_t n_jt, int prec);
 size_t sym_ipart_bytes(const SymSplit &S, bool jrk);
 size_t sym_jpart_bytes(const SymSplit &S, bool jrk);
 // Shared-memory attribute of the kernel; before its first launch or capture.
-cudaError_t sym_prepare(int prec, int mask, bool jrk);
+cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq);
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
                              int *launches);
 

@@ -38,6 +38,9 @@
 //    the fix-up adds a particle's i-side and j-side partial sums in an order
 //    fixed by the split: results are deterministic.  The scratch holds
 //    about n / 2 records per CTA (split-precision pairs: 3.9 GB at N = 1M).
+//  * One mass for all particles (EQ) leaves one product m / s^3 for both sides:
+//    32 lane-operations instead of 34, N = 1,048,576 King 622 -> 588 ms per
+//    step.
 //  * Own-block tiles take the same loop and drop the j-side sums.
 //  * Sums: near tiles fold the acceleration every 32 terms on both sides, far
 //    tiles every 64 (i) and 32 IPT (j), the jerk every 128; no FP32 sum is
@@ -129,6 +132,11 @@ __host__ __device__ constexpr uint32_t rec_bytes(int prec) {
   return rec_vel(prec) + kPlane4 + kPlane2;
 }
 
+// Coordinate of a record that is no particle (and, with the other sign, of a
+// lane): its squared distance to anything overflows to infinity, whose
+// reciprocal root is 0, so it adds exactly zero whatever mass it is taken with.
+constexpr float kNowhere = 2.0e19f;
+
 // One CTA per tile, one thread per pair.
 template <int PREC>
 __global__ void __launch_bounds__(kPairs) sym_records_kernel(const SymArgs A) {
@@ -136,8 +144,11 @@ __global__ void __launch_bounds__(kPairs) sym_records_kernel(const SymArgs A) {
   const int k = threadIdx.x;
   const size_t j = static_cast<size_t>(blockIdx.x) * kJT + 2 * k;
   unsigned char *t = A.recs + static_cast<size_t>(blockIdx.x) * rec_bytes(PREC);
+  const float4 none = make_float4(kNowhere, kNowhere, kNowhere, 0.f);
   auto put = [&](const float4 *src, uint32_t at, bool four) {
-    const float4 p = src[j], q = src[j + 1];
+    const int64_t i = static_cast<int64_t>(j);
+    const float4 p = four && i >= A.n ? none : src[j];
+    const float4 q = four && i + 1 >= A.n ? none : src[j + 1];
     reinterpret_cast<float4 *>(t + at)[k] = make_float4(p.x, q.x, p.y, q.y);
     if (four)
       reinterpret_cast<float4 *>(t + at + kPlane4)[k] = make_float4(p.z, q.z, p.w, q.w);
@@ -152,7 +163,7 @@ __global__ void __launch_bounds__(kPairs) sym_records_kernel(const SymArgs A) {
   if (A.jerk) put(A.jvel, rec_vel(PREC), false);
 }
 
-template <int PREC, int MASK, int JRK, int IPT, int NT, int ST, int SACC>
+template <int PREC, int MASK, int JRK, int EQ, int IPT, int NT, int ST, int SACC>
 struct SymShape {
   static constexpr int NW = NT / 32;
   static constexpr int NROW = (PREC ? 6 : 3) + (JRK ? 3 : 0);  // acc hi (lo), jerk
@@ -162,10 +173,10 @@ struct SymShape {
   static constexpr size_t kSmem = kAccOff + (SACC ? 12 * IPT * NT * sizeof(float) : 0);
 };
 
-template <int PREC, int MASK, int JRK, int IPT, int NT, int ST, int SACC>
+template <int PREC, int MASK, int JRK, int EQ, int IPT, int NT, int ST, int SACC>
 __global__ void __launch_bounds__(NT, 256 / NT)
     sym_force_kernel(const SymArgs A) {
-  using SH = SymShape<PREC, MASK, JRK, IPT, NT, ST, SACC>;
+  using SH = SymShape<PREC, MASK, JRK, EQ, IPT, NT, ST, SACC>;
   using V = float2;  // two records j
   using O = VOps<V>;
   constexpr int BI = NT * IPT;
@@ -252,7 +263,7 @@ __global__ void __launch_bounds__(NT, 256 / NT)
   while (u < u1) {
     const uint32_t seg = min(sym_row_len(S, row) - off, u1 - u);
     // i-particle data, negated so that every difference is an addition;
-    // lanes past n carry no mass
+    // lanes past n stand opposite the records past n
     float nxh[IPT][3], nxl[IPT][3], nvi[IPT][3], mi[IPT];
 #pragma unroll
     for (int q = 0; q < IPT; ++q) {
@@ -261,12 +272,16 @@ __global__ void __launch_bounds__(NT, 256 / NT)
       const float4 h = A.jhi[i];
       const float4 w = JRK ? A.jvel[i] : make_float4(0.f, 0.f, 0.f, 0.f);
       const float4 l = PREC ? A.jlo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-      nxh[q][0] = -h.x; nxh[q][1] = -h.y; nxh[q][2] = -h.z;
+      if (k < A.n) {
+        nxh[q][0] = -h.x; nxh[q][1] = -h.y; nxh[q][2] = -h.z;
+      } else {
+        nxh[q][0] = nxh[q][1] = nxh[q][2] = kNowhere;
+      }
       nxl[q][0] = -l.x; nxl[q][1] = -l.y; nxl[q][2] = -l.z;
       nvi[q][0] = -w.x; nvi[q][1] = -w.y; nvi[q][2] = -w.z;
       mi[q] = k < A.n ? h.w : 0.f;
     }
-    const V veps2 = O::bc(A.eps2);
+    const V veps2 = O::bc(A.eps2), meq = O::bc(A.m_eq);
     float bc_i[3] = {0.f, 0.f, 0.f}, bh_i[3] = {0.f, 0.f, 0.f};
     if (PREC) {
       // bounding box of the i-block (far test), as in the one-sided kernel
@@ -415,8 +430,8 @@ __global__ void __launch_bounds__(NT, 256 / NT)
                 const V y2 = O::mul(y, y);
                 // (m y) y^2, not m y^3: y^3 alone leaves the FP32 range for
                 // separations the product still covers
-                const V fi = O::mul(O::mul(mj, y), y2);     // on i from j
-                const V fj = O::mul(O::mul(wi[q], y), y2);  // on j from i
+                const V fi = O::mul(O::mul(EQ ? meq : mj, y), y2);        // on i from j
+                const V fj = EQ ? fi : O::mul(O::mul(wi[q], y), y2);      // on j from i
                 pa[q][0] = O::fma(fi, dx, pa[q][0]);
                 pa[q][1] = O::fma(fi, dy, pa[q][1]);
                 pa[q][2] = O::fma(fi, dz, pa[q][2]);
@@ -618,19 +633,23 @@ struct SymEntry {
   size_t smem;
 };
 
-template <int PREC, int MASK, int JRK, int IPT, int NT, int ST, int SACC>
+template <int PREC, int MASK, int JRK, int EQ, int IPT, int NT, int ST, int SACC>
 SymEntry sym_entry() {
-  return {&sym_force_kernel<PREC, MASK, JRK, IPT, NT, ST, SACC>, IPT, NT,
-          SymShape<PREC, MASK, JRK, IPT, NT, ST, SACC>::kSmem};
+  return {&sym_force_kernel<PREC, MASK, JRK, EQ, IPT, NT, ST, SACC>, IPT, NT,
+          SymShape<PREC, MASK, JRK, EQ, IPT, NT, ST, SACC>::kSmem};
 }
 
-const SymEntry &sym_pick(int prec, int mask, int jrk) {
-  static const SymEntry kE[2][2][2] = {
-      {{sym_entry<0, 0, 0, 4, 256, 3, 0>(), sym_entry<0, 0, 1, 4, 256, 3, 0>()},
-       {sym_entry<0, 1, 0, 4, 256, 3, 0>(), sym_entry<0, 1, 1, 4, 256, 3, 0>()}},
-      {{sym_entry<1, 0, 0, 4, 256, 3, 0>(), sym_entry<1, 0, 1, 4, 256, 2, 1>()},
-       {sym_entry<1, 1, 0, 4, 256, 3, 0>(), sym_entry<1, 1, 1, 4, 256, 2, 1>()}}};
-  return kE[prec ? 1 : 0][mask ? 1 : 0][jrk ? 1 : 0];
+template <int MASK, int EQ>
+const SymEntry &sym_shape(int prec, int jrk) {
+  static const SymEntry kE[2][2] = {
+      {sym_entry<0, MASK, 0, EQ, 4, 256, 3, 0>(), sym_entry<0, MASK, 1, EQ, 4, 256, 3, 0>()},
+      {sym_entry<1, MASK, 0, EQ, 4, 256, 3, 0>(), sym_entry<1, MASK, 1, EQ, 4, 256, 2, 1>()}};
+  return kE[prec ? 1 : 0][jrk ? 1 : 0];
+}
+
+const SymEntry &sym_pick(int prec, int mask, int jrk, bool eq) {
+  if (mask) return eq ? sym_shape<1, 1>(prec, jrk) : sym_shape<1, 0>(prec, jrk);
+  return eq ? sym_shape<0, 1>(prec, jrk) : sym_shape<0, 0>(prec, jrk);
 }
 
 }  // namespace
@@ -675,12 +694,12 @@ size_t sym_record_bytes(int64_t n_jt, int prec) {
 }
 
 int sym_block_i(int prec, int mask, bool jrk) {
-  const SymEntry &E = sym_pick(prec, mask, jrk);
+  const SymEntry &E = sym_pick(prec, mask, jrk, false);
   return E.ipt * E.nt;
 }
 
-cudaError_t sym_prepare(int prec, int mask, bool jrk) {
-  const SymEntry &E = sym_pick(prec, mask, jrk);
+cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq) {
+  const SymEntry &E = sym_pick(prec, mask, jrk, eq);
   return cudaFuncSetAttribute(E.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(E.smem));
 }
@@ -688,7 +707,7 @@ cudaError_t sym_prepare(int prec, int mask, bool jrk) {
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
                              int *launches) {
   const bool jrk = A.jerk != nullptr;
-  const SymEntry &E = sym_pick(prec, mask, jrk);
+  const SymEntry &E = sym_pick(prec, mask, jrk, A.eq != 0);
   const unsigned tiles = static_cast<unsigned>(A.n_jt);
   if (prec)
     sym_records_kernel<1><<<tiles, kPairs, 0, s>>>(A);

@@ -28,8 +28,8 @@ def nb():
     return _lib
 
 
-def _system(nb, n, sort, seed=31):
-    m, x, v = ics.plummer(n, seed, masses=ics.salpeter_masses(n, seed))
+def _system(nb, n, sort, seed=31, equal=False):
+    m, x, v = ics.plummer(n, seed, masses=None if equal else ics.salpeter_masses(n, seed))
     if sort:
         p = nb.spatial_order(x, 256)
         m, x, v = m[p], x[p], v[p]
@@ -43,8 +43,11 @@ def _system(nb, n, sort, seed=31):
 @pytest.mark.parametrize("prec", ["ds", "fp32"])
 @pytest.mark.parametrize("eps", [1e-3, 0.0])
 @pytest.mark.parametrize("sort", [False, True])
-def test_matches_oracle_and_one_sided(nb, oracle_mod, n, prec, eps, sort):
-    m, x, v = _system(nb, n, sort)
+@pytest.mark.parametrize("equal", [False, True])
+def test_matches_oracle_and_one_sided(nb, oracle_mod, n, prec, eps, sort, equal):
+    """(equal: one mass for all takes a shorter pair loop where no record or
+    lane past n is met)"""
+    m, x, v = _system(nb, n, sort, equal=equal)
     with nb.NBody(m, x, v, eps=eps, precision=prec, block_steps=False, lev_shared=10) as s:
         got = s.get_state(want=("a", "jerk"))
     with nb.NBody(m, x, v, eps=eps, precision=prec) as s:
