@@ -1360,20 +1360,9 @@ struct SymArrays {
   const double *m;
 };
 
-// Acceleration of every particle into S.a: the pair-symmetric kernel, or
-// the acceleration-only kernel of the built-in shape for n (or its
-// acceleration-only counterpart).
-nb_status queue_acc_all(nb_ctx *c, const SymArrays &S, cudaStream_t s, int64_t *launches,
-                        bool stepping) {
-  SymArgs SA;
-  if (stepping && sym_ready(c, false, &SA)) {
-    SA.acc = S.a;
-    SA.jerk = nullptr;
-    int nl = 0;
-    NB_CUDA(launch_sym_force(c->cfg.precision, eps_masks(c->cfg.eps), SA, s, &nl));
-    *launches += nl;
-    return NB_OK;
-  }
+// Acceleration of every particle into S.a by the acceleration-only kernel of
+// the built-in shape for n (or its acceleration-only counterpart).
+nb_status queue_acc_all(nb_ctx *c, const SymArrays &S, cudaStream_t s, int64_t *launches) {
   const int v = acc_shape(choose_variant(c->cfg.precision, eps_masks(c->cfg.eps), c->n,
                                          c->n_jt, c->num_sms));
   if (!has_acc_only(v)) return fail(NB_ERR_STATE, "force shape %d has no acceleration-only kernel", v);
@@ -1401,28 +1390,47 @@ nb_status queue_acc_all(nb_ctx *c, const SymArrays &S, cudaStream_t s, int64_t *
   return NB_OK;
 }
 
-nb_status queue_kick_drift(nb_ctx *c, const SymArrays &S, cudaStream_t s, double h, double d,
-                           bool rec, int64_t *launches) {
-  NB_CUDA(launch_kick_drift(c->n, c->n_jt, h, d, rec, c->ext, S.a, S.v, S.x, S.m,
-                            c->cfg.precision, c->jhi, c->jlo, c->jvel, c->jrel, c->tinfo, s));
+// With P set (the pair-symmetric kernel's arguments for these arrays) its
+// records are written too, and a already carries the external field.
+nb_status queue_kick_drift(nb_ctx *c, const SymArrays &S, const SymArgs *P, cudaStream_t s,
+                           double h, double d, bool rec, int64_t *launches) {
+  NB_CUDA(launch_kick_drift(c->n, c->n_jt, h, d, rec, P ? ExtField() : c->ext, S.a, S.v, S.x,
+                            S.m, c->cfg.precision, c->jhi, c->jlo, c->jvel, c->jrel, c->tinfo,
+                            P ? P->recs : nullptr, s));
   *launches += 1;
   return NB_OK;
 }
 
-// One step: the stages' kick-drift + force with the kicks between two
-// drifts merged, then the closing half kick.
-nb_status queue_symplectic_step(nb_ctx *c, const SymArrays &A, cudaStream_t s, const double *w,
-                                int S, double dt, int64_t *launches) {
-  for (int k = 0; k < S; ++k) {
-    const double h = 0.5 * dt * ((k > 0 ? w[k - 1] : 0.0) + w[k]);
-    nb_status st = queue_kick_drift(c, A, s, h, w[k] * dt, true, launches);
-    if (st == NB_OK) st = queue_acc_all(c, A, s, launches, true);
-    if (st != NB_OK) return st;
-  }
-  return queue_kick_drift(c, A, s, 0.5 * dt * w[S - 1], 0.0, false, launches);
+// a = A(x) from records that queue_kick_drift left, then v += kick a.
+nb_status queue_acc_sym(nb_ctx *c, const SymArgs &P, cudaStream_t s, double kick,
+                        int64_t *launches) {
+  SymArgs A = P;
+  A.kick = kick;
+  int nl = 0;
+  NB_CUDA(launch_sym_force(c->cfg.precision, eps_masks(c->cfg.eps), A, s, &nl, false));
+  *launches += nl;
+  return NB_OK;
 }
 
-nb_status capture_symplectic(nb_ctx *c, const SymArrays &A, const double *w, int S, double dt) {
+// One step: the stages' kick-drift + force with the kicks between two
+// drifts merged, then the closing half kick (with the pair-symmetric kernel
+// in the last stage's fix-up: three launches per stage and no other).
+nb_status queue_symplectic_step(nb_ctx *c, const SymArrays &A, const SymArgs *P, cudaStream_t s,
+                                const double *w, int S, double dt, int64_t *launches) {
+  const double close = 0.5 * dt * w[S - 1];
+  for (int k = 0; k < S; ++k) {
+    const double h = 0.5 * dt * ((k > 0 ? w[k - 1] : 0.0) + w[k]);
+    nb_status st = queue_kick_drift(c, A, P, s, h, w[k] * dt, true, launches);
+    if (st == NB_OK)
+      st = P ? queue_acc_sym(c, *P, s, k == S - 1 ? close : 0.0, launches)
+             : queue_acc_all(c, A, s, launches);
+    if (st != NB_OK) return st;
+  }
+  return P ? NB_OK : queue_kick_drift(c, A, P, s, close, 0.0, false, launches);
+}
+
+nb_status capture_symplectic(nb_ctx *c, const SymArrays &A, const SymArgs *P, const double *w,
+                             int S, double dt) {
   if (c->sym_graph) {
     cudaGraphExecDestroy(c->sym_graph);
     c->sym_graph = nullptr;
@@ -1433,7 +1441,7 @@ nb_status capture_symplectic(nb_ctx *c, const SymArrays &A, const double *w, int
   int64_t nl = 0;
   cudaError_t e = cudaStreamBeginCapture(cs, cudaStreamCaptureModeThreadLocal);
   nb_status qs = NB_ERR_CUDA;
-  if (e == cudaSuccess) qs = queue_symplectic_step(c, A, cs, w, S, dt, &nl);
+  if (e == cudaSuccess) qs = queue_symplectic_step(c, A, P, cs, w, S, dt, &nl);
   cudaError_t e2 = cudaStreamEndCapture(cs, &g);
   cudaStreamDestroy(cs);
   if (qs != NB_OK && qs != NB_ERR_CUDA) {
@@ -1714,9 +1722,19 @@ extern "C" nb_status nb_symplectic(nb_ctx *c, int32_t order, double dt, int64_t 
   // the acceleration at the current positions, then nsteps replays of one
   // step's graph
   int64_t nl = 0;
-  s = queue_kick_drift(c, A, c->stream, 0.0, 0.0, true, &nl);
   // with nsteps = 0 the call only refreshes A(x), with the sums nb_init makes
-  if (s == NB_OK) s = queue_acc_all(c, A, c->stream, &nl, nsteps > 0);
+  SymArgs SA;
+  const SymArgs *P = nsteps > 0 && sym_ready(c, false, &SA) ? &SA : nullptr;
+  if (P) {
+    SA.acc = A.a;
+    SA.jerk = nullptr;
+    SA.ext = c->ext;
+    SA.x = A.x;
+    SA.v = A.v;
+  }
+  s = queue_kick_drift(c, A, P, c->stream, 0.0, 0.0, true, &nl);
+  if (s == NB_OK)
+    s = P ? queue_acc_sym(c, *P, c->stream, 0.0, &nl) : queue_acc_all(c, A, c->stream, &nl);
   if (s != NB_OK) return s;
   c->launches += nl;
   c->interactions += c->n * c->n;
@@ -1728,7 +1746,7 @@ extern "C" nb_status nb_symplectic(nb_ctx *c, int32_t order, double dt, int64_t 
   if (nsteps > 0) {
     if (!c->sym_graph || c->sym_order != order || c->sym_dt != dt ||
         c->sym_graph_part != c->part || c->sym_graph_stale || c->sym_graph_x != A.x) {
-      s = capture_symplectic(c, A, w, S, dt);
+      s = capture_symplectic(c, A, P, w, S, dt);
       if (s != NB_OK) return s;
       c->sym_order = order;
       c->sym_dt = dt;
@@ -1741,7 +1759,7 @@ extern "C" nb_status nb_symplectic(nb_ctx *c, int32_t order, double dt, int64_t 
     c->interactions += nsteps * S * c->n * c->n;
   }
   // the acceleration left in the state is the total one at the final x
-  if (c->ext.on) {
+  if (c->ext.on && !P) {
     NB_CUDA(launch_ext_add(c->n, c->ext, A.x, A.a, c->stream));
     c->launches += 1;
   }

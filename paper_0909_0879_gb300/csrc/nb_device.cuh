@@ -137,15 +137,55 @@ __device__ __forceinline__ float4 store_records(int64_t i, const double xp[3],
   return h;
 }
 
+// Records of the pair-symmetric kernel (nb_symforce.cu): a tile is 128 pairs
+// of records, the two values of a component side by side, so that a packed
+// instruction takes two records with one register pair and no moves.  Planes
+// (bytes from the tile's start): position (x0 x1 y0 y1), (z0 z1 m0 m1); split
+// precision also the low words (x y), (z) and the tile-relative position like
+// the first two; velocity (x y), (z) last, so that the acceleration kernel
+// copies less.
+constexpr int kPairs = kJT / 2;
+constexpr uint32_t kPlane4 = kPairs * 16, kPlane2 = kPairs * 8;
+__host__ __device__ constexpr uint32_t rec_lo() { return 2 * kPlane4; }
+__host__ __device__ constexpr uint32_t rec_rel() { return rec_lo() + kPlane4 + kPlane2; }
+__host__ __device__ constexpr uint32_t rec_vel(int prec) {
+  return prec ? rec_rel() + 2 * kPlane4 : 2 * kPlane4;
+}
+__host__ __device__ constexpr uint32_t rec_bytes(int prec) {
+  return rec_vel(prec) + kPlane4 + kPlane2;
+}
+
+// Coordinate of a record that is no particle (and, with the other sign, of a
+// lane): its squared distance to anything overflows to infinity, whose
+// reciprocal root is 0, so it adds exactly zero whatever mass it is taken with.
+constexpr float kNowhere = 2.0e19f;
+
+// Record t of a tile into the four- or three-value planes at byte `at`.
+__device__ __forceinline__ void put_rec4(unsigned char *tile, uint32_t at, int t, float4 p) {
+  float *f = reinterpret_cast<float *>(tile + at) + 4 * (t >> 1) + (t & 1);
+  f[0] = p.x;
+  f[2] = p.y;
+  f = reinterpret_cast<float *>(tile + at + kPlane4) + 4 * (t >> 1) + (t & 1);
+  f[0] = p.z;
+  f[2] = p.w;
+}
+__device__ __forceinline__ void put_rec3(unsigned char *tile, uint32_t at, int t, float4 p) {
+  float *f = reinterpret_cast<float *>(tile + at) + 4 * (t >> 1) + (t & 1);
+  f[0] = p.x;
+  f[2] = p.y;
+  reinterpret_cast<float *>(tile + at + kPlane4)[t] = p.z;
+}
+
 // Frame of one tile of kJT records (called by all kJT threads of a CTA,
 // thread t holding record j = tile * kJT + t): the bounding box of the
 // high words, its FP32 centre O_t, half-widths and radius R_t into
 // tinfo[2 tile], tinfo[2 tile + 1], and every record's position relative
 // to O_t into jrel.  The half-widths cover the box about O_t, the low
 // words (below half an ulp of the high word) and the rounding of O_t.
-__device__ __forceinline__ void tile_frame(int64_t tile, int64_t j, bool real, float4 h,
-                                           float4 l, float4 *__restrict__ jrel,
-                                           float4 *__restrict__ tinfo) {
+// Returns the record's relative position.
+__device__ __forceinline__ float4 tile_frame(int64_t tile, int64_t j, bool real, float4 h,
+                                             float4 l, float4 *__restrict__ jrel,
+                                             float4 *__restrict__ tinfo) {
   __shared__ float smn[3][kJT / 32], smx[3][kJT / 32];
   __shared__ float4 s_o;
   const int tid = threadIdx.x, lane = tid & 31, wid = tid >> 5;
@@ -187,12 +227,13 @@ __device__ __forceinline__ void tile_frame(int64_t tile, int64_t j, bool real, f
     s_o = make_float4(o[0], o[1], o[2], 0.f);
   }
   __syncthreads();
+  float4 rel = make_float4(1.0e15f, 1.0e15f, 1.0e15f, 0.f);
   if (real) {
     const float4 o = s_o;
-    jrel[j] = make_float4((h.x - o.x) + l.x, (h.y - o.y) + l.y, (h.z - o.z) + l.z, h.w);
-  } else {
-    jrel[j] = make_float4(1.0e15f, 1.0e15f, 1.0e15f, 0.f);
+    rel = make_float4((h.x - o.x) + l.x, (h.y - o.y) + l.y, (h.z - o.z) + l.z, h.w);
   }
+  jrel[j] = rel;
+  return rel;
 }
 
 // Error-free addition of x into the unevaluated sum hi + lo (two-sum).

@@ -189,6 +189,12 @@ struct SymArgs {
   SymSplit split;
   // Device-resident mode: a launch does nothing unless ctl[kCtlNact] == n.
   const int64_t *ctl = nullptr;
+  // Symplectic steps: with ext on, acc also carries the field at x; with kick
+  // set, v += kick acc follows.
+  ExtField ext;
+  const double *x = nullptr;
+  double *v = nullptr;
+  double kick = 0.0;
 };
 // i-particles per block of the kernel for this precision / masking / output.
 int sym_block_i(int prec, int mask, bool jrk);
@@ -199,8 +205,9 @@ size_t sym_ipart_bytes(const SymSplit &S, bool jrk);
 size_t sym_jpart_bytes(const SymSplit &S, bool jrk);
 // Shared-memory attribute of the kernel; before its first launch or capture.
 cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq);
+// with_records false: recs already hold the positions (launch_kick_drift).
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
-                             int *launches);
+                             int *launches, bool with_records = true);
 
 // --- Hermite and bookkeeping kernels (nb_hermite.cu) ---
 // The j-records of every particle at t_next and, with jrel set, per
@@ -351,11 +358,13 @@ cudaError_t launch_shard_import(int64_t n_act, int64_t lo, int64_t hi, const int
 int symplectic_stages(int order, double *w);
 // v += h (a + a_ext(x)), x += d v for every particle (a factor of 0 skips
 // its update; a_ext only when E.on); with rec set also the j-records and,
-// when jrel is set, the tile frames.
+// when jrel is set, the tile frames, and, when recs is set, the records of
+// the pair-symmetric kernel.
 cudaError_t launch_kick_drift(int64_t n, int64_t n_jt, double h, double d, bool rec,
                               const ExtField &E, const double *a, double *v, double *x,
                               const double *m, int prec, float4 *jhi, float4 *jlo,
-                              float4 *jvel, float4 *jrel, float4 *tinfo, cudaStream_t s);
+                              float4 *jvel, float4 *jrel, float4 *tinfo, unsigned char *recs,
+                              cudaStream_t s);
 // Rows of w doubles: dst[k] = src[perm[k]], or with scatter dst[perm[k]] =
 // src[k].
 cudaError_t launch_permute(int64_t n, const int64_t *perm, const double *src, double *dst,

@@ -73,6 +73,14 @@ namespace {
 using dev::DsAcc;
 using dev::ds_add;
 using dev::VOps;
+using dev::kNowhere;
+using dev::kPairs;
+using dev::kPlane2;
+using dev::kPlane4;
+using dev::rec_bytes;
+using dev::rec_lo;
+using dev::rec_rel;
+using dev::rec_vel;
 
 // Row of unit u and the unit's offset in it: tile offset `off` of row ib is
 // tile off % TB of the block at ring distance off / TB.
@@ -114,28 +122,6 @@ __host__ __device__ __forceinline__ uint32_t sym_tile(const SymSplit &S, uint32_
   if (b >= S.nb) b -= S.nb;
   return b * S.tb + (off - d * S.tb);
 }
-
-// Record layout of a tile: 128 pairs of records, the two values of a
-// component side by side, so that a packed instruction takes two records
-// with one register pair and no moves.  Planes (bytes from the tile's
-// start): position (x0 x1 y0 y1), (z0 z1 m0 m1); split precision also the
-// low words (x y), (z) and the tile-relative position like the first two;
-// velocity (x y), (z) last, so that the acceleration kernel copies less.
-constexpr int kPairs = kJT / 2;
-constexpr uint32_t kPlane4 = kPairs * 16, kPlane2 = kPairs * 8;
-__host__ __device__ constexpr uint32_t rec_lo() { return 2 * kPlane4; }
-__host__ __device__ constexpr uint32_t rec_rel() { return rec_lo() + kPlane4 + kPlane2; }
-__host__ __device__ constexpr uint32_t rec_vel(int prec) {
-  return prec ? rec_rel() + 2 * kPlane4 : 2 * kPlane4;
-}
-__host__ __device__ constexpr uint32_t rec_bytes(int prec) {
-  return rec_vel(prec) + kPlane4 + kPlane2;
-}
-
-// Coordinate of a record that is no particle (and, with the other sign, of a
-// lane): its squared distance to anything overflows to infinity, whose
-// reciprocal root is 0, so it adds exactly zero whatever mass it is taken with.
-constexpr float kNowhere = 2.0e19f;
 
 // One CTA per tile, one thread per pair.
 template <int PREC>
@@ -564,66 +550,110 @@ __global__ void __launch_bounds__(NT, 256 / NT)
 }
 
 // Sums of every particle: its i-side partial sums (ascending CTAs), then
-// the j-side ones by ring distance, in split precision; one CTA per tile,
-// one thread per particle.
+// the j-side ones by ring distance, in split precision; then, for a symplectic
+// step, the external field at x and the closing kick v += kick a.
+//
+// Bound: latency of the chain of loads and additions (about nb / 2 links)
+// and, with the field, the FP64 pipe.  One thread per (particle, component)
+// and 32 particles per CTA: six or three short chains instead of one long
+// one, and the field's particles spread over all SMs.  The partial sums'
+// places (divisions) are worked out once per CTA, into a list of those that
+// exist.  N = 20,011, acceleration, with the field: 20 us + 18 us per kick
+// for the field with a thread per particle and 256 particles per CTA -> 17.8 us
+// with everything in it; N = 100,003, jerk, FP32: 52 us.
+constexpr int kFixP = 32, kFixList = 192;
+
 template <int NC>
-__global__ void __launch_bounds__(kJT) sym_fixup_kernel(const SymArgs A) {
+__global__ void __launch_bounds__(kFixP *NC) sym_fixup_kernel(const SymArgs A) {
   if (A.ctl && A.ctl[kCtlNact] != A.n) return;
+  __shared__ uint32_t s_raw[kFixList], s_src[kFixList], s_n;
+  __shared__ double s_a[3][kFixP];
+  constexpr uint32_t kNone = 0xffffffffu;
   const SymSplit S = A.split;
-  const uint32_t jt = blockIdx.x, t = threadIdx.x;
+  const uint32_t tid = threadIdx.x, c = tid / kFixP, pl = tid - c * kFixP, lane = tid & 31;
+  const uint32_t jt = blockIdx.x / (kJT / kFixP);
+  const uint32_t t = (blockIdx.x - jt * (kJT / kFixP)) * kFixP + pl;
   const uint32_t BI = S.tb * kJT;
   const uint32_t row = jt / S.tb, jo = jt - row * S.tb;
-  float h[NC], l[NC];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) h[c] = l[c] = 0.f;
-  {
-    const uint32_t us = sym_row_start(S, row), ue = us + sym_row_len(S, row) - 1;
-    const uint32_t p1 = sym_owner(S, ue);
-    for (uint32_t p = sym_owner(S, us); p <= p1; ++p) {
-      uint32_t o;
-      const uint32_t fr = sym_row(S, sym_begin(S, p), &o);
-      const float2 *src = A.ipart + (static_cast<size_t>(p) * S.irows + (row - fr)) * NC * BI +
-                          jo * kJT + t;
-#pragma unroll
-      for (int c = 0; c < NC; ++c) {
-        const float2 w = src[c * BI];
-        dev::ds_add_pair(h[c], l[c], w.x, w.y, h[c], l[c]);
+
+  // adds base[place(k) * stride] for k = 0 .. count - 1, without the kNone ones
+  auto sum = [&](uint32_t count, auto place, const float2 *base, size_t stride, float &h,
+                 float &l) {
+    for (uint32_t b = 0; b < count; b += kFixList) {
+      const uint32_t m = min(count - b, static_cast<uint32_t>(kFixList));
+      __syncthreads();
+      for (uint32_t k = tid; k < m; k += kFixP * NC) s_raw[k] = place(b + k);
+      __syncthreads();
+      if (tid < 32) {
+        uint32_t cnt = 0;
+        for (uint32_t k0 = 0; k0 < m; k0 += 32) {
+          const uint32_t v = k0 + lane < m ? s_raw[k0 + lane] : kNone;
+          const uint32_t mk = __ballot_sync(0xffffffffu, v != kNone);
+          if (v != kNone) s_src[cnt + __popc(mk & ((1u << lane) - 1))] = v;
+          cnt += __popc(mk);
+        }
+        if (lane == 0) s_n = cnt;
+      }
+      __syncthreads();
+      const uint32_t cnt = s_n;
+#pragma unroll 8
+      for (uint32_t k = 0; k < cnt; ++k) {
+        const float2 w = base[s_src[k] * stride];
+        dev::ds_add_pair(h, l, w.x, w.y, h, l);
       }
     }
-  }
-  float gh[NC], gl[NC];
-#pragma unroll
-  for (int c = 0; c < NC; ++c) gh[c] = gl[c] = 0.f;
-  uint32_t last = 0xffffffffu;
-#pragma unroll 4
-  for (uint32_t d = 1; d <= S.nb / 2; ++d) {
+  };
+
+  float h = 0.f, l = 0.f, gh = 0.f, gl = 0.f;
+  const uint32_t us = sym_row_start(S, row), ue = us + sym_row_len(S, row) - 1;
+  const uint32_t p0 = sym_owner(S, us);
+  sum(sym_owner(S, ue) - p0 + 1,
+      [&](uint32_t k) {
+        uint32_t o;
+        return (p0 + k) * S.irows + (row - sym_row(S, sym_begin(S, p0 + k), &o));
+      },
+      A.ipart + static_cast<size_t>(c) * BI + jo * kJT + t, static_cast<size_t>(NC) * BI, h, l);
+  // owner of this tile as seen from the row at ring distance d (kNone: not
+  // that row's)
+  auto owner = [&](uint32_t d) {
     const uint32_t r = row >= d ? row - d : row + S.nb - d;
     const uint32_t o = d * S.tb + jo;
-    if (o >= sym_row_len(S, r)) continue;
-    const uint32_t p = sym_owner(S, sym_row_start(S, r) + o);
-    if (p == last) continue;  // one slot for all rows of a CTA
-    last = p;
-    uint32_t fo;
-    const uint32_t fr = sym_row(S, sym_begin(S, p), &fo);
-    const uint32_t sb = fr * S.tb;
-    const uint32_t sl = jt + (jt < sb ? S.nb * S.tb : 0) - sb;
-    const float2 *src = A.jpart + (static_cast<size_t>(p) * S.jslots + sl) * NC * kJT + t;
-#pragma unroll
-    for (int c = 0; c < NC; ++c) {
-      const float2 w = src[c * kJT];
-      dev::ds_add_pair(gh[c], gl[c], w.x, w.y, gh[c], gl[c]);
-    }
-  }
+    return o >= sym_row_len(S, r) ? kNone : sym_owner(S, sym_row_start(S, r) + o);
+  };
+  sum(S.nb / 2,
+      [&](uint32_t k) {
+        const uint32_t p = owner(k + 1);
+        // one slot for all rows of a CTA
+        if (p == kNone || (k > 0 && p == owner(k))) return kNone;
+        uint32_t fo;
+        const uint32_t sb = sym_row(S, sym_begin(S, p), &fo) * S.tb;
+        return p * S.jslots + (jt + (jt < sb ? S.nb * S.tb : 0) - sb);
+      },
+      A.jpart + static_cast<size_t>(c) * kJT + t, static_cast<size_t>(NC) * kJT, gh, gl);
+
   const int64_t i = static_cast<int64_t>(jt) * kJT + t;
-  if (i >= A.n) return;
+  const bool real = i < A.n;
+  dev::ds_add_pair(h, l, -gh, -gl, h, l);
+  double val = dev::ds_to_double(h, l, A.G);
+  if (A.ext.on) {
+    if (c < 3) s_a[c][pl] = val;
+    __syncthreads();
+    if (c == 0 && real) {
+      const double xv[3] = {A.x[3 * i], A.x[3 * i + 1], A.x[3 * i + 2]};
+      double at[3] = {s_a[0][pl], s_a[1][pl], s_a[2][pl]};
+      dev::ext_field(A.ext, xv, nullptr, at, nullptr, nullptr);
 #pragma unroll
-  for (int c = 0; c < NC; ++c) {
-    dev::ds_add_pair(h[c], l[c], -gh[c], -gl[c], h[c], l[c]);
-    const double val = dev::ds_to_double(h[c], l[c], A.G);
-    if (c < 3)
-      A.acc[3 * i + c] = val;
-    else
-      A.jerk[3 * i + c - 3] = val;
+      for (int q = 0; q < 3; ++q) s_a[q][pl] = at[q];
+    }
+    __syncthreads();
+    if (c < 3) val = s_a[c][pl];
+  }
+  if (!real) return;
+  if (c < 3) {
+    A.acc[3 * i + c] = val;
+    if (A.kick != 0.0) A.v[3 * i + c] = fma(A.kick, val, A.v[3 * i + c]);
+  } else {
+    A.jerk[3 * i + c - 3] = val;
   }
 }
 
@@ -705,22 +735,26 @@ cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq) {
 }
 
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
-                             int *launches) {
+                             int *launches, bool with_records) {
   const bool jrk = A.jerk != nullptr;
   const SymEntry &E = sym_pick(prec, mask, jrk, A.eq != 0);
   const unsigned tiles = static_cast<unsigned>(A.n_jt);
-  if (prec)
-    sym_records_kernel<1><<<tiles, kPairs, 0, s>>>(A);
-  else
-    sym_records_kernel<0><<<tiles, kPairs, 0, s>>>(A);
+  if (with_records) {
+    if (prec)
+      sym_records_kernel<1><<<tiles, kPairs, 0, s>>>(A);
+    else
+      sym_records_kernel<0><<<tiles, kPairs, 0, s>>>(A);
+    if (launches) *launches += 1;
+  }
   E.fn<<<A.split.ctas, E.nt, E.smem, s>>>(A);
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;
+  const unsigned ctas = tiles * (kJT / kFixP);
   if (jrk)
-    sym_fixup_kernel<6><<<tiles, kJT, 0, s>>>(A);
+    sym_fixup_kernel<6><<<ctas, 6 * kFixP, 0, s>>>(A);
   else
-    sym_fixup_kernel<3><<<tiles, kJT, 0, s>>>(A);
-  if (launches) *launches += 3;
+    sym_fixup_kernel<3><<<ctas, 3 * kFixP, 0, s>>>(A);
+  if (launches) *launches += 2;
   return cudaGetLastError();
 }
 

@@ -30,14 +30,16 @@ constexpr double kY6W3 = 0.784513610477557263820;
 // v += h (a + a_ext(x)) and x += d v in FP64 (each skipped when its factor
 // is 0; a_ext only with the field on), then, with rec set, the particle's
 // j-records and (split precision) the tile's frame for the far-field test
-// of the force kernel.
+// of the force kernel; with recs set also the pair-symmetric kernel's records
+// (a launch of its own for them took 2.7 us at N = 20,011).
 __global__ void __launch_bounds__(kJT)
     kick_drift_kernel(int64_t n, double h, double d, int rec, const ExtField E,
                       const double *__restrict__ a, double *__restrict__ v,
                       double *__restrict__ x,
                       const double *__restrict__ m, int prec, float4 *__restrict__ jhi,
                       float4 *__restrict__ jlo, float4 *__restrict__ jvel,
-                      float4 *__restrict__ jrel, float4 *__restrict__ tinfo) {
+                      float4 *__restrict__ jrel, float4 *__restrict__ tinfo,
+                      unsigned char *__restrict__ recs) {
   const int64_t j = static_cast<int64_t>(blockIdx.x) * kJT + threadIdx.x;
   const bool real = j < n;
   float4 hr = make_float4(0.f, 0.f, 0.f, 0.f), lr = hr;
@@ -68,7 +70,18 @@ __global__ void __launch_bounds__(kJT)
   } else if (rec) {
     hr = jhi[j];  // padding record (zero mass, far away)
   }
-  if (rec && jrel) dev::tile_frame(blockIdx.x, j, real, hr, lr, jrel, tinfo);
+  float4 rel = hr;
+  if (rec && jrel) rel = dev::tile_frame(blockIdx.x, j, real, hr, lr, jrel, tinfo);
+  if (rec && recs) {
+    const int t = threadIdx.x;
+    const float4 none = make_float4(dev::kNowhere, dev::kNowhere, dev::kNowhere, 0.f);
+    unsigned char *tile = recs + static_cast<size_t>(blockIdx.x) * dev::rec_bytes(prec);
+    dev::put_rec4(tile, 0, t, real ? hr : none);
+    if (prec) {
+      dev::put_rec3(tile, dev::rec_lo(), t, lr);
+      dev::put_rec4(tile, dev::rec_rel(), t, real ? rel : none);
+    }
+  }
 }
 
 __global__ void ext_add_kernel(int64_t n, const ExtField E, const double *__restrict__ x,
@@ -120,10 +133,11 @@ int symplectic_stages(int order, double *w) {
 cudaError_t launch_kick_drift(int64_t n, int64_t n_jt, double h, double d, bool rec,
                               const ExtField &E, const double *a, double *v, double *x,
                               const double *m, int prec, float4 *jhi, float4 *jlo,
-                              float4 *jvel, float4 *jrel, float4 *tinfo, cudaStream_t s) {
+                              float4 *jvel, float4 *jrel, float4 *tinfo, unsigned char *recs,
+                              cudaStream_t s) {
   if (n_jt <= 0) return cudaSuccess;
   kick_drift_kernel<<<static_cast<unsigned>(n_jt), kJT, 0, s>>>(
-      n, h, d, rec ? 1 : 0, E, a, v, x, m, prec, jhi, jlo, jvel, jrel, tinfo);
+      n, h, d, rec ? 1 : 0, E, a, v, x, m, prec, jhi, jlo, jvel, jrel, tinfo, recs);
   return cudaGetLastError();
 }
 

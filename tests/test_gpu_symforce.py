@@ -123,3 +123,38 @@ def test_one_sided_where_rows_or_shapes_are_asked_for_and_without_scratch(nb):
             assert np.isfinite(s.get_state(want=("x",))["x"]).all()
     finally:
         del os.environ["NB_TEST_MAX_BYTES"]
+
+
+@pytest.mark.parametrize("n", [MIN_N + 1, 17 * 1024 + 300])
+@pytest.mark.parametrize("order", [2, 6])
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+@pytest.mark.parametrize("field", [False, True])
+def test_symplectic_steps_match_one_sided(nb, n, order, prec, field):
+    """Records written by the kick-drift and field and closing kick in the
+    fix-up: two steps against the one-sided path, which keeps them in
+    launches of their own (no room for the pair-symmetric scratch).  The pair
+    sums differ by at most 2 TOL of the largest pair acceleration, and a
+    velocity by the sum of its kicks (|h| adds up to at most 6 dt per step)."""
+    m, x, v = _system(nb, n, False)
+    m, x = m * 0.00431, x * 0.01 + np.array([8.5, 0.0, 0.0])
+    v = v * 0.65 + np.array([0.0, 22.0, 0.0])
+    dt, res = 2.0**-12, {}
+    for side in ("pairs", "one"):
+        if side == "one":
+            os.environ["NB_TEST_MAX_BYTES"] = str(32 << 20)
+        try:
+            with nb.NBody(m, x, v, eps=1e-4, precision=prec) as s:
+                pair = np.abs(s.get_state(want=("a",))["a"]).max()
+                if field:
+                    s.set_external({})
+                s.set_symplectic_layout("as_given")
+                s.symplectic(order, dt, 2)
+                res[side] = s.get_state(want=("x", "v", "a"))
+        finally:
+            os.environ.pop("NB_TEST_MAX_BYTES", None)
+    da = 2 * TOL[prec][0] * pair
+    dv = 2 * 6 * dt * da
+    for k, bar in (("a", 2 * da), ("v", dv), ("x", 2 * 6 * dt * dv + 1e-15 * 9)):
+        err = np.abs(res["pairs"][k] - res["one"][k]).max()
+        assert err <= bar, (k, err, bar)
+    assert not np.array_equal(res["pairs"]["a"], res["one"]["a"])  # two routes
