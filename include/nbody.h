@@ -460,7 +460,9 @@ int64_t nb_batched_launch_count(const nb_batch *b);
  * symplectic scheme, kick-drift-kick form) in FP32, with the adjoint of the
  * force sum.  All pointers are caller-owned device arrays (float32):
  * x, v (n,3) row-major, m (n).  Work is queued on `stream` (NULL = default
- * stream); nothing is allocated.  Errors: NB_ERR_INVALID_ARG for n outside
+ * stream); nothing is allocated.  The force of nb_lf_forward_lent and
+ * nb_lf_backward_lent evaluates each pair of particles once where the caller
+ * lends scratch for it.  Errors: NB_ERR_INVALID_ARG for n outside
  * [1, 2^30], eps < 0, G <= 0, a NULL pointer or a bad step count;
  * NB_ERR_CUDA for a failed launch.
  * ---------------------------------------------------------------------- */
@@ -483,6 +485,10 @@ nb_status nb_lf_acc_vjp(int64_t n, const float *d_x, const float *d_m,
 int64_t nb_lf_ckpt_floats(int64_t n, int64_t nsteps, int32_t ckpt_every);
 int64_t nb_lf_work_floats(int64_t n, int32_t ckpt_every);
 
+/* Bytes of scratch with which the current device's *_lent calls below take
+ * the pair-symmetric force; 0 when n is too small (or too large) for it. */
+int64_t nb_lf_scratch_bytes(int64_t n);
+
 /* nsteps KDK steps of dt in place on d_x, d_v (d_acc (n,3) receives the
  * final acceleration).  If d_ckpt is not NULL, (x, v) at every step that is
  * a multiple of ckpt_every is stored in it (nb_lf_ckpt_floats floats). */
@@ -490,6 +496,17 @@ nb_status nb_lf_forward(int64_t n, const float *d_m, float *d_x, float *d_v,
                         float *d_acc, int64_t nsteps, float dt, float eps,
                         float G, int32_t ckpt_every, float *d_ckpt,
                         void *stream);
+
+/* nb_lf_forward with scratch on loan (device memory on a 256-byte boundary,
+ * in use until the call's work on `stream` is done): with at least
+ * nb_lf_scratch_bytes(n) bytes of it the forces are the pair-symmetric ones,
+ * equal to the others' up to FP32 rounding; with less, or NULL, the same as
+ * nb_lf_forward. */
+nb_status nb_lf_forward_lent(int64_t n, const float *d_m, float *d_x,
+                             float *d_v, float *d_acc, int64_t nsteps,
+                             float dt, float eps, float G, int32_t ckpt_every,
+                             float *d_ckpt, void *d_scratch,
+                             int64_t scratch_bytes, void *stream);
 
 /* Reverse pass of nb_lf_forward from its checkpoints: on entry d_lx, d_lv
  * hold dL/dx(T), dL/dv(T); on exit dL/dx(0), dL/dv(0), and d_lm (n) holds
@@ -499,6 +516,16 @@ nb_status nb_lf_backward(int64_t n, const float *d_m, const float *d_ckpt,
                          int64_t nsteps, float dt, float eps, float G,
                          int32_t ckpt_every, float *d_lx, float *d_lv,
                          float *d_lm, float *d_work, void *stream);
+
+/* nb_lf_backward with scratch on loan for re-running the segments, as
+ * nb_lf_forward_lent (lend it to both or to neither: the re-run then repeats
+ * the forward pass bit for bit). */
+nb_status nb_lf_backward_lent(int64_t n, const float *d_m,
+                              const float *d_ckpt, int64_t nsteps, float dt,
+                              float eps, float G, int32_t ckpt_every,
+                              float *d_lx, float *d_lv, float *d_lm,
+                              float *d_work, void *d_scratch,
+                              int64_t scratch_bytes, void *stream);
 
 /* ------------------------------------------------------------------------
  * i-split shards (the paper's two-GPU version of its code, Sec. 4, splits

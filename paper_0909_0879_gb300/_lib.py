@@ -119,6 +119,11 @@ SIGNATURES = [
                                 C.c_float, _i32, _vp, _vp]),
     ("nb_lf_backward", C.c_int, [_i64, _vp, _vp, _i64, C.c_float, C.c_float, C.c_float, _i32,
                                  _vp, _vp, _vp, _vp, _vp]),
+    ("nb_lf_scratch_bytes", _i64, [_i64]),
+    ("nb_lf_forward_lent", C.c_int, [_i64, _vp, _vp, _vp, _vp, _i64, C.c_float, C.c_float,
+                                     C.c_float, _i32, _vp, _vp, _i64, _vp]),
+    ("nb_lf_backward_lent", C.c_int, [_i64, _vp, _vp, _i64, C.c_float, C.c_float, C.c_float,
+                                      _i32, _vp, _vp, _vp, _vp, _vp, _i64, _vp]),
     ("nb_shard_set", C.c_int, [_vp, _i32, _i32, _vp]),
     ("nb_shard_offsets", C.c_int, [_vp, _vp]),
     ("nb_shard_export", C.c_int, [_vp, _vp, _P(_i64)]),
@@ -645,15 +650,26 @@ def lf_work_floats(n, ckpt_every) -> int:
     return int(load().nb_lf_work_floats(int(n), int(ckpt_every)))
 
 
+def lf_scratch_bytes(n) -> int:
+    return int(load().nb_lf_scratch_bytes(int(n)))
+
+
+def _lent(scratch):
+    return (None, 0) if scratch is None else (_ptr(scratch), scratch.numel())
+
+
 def lf_forward(n, d_m, d_x, d_v, d_acc, nsteps, dt, d_ckpt, *, eps, G=1.0, ckpt_every=8,
-               stream=None):
-    _check(load().nb_lf_forward(int(n), _ptr(d_m), _ptr(d_x), _ptr(d_v), _ptr(d_acc),
-                                int(nsteps), float(dt), float(eps), float(G), int(ckpt_every),
-                                _ptr(d_ckpt), _stream_ptr(stream)))
+               stream=None, scratch=None):
+    """``scratch``: a uint8 tensor of lf_scratch_bytes(n) bytes for the pair-symmetric force."""
+    _check(load().nb_lf_forward_lent(int(n), _ptr(d_m), _ptr(d_x), _ptr(d_v), _ptr(d_acc),
+                                     int(nsteps), float(dt), float(eps), float(G),
+                                     int(ckpt_every), _ptr(d_ckpt), *_lent(scratch),
+                                     _stream_ptr(stream)))
 
 
 def lf_backward(n, d_m, d_ckpt, nsteps, dt, d_lx, d_lv, d_lm, d_work, *, eps, G=1.0,
-                ckpt_every=8, stream=None):
-    _check(load().nb_lf_backward(int(n), _ptr(d_m), _ptr(d_ckpt), int(nsteps), float(dt),
-                                 float(eps), float(G), int(ckpt_every), _ptr(d_lx), _ptr(d_lv),
-                                 _ptr(d_lm), _ptr(d_work), _stream_ptr(stream)))
+                ckpt_every=8, stream=None, scratch=None):
+    _check(load().nb_lf_backward_lent(int(n), _ptr(d_m), _ptr(d_ckpt), int(nsteps), float(dt),
+                                      float(eps), float(G), int(ckpt_every), _ptr(d_lx),
+                                      _ptr(d_lv), _ptr(d_lm), _ptr(d_work), *_lent(scratch),
+                                      _stream_ptr(stream)))

@@ -14,6 +14,18 @@ import torch
 from . import _lib
 
 
+def _scratch(n, device):
+    """Memory for the pair-symmetric force, or None (small n, or no room: the
+    one-sided force needs none)."""
+    size = _lib.lf_scratch_bytes(n)
+    if size == 0:
+        return None
+    try:
+        return torch.empty(size, dtype=torch.uint8, device=device)
+    except torch.OutOfMemoryError:
+        return None
+
+
 class LeapfrogFunction(torch.autograd.Function):
     @staticmethod
     def forward(ctx, x0, v0, m, nsteps: int, dt: float, eps: float, G: float, ckpt_every: int):
@@ -29,7 +41,7 @@ class LeapfrogFunction(torch.autograd.Function):
         ckpt = torch.empty(_lib.lf_ckpt_floats(n, nsteps, ckpt_every), dtype=torch.float32,
                            device=x.device)
         _lib.lf_forward(n, mm, x, v, acc, nsteps, dt, ckpt, eps=eps, G=G, ckpt_every=ckpt_every,
-                        stream=stream)
+                        stream=stream, scratch=_scratch(n, x.device))
         ctx.save_for_backward(mm, ckpt)
         ctx.cfg = (n, nsteps, dt, eps, G, ckpt_every)
         return x, v
@@ -46,7 +58,8 @@ class LeapfrogFunction(torch.autograd.Function):
         lm = torch.empty(n, dtype=torch.float32, device=dev)
         work = torch.empty(_lib.lf_work_floats(n, ckpt_every), dtype=torch.float32, device=dev)
         _lib.lf_backward(n, mm, ckpt, nsteps, dt, lx, lv, lm, work, eps=eps, G=G,
-                         ckpt_every=ckpt_every, stream=torch.cuda.current_stream(dev))
+                         ckpt_every=ckpt_every, stream=torch.cuda.current_stream(dev),
+                         scratch=_scratch(n, dev))
         return lx, lv, lm, None, None, None, None, None
 
 

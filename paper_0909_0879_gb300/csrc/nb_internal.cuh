@@ -195,6 +195,9 @@ struct SymArgs {
   const double *x = nullptr;
   double *v = nullptr;
   double kick = 0.0;
+  // The acceleration in FP32 in place of acc; NaN should the force kernel have
+  // reported an error in *err.
+  float *acc_f = nullptr;
 };
 // i-particles per block of the kernel for this precision / masking / output.
 int sym_block_i(int prec, int mask, bool jrk);

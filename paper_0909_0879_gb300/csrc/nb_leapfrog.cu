@@ -22,7 +22,7 @@
 // steps; the reverse pass re-runs each segment from its checkpoint, keeping
 // the segment's positions, then walks it backwards.
 #include "../../include/nbody.h"
-#include "nb_internal.cuh"
+#include "nb_device.cuh"
 
 #include <algorithm>
 #include <cmath>
@@ -466,6 +466,43 @@ __global__ void lf_step_kernel(int64_t n3, const float *x_in, float *x_out, cons
   x_out[q] = fmaf(vq, dt, xq);
 }
 
+// The same for a run with the pair-symmetric force, one CTA per 256-record
+// tile and one thread per particle: the step (with move set), then the new
+// position's records for the force kernel.
+__global__ void __launch_bounds__(kJT)
+    lf_sym_step_kernel(int64_t n, const float *x_in, float *x_out, const float *v_in, float *v_out,
+                       const float *__restrict__ a, float h, float dt, int move, int close,
+                       float *__restrict__ ck_x, float *__restrict__ ck_v,
+                       const float *__restrict__ m, float4 *__restrict__ jhi,
+                       unsigned char *__restrict__ recs) {
+  const int64_t j = static_cast<int64_t>(blockIdx.x) * kJT + threadIdx.x;
+  float4 r = make_float4(dev::kNowhere, dev::kNowhere, dev::kNowhere, 0.f);
+  if (j < n) {
+    float xn[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const int64_t q = 3 * j + c;
+      xn[c] = x_in[q];
+      if (move) {
+        const float aq = a[q];
+        float vq = v_in[q];
+        if (close) vq = fmaf(aq, h, vq);
+        if (ck_x) {
+          ck_x[q] = xn[c];
+          ck_v[q] = vq;
+        }
+        vq = fmaf(aq, h, vq);
+        v_out[q] = vq;
+        xn[c] = fmaf(vq, dt, xn[c]);
+        x_out[q] = xn[c];
+      }
+    }
+    r = make_float4(xn[0], xn[1], xn[2], m[j]);
+  }
+  jhi[j] = r;
+  dev::put_rec4(recs + static_cast<size_t>(blockIdx.x) * dev::rec_bytes(0), 0, threadIdx.x, r);
+}
+
 struct LfCtx {
   int64_t n;
   const float *m;
@@ -474,7 +511,73 @@ struct LfCtx {
   int sms;
   cudaStream_t s;
   int64_t launches;
+  // the pair-symmetric force, when the caller lent the scratch for it
+  bool sym = false;
+  SymArgs S;
+  float4 *jhi = nullptr;
 };
+
+// Smallest n of the pair-symmetric force (nb_symforce.cu) for the forward
+// steps, and the most scratch it may ask for (1.9 kB per particle).  A step
+// with it against the one-sided shapes, N = 16,384 / 16,385 (a block more) /
+// 20,000 / 60,000 / 131,101 / 262,144: 0.108 / 0.129 / 0.152 / 1.05 / 4.90 /
+// 19.2 ms against 0.133 / 0.137 / 0.225 / 1.61 / 6.57 / 25.8; its sums fold in
+// split precision, error against 64 bits 3 .. 4e-8 against 1.2 .. 4.6e-7.
+constexpr int64_t kLfSymMin = 16384;
+constexpr int64_t kLfSymMaxBytes = int64_t(16) << 30;
+
+struct LfSymLayout {
+  SymSplit split;
+  size_t recs, ipart, jpart, err, bytes;  // offsets behind the records jhi
+};
+
+bool lf_sym_layout(int64_t n, int mask, int sms, LfSymLayout *L) {
+  if (n < kLfSymMin) return false;
+  const int64_t n_jt = (n + kJT - 1) / kJT;
+  if (!sym_split(n_jt, sym_block_i(0, mask, false), sms, &L->split)) return false;
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  L->recs = up(static_cast<size_t>(n_jt) * kJT * sizeof(float4));
+  L->ipart = L->recs + up(sym_record_bytes(n_jt, 0));
+  L->jpart = L->ipart + up(sym_ipart_bytes(L->split, false));
+  L->err = L->jpart + up(sym_jpart_bytes(L->split, false));
+  L->bytes = L->err + 256;
+  return L->bytes <= static_cast<size_t>(kLfSymMaxBytes);
+}
+
+int lf_sms() {
+  // A failed query leaves its error for the launch's error check to report.
+  int dev = 0, sms = 0;
+  if (cudaGetDevice(&dev) == cudaSuccess)
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  return sms < 1 ? 1 : sms;
+}
+
+// Takes the pair-symmetric force where the scratch suffices.
+cudaError_t lf_lend(LfCtx &C, void *scratch, int64_t bytes) {
+  LfSymLayout L;
+  if (!scratch || reinterpret_cast<uintptr_t>(scratch) % 256 != 0 ||
+      !lf_sym_layout(C.n, C.mask, C.sms, &L) || bytes < static_cast<int64_t>(L.bytes))
+    return cudaSuccess;
+  unsigned char *b = static_cast<unsigned char *>(scratch);
+  C.jhi = reinterpret_cast<float4 *>(b);
+  C.S = SymArgs();
+  C.S.jhi = C.jhi;
+  C.S.jlo = C.S.jvel = C.S.jrel = C.S.tinfo = nullptr;
+  C.S.n_jt = (C.n + kJT - 1) / kJT;
+  C.S.n = C.n;
+  C.S.eps2 = C.eps2;
+  C.S.G = C.G;
+  C.S.acc = C.S.jerk = nullptr;
+  C.S.recs = b + L.recs;
+  C.S.ipart = reinterpret_cast<float2 *>(b + L.ipart);
+  C.S.jpart = reinterpret_cast<float2 *>(b + L.jpart);
+  C.S.err = reinterpret_cast<int *>(b + L.err);
+  C.S.split = L.split;
+  C.sym = true;
+  cudaError_t e = sym_prepare(0, C.mask, false, false);
+  if (e == cudaSuccess) e = cudaMemsetAsync(C.S.err, 0, sizeof(int), C.s);
+  return e;
+}
 
 // N >= kLfWideMin takes the wide shape (4 particles per thread, records
 // broadcast) for the force.
@@ -547,7 +650,24 @@ cudaError_t lf_eval(LfCtx &C, const float *x, const LfTail &T) {
   return cudaGetLastError();
 }
 
+// acc = A(x_out) after the step that leads there (with v_in set), or A(x_in).
+cudaError_t lf_sym_eval(LfCtx &C, const float *x_in, float *x_out, const float *v_in, float *v_out,
+                        float *acc, float h, float dt, bool close, float *ck) {
+  lf_sym_step_kernel<<<static_cast<unsigned>(C.S.n_jt), kJT, 0, C.s>>>(
+      C.n, x_in, x_out, v_in, v_out, acc, h, dt, v_in ? 1 : 0, close ? 1 : 0, ck,
+      ck ? ck + 3 * C.n : nullptr, C.m, C.jhi, C.S.recs);
+  ++C.launches;
+  cudaError_t e = cudaGetLastError();
+  if (e != cudaSuccess) return e;
+  C.S.acc_f = acc;
+  int nl = 0;
+  e = launch_sym_force(0, C.mask, C.S, C.s, &nl, false);
+  C.launches += nl;
+  return e;
+}
+
 cudaError_t lf_acc(LfCtx &C, const float *x, float *acc) {
+  if (C.sym) return lf_sym_eval(C, x, nullptr, nullptr, nullptr, acc, 0.f, 0.f, false, nullptr);
   if (C.n < kLfWideMin) {
     LfTail T;
     T.acc = acc;
@@ -590,12 +710,18 @@ cudaError_t lf_kick(LfCtx &C, float *x, float *v, const float *a, float h, float
   return cudaGetLastError();
 }
 
-// The drift of one KDK step with the kicks around it: from A(x_in) (computed
-// here below kLfWideMin, where x_out must differ from x_in; above it acc
-// holds A(x_in) and receives A(x_out)).  The step's own closing kick is left
+// Whether acc carries A(x) from one half step to the next (and x_in may be
+// x_out), or every half step computes it.
+bool lf_carries(const LfCtx &C) { return C.sym || C.n >= kLfWideMin; }
+
+// The drift of one KDK step with the kicks around it: from A(x_in) (where
+// lf_carries, acc holds it and receives A(x_out); otherwise it is computed
+// here and x_out must differ from x_in).  The step's own closing kick is left
 // to the next call (close) or to the end of the run.
 cudaError_t lf_half_step(LfCtx &C, const float *x_in, float *x_out, const float *v_in,
                          float *v_out, float *acc, float dt, bool close, float *ck) {
+  if (C.sym)
+    return lf_sym_eval(C, x_in, x_out, v_in, v_out, acc, 0.5f * dt, dt, close, ck);
   if (C.n < kLfWideMin) {
     LfTail T;
     T.v_in = v_in;
@@ -640,12 +766,7 @@ LfCtx make_ctx(int64_t n, const float *m, float eps, float G, void *stream) {
   C.mask = eps * eps < FLT_MIN ? 1 : 0;
   C.eps2 = C.mask ? 0.f : eps * eps;
   C.G = G;
-  // A failed query leaves its error for the launch's error check to report.
-  int dev = 0;
-  C.sms = 0;
-  if (cudaGetDevice(&dev) == cudaSuccess)
-    cudaDeviceGetAttribute(&C.sms, cudaDevAttrMultiProcessorCount, dev);
-  if (C.sms < 1) C.sms = 1;
+  C.sms = lf_sms();
   C.s = static_cast<cudaStream_t>(stream);
   C.launches = 0;
   return C;
@@ -692,9 +813,24 @@ int64_t nb_lf_work_floats(int64_t n, int32_t ckpt_every) {
   return (static_cast<int64_t>(ckpt_every) + 1) * 3 * n + 6 * n;
 }
 
+int64_t nb_lf_scratch_bytes(int64_t n) {
+  LfSymLayout L;
+  return n >= kLfSymMin && n <= (int64_t(1) << 30) && lf_sym_layout(n, 0, lf_sms(), &L)
+             ? static_cast<int64_t>(L.bytes)
+             : 0;
+}
+
 nb_status nb_lf_forward(int64_t n, const float *d_m, float *d_x, float *d_v, float *d_acc,
                         int64_t nsteps, float dt, float eps, float G, int32_t ckpt_every,
                         float *d_ckpt, void *stream) {
+  return nb_lf_forward_lent(n, d_m, d_x, d_v, d_acc, nsteps, dt, eps, G, ckpt_every, d_ckpt,
+                            nullptr, 0, stream);
+}
+
+nb_status nb_lf_forward_lent(int64_t n, const float *d_m, float *d_x, float *d_v, float *d_acc,
+                             int64_t nsteps, float dt, float eps, float G, int32_t ckpt_every,
+                             float *d_ckpt, void *d_scratch, int64_t scratch_bytes,
+                             void *stream) {
   nb_status s = lf_check(n, eps, G, d_m, d_x);
   if (s != NB_OK) return s;
   if (!d_v || !d_acc || nsteps < 0 || ckpt_every < 1 || !(std::isfinite(dt)))
@@ -704,8 +840,8 @@ nb_status nb_lf_forward(int64_t n, const float *d_m, float *d_x, float *d_v, flo
   auto ck = [&](int64_t st) {
     return d_ckpt && st % ckpt_every == 0 ? d_ckpt + (st / ckpt_every) * 6 * n : nullptr;
   };
-  cudaError_t e = cudaSuccess;
-  if (n < kLfWideMin) {
+  cudaError_t e = lf_lend(C, d_scratch, scratch_bytes);
+  if (!lf_carries(C)) {
     // every force evaluation ends with the drift to the next positions, which
     // go to the other of d_x and d_acc (free until the last evaluation)
     float *cur = d_x, *other = d_acc;
@@ -726,7 +862,7 @@ nb_status nb_lf_forward(int64_t n, const float *d_m, float *d_x, float *d_v, flo
     if (e == cudaSuccess) e = lf_eval(C, d_x, T);
     return e == cudaSuccess ? NB_OK : lf_err(e);
   }
-  e = lf_acc(C, d_x, d_acc);
+  if (e == cudaSuccess) e = lf_acc(C, d_x, d_acc);
   for (int64_t st = 0; st < nsteps && e == cudaSuccess; ++st)
     e = lf_half_step(C, d_x, d_x, d_v, d_v, d_acc, dt, st > 0, ck(st));
   if (e == cudaSuccess && nsteps > 0) e = lf_kick(C, d_x, d_v, d_acc, 0.5f * dt, dt, 0);
@@ -736,6 +872,14 @@ nb_status nb_lf_forward(int64_t n, const float *d_m, float *d_x, float *d_v, flo
 nb_status nb_lf_backward(int64_t n, const float *d_m, const float *d_ckpt, int64_t nsteps,
                          float dt, float eps, float G, int32_t ckpt_every, float *d_lx,
                          float *d_lv, float *d_lm, float *d_work, void *stream) {
+  return nb_lf_backward_lent(n, d_m, d_ckpt, nsteps, dt, eps, G, ckpt_every, d_lx, d_lv, d_lm,
+                             d_work, nullptr, 0, stream);
+}
+
+nb_status nb_lf_backward_lent(int64_t n, const float *d_m, const float *d_ckpt, int64_t nsteps,
+                              float dt, float eps, float G, int32_t ckpt_every, float *d_lx,
+                              float *d_lv, float *d_lm, float *d_work, void *d_scratch,
+                              int64_t scratch_bytes, void *stream) {
   nb_status s = lf_check(n, eps, G, d_m, d_ckpt);
   if (s != NB_OK) return s;
   if (!d_lx || !d_lv || !d_lm || !d_work || nsteps < 0 || ckpt_every < 1)
@@ -746,7 +890,8 @@ nb_status nb_lf_backward(int64_t n, const float *d_m, const float *d_ckpt, int64
   float *xs = d_work;                               // (ckpt_every + 1) positions
   float *v = d_work + (ckpt_every + 1) * n3;        // velocity during recompute
   float *acc = v + n3;                              // acceleration during recompute
-  cudaError_t e = cudaMemsetAsync(d_lm, 0, n * sizeof(float), C.s);
+  cudaError_t e = lf_lend(C, d_scratch, scratch_bytes);
+  if (e == cudaSuccess) e = cudaMemsetAsync(d_lm, 0, n * sizeof(float), C.s);
   const int64_t K = (nsteps + ckpt_every - 1) / ckpt_every;
   for (int64_t seg = K - 1; seg >= 0 && e == cudaSuccess; --seg) {
     const int64_t s0 = seg * ckpt_every;
@@ -757,7 +902,7 @@ nb_status nb_lf_backward(int64_t n, const float *d_m, const float *d_ckpt, int64
     // of the others are the next one's checkpoint
     const int64_t upto = seg == K - 1 ? L : L - 1;
     auto pos = [&](int64_t q) -> const float * { return q == 0 ? slot : xs + q * n3; };
-    if (upto > 0 && n >= kLfWideMin) e = lf_acc(C, slot, acc);
+    if (upto > 0 && lf_carries(C)) e = lf_acc(C, slot, acc);
     for (int64_t q = 0; q < upto && e == cudaSuccess; ++q)
       e = lf_half_step(C, pos(q), xs + (q + 1) * n3, q == 0 ? slot + n3 : v, v, acc, dt, q > 0,
                        nullptr);

@@ -649,7 +649,9 @@ __global__ void __launch_bounds__(kFixP *NC) sym_fixup_kernel(const SymArgs A) {
     if (c < 3) val = s_a[c][pl];
   }
   if (!real) return;
-  if (c < 3) {
+  if (NC == 3 && A.acc_f) {
+    A.acc_f[3 * i + c] = *A.err ? __int_as_float(0x7fffffff) : static_cast<float>(val);
+  } else if (c < 3) {
     A.acc[3 * i + c] = val;
     if (A.kick != 0.0) A.v[3 * i + c] = fma(A.kick, val, A.v[3 * i + c]);
   } else {

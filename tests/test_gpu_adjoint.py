@@ -203,3 +203,54 @@ def test_short_runs_and_segments(torch_cuda, oracle_mod, nsteps, ckpt):
     assert torch.equal(xw, xT.detach()) and torch.equal(vw, vT.detach())
     ra = oracle_mod.acc(mr, xw.double().cpu().numpy(), eps)
     assert rel_l2(acc.double().cpu().numpy(), ra) < 1e-5
+
+
+@pytest.mark.parametrize("n", [16384, 16385, 17 * 1024 + 300])
+@pytest.mark.parametrize("eps", [0.05, 0.0])
+def test_lent_scratch_takes_each_pair_once(torch_cuda, n, eps):
+    """The forward steps with scratch on loan: accelerations against FP64 sums
+    of the same FP32 inputs (a term is off by at most ~15 u, a chain of 64
+    terms by 64 u of their absolute sum, u = 2^-24), two steps and their
+    gradient against the run without it (a kick is off by twice that, plus
+    the roundings of x and v; a pair's tidal tensor by a few of the offset in
+    x over its distance), and too little scratch changes no bit."""
+    torch = torch_cuda
+    from paper_0909_0879_gb300 import _lib
+
+    m, x, v = ics.plummer(n, 7, masses=ics.salpeter_masses(n, 7))
+    X, V, M = [torch.tensor(a, dtype=torch.float32, device="cuda") for a in (x, v, m)]
+    size = _lib.lf_scratch_bytes(n)
+    assert size > 0 and _lib.lf_scratch_bytes(16383) == 0
+    u, dt = 2.0**-24, 2.0**-9
+    idx = torch.cat([torch.arange(64), torch.arange(n - 64, n),
+                     torch.arange(100, n, 97)]).cuda()
+    d = X.double()[None] - X.double()[idx][:, None]
+    s2 = (d * d).sum(-1) + eps * eps
+    t = torch.where(s2 > 0, M.double() * s2**-1.5, 0.0)[..., None] * d
+    ref, size_of = t.sum(1), t.abs().sum(1)
+    out = {}
+    for side, lent in (("one", None), ("pairs", size), ("little", size - 256)):
+        sc = None if lent is None else torch.empty(lent, dtype=torch.uint8, device="cuda")
+        acc, xs, vs = torch.empty_like(X), X.clone(), V.clone()
+        _lib.lf_forward(n, M, xs, vs, acc, 0, dt, None, eps=eps, scratch=sc)
+        a0 = acc.clone()
+        ck = torch.empty(_lib.lf_ckpt_floats(n, 2, 2), dtype=torch.float32, device="cuda")
+        _lib.lf_forward(n, M, xs, vs, acc, 2, dt, ck, eps=eps, ckpt_every=2, scratch=sc)
+        lx, lv, lm = X.clone(), V.clone(), torch.empty_like(M)
+        work = torch.empty(_lib.lf_work_floats(n, 2), dtype=torch.float32, device="cuda")
+        _lib.lf_backward(n, M, ck, 2, dt, lx, lv, lm, work, eps=eps, ckpt_every=2, scratch=sc)
+        out[side] = [a.double() for a in (a0, xs, vs, acc, lx, lv, lm)]
+    assert all(torch.equal(a, b) for a, b in zip(out["one"], out["little"]))
+    assert not torch.equal(out["one"][0], out["pairs"][0])
+    err = (out["pairs"][0][idx] - ref).abs()
+    assert bool((err <= 80 * u * size_of).all()), (err / size_of).max().item() / u
+    da = 2 * 80 * u * size_of.max().item()
+    dv = 2 * dt * da + 8 * u * V.abs().max().item()
+    assert (out["pairs"][2] - out["one"][2]).abs().max().item() <= dv
+    dx = 2 * dt * dv + 8 * u * X.abs().max().item()
+    assert (out["pairs"][1] - out["one"][1]).abs().max().item() <= dx
+    gap = min(torch.where(r > 0, r, 9.0).min().item()
+              for r in (torch.cdist(c, X.double()) for c in X.double().split(1024)))
+    bar = 1e-5 + 12 * dx / np.hypot(gap, eps)
+    for a, b in zip(out["pairs"][4:], out["one"][4:]):
+        assert ((a - b).norm() <= bar * b.norm()).item()
