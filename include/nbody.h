@@ -585,16 +585,16 @@ nb_status nb_shard_import(nb_ctx *ctx, const double *d_rec, int64_t n_rec);
  *
  * Scratch: the partial sums of i-blocks split across CTAs live in one
  * static device array of 2^20 doubles (8 MiB) that every GPU loading the
- * library holds until the process exits; a launch uses at most 341 CTAs so
- * that they fit, whatever n and n_idx are.  Every call shares that array
+ * library holds until the process exits; a call splits its work into at most
+ * 341 ranges so that they fit, whatever n and n_idx are.  Every call shares that array
  * and it keeps the last call's contents; each call writes every partial it
  * later reads, so nothing needs clearing, but calls whose work overlaps on
  * the GPU (other streams, or other host threads on the same device) race on
  * it and must be serialised by the caller.
  *
  * The first call on each device resolves the array's device address
- * (cudaGetSymbolAddress, with that device current) and the kernel's
- * occupancy; make that first call before any stream capture begins.
+ * (cudaGetSymbolAddress, with that device current) and its SM count; make
+ * that first call before any stream capture begins.
  * Errors: NB_ERR_INVALID_ARG for n outside [1, 2^31-1], n_idx outside
  * [0, 2^31-1] (or above n without an index list), a NULL pointer, eps < 0,
  * G <= 0 or an unknown precision; NB_ERR_CUDA for a failed launch or set-up,

@@ -18,7 +18,7 @@
 // converts them to FP32 or double-single records in shared memory, and
 // zero-fills records past n, so no padded copy is needed.
 #include "../../include/nbody.h"
-#include "nb_internal.cuh"
+#include "nb_device.cuh"
 
 #include <cstring>
 #include <mutex>
@@ -26,14 +26,33 @@
 namespace nbi {
 namespace {
 
-constexpr int kNaNT = 256;    // threads per CTA
 constexpr int kNaJT = 256;    // j-records per tile
 constexpr int kNaFold = 32;   // j per thread between acceleration folds
-// Partial-sum scratch: 8 MiB of doubles, enough for kNaMaxCtas CTAs of
+// Partial-sum scratch: 8 MiB of doubles, enough for kNaMaxParts ranges of
 // 2 slots x 6 components x 256 i-particles.
 constexpr size_t kNaScratchDoubles = size_t(1) << 20;
-constexpr int kNaBI = kNaNT;  // one i-particle per thread
-constexpr int kNaMaxCtas = static_cast<int>(kNaScratchDoubles / (2 * 6 * kNaBI));
+constexpr int kNaBI = 256;  // i-particles per block of the split
+constexpr int kNaMaxParts = static_cast<int>(kNaScratchDoubles / (2 * 6 * kNaBI));
+// The (i-block, j-tile) units are cut into ranges; a range is run by 256 / NT
+// CTAs of NT threads, one particle per thread, each with its slice of the
+// i-particles.  Bound: issue slots, 40 per pair (32 FP32, three shared loads,
+// the rest loop and tile staging; issue 93 % active on the fullest SMs), so
+// what counts is how evenly the CTAs fill the SMs:
+//  * split precision: at most two ranges per SM in one slice each; with no
+//    more than one range for two SMs, two slices (N = 2,047: 19 against 25
+//    us; N = 3,000: 27 against 26).
+//  * FP32: always 341 ranges, which its sums depend on, in two slices: 5
+//    CTAs on the fullest SM of 4.5 on average, in place of 3 of 2.2.
+// Four slices of 64 threads balance better and run slower (N = 60,000 split
+// precision 5.29 against 4.33 ms), as do two particles per thread in FP32
+// (4.54 against 3.83; eight or nine warps per SM do not cover the latencies).
+// With conversions on the integer pipe, the fix-up per component (14 -> 4 us)
+// and one launch shape for every N before: N = 1,000 / 4,000 / 8,000 / 60,000,
+// eps = 0, split precision 28 / 52 / 121 / 4,538 -> 19 / 39 / 113 / 4,512 us,
+// FP32 24 / 44 / 120 / 4,789 -> 17 / 34 / 98 / 4,176 us; 700 of 60,000
+// particles 159 -> 96 us.
+constexpr int kNaSmallNT = 128;
+constexpr int kNaBatch = 2;  // records a thread has in flight while it stages a tile
 
 static __device__ __align__(256) double g_noalloc_part[kNaScratchDoubles];
 
@@ -48,24 +67,20 @@ struct NaArgs {
   double *part;  // device address of g_noalloc_part
 };
 
-__device__ __forceinline__ void na_ds_add(float &hi, float &lo, float x) {
-  const float s = hi + x;
-  const float bp = s - hi;
-  const float e = (hi - (s - bp)) + (x - bp);
-  hi = s;
-  lo += e;
-}
-
 __host__ __device__ __forceinline__ int na_owner(uint64_t u, uint64_t U, int P) {
   return static_cast<int>(((u + 1) * static_cast<uint64_t>(P) - 1) / U);
 }
 
-template <int PREC, int MASK>
-__global__ void __launch_bounds__(kNaNT, 2)
+template <int PREC, int MASK, int NT>
+__global__ void __launch_bounds__(NT, 512 / NT)
     noalloc_force_kernel(const NaArgs A, const uint64_t U, const int P) {
-  __shared__ float4 s_hi[kNaJT], s_lo[kNaJT], s_v[kNaJT];
+  constexpr int kSlices = kNaBI / NT;
+  constexpr int kBatch = kNaJT / NT < kNaBatch ? kNaJT / NT : kNaBatch;
+  constexpr int kUnroll = PREC ? 8 : 4;
+  __shared__ float4 s_hi[kNaJT], s_lo[PREC ? kNaJT : 1], s_v[kNaJT];
   const int tid = threadIdx.x;
-  const int p = blockIdx.x;
+  const int p = blockIdx.x / kSlices;
+  const int at = blockIdx.x % kSlices * NT + tid;  // particle in the i-block
   const uint64_t u0 = U * static_cast<uint64_t>(p) / static_cast<uint64_t>(P);
   const uint64_t u1 = U * static_cast<uint64_t>(p + 1) / static_cast<uint64_t>(P);
   if (u0 >= u1) return;
@@ -78,41 +93,59 @@ __global__ void __launch_bounds__(kNaNT, 2)
     const uint64_t jt0 = u % n_jt;
     const uint64_t seg = (n_jt - jt0) < (u1 - u) ? (n_jt - jt0) : (u1 - u);
     const bool full = (jt0 == 0) && (seg == n_jt);
-    const int64_t k = static_cast<int64_t>(ib) * kNaBI + tid;
+    const int64_t k = static_cast<int64_t>(ib) * kNaBI + at;
     const int64_t i = k < A.n_i ? (A.idx ? A.idx[k] : k) : 0;
     float xh[3], xl[3], vi[3];
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       const double xc = A.x[3 * i + c];
-      xh[c] = __double2float_rn(xc);
-      xl[c] = PREC ? __double2float_rn(xc - static_cast<double>(xh[c])) : 0.f;
-      vi[c] = __double2float_rn(A.v[3 * i + c]);
+      xh[c] = dev::d2f_rn(xc);
+      xl[c] = PREC ? dev::d2f_rn(xc - dev::f2d(xh[c])) : 0.f;
+      vi[c] = dev::d2f_rn(A.v[3 * i + c]);
     }
     float ah[3] = {0, 0, 0}, al[3] = {0, 0, 0}, p1[3] = {0, 0, 0}, p2[3] = {0, 0, 0};
     float jh[3] = {0, 0, 0}, jl[3] = {0, 0, 0};
     for (uint64_t t = 0; t < seg; ++t) {
-      const int64_t j = static_cast<int64_t>(jt0 + t) * kNaJT + tid;
-      if (j < A.n) {
-        const double x0 = A.x[3 * j], x1 = A.x[3 * j + 1], x2 = A.x[3 * j + 2];
-        const float h0 = __double2float_rn(x0), h1 = __double2float_rn(x1),
-                    h2 = __double2float_rn(x2);
-        s_hi[tid] = make_float4(h0, h1, h2, __double2float_rn(A.m[j]));
-        s_lo[tid] = make_float4(__double2float_rn(x0 - static_cast<double>(h0)),
-                                __double2float_rn(x1 - static_cast<double>(h1)),
-                                __double2float_rn(x2 - static_cast<double>(h2)), 0.f);
-        s_v[tid] = make_float4(__double2float_rn(A.v[3 * j]), __double2float_rn(A.v[3 * j + 1]),
-                               __double2float_rn(A.v[3 * j + 2]), 0.f);
-      } else {
-        // past the end: zero mass far away adds exactly zero
-        s_hi[tid] = make_float4(1.0e15f, 1.0e15f, 1.0e15f, 0.f);
-        s_lo[tid] = make_float4(0.f, 0.f, 0.f, 0.f);
-        s_v[tid] = make_float4(0.f, 0.f, 0.f, 0.f);
+      const int64_t j0 = static_cast<int64_t>(jt0 + t) * kNaJT;
+#pragma unroll 1
+      for (int w0 = tid; w0 < kNaJT; w0 += kBatch * NT) {
+        double raw[kBatch][7];
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+          const int64_t j = j0 + w0 + q * NT;
+          if (j < A.n) {
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              raw[q][c] = A.x[3 * j + c];
+              raw[q][3 + c] = A.v[3 * j + c];
+            }
+            raw[q][6] = A.m[j];
+          } else {
+            // past the end: zero mass far away adds exactly zero
+            raw[q][0] = raw[q][1] = raw[q][2] = 1.0e15;
+            raw[q][3] = raw[q][4] = raw[q][5] = raw[q][6] = 0.0;
+          }
+        }
+#pragma unroll
+        for (int q = 0; q < kBatch; ++q) {
+          const int w = w0 + q * NT;
+          float h[3], l[3];
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            h[c] = dev::d2f_rn(raw[q][c]);
+            l[c] = PREC ? dev::d2f_rn(raw[q][c] - dev::f2d(h[c])) : 0.f;
+          }
+          s_hi[w] = make_float4(h[0], h[1], h[2], dev::d2f_rn(raw[q][6]));
+          if (PREC) s_lo[w] = make_float4(l[0], l[1], l[2], 0.f);
+          s_v[w] = make_float4(dev::d2f_rn(raw[q][3]), dev::d2f_rn(raw[q][4]),
+                               dev::d2f_rn(raw[q][5]), 0.f);
+        }
       }
       __syncthreads();
 #pragma unroll 1
       for (int c0 = 0; c0 < kNaJT; c0 += kNaFold) {
         float pa[3] = {0, 0, 0};
-#pragma unroll 4
+#pragma unroll (kUnroll)
         for (int jj = c0; jj < c0 + kNaFold; ++jj) {
           const float4 hj = s_hi[jj];
           const float4 wj = s_v[jj];
@@ -151,7 +184,7 @@ __global__ void __launch_bounds__(kNaNT, 2)
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           if (PREC)
-            na_ds_add(ah[c], al[c], pa[c]);
+            dev::ds_add(ah[c], al[c], pa[c]);
           else
             ah[c] += pa[c];
         }
@@ -161,7 +194,7 @@ __global__ void __launch_bounds__(kNaNT, 2)
         const float jt = fmaf(-3.f, p2[c], p1[c]);
         p1[c] = p2[c] = 0.f;
         if (PREC)
-          na_ds_add(jh[c], jl[c], jt);
+          dev::ds_add(jh[c], jl[c], jt);
         else
           jh[c] += jt;
       }
@@ -184,61 +217,66 @@ __global__ void __launch_bounds__(kNaNT, 2)
         const int slot = (ib == ib_first) ? 0 : 1;
         double *dst = A.part + static_cast<size_t>(p * 2 + slot) * 6 * kNaBI;
 #pragma unroll
-        for (int c = 0; c < 6; ++c) dst[static_cast<size_t>(c) * kNaBI + tid] = o[c];
+        for (int c = 0; c < 6; ++c) dst[static_cast<size_t>(c) * kNaBI + at] = o[c];
       }
     }
     u += seg;
   }
 }
 
-__global__ void noalloc_fixup_kernel(const double *__restrict__ part, int64_t n_i,
-                                     uint64_t n_jt, uint64_t U, int P, double G,
-                                     double *__restrict__ acc, double *__restrict__ jerk) {
-  const int64_t k = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
+// Sums of the i-blocks that several ranges share, ascending ranges; one
+// thread per (particle, component).
+constexpr int kNaFixP = 32;
+
+__global__ void __launch_bounds__(6 * kNaFixP)
+    noalloc_fixup_kernel(const double *__restrict__ part, int64_t n_i, uint64_t n_jt, uint64_t U,
+                         int P, double G, double *__restrict__ acc, double *__restrict__ jerk) {
+  const int c = threadIdx.x / kNaFixP;
+  const int64_t k = static_cast<int64_t>(blockIdx.x) * kNaFixP + threadIdx.x % kNaFixP;
   if (k >= n_i) return;
   const uint64_t ib = static_cast<uint64_t>(k) / kNaBI;
   const int kk = static_cast<int>(static_cast<uint64_t>(k) % kNaBI);
   const int plo = na_owner(ib * n_jt, U, P);
   const int phi = na_owner((ib + 1) * n_jt - 1, U, P);
   if (plo == phi) return;
-  double s[6] = {0, 0, 0, 0, 0, 0};
-  for (int p = plo; p <= phi; ++p) {
-    const uint64_t u0p = U * static_cast<uint64_t>(p) / static_cast<uint64_t>(P);
-    const int slot = (u0p / n_jt == ib) ? 0 : 1;
-    const double *src = part + static_cast<size_t>(p * 2 + slot) * 6 * kNaBI;
-#pragma unroll
-    for (int c = 0; c < 6; ++c) s[c] += src[static_cast<size_t>(c) * kNaBI + kk];
+  // only the first range can have begun in an earlier block
+  const uint64_t u0 = U * static_cast<uint64_t>(plo) / static_cast<uint64_t>(P);
+  const double *src = part + (static_cast<size_t>(plo) * 2 * 6 + c) * kNaBI + kk;
+  double s = src[u0 < ib * n_jt ? 6 * kNaBI : 0];
+#pragma unroll 4
+  for (int p = plo + 1; p <= phi; ++p) {
+    src += 2 * 6 * kNaBI;
+    s += *src;
   }
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    acc[3 * k + c] = G * s[c];
-    jerk[3 * k + c] = G * s[3 + c];
-  }
+  if (c < 3)
+    acc[3 * k + c] = G * s;
+  else
+    jerk[3 * k + c - 3] = G * s;
 }
 
-// Per-device set-up: the device address of the scratch array and the
-// resident CTA count, resolved once with that device current.
+// The device address of the scratch array and the SM count, resolved once
+// with that device current.
 struct NaDevice {
-  bool ready = false;
   double *part = nullptr;
   int num_sms = 0;
-  int per_sm[4] = {0, 0, 0, 0};
 };
 constexpr int kNaMaxDevices = 64;
 std::mutex g_na_mu;
 NaDevice g_na_dev[kNaMaxDevices];
 
 using NaKernel = void (*)(const NaArgs, const uint64_t, const int);
-NaKernel na_kernel(int prec, int mask) {
-  if (prec)
-    return mask ? &noalloc_force_kernel<1, 1> : &noalloc_force_kernel<1, 0>;
-  return mask ? &noalloc_force_kernel<0, 1> : &noalloc_force_kernel<0, 0>;
+NaKernel na_kernel(int prec, int mask, int nt) {
+  if (!prec)
+    return mask ? &noalloc_force_kernel<0, 1, kNaSmallNT> : &noalloc_force_kernel<0, 0, kNaSmallNT>;
+  if (nt == kNaSmallNT)
+    return mask ? &noalloc_force_kernel<1, 1, kNaSmallNT> : &noalloc_force_kernel<1, 0, kNaSmallNT>;
+  return mask ? &noalloc_force_kernel<1, 1, kNaBI> : &noalloc_force_kernel<1, 0, kNaBI>;
 }
 
-int na_setup(int dev, NaDevice **out) {
+int na_setup(int dev, NaDevice *out) {
   std::lock_guard<std::mutex> lk(g_na_mu);
   NaDevice &D = g_na_dev[dev];
-  if (!D.ready) {
+  if (!D.part) {
     void *ptr = nullptr;
     cudaError_t e = cudaGetSymbolAddress(&ptr, g_noalloc_part);
     if (e != cudaSuccess)
@@ -247,19 +285,9 @@ int na_setup(int dev, NaDevice **out) {
     e = cudaDeviceGetAttribute(&D.num_sms, cudaDevAttrMultiProcessorCount, dev);
     if (e != cudaSuccess)
       return set_error(NB_ERR_CUDA, "device attribute query failed: %s", cudaGetErrorString(e));
-    for (int prec = 0; prec < 2; ++prec)
-      for (int mask = 0; mask < 2; ++mask) {
-        int nb = 1;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&nb, na_kernel(prec, mask), kNaNT, 0) !=
-                cudaSuccess ||
-            nb < 1)
-          nb = 1;
-        D.per_sm[prec * 2 + mask] = nb;
-      }
     D.part = static_cast<double *>(ptr);
-    D.ready = true;
   }
-  *out = &D;
+  *out = D;
   return NB_OK;
 }
 
@@ -296,21 +324,17 @@ extern "C" nb_status nb_force_jerk_noalloc(int64_t n, const double *d_m, const d
         set_error(NB_ERR_CUDA, "cudaGetDevice failed: %s", cudaGetErrorString(e)));
   if (dev < 0 || dev >= kNaMaxDevices)
     return static_cast<nb_status>(set_error(NB_ERR_INVALID_ARG, "device index %d too large", dev));
-  NaDevice *D = nullptr;
+  NaDevice D;
   int st = na_setup(dev, &D);
   if (st != NB_OK) return static_cast<nb_status>(st);
   const int mask = eps_masks(eps);
   const uint64_t n_jt = static_cast<uint64_t>((n + kNaJT - 1) / kNaJT);
   const uint64_t n_ib = static_cast<uint64_t>((n_idx + kNaBI - 1) / kNaBI);
   const uint64_t U = n_ib * n_jt;
-  int64_t P = static_cast<int64_t>(D->num_sms) * D->per_sm[precision * 2 + mask];
-  if (P > kNaMaxCtas) P = kNaMaxCtas;
-  if (static_cast<int64_t>(U) < P) P = static_cast<int64_t>(U);
-  const size_t need = static_cast<size_t>(P) * 2 * 6 * kNaBI;
-  if (need > kNaScratchDoubles)
-    return static_cast<nb_status>(set_error(
-        NB_ERR_INVALID_ARG, "partial sums of %lld CTAs exceed the %zu-double no-alloc scratch",
-        static_cast<long long>(P), kNaScratchDoubles));
+  uint64_t most = kNaMaxParts;
+  if (precision && most > 2 * static_cast<uint64_t>(D.num_sms)) most = 2 * D.num_sms;
+  const int P = static_cast<int>(U < most ? U : most);
+  const int nt = !precision || 2 * P <= D.num_sms ? kNaSmallNT : kNaBI;
   NaArgs A;
   A.n = n;
   A.m = d_m;
@@ -322,7 +346,7 @@ extern "C" nb_status nb_force_jerk_noalloc(int64_t n, const double *d_m, const d
   A.G = G;
   A.acc = d_acc;
   A.jerk = d_jerk;
-  A.part = D->part;
+  A.part = D.part;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   // An error left pending by earlier work on this thread would be returned
   // by the launch check below and blamed on this call: report it as what it
@@ -332,14 +356,13 @@ extern "C" nb_status nb_force_jerk_noalloc(int64_t n, const double *d_m, const d
     return static_cast<nb_status>(set_error(
         NB_ERR_CUDA, "a CUDA error from earlier work is pending (left set): %s",
         cudaGetErrorString(e)));
-  na_kernel(precision, mask)<<<static_cast<unsigned>(P), kNaNT, 0, s>>>(A, U,
-                                                                         static_cast<int>(P));
+  na_kernel(precision, mask, nt)<<<static_cast<unsigned>(P * (kNaBI / nt)), nt, 0, s>>>(A, U, P);
   e = cudaGetLastError();
   if (e == cudaSuccess && !(U % static_cast<uint64_t>(P) == 0 &&
                             (U / static_cast<uint64_t>(P)) % n_jt == 0)) {
-    const int64_t nb = (n_idx + 255) / 256;
-    noalloc_fixup_kernel<<<static_cast<unsigned>(nb), 256, 0, s>>>(
-        D->part, n_idx, n_jt, U, static_cast<int>(P), G, d_acc, d_jerk);
+    const int64_t nb = (n_idx + kNaFixP - 1) / kNaFixP;
+    noalloc_fixup_kernel<<<static_cast<unsigned>(nb), 6 * kNaFixP, 0, s>>>(
+        D.part, n_idx, n_jt, U, P, G, d_acc, d_jerk);
     e = cudaGetLastError();
   }
   if (e != cudaSuccess)

@@ -162,3 +162,13 @@ def test_noalloc_rejects_bad_sizes(cuda):
         assert e.value.status == _lib.NB_ERR_INVALID_ARG
     with pytest.raises(ValueError):
         _lib.force_jerk_noalloc(10, d, d, d, None, 1, d, d, eps=1e-3, precision="DS")
+
+
+@pytest.mark.parametrize("n", [255, 257, 2048, 2049])
+def test_noalloc_slices_of_i_blocks(cuda, oracle_mod, n):
+    """A particle short of a block and one over it, and both sides of the
+    line between two slices per range and one (64 and 81 units)."""
+    eps = 1e-3
+    m, x, v = ics.plummer(n, n, masses=ics.salpeter_masses(n, n))
+    idx_list = [np.arange(n, dtype=np.int32), ics.random_active_subset(n, n - 100, 3)]
+    _run_case(cuda, oracle_mod, m, x, v, eps, idx_list, pass_idx=(False, True))
