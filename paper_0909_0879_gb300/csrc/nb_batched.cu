@@ -13,7 +13,9 @@
 //
 // Threads per i-particle adapt to the cluster size: small clusters spread
 // each i-particle's j-range over up to 32 lanes and meet by a warp-shuffle
-// butterfly, so a 16-body cluster still occupies the whole CTA.
+// butterfly, so a 16-body cluster still occupies the whole CTA.  Where few
+// clusters would keep the GPU waiting for the largest ones, the CTAs of a
+// thread-block cluster share each of those.
 #include "../../include/nbody.h"
 #include "nb_device.cuh"
 
@@ -44,6 +46,7 @@ struct BatchArgs {
   int nsteps;             // steps per launch (>= 1)
   int cap;                // shared-memory record capacity
   int init_only;          // 1: evaluate a, j at the current state only
+  int n_large, teams;     // batched_team_kernel; its second counter is queue[1]
 };
 
 __device__ __forceinline__ void bds_add(float &hi, float &lo, float x) {
@@ -116,59 +119,119 @@ __device__ __forceinline__ void bherm_component(const BHermCoef &K, double x0, d
   v1 = vp + (K.v_s * snap + K.v_c * crackle);
 }
 
-template <int PREC, int IPT, int NT, int MASK, int PACK>
-__global__ void __launch_bounds__(NT, 2) batched_hermite_kernel(const BatchArgs B) {
+// The CTAs of a thread-block cluster as a group with one cluster of particles.
+namespace team {
+
+__device__ __forceinline__ uint32_t rank() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+  return r;
+}
+__device__ __forceinline__ uint32_t size() {
+  uint32_t r;
+  asm("mov.u32 %0, %%cluster_nctarank;" : "=r"(r));
+  return r;
+}
+// Everything written before it (shared memory of any CTA, global memory) is
+// seen by all of them after it.
+__device__ __forceinline__ void sync() {
+  asm volatile(
+      "barrier.cluster.arrive.release;\n\t"
+      "barrier.cluster.wait.acquire;" ::
+          : "memory");
+}
+__device__ __forceinline__ uint32_t addr_of(const void *p, uint32_t r) {
+  uint32_t a;
+  asm("mapa.shared::cluster.u32 %0, %1, %2;"
+      : "=r"(a)
+      : "r"(static_cast<uint32_t>(__cvta_generic_to_shared(p))), "r"(r));
+  return a;
+}
+__device__ __forceinline__ void put(float4 *p, float4 v, uint32_t r) {
+  asm volatile("st.shared::cluster.v4.f32 [%0], {%1, %2, %3, %4};" ::"r"(addr_of(p, r)),
+               "f"(v.x), "f"(v.y), "f"(v.z), "f"(v.w)
+               : "memory");
+}
+__device__ __forceinline__ void put(int *p, int v, uint32_t r) {
+  asm volatile("st.shared::cluster.s32 [%0], %1;" ::"r"(addr_of(p, r)), "r"(v) : "memory");
+}
+
+}  // namespace team
+
+// One cluster, nsteps steps, by a CTA of NT threads or (TEAM) by the CTAs of
+// a thread-block cluster: each takes an equal run of the i-particles and puts
+// their records into every CTA's shared memory.  A particle's sum is the same
+// in either case, and for every IPT: its threads tpi and their order follow
+// from n, NT and TPI_IPT alone.
+template <int PREC, int IPT, int NT, int MASK, int PACK, int TEAM, int TPI_IPT = IPT>
+__device__ __forceinline__ void batched_cluster(const BatchArgs &B, int c, float4 *srec) {
   using V = typename std::conditional<PACK != 0, float2, float>::type;
   using O = dev::VOps<V>;
   constexpr int W = O::W;
   static_assert(IPT % W == 0, "packed kernels need an even IPT");
   constexpr int NQ = IPT / W;
   constexpr int NARR = PREC ? 3 : 2;
-  extern __shared__ __align__(16) float4 srec[];
-  __shared__ int s_item;
   const int tid = threadIdx.x;
-  const float eps2 = B.eps2;
-  for (;;) {
-    if (tid == 0) s_item = atomicAdd(B.queue, 1);
-    __syncthreads();
-    const int item = s_item;
-    if (item >= B.n_items) return;  // uniform
-    const int c = B.order[item];
-    const int64_t base = B.off[c];
-    const int n = static_cast<int>(B.off[c + 1] - base);
-    int tpi = 1;
-    while (tpi < 32 && (NT / (tpi * 2)) * IPT >= n) tpi *= 2;
-    const int ng = NT / tpi;
-    const int bi = ng * IPT;
-    const int g = tid / tpi;
-    const int r = tid % tpi;
-    float4 *s_hi = srec;
-    float4 *s_lo = srec + B.cap;
-    float4 *s_v = srec + (NARR - 1) * B.cap;
-    float2 *s_f = reinterpret_cast<float2 *>(srec + NARR * B.cap);  // bi x 6 sums
-    const double dt = B.init_only ? 0.0 : B.dt;
-    const int nsteps = B.init_only ? 1 : B.nsteps;
-    // corrector coefficients of the shared step (dt a power of two: exact;
-    // the host gives 1/dt^2, 1/dt^3)
-    const BHermCoef K = bherm_coef(dt, B.idt2, B.idt3);
-
-    for (int step = 0; step < nsteps; ++step) {
-      for (int p = tid; p < n; p += NT) {
-        double xp[3], vp[3];
-        bpredict(B.x, B.v, B.a, B.jk, base + p, dt, xp, vp);
-        // conversions on the integer pipe (bit-identical to the hardware ones)
-        const float hx = dev::d2f_rn(xp[0]);
-        const float hy = dev::d2f_rn(xp[1]);
-        const float hz = dev::d2f_rn(xp[2]);
-        s_hi[p] = make_float4(hx, hy, hz, dev::d2f_rn(B.m[base + p]));
-        if (PREC)
-          s_lo[p] = make_float4(dev::d2f_rn(xp[0] - dev::f2d(hx)),
-                                dev::d2f_rn(xp[1] - dev::f2d(hy)),
-                                dev::d2f_rn(xp[2] - dev::f2d(hz)), 0.f);
-        s_v[p] = make_float4(dev::d2f_rn(vp[0]), dev::d2f_rn(vp[1]), dev::d2f_rn(vp[2]), 0.f);
-      }
+  auto sync_all = [&] {
+    if (TEAM)
+      team::sync();
+    else
       __syncthreads();
-      for (int i0 = 0; i0 < n; i0 += bi) {
+  };
+  const float eps2 = B.eps2;
+  const int64_t base = B.off[c];
+  const int n = static_cast<int>(B.off[c + 1] - base);
+  int tpi = 1;
+  while (tpi < 32 && (NT / (tpi * 2)) * TPI_IPT >= n) tpi *= 2;
+  const int g = tid / tpi;
+  const int r = tid % tpi;
+  // the i-particles in equal passes, each packed onto as few warps as hold it:
+  // the idle warps cost no issue slots (600 particles in two passes of 512
+  // slots: 41 % of them padding; 4,096 clusters 19.7 -> 18.9 ms)
+  const int parts = TEAM ? static_cast<int>(team::size()) : 1;
+  const int part = TEAM ? static_cast<int>(team::rank()) : 0;
+  const int lo = n * part / parts, hi = n * (part + 1) / parts;  // this CTA's i-particles
+  const int most = NT / tpi * IPT;
+  const int passes = max(1, (hi - lo + most - 1) / most);
+  const int per = max(1, (hi - lo + passes - 1) / passes);
+  float4 *s_hi = srec;
+  float4 *s_lo = srec + B.cap;
+  float4 *s_v = srec + (NARR - 1) * B.cap;
+  float2 *s_f = reinterpret_cast<float2 *>(srec + NARR * B.cap);  // per x 6 sums
+  auto put = [&](float4 *p, float4 w) {
+    if (TEAM)
+      for (int q = 0; q < parts; ++q) team::put(p, w, q);
+    else
+      *p = w;
+  };
+  const double dt = B.init_only ? 0.0 : B.dt;
+  const int nsteps = B.init_only ? 1 : B.nsteps;
+  // corrector coefficients of the shared step (dt a power of two: exact;
+  // the host gives 1/dt^2, 1/dt^3)
+  const BHermCoef K = bherm_coef(dt, B.idt2, B.idt3);
+
+  for (int step = 0; step < nsteps; ++step) {
+    for (int p = lo + tid; p < hi; p += NT) {
+      double xp[3], vp[3];
+      bpredict(B.x, B.v, B.a, B.jk, base + p, dt, xp, vp);
+      // conversions on the integer pipe (bit-identical to the hardware ones)
+      const float hx = dev::d2f_rn(xp[0]);
+      const float hy = dev::d2f_rn(xp[1]);
+      const float hz = dev::d2f_rn(xp[2]);
+      put(s_hi + p, make_float4(hx, hy, hz, dev::d2f_rn(B.m[base + p])));
+      if (PREC)
+        put(s_lo + p, make_float4(dev::d2f_rn(xp[0] - dev::f2d(hx)),
+                                  dev::d2f_rn(xp[1] - dev::f2d(hy)),
+                                  dev::d2f_rn(xp[2] - dev::f2d(hz)), 0.f));
+      put(s_v + p,
+          make_float4(dev::d2f_rn(vp[0]), dev::d2f_rn(vp[1]), dev::d2f_rn(vp[2]), 0.f));
+    }
+    sync_all();
+    for (int i0 = lo; i0 < hi; i0 += per) {
+      const int lim = min(hi, i0 + per);  // i-particles of this pass
+      const int ng = (lim - i0 + IPT - 1) / IPT;
+      // warps without a particle go on to the corrector
+      if ((tid & ~31) / tpi < ng) {
         // i-data negated, so that every difference is an addition (a - b and
         // a + (-b) round alike); two i-particles per packed FP32x2 lane
         // pair when PACK (per-lane IEEE rounding: the same bits as scalar)
@@ -176,7 +239,7 @@ __global__ void __launch_bounds__(NT, 2) batched_hermite_kernel(const BatchArgs 
 #pragma unroll
         for (int q = 0; q < IPT; ++q) {
           const int i = i0 + g + q * ng;
-          const int ii = i < n ? i : 0;
+          const int ii = i < lim ? i : 0;
           const float4 h = s_hi[ii];
           const float4 w = s_v[ii];
           const float4 l = PREC ? s_lo[ii] : make_float4(0.f, 0.f, 0.f, 0.f);
@@ -290,43 +353,87 @@ __global__ void __launch_bounds__(NT, 2) batched_hermite_kernel(const BatchArgs 
           // hand the sums to consecutive threads so that the FP64
           // corrector runs on full warps (an FP64 instruction costs the SM
           // the same whatever the number of active lanes)
-          if (r == 0) {
+          if (r == 0 && g < ng) {
 #pragma unroll
             for (int k = 0; k < 6; ++k) s_f[(g + q * ng) * 6 + k] = make_float2(oh[k], ol[k]);
           }
         }
-        __syncthreads();
-        for (int t = tid; t < bi; t += NT) {
-          const int i = i0 + t;
-          if (i >= n) break;
-          const int64_t gi = base + i;
-          double o[6];
-#pragma unroll
-          for (int k = 0; k < 6; ++k)
-            o[k] = dev::f2d(s_f[t * 6 + k].x) + dev::f2d(s_f[t * 6 + k].y);
-          if (B.init_only) {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-              B.a[3 * gi + k] = B.G * o[k];
-              B.jk[3 * gi + k] = B.G * o[3 + k];
-            }
-          } else {
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-              double x1, v1;
-              bherm_component(K, B.x[3 * gi + k], B.v[3 * gi + k], B.a[3 * gi + k],
-                              B.jk[3 * gi + k], B.G * o[k], B.G * o[3 + k], x1, v1);
-              B.x[3 * gi + k] = x1;
-              B.v[3 * gi + k] = v1;
-              B.a[3 * gi + k] = B.G * o[k];
-              B.jk[3 * gi + k] = B.G * o[3 + k];
-            }
-          }
-        }
-        __syncthreads();  // s_f is reused by the next i-block
       }
       __syncthreads();
+      for (int t = tid; t < lim - i0; t += NT) {
+        const int i = i0 + t;
+        const int64_t gi = base + i;
+        double o[6];
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+          o[k] = dev::f2d(s_f[t * 6 + k].x) + dev::f2d(s_f[t * 6 + k].y);
+        if (B.init_only) {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            B.a[3 * gi + k] = B.G * o[k];
+            B.jk[3 * gi + k] = B.G * o[3 + k];
+          }
+        } else {
+#pragma unroll
+          for (int k = 0; k < 3; ++k) {
+            double x1, v1;
+            bherm_component(K, B.x[3 * gi + k], B.v[3 * gi + k], B.a[3 * gi + k],
+                            B.jk[3 * gi + k], B.G * o[k], B.G * o[3 + k], x1, v1);
+            B.x[3 * gi + k] = x1;
+            B.v[3 * gi + k] = v1;
+            B.a[3 * gi + k] = B.G * o[k];
+            B.jk[3 * gi + k] = B.G * o[3 + k];
+          }
+        }
+      }
+      __syncthreads();  // s_f is reused by the next i-block
     }
+    sync_all();  // the records are written again
+  }
+}
+
+template <int PREC, int IPT, int NT, int MASK, int PACK>
+__global__ void __launch_bounds__(NT, 2) batched_hermite_kernel(const BatchArgs B) {
+  extern __shared__ __align__(16) float4 srec[];
+  __shared__ int s_item;
+  for (;;) {
+    if (threadIdx.x == 0) s_item = atomicAdd(B.queue, 1);
+    __syncthreads();
+    const int item = s_item;
+    if (item >= B.n_items) return;  // uniform
+    batched_cluster<PREC, IPT, NT, MASK, PACK, 0>(B, B.order[item], srec);
+  }
+}
+
+// The same in thread-block clusters: the first B.teams of them share each of
+// the B.n_large largest clusters (the queue's head) among their CTAs, the
+// others' CTAs, and the teams' when no large cluster is left, take one each
+// of the rest.  Sums and bits are those of the kernel above.
+template <int PREC, int IPT, int NT, int MASK, int PACK>
+__global__ void __launch_bounds__(NT, 2) batched_team_kernel(const BatchArgs B) {
+  extern __shared__ __align__(16) float4 srec[];
+  __shared__ int s_item;
+  const uint32_t parts = team::size();
+  if (blockIdx.x / parts < static_cast<uint32_t>(B.teams)) {
+    team::sync();  // every CTA's shared memory is there
+    for (;;) {
+      if (team::rank() == 0 && threadIdx.x == 0) {
+        const int item = atomicAdd(B.queue + 1, 1);
+        for (uint32_t q = 0; q < parts; ++q) team::put(&s_item, item, q);
+      }
+      team::sync();
+      const int item = s_item;
+      if (item >= B.n_large) break;  // the whole team
+      batched_cluster<PREC, 1, NT, MASK, 0, 1, IPT>(B, B.order[item], srec);
+    }
+  }
+  for (;;) {
+    __syncthreads();  // s_item has been read
+    if (threadIdx.x == 0) s_item = B.n_large + atomicAdd(B.queue, 1);
+    __syncthreads();
+    const int item = s_item;
+    if (item >= B.n_items) return;
+    batched_cluster<PREC, IPT, NT, MASK, PACK, 0>(B, B.order[item], srec);
   }
 }
 
@@ -389,6 +496,16 @@ const BEntry kBTable[] = {
 };
 constexpr int kNumBVariants = sizeof(kBTable) / sizeof(kBTable[0]);
 
+// batched_team_kernel for the default shapes, by precision and masking.
+constexpr int kTeamNT = 256, kTeamIpt = 2;
+BKernel team_kernel(int prec, int mask) {
+  if (prec)
+    return mask ? &batched_team_kernel<1, kTeamIpt, kTeamNT, 1, 0>
+                : &batched_team_kernel<1, kTeamIpt, kTeamNT, 0, 0>;
+  return mask ? &batched_team_kernel<0, kTeamIpt, kTeamNT, 1, 0>
+              : &batched_team_kernel<0, kTeamIpt, kTeamNT, 0, 0>;
+}
+
 }  // namespace
 }  // namespace nbi
 
@@ -398,6 +515,9 @@ struct nb_batch {
   int32_t n_clusters = 0;
   int64_t n = 0;
   int max_n = 0;
+  int team = 0;         // CTAs that share a large cluster (0: none is shared)
+  int n_large = 0;      // clusters that are shared
+  double large = 0.0;   // their part of the work
   nb_config cfg{};
   cudaStream_t stream = nullptr;
   int num_sms = 0;
@@ -433,6 +553,9 @@ nb_status bfail(nb_status s, const char *msg, cudaError_t e = cudaSuccess) {
     if (e_ != cudaSuccess) return bfail(NB_ERR_CUDA, #call, e_); \
   } while (0)
 
+// Stands for batched_team_kernel where a shape's index is asked for.
+constexpr int kTeamShape = -2;
+
 int pick_bvariant(const nb_batch *b) {
   if (b->variant >= 0) return b->variant;
   const int mask = eps_masks(b->cfg.eps);
@@ -443,6 +566,60 @@ int pick_bvariant(const nb_batch *b) {
 size_t bsmem(const BEntry &E, int cap) {
   return static_cast<size_t>(E.prec ? 3 : 2) * cap * sizeof(float4) +
          static_cast<size_t>(E.threads) * E.ipt * 6 * sizeof(float2);
+}
+
+// A cluster's time goes with n^2 and a run lasts at least as long as its
+// longest cluster.  Where that has more than twice the mean load of a CTA, sum
+// n^2 / (2 SMs), the clusters above the mean are shared by teams of 4 or 8
+// CTAs (at twice the mean or less a team of two gains nothing: 1,500 clusters
+// 7.38 against 7.36 ms); as many teams as the large clusters' part of the
+// work.  Clusters of up to 256 gain nothing from it.  20 steps of clusters of
+// 16 .. 1,024, split precision, 50 / 150 / 400 / 1,000 clusters: 4.23 / 4.23 /
+// 4.32 / 5.93 -> 0.85 / 1.20 / 2.69 / 5.33 ms.
+constexpr int kTeamMin = 256, kTeamMost = 8;
+
+void pick_team(nb_batch *b, const int64_t *offsets) {
+  double load = 0.0;
+  auto cost = [&](int32_t c) {
+    const double n = static_cast<double>(offsets[c + 1] - offsets[c]);
+    return n * n;
+  };
+  for (int32_t c = 0; c < b->n_clusters; ++c) load += cost(c);
+  const double mean = load / (2.0 * b->num_sms);
+  const double line = std::max(static_cast<double>(kTeamMin) * kTeamMin, mean);
+  double large = 0.0;
+  for (int32_t c = 0; c < b->n_clusters; ++c)
+    if (cost(c) > line) {
+      b->n_large += 1;
+      large += cost(c);
+    }
+  const double top = static_cast<double>(b->max_n) * b->max_n;
+  if (b->n_large == 0 || top <= 2.0 * mean) return;
+  b->large = large / load;
+  b->team = top > 4.0 * mean ? kTeamMost : 4;
+}
+
+// Teams that fit the device at once (0: none does).
+int team_config(nb_batch *b, cudaLaunchConfig_t *cfg, cudaLaunchAttribute *at) {
+  const BKernel fn = team_kernel(b->cfg.precision, eps_masks(b->cfg.eps));
+  *cfg = cudaLaunchConfig_t();
+  cfg->blockDim = dim3(kTeamNT);
+  cfg->gridDim = dim3(b->team);
+  cfg->dynamicSmemBytes = bsmem(kBTable[pick_bvariant(b)], b->max_n);
+  cfg->stream = b->stream;
+  at->id = cudaLaunchAttributeClusterDimension;
+  at->val.clusterDim.x = b->team;
+  at->val.clusterDim.y = at->val.clusterDim.z = 1;
+  cfg->attrs = at;
+  cfg->numAttrs = 1;
+  int n = 0;
+  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(cfg->dynamicSmemBytes)) != cudaSuccess ||
+      cudaOccupancyMaxActiveClusters(&n, fn, cfg) != cudaSuccess) {
+    cudaGetLastError();  // a refused query is not this call's error
+    return 0;
+  }
+  return n;
 }
 
 int bgrid(nb_batch *b, int v) {
@@ -460,7 +637,6 @@ int bgrid(nb_batch *b, int v) {
 
 nb_status launch_batch(nb_batch *b, int v, int grid, int32_t n_items, const int32_t *order,
                        int *counter, int nsteps, int init_only) {
-  const BEntry &E = kBTable[v];
   BatchArgs A;
   A.n_items = n_items;
   A.off = b->off;
@@ -479,7 +655,18 @@ nb_status launch_batch(nb_batch *b, int v, int grid, int32_t n_items, const int3
   A.nsteps = nsteps;
   A.cap = b->max_n;
   A.init_only = init_only;
-  E.fn<<<grid, E.threads, bsmem(E, b->max_n), b->stream>>>(A);
+  if (v == kTeamShape) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    if (team_config(b, &cfg, &at) < 1) return bfail(NB_ERR_CUDA, "no thread-block cluster fits");
+    cfg.gridDim = dim3(grid);
+    const int most = std::min(grid / b->team, b->n_large);
+    A.n_large = b->n_large;
+    A.teams = std::min(most, 1 + static_cast<int>(b->large * (grid / b->team)));
+    BCUDA(cudaLaunchKernelEx(&cfg, team_kernel(b->cfg.precision, eps_masks(b->cfg.eps)), A));
+  } else {
+    kBTable[v].fn<<<grid, kBTable[v].threads, bsmem(kBTable[v], b->max_n), b->stream>>>(A);
+  }
   BCUDA(cudaGetLastError());
   b->launches += 1;
   return NB_OK;
@@ -497,10 +684,10 @@ nb_status queue_persistent(nb_batch *b, int64_t nsteps, int v, int grid) {
   const int S = std::max(1, b->steps_per_launch);
   const int64_t nl = (nsteps + S - 1) / S;
   if (nl > b->n_counters) return bfail(NB_ERR_INVALID_ARG, "too many launches for the counter array");
-  BCUDA(cudaMemsetAsync(b->counters, 0, sizeof(int) * nl, b->stream));
+  BCUDA(cudaMemsetAsync(b->counters, 0, 2 * sizeof(int) * nl, b->stream));
   for (int64_t k = 0; k < nl; ++k) {
     const int s = static_cast<int>(std::min<int64_t>(S, nsteps - k * S));
-    nb_status st = launch_batch(b, v, grid, b->n_clusters, b->order, b->counters + k, s, 0);
+    nb_status st = launch_batch(b, v, grid, b->n_clusters, b->order, b->counters + 2 * k, s, 0);
     if (st != NB_OK) return st;
   }
   return NB_OK;
@@ -579,7 +766,7 @@ nb_status nb_batched_init(nb_batch **out, int32_t n_clusters, const int64_t *off
       (st = alloc(reinterpret_cast<void **>(&b->off), (n_clusters + 1) * sizeof(int64_t))) ||
       (st = alloc(reinterpret_cast<void **>(&b->order), n_clusters * sizeof(int32_t))) ||
       (st = alloc(reinterpret_cast<void **>(&b->ident), n_clusters * sizeof(int32_t))) ||
-      (st = alloc(reinterpret_cast<void **>(&b->counters), b->n_counters * sizeof(int))) ||
+      (st = alloc(reinterpret_cast<void **>(&b->counters), 2 * b->n_counters * sizeof(int))) ||
       (st = alloc(reinterpret_cast<void **>(&b->ekin), n_clusters * sizeof(double))) ||
       (st = alloc(reinterpret_cast<void **>(&b->epot), n_clusters * sizeof(double))))
     return cleanup(st);
@@ -598,6 +785,7 @@ nb_status nb_batched_init(nb_batch **out, int32_t n_clusters, const int64_t *off
   std::stable_sort(order.begin(), order.end(), [&](int32_t p, int32_t q) {
     return (offsets[p + 1] - offsets[p]) > (offsets[q + 1] - offsets[q]);
   });
+  pick_team(b, offsets);
   cudaStream_t s = b->stream;
   if (cudaMemcpyAsync(b->m, m, n * sizeof(double), cudaMemcpyHostToDevice, s) ||
       cudaMemcpyAsync(b->x, x, n3, cudaMemcpyHostToDevice, s) ||
@@ -609,7 +797,7 @@ nb_status nb_batched_init(nb_batch **out, int32_t n_clusters, const int64_t *off
                       cudaMemcpyHostToDevice, s) ||
       cudaMemcpyAsync(b->ident, ident.data(), n_clusters * sizeof(int32_t),
                       cudaMemcpyHostToDevice, s) ||
-      cudaMemsetAsync(b->counters, 0, b->n_counters * sizeof(int), s))
+      cudaMemsetAsync(b->counters, 0, 2 * b->n_counters * sizeof(int), s))
     return cleanup(bfail(NB_ERR_CUDA, "initial copies failed"));
   const int vv = pick_bvariant(b);
   st = launch_batch(b, vv, bgrid(b, vv), n_clusters, b->order, b->counters, 1, 1);
@@ -662,8 +850,17 @@ nb_status nb_batched_run(nb_batch *b, int64_t nsteps) {
   if (!b) return bfail(NB_ERR_INVALID_ARG, "null batch");
   if (nsteps < 0) return bfail(NB_ERR_INVALID_ARG, "negative step count");
   if (nsteps == 0) return NB_OK;
-  const int v = pick_bvariant(b);
-  const int grid = bgrid(b, v);
+  // the built-in shape and grid, and a cluster that is worth sharing
+  int v = pick_bvariant(b), grid = 0;
+  if (b->team > 0 && b->variant < 0 && b->grid_cap == 0) {
+    cudaLaunchConfig_t cfg;
+    cudaLaunchAttribute at;
+    grid = b->team * std::min(team_config(b, &cfg, &at), b->n_clusters);
+  }
+  if (grid > 0)
+    v = kTeamShape;
+  else
+    grid = bgrid(b, v);
   if (!b->use_graph) return queue_persistent(b, nsteps, v, grid);
   const int key[4] = {v, b->steps_per_launch, b->grid_cap, grid};
   if (!b->graph || b->graph_steps != nsteps || std::memcmp(key, b->graph_key, sizeof(key)) != 0) {

@@ -189,3 +189,26 @@ def test_batched_packed_variants_bitwise_equal_scalar(nb):
         for key in res[0]:
             assert np.array_equal(res[0][key], res[1][key]), (k, j, key)
     assert compared >= 4
+
+
+@pytest.mark.parametrize("sizes", [[257, 1, 16], [1023, 300, 257, 256, 31] * 3, [4096, 513],
+                                   [700] * 700 + [1024]])
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+@pytest.mark.parametrize("eps", [1e-3, 0.0])
+def test_batched_shared_clusters_bitwise_equal(nb, sizes, prec, eps):
+    """Large clusters shared by the CTAs of a thread-block cluster: one just
+    past the line, uneven shares, two passes per CTA; the last batch has no
+    cluster above twice the mean load and shares none.  Bits as with a CTA
+    per cluster."""
+    off = np.concatenate([[0], np.cumsum(sizes)]).astype(np.int64)
+    parts = [ics.plummer(k, (3, c)) if k > 1 else (np.ones(1), np.zeros((1, 3)), np.zeros((1, 3)))
+             for c, k in enumerate(sizes)]
+    m, x, v = (np.concatenate([p[q] for p in parts]) for q in range(3))
+    res = []
+    for run in ("run", "run_per_cluster"):
+        with nb.Batch(off, m, x, v, eps=eps, lev_shared=9, precision=prec) as b:
+            getattr(b, run)(3)
+            b.run(2) if run == "run" else b.run_per_cluster(2)
+            res.append(b.get_state())
+    for k in res[0]:
+        assert np.array_equal(res[0][k], res[1][k]), k
