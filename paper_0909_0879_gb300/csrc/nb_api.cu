@@ -301,7 +301,7 @@ struct nb_ctx {
   size_t sym_i_cap = 0, sym_j_cap = 0;
   bool sym_off = false;
   bool eq_mass = false;  // every mass is m_eq
-  double m_eq = 0.0;
+  double m_eq = 0.0, m_mean = 0.0;
   double *red = nullptr;        // energy scratch
   unsigned char *en_rec = nullptr;  // records of the split-precision energy
   int *err = nullptr;           // device error word
@@ -572,7 +572,8 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
   A->eps2 = eps2_f32(c->cfg.eps);
   A->G = c->cfg.G;
   A->eq = c->eq_mass ? 1 : 0;
-  A->m_eq = static_cast<float>(c->m_eq);
+  A->m_eq = c->m_eq;
+  A->sexp = sym_exponent(c->m_mean, A->eps2);
   A->recs = c->sym_rec;
   A->ipart = c->sym_i;
   A->jpart = c->sym_j;
@@ -743,6 +744,7 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x,
   c->cfg = *cfg;
   c->n = n;
   c->m_eq = m[0];
+  c->m_mean = std::accumulate(m, m + n, 0.0) / static_cast<double>(n);
   c->eq_mass = std::all_of(m, m + n, [&](double q) { return q == m[0]; });
   c->n_jt = (n + kJT - 1) / kJT;
   c->n_pad = c->n_jt * kJT;
@@ -1396,7 +1398,7 @@ nb_status queue_kick_drift(nb_ctx *c, const SymArrays &S, const SymArgs *P, cuda
                            double h, double d, bool rec, int64_t *launches) {
   NB_CUDA(launch_kick_drift(c->n, c->n_jt, h, d, rec, P ? ExtField() : c->ext, S.a, S.v, S.x,
                             S.m, c->cfg.precision, c->jhi, c->jlo, c->jvel, c->jrel, c->tinfo,
-                            P ? P->recs : nullptr, s));
+                            P ? P->recs : nullptr, P ? P->sexp : 0, s));
   *launches += 1;
   return NB_OK;
 }

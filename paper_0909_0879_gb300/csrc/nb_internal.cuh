@@ -181,8 +181,9 @@ struct SymArgs {
   float eps2;
   double G;
   double *acc, *jerk;    // (n, 3); jerk null: acceleration only
-  int eq = 0;            // every mass is m_eq (as the records hold it)
-  float m_eq = 0.f;
+  int eq = 0;            // every mass is m_eq
+  double m_eq = 0.0;
+  int sexp = 0;          // sym_exponent
   unsigned char *recs;   // the records in pairs (scratch)
   float2 *ipart, *jpart; // partial sums (hi, lo pairs; scratch)
   int *err;
@@ -198,7 +199,14 @@ struct SymArgs {
   // The acceleration in FP32 in place of acc; NaN should the force kernel have
   // reported an error in *err.
   float *acc_f = nullptr;
+  // set by launch_sym_force: 2^sexp, 2^(3 sexp), and what the sums are taken by
+  float sc = 1.f, sm = 1.f;
+  double g_acc = 0.0, g_jerk = 0.0;
 };
+// The pair kernel works on positions times 2^s and masses times 2^(3 s) (exact),
+// s = sym_exponent: with 2^(-3 s) near the mean mass, 1 / r^3 of the scaled
+// positions has the FP32 range that mass / r^3 has.
+int sym_exponent(double mean_mass, float eps2);
 // i-particles per block of the kernel for this precision / masking / output.
 int sym_block_i(int prec, int mask, bool jrk);
 // False when n_jt tiles are too few (or too many) for a ring of such blocks.
@@ -362,12 +370,12 @@ int symplectic_stages(int order, double *w);
 // v += h (a + a_ext(x)), x += d v for every particle (a factor of 0 skips
 // its update; a_ext only when E.on); with rec set also the j-records and,
 // when jrel is set, the tile frames, and, when recs is set, the records of
-// the pair-symmetric kernel.
+// the pair-symmetric kernel (scaled by sexp).
 cudaError_t launch_kick_drift(int64_t n, int64_t n_jt, double h, double d, bool rec,
                               const ExtField &E, const double *a, double *v, double *x,
                               const double *m, int prec, float4 *jhi, float4 *jlo,
                               float4 *jvel, float4 *jrel, float4 *tinfo, unsigned char *recs,
-                              cudaStream_t s);
+                              int sexp, cudaStream_t s);
 // Rows of w doubles: dst[k] = src[perm[k]], or with scatter dst[perm[k]] =
 // src[k].
 cudaError_t launch_permute(int64_t n, const int64_t *perm, const double *src, double *dst,

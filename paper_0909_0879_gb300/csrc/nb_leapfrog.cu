@@ -474,7 +474,7 @@ __global__ void __launch_bounds__(kJT)
                        const float *__restrict__ a, float h, float dt, int move, int close,
                        float *__restrict__ ck_x, float *__restrict__ ck_v,
                        const float *__restrict__ m, float4 *__restrict__ jhi,
-                       unsigned char *__restrict__ recs) {
+                       unsigned char *__restrict__ recs, float sc, float sm) {
   const int64_t j = static_cast<int64_t>(blockIdx.x) * kJT + threadIdx.x;
   float4 r = make_float4(dev::kNowhere, dev::kNowhere, dev::kNowhere, 0.f);
   if (j < n) {
@@ -500,6 +500,7 @@ __global__ void __launch_bounds__(kJT)
     r = make_float4(xn[0], xn[1], xn[2], m[j]);
   }
   jhi[j] = r;
+  if (j < n) r = make_float4(r.x * sc, r.y * sc, r.z * sc, r.w * sm);
   dev::put_rec4(recs + static_cast<size_t>(blockIdx.x) * dev::rec_bytes(0), 0, threadIdx.x, r);
 }
 
@@ -520,8 +521,8 @@ struct LfCtx {
 // Smallest n of the pair-symmetric force (nb_symforce.cu) for the forward
 // steps, and the most scratch it may ask for (1.9 kB per particle).  A step
 // with it against the one-sided shapes, N = 16,384 / 16,385 (a block more) /
-// 20,000 / 60,000 / 131,101 / 262,144: 0.108 / 0.129 / 0.152 / 1.05 / 4.90 /
-// 19.2 ms against 0.133 / 0.137 / 0.225 / 1.61 / 6.57 / 25.8; its sums fold in
+// 20,000 / 60,000 / 131,101 / 262,144: 0.105 / 0.126 / 0.148 / 1.03 / 4.81 /
+// 18.9 ms against 0.133 / 0.137 / 0.225 / 1.61 / 6.57 / 25.8; its sums fold in
 // split precision, error against 64 bits 3 .. 4e-8 against 1.2 .. 4.6e-7.
 constexpr int64_t kLfSymMin = 16384;
 constexpr int64_t kLfSymMaxBytes = int64_t(16) << 30;
@@ -567,6 +568,7 @@ cudaError_t lf_lend(LfCtx &C, void *scratch, int64_t bytes) {
   C.S.n = C.n;
   C.S.eps2 = C.eps2;
   C.S.G = C.G;
+  C.S.sexp = sym_exponent(1.0 / static_cast<double>(C.n), C.eps2);  // masses of about 1 / n
   C.S.acc = C.S.jerk = nullptr;
   C.S.recs = b + L.recs;
   C.S.ipart = reinterpret_cast<float2 *>(b + L.ipart);
@@ -655,7 +657,8 @@ cudaError_t lf_sym_eval(LfCtx &C, const float *x_in, float *x_out, const float *
                         float *acc, float h, float dt, bool close, float *ck) {
   lf_sym_step_kernel<<<static_cast<unsigned>(C.S.n_jt), kJT, 0, C.s>>>(
       C.n, x_in, x_out, v_in, v_out, acc, h, dt, v_in ? 1 : 0, close ? 1 : 0, ck,
-      ck ? ck + 3 * C.n : nullptr, C.m, C.jhi, C.S.recs);
+      ck ? ck + 3 * C.n : nullptr, C.m, C.jhi, C.S.recs, std::ldexp(1.f, C.S.sexp),
+      std::ldexp(1.f, 3 * C.S.sexp));
   ++C.launches;
   cudaError_t e = cudaGetLastError();
   if (e != cudaSuccess) return e;

@@ -7,9 +7,9 @@
 // particles: i takes m_j / s^3 (d, c), j takes -m_i / s^3 (d, c).
 //
 // Bound: FP32 pipe and, with packed instructions holding the issue port for
-// two cycles, the issue slots of everything else.  Per pair 20
-// lane-operations are shared and 7 belong to each side: 34 for two
-// interactions against 2 x 26 in the one-sided kernel (acceleration only 17
+// two cycles, the issue slots of everything else.  Per pair 19
+// lane-operations are shared and 7 belong to each side: 33 for two
+// interactions against 2 x 26 in the one-sided kernel (acceleration only 16
 // against 2 x 12; split-precision near tiles 6 more, shared).
 //
 // Design:
@@ -38,9 +38,12 @@
 //    the fix-up adds a particle's i-side and j-side partial sums in an order
 //    fixed by the split: results are deterministic.  The scratch holds
 //    about n / 2 records per CTA (split-precision pairs: 3.9 GB at N = 1M).
-//  * One mass for all particles (EQ) leaves one product m / s^3 for both sides:
-//    32 lane-operations instead of 34, N = 1,048,576 King 622 -> 588 ms per
-//    step.
+//  * m / r^3 is m (1 / r^3) on scaled positions and masses (sym_exponent), one
+//    product less than (m y) y^2, whose FP32 range it has.  One mass for all
+//    particles (EQ) comes in after the sums and leaves one 1 / r^3 for both
+//    sides, 31 lane-operations (acceleration 14).  N = 1,048,576 King with EQ
+//    622 -> 568 ms per step (577 without the scaling), N = 65,536 acceleration
+//    (masses of a power law, near tiles) 1.68 -> 1.64 ms.
 //  * Own-block tiles take the same loop and drop the j-side sums.
 //  * Sums: near tiles fold the acceleration every 32 terms on both sides, far
 //    tiles every 64 (i) and 32 IPT (j), the jerk every 128; no FP32 sum is
@@ -58,14 +61,16 @@
 //    100,003).
 //
 // Measured (GB300, per evaluation, one-sided kernel -> this one):
-//   N = 1,048,576 King, split precision, jerk     848 -> 621 ms
-//   N = 100,003 sphere, FP32, jerk                7.86 -> 5.74 ms
-//   N = 65,536 sphere, acceleration, DS           2.39 -> 1.70 ms
-//   N = 16,384, acceleration DS / FP32            0.183 / 0.138 -> 0.150 / 0.113
+//   N = 1,048,576 King, split precision, jerk, EQ 848 -> 568 ms
+//   N = 100,003 sphere, FP32, jerk                7.86 -> 5.60 ms
+//   N = 65,536 sphere, acceleration, DS           2.39 -> 1.64 ms
+//   N = 131,101, acceleration, FP32               6.57 -> 4.81 ms
+//   N = 16,384, acceleration, FP32                0.133 -> 0.105 ms
 #include "nb_device.cuh"
 #include "nb_pipe.cuh"
 
 #include <algorithm>
+#include <cmath>
 
 namespace nbi {
 namespace {
@@ -131,22 +136,25 @@ __global__ void __launch_bounds__(kPairs) sym_records_kernel(const SymArgs A) {
   const size_t j = static_cast<size_t>(blockIdx.x) * kJT + 2 * k;
   unsigned char *t = A.recs + static_cast<size_t>(blockIdx.x) * rec_bytes(PREC);
   const float4 none = make_float4(kNowhere, kNowhere, kNowhere, 0.f);
-  auto put = [&](const float4 *src, uint32_t at, bool four) {
+  auto scaled = [](float4 p, float s, float w) {
+    return make_float4(p.x * s, p.y * s, p.z * s, p.w * w);
+  };
+  auto put = [&](const float4 *src, uint32_t at, bool four, float s) {
     const int64_t i = static_cast<int64_t>(j);
-    const float4 p = four && i >= A.n ? none : src[j];
-    const float4 q = four && i + 1 >= A.n ? none : src[j + 1];
+    const float4 p = four && i >= A.n ? none : scaled(src[j], s, A.sm);
+    const float4 q = four && i + 1 >= A.n ? none : scaled(src[j + 1], s, A.sm);
     reinterpret_cast<float4 *>(t + at)[k] = make_float4(p.x, q.x, p.y, q.y);
     if (four)
       reinterpret_cast<float4 *>(t + at + kPlane4)[k] = make_float4(p.z, q.z, p.w, q.w);
     else
       reinterpret_cast<float2 *>(t + at + kPlane4)[k] = make_float2(p.z, q.z);
   };
-  put(A.jhi, 0, true);
+  put(A.jhi, 0, true, A.sc);
   if (PREC) {
-    put(A.jlo, rec_lo(), false);
-    put(A.jrel, rec_rel(), true);
+    put(A.jlo, rec_lo(), false, A.sc);
+    put(A.jrel, rec_rel(), true, A.sc);
   }
-  if (A.jerk) put(A.jvel, rec_vel(PREC), false);
+  if (A.jerk) put(A.jvel, rec_vel(PREC), false, 1.f);
 }
 
 template <int PREC, int MASK, int JRK, int EQ, int IPT, int NT, int ST, int SACC>
@@ -259,15 +267,15 @@ __global__ void __launch_bounds__(NT, 256 / NT)
       const float4 w = JRK ? A.jvel[i] : make_float4(0.f, 0.f, 0.f, 0.f);
       const float4 l = PREC ? A.jlo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
       if (k < A.n) {
-        nxh[q][0] = -h.x; nxh[q][1] = -h.y; nxh[q][2] = -h.z;
+        nxh[q][0] = -h.x * A.sc; nxh[q][1] = -h.y * A.sc; nxh[q][2] = -h.z * A.sc;
       } else {
         nxh[q][0] = nxh[q][1] = nxh[q][2] = kNowhere;
       }
-      nxl[q][0] = -l.x; nxl[q][1] = -l.y; nxl[q][2] = -l.z;
+      nxl[q][0] = -l.x * A.sc; nxl[q][1] = -l.y * A.sc; nxl[q][2] = -l.z * A.sc;
       nvi[q][0] = -w.x; nvi[q][1] = -w.y; nvi[q][2] = -w.z;
-      mi[q] = k < A.n ? h.w : 0.f;
+      mi[q] = k < A.n ? h.w * A.sm : 0.f;
     }
-    const V veps2 = O::bc(A.eps2), meq = O::bc(A.m_eq);
+    const V veps2 = O::bc(A.eps2 * A.sc * A.sc);
     float bc_i[3] = {0.f, 0.f, 0.f}, bh_i[3] = {0.f, 0.f, 0.f};
     if (PREC) {
       // bounding box of the i-block (far test), as in the one-sided kernel
@@ -327,15 +335,15 @@ __global__ void __launch_bounds__(NT, 256 / NT)
       if (PREC && live) {
         const float4 to = __ldg(&A.tinfo[2 * jt]);
         const float4 th = __ldg(&A.tinfo[2 * jt + 1]);
-        ox[0] = to.x; ox[1] = to.y; ox[2] = to.z;
-        const float hw[3] = {th.x, th.y, th.z};
+        ox[0] = to.x * A.sc; ox[1] = to.y * A.sc; ox[2] = to.z * A.sc;
+        const float hw[3] = {th.x * A.sc, th.y * A.sc, th.z * A.sc};
         float d2 = 0.f;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
           const float d = fmaxf(0.f, fabsf(bc_i[c] - ox[c]) - (bh_i[c] + hw[c]));
           d2 = fmaf(d, d, d2);
         }
-        const float lim = kRelKappa * to.w * (1.0f + 1.0e-5f);
+        const float lim = kRelKappa * (to.w * A.sc) * (1.0f + 1.0e-5f);
         far = d2 >= lim * lim;
       }
 
@@ -413,11 +421,12 @@ __global__ void __launch_bounds__(NT, 256 / NT)
                 }
                 const V r2 = O::fma(dx, dx, O::fma(dy, dy, O::fma(dz, dz, veps2)));
                 const V y = O::template rsq<MASK>(r2);
-                const V y2 = O::mul(y, y);
-                // (m y) y^2, not m y^3: y^3 alone leaves the FP32 range for
-                // separations the product still covers
-                const V fi = O::mul(O::mul(EQ ? meq : mj, y), y2);        // on i from j
-                const V fj = EQ ? fi : O::mul(O::mul(wi[q], y), y2);      // on j from i
+                // k = y^2, f = y^3; the jerk kernel for equal masses has -3 y^2
+                // and 9 y^3 instead (the sums' factor makes up for it)
+                const V ym = EQ && JRK ? O::mul(y, O::bc(-3.f)) : y;
+                const V k2 = O::mul(ym, y), y3 = O::mul(ym, k2);
+                const V fi = EQ ? y3 : O::mul(mj, y3);    // on i from j
+                const V fj = EQ ? y3 : O::mul(wi[q], y3);  // on j from i
                 pa[q][0] = O::fma(fi, dx, pa[q][0]);
                 pa[q][1] = O::fma(fi, dy, pa[q][1]);
                 pa[q][2] = O::fma(fi, dz, pa[q][2]);
@@ -429,7 +438,7 @@ __global__ void __launch_bounds__(NT, 256 / NT)
                   V uy = O::add(vyj, vi[q][1]);
                   V uz = O::add(vzj, vi[q][2]);
                   const V rv = O::fma(dx, ux, O::fma(dy, uy, O::mul(dz, uz)));
-                  const V a3 = O::mul(O::mul(rv, y2), O::bc(-3.f));
+                  const V a3 = EQ ? O::mul(rv, k2) : O::mul(O::mul(rv, k2), O::bc(-3.f));
                   ux = O::fma(a3, dx, ux);
                   uy = O::fma(a3, dy, uy);
                   uz = O::fma(a3, dz, uz);
@@ -634,7 +643,7 @@ __global__ void __launch_bounds__(kFixP *NC) sym_fixup_kernel(const SymArgs A) {
   const int64_t i = static_cast<int64_t>(jt) * kJT + t;
   const bool real = i < A.n;
   dev::ds_add_pair(h, l, -gh, -gl, h, l);
-  double val = dev::ds_to_double(h, l, A.G);
+  double val = dev::ds_to_double(h, l, c < 3 ? A.g_acc : A.g_jerk);
   if (A.ext.on) {
     if (c < 3) s_a[c][pl] = val;
     __syncthreads();
@@ -736,9 +745,27 @@ cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq) {
                               static_cast<int>(E.smem));
 }
 
-cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
+int sym_exponent(double mean_mass, float eps2) {
+  if (!(mean_mass > 0.0) || !std::isfinite(mean_mass)) return 0;
+  int s = static_cast<int>(std::lround(std::log2(mean_mass) / -3.0));
+  // positions up to 1e13 keep a finite square, and 2^(3 s) is a float
+  s = std::max(-40, std::min(20, s));
+  if (eps2 > 0.f) {  // eps^2 stays a normal number
+    const int e = std::ilogb(eps2);
+    s = std::max(s, (-122 - e) / 2);
+    s = std::min(s, (120 - e) / 2);
+  }
+  return s;
+}
+
+cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A0, cudaStream_t s,
                              int *launches, bool with_records) {
+  SymArgs A = A0;
   const bool jrk = A.jerk != nullptr;
+  A.sc = static_cast<float>(std::ldexp(1.0, A.sexp));
+  A.sm = static_cast<float>(std::ldexp(1.0, 3 * A.sexp));
+  A.g_jerk = A.eq ? A.G * std::ldexp(A.m_eq, 3 * A.sexp) / (jrk ? 9.0 : 1.0) : A.G;
+  A.g_acc = std::ldexp(A.g_jerk, -A.sexp);
   const SymEntry &E = sym_pick(prec, mask, jrk, A.eq != 0);
   const unsigned tiles = static_cast<unsigned>(A.n_jt);
   if (with_records) {

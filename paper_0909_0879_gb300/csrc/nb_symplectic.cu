@@ -15,6 +15,8 @@
 // so a step takes S force evaluations and leaves x, v at the same instant.
 #include "nb_device.cuh"
 
+#include <cmath>
+
 namespace nbi {
 namespace {
 
@@ -39,7 +41,7 @@ __global__ void __launch_bounds__(kJT)
                       const double *__restrict__ m, int prec, float4 *__restrict__ jhi,
                       float4 *__restrict__ jlo, float4 *__restrict__ jvel,
                       float4 *__restrict__ jrel, float4 *__restrict__ tinfo,
-                      unsigned char *__restrict__ recs) {
+                      unsigned char *__restrict__ recs, float sc, float sm) {
   const int64_t j = static_cast<int64_t>(blockIdx.x) * kJT + threadIdx.x;
   const bool real = j < n;
   float4 hr = make_float4(0.f, 0.f, 0.f, 0.f), lr = hr;
@@ -76,10 +78,11 @@ __global__ void __launch_bounds__(kJT)
     const int t = threadIdx.x;
     const float4 none = make_float4(dev::kNowhere, dev::kNowhere, dev::kNowhere, 0.f);
     unsigned char *tile = recs + static_cast<size_t>(blockIdx.x) * dev::rec_bytes(prec);
-    dev::put_rec4(tile, 0, t, real ? hr : none);
+    auto scaled = [&](float4 p) { return make_float4(p.x * sc, p.y * sc, p.z * sc, p.w * sm); };
+    dev::put_rec4(tile, 0, t, real ? scaled(hr) : none);
     if (prec) {
-      dev::put_rec3(tile, dev::rec_lo(), t, lr);
-      dev::put_rec4(tile, dev::rec_rel(), t, real ? rel : none);
+      dev::put_rec3(tile, dev::rec_lo(), t, scaled(lr));
+      dev::put_rec4(tile, dev::rec_rel(), t, real ? scaled(rel) : none);
     }
   }
 }
@@ -134,10 +137,11 @@ cudaError_t launch_kick_drift(int64_t n, int64_t n_jt, double h, double d, bool 
                               const ExtField &E, const double *a, double *v, double *x,
                               const double *m, int prec, float4 *jhi, float4 *jlo,
                               float4 *jvel, float4 *jrel, float4 *tinfo, unsigned char *recs,
-                              cudaStream_t s) {
+                              int sexp, cudaStream_t s) {
   if (n_jt <= 0) return cudaSuccess;
   kick_drift_kernel<<<static_cast<unsigned>(n_jt), kJT, 0, s>>>(
-      n, h, d, rec ? 1 : 0, E, a, v, x, m, prec, jhi, jlo, jvel, jrel, tinfo, recs);
+      n, h, d, rec ? 1 : 0, E, a, v, x, m, prec, jhi, jlo, jvel, jrel, tinfo, recs,
+      std::ldexp(1.f, sexp), std::ldexp(1.f, 3 * sexp));
   return cudaGetLastError();
 }
 

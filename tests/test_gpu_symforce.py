@@ -158,3 +158,21 @@ def test_symplectic_steps_match_one_sided(nb, n, order, prec, field):
         err = np.abs(res["pairs"][k] - res["one"][k]).max()
         assert err <= bar, (k, err, bar)
     assert not np.array_equal(res["pairs"]["a"], res["one"]["a"])  # two routes
+
+
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+@pytest.mark.parametrize("equal", [False, True])
+@pytest.mark.parametrize("power", [-60, 30, 90])
+def test_scaled_masses_scale_the_sums_exactly(nb, prec, equal, power):
+    """Masses times a power of two take another internal scale of positions
+    and masses; every operation scales exactly, so the sums do too."""
+    m, x, v = _system(nb, MIN_N + 1, False, equal=equal)
+    res = []
+    for mm in (m, m * 2.0**power):
+        with nb.NBody(mm, x, v, eps=1e-3, precision=prec, block_steps=False, lev_shared=10) as s:
+            a = s.get_state(want=("a", "jerk"))
+            s.set_symplectic_layout("as_given")
+            s.symplectic(2, 0.0, 1)
+            res.append((a["a"], a["jerk"], s.get_state(want=("a",))["a"]))
+    for one, two in zip(*res):
+        assert np.array_equal(one * 2.0**power, two)
