@@ -526,7 +526,7 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
   if (c->sym_off || c->n < kSymMin) return false;
   const int prec = c->cfg.precision, mask = eps_masks(c->cfg.eps);
   SymSplit S;
-  if (!sym_split(c->n_jt, sym_block_i(prec, mask, jrk), c->num_sms, &S)) return false;
+  if (!sym_split(c->n_jt, sym_block_i(prec, mask, jrk, c->n_jt), c->num_sms, &S)) return false;
   const size_t ib = sym_ipart_bytes(S, jrk), jb = sym_jpart_bytes(S, jrk);
   const size_t rb = sym_record_bytes(c->n_jt, prec);
   if (ib > c->sym_i_cap || jb > c->sym_j_cap) {
@@ -538,8 +538,8 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
     if (ok && !c->sym_rec) ok = scratch_alloc(reinterpret_cast<void **>(&c->sym_rec), rb);
     if (ok) ok = scratch_alloc(reinterpret_cast<void **>(&ni), ib) &&
                  scratch_alloc(reinterpret_cast<void **>(&nj), jb);
-    if (ok) ok = sym_prepare(prec, mask, true, c->eq_mass) == cudaSuccess &&
-                 sym_prepare(prec, mask, false, c->eq_mass) == cudaSuccess;
+    if (ok) ok = sym_prepare(prec, mask, true, c->eq_mass, c->n_jt) == cudaSuccess &&
+                 sym_prepare(prec, mask, false, c->eq_mass, c->n_jt) == cudaSuccess;
     if (!ok) {
       cudaGetLastError();  // a refused query is not this call's error
       if (ni) cudaFree(ni);

@@ -208,14 +208,14 @@ struct SymArgs {
 // positions has the FP32 range that mass / r^3 has.
 int sym_exponent(double mean_mass, float eps2);
 // i-particles per block of the kernel for this precision / masking / output.
-int sym_block_i(int prec, int mask, bool jrk);
+int sym_block_i(int prec, int mask, bool jrk, int64_t n_jt);
 // False when n_jt tiles are too few (or too many) for a ring of such blocks.
 bool sym_split(int64_t n_jt, int bi, int ctas, SymSplit *out);
 size_t sym_record_bytes(int64_t n_jt, int prec);
 size_t sym_ipart_bytes(const SymSplit &S, bool jrk);
 size_t sym_jpart_bytes(const SymSplit &S, bool jrk);
 // Shared-memory attribute of the kernel; before its first launch or capture.
-cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq);
+cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq, int64_t n_jt);
 // with_records false: recs already hold the positions (launch_kick_drift).
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
                              int *launches, bool with_records = true);

@@ -521,8 +521,8 @@ struct LfCtx {
 // Smallest n of the pair-symmetric force (nb_symforce.cu) for the forward
 // steps, and the most scratch it may ask for (1.9 kB per particle).  A step
 // with it against the one-sided shapes, N = 16,384 / 16,385 (a block more) /
-// 20,000 / 60,000 / 131,101 / 262,144: 0.105 / 0.126 / 0.148 / 1.03 / 4.81 /
-// 18.9 ms against 0.133 / 0.137 / 0.225 / 1.61 / 6.57 / 25.8; its sums fold in
+// 20,000 / 60,000 / 131,101 / 262,144: 0.105 / 0.126 / 0.148 / 1.03 / 4.62 /
+// 17.7 ms against 0.133 / 0.137 / 0.225 / 1.61 / 6.57 / 25.8; its sums fold in
 // split precision, error against 64 bits 3 .. 4e-8 against 1.2 .. 4.6e-7.
 constexpr int64_t kLfSymMin = 16384;
 constexpr int64_t kLfSymMaxBytes = int64_t(16) << 30;
@@ -535,7 +535,7 @@ struct LfSymLayout {
 bool lf_sym_layout(int64_t n, int mask, int sms, LfSymLayout *L) {
   if (n < kLfSymMin) return false;
   const int64_t n_jt = (n + kJT - 1) / kJT;
-  if (!sym_split(n_jt, sym_block_i(0, mask, false), sms, &L->split)) return false;
+  if (!sym_split(n_jt, sym_block_i(0, mask, false, n_jt), sms, &L->split)) return false;
   auto up = [](size_t b) { return (b + 255) / 256 * 256; };
   L->recs = up(static_cast<size_t>(n_jt) * kJT * sizeof(float4));
   L->ipart = L->recs + up(sym_record_bytes(n_jt, 0));
@@ -576,7 +576,7 @@ cudaError_t lf_lend(LfCtx &C, void *scratch, int64_t bytes) {
   C.S.err = reinterpret_cast<int *>(b + L.err);
   C.S.split = L.split;
   C.sym = true;
-  cudaError_t e = sym_prepare(0, C.mask, false, false);
+  cudaError_t e = sym_prepare(0, C.mask, false, false, C.S.n_jt);
   if (e == cudaSuccess) e = cudaMemsetAsync(C.S.err, 0, sizeof(int), C.s);
   return e;
 }
@@ -817,10 +817,14 @@ int64_t nb_lf_work_floats(int64_t n, int32_t ckpt_every) {
 }
 
 int64_t nb_lf_scratch_bytes(int64_t n) {
-  LfSymLayout L;
-  return n >= kLfSymMin && n <= (int64_t(1) << 30) && lf_sym_layout(n, 0, lf_sms(), &L)
-             ? static_cast<int64_t>(L.bytes)
-             : 0;
+  int64_t most = 0;
+  if (n < kLfSymMin || n > (int64_t(1) << 30)) return 0;
+  const int sms = lf_sms();
+  for (int mask = 0; mask < 2; ++mask) {
+    LfSymLayout L;
+    if (lf_sym_layout(n, mask, sms, &L)) most = std::max(most, static_cast<int64_t>(L.bytes));
+  }
+  return most;
 }
 
 nb_status nb_lf_forward(int64_t n, const float *d_m, float *d_x, float *d_v, float *d_acc,

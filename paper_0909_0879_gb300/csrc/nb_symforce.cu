@@ -51,7 +51,8 @@
 //    fold is split precision.  Against FP64 over 12 clusters of N = 33,000
 //    (Salpeter masses): acceleration rms error 4.75e-8 against 4.79e-8
 //    one-sided, jerk 3.5e-7 against 4.9e-7.
-//  * One CTA of 8 warps per SM, IPT = 4.  The jerk kernel in split precision
+//  * One CTA of 8 warps per SM, IPT = 4 (8 for the FP32 acceleration of many
+//    particles, see sym_pick).  The jerk kernel in split precision
 //    keeps its i-side split-precision accumulators in shared memory (two
 //    copy stages make room): 41.0 against 42.0 ms (N = 262,144 King, spatial
 //    order) with them in registers.  Measured and not taken: IPT 3 / 2 with
@@ -64,7 +65,7 @@
 //   N = 1,048,576 King, split precision, jerk, EQ 848 -> 568 ms
 //   N = 100,003 sphere, FP32, jerk                7.86 -> 5.60 ms
 //   N = 65,536 sphere, acceleration, DS           2.39 -> 1.64 ms
-//   N = 131,101, acceleration, FP32               6.57 -> 4.81 ms
+//   N = 131,101, acceleration, FP32               6.57 -> 4.62 ms
 //   N = 16,384, acceleration, FP32                0.133 -> 0.105 ms
 #include "nb_device.cuh"
 #include "nb_pipe.cuh"
@@ -688,7 +689,24 @@ const SymEntry &sym_shape(int prec, int jrk) {
   return kE[prec ? 1 : 0][jrk ? 1 : 0];
 }
 
-const SymEntry &sym_pick(int prec, int mask, int jrk, bool eq) {
+// The FP32 acceleration takes eight i-particles per thread from N = 65,536
+// (generic masses: N = 65,536 1.209 -> 1.163, N = 131,101 4.81 -> 4.62, N = 262,144
+// 18.9 -> 17.7 ms): the loads, turns and address arithmetic of a record pair
+// serve twice the pairs.  Below it the ring of 2,048-particle blocks divides
+// worse (N = 16,385 0.126 against 0.144 ms, 24,000 0.193 against 0.227,
+// 60,000 1.033 against 1.037), with eps = 0 there is nothing in it (N = 65,536
+// 1.27 both), and in split precision the records' sums of 64 terms between
+// folds cost accuracy (rms 4.55e-8 against 4.27e-8, N = 66,000).
+constexpr int64_t kWideTiles = 65536 / kJT;
+
+template <int EQ>
+const SymEntry &sym_wide() {
+  static const SymEntry kE = sym_entry<0, 0, 0, EQ, 8, 256, 4, 0>();
+  return kE;
+}
+
+const SymEntry &sym_pick(int prec, int mask, int jrk, bool eq, int64_t n_jt) {
+  if (!prec && !mask && !jrk && n_jt >= kWideTiles) return eq ? sym_wide<1>() : sym_wide<0>();
   if (mask) return eq ? sym_shape<1, 1>(prec, jrk) : sym_shape<1, 0>(prec, jrk);
   return eq ? sym_shape<0, 1>(prec, jrk) : sym_shape<0, 0>(prec, jrk);
 }
@@ -734,13 +752,13 @@ size_t sym_record_bytes(int64_t n_jt, int prec) {
   return static_cast<size_t>(n_jt) * rec_bytes(prec);
 }
 
-int sym_block_i(int prec, int mask, bool jrk) {
-  const SymEntry &E = sym_pick(prec, mask, jrk, false);
+int sym_block_i(int prec, int mask, bool jrk, int64_t n_jt) {
+  const SymEntry &E = sym_pick(prec, mask, jrk, false, n_jt);
   return E.ipt * E.nt;
 }
 
-cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq) {
-  const SymEntry &E = sym_pick(prec, mask, jrk, eq);
+cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq, int64_t n_jt) {
+  const SymEntry &E = sym_pick(prec, mask, jrk, eq, n_jt);
   return cudaFuncSetAttribute(E.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(E.smem));
 }
@@ -766,7 +784,7 @@ cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A0, cudaStream_t
   A.sm = static_cast<float>(std::ldexp(1.0, 3 * A.sexp));
   A.g_jerk = A.eq ? A.G * std::ldexp(A.m_eq, 3 * A.sexp) / (jrk ? 9.0 : 1.0) : A.G;
   A.g_acc = std::ldexp(A.g_jerk, -A.sexp);
-  const SymEntry &E = sym_pick(prec, mask, jrk, A.eq != 0);
+  const SymEntry &E = sym_pick(prec, mask, jrk, A.eq != 0, A.n_jt);
   const unsigned tiles = static_cast<unsigned>(A.n_jt);
   if (with_records) {
     if (prec)

@@ -176,3 +176,27 @@ def test_scaled_masses_scale_the_sums_exactly(nb, prec, equal, power):
             res.append((a["a"], a["jerk"], s.get_state(want=("a",))["a"]))
     for one, two in zip(*res):
         assert np.array_equal(one * 2.0**power, two)
+
+
+# whole blocks of 2,048 (even ring), one particle more, a last block of two tiles
+@pytest.mark.parametrize("n", [65536, 65537, 67 * 1024 + 300])
+@pytest.mark.parametrize("equal", [False, True])
+def test_wide_blocks_against_fp64_sums(nb, n, equal):
+    """FP32 acceleration with eight i-particles per thread, sums of the same
+    FP32 inputs: a term is off by at most ~15 u, a chain of 256 terms by
+    256 u of their absolute sum (u = 2^-24)."""
+    import torch
+
+    m, x, v = (a.astype(np.float32).astype(np.float64) for a in _system(nb, n, False, equal=equal))
+    eps = 1e-2
+    with nb.NBody(m, x, v, eps=eps, precision="fp32") as s:
+        s.set_symplectic_layout("as_given")
+        s.symplectic(2, 0.0, 1)
+        got = torch.from_numpy(s.get_state(want=("a",))["a"]).cuda()
+    X, M = torch.from_numpy(x).cuda(), torch.from_numpy(m).cuda()
+    idx = torch.cat([torch.arange(64), torch.arange(n - 64, n), torch.arange(100, n, 401)]).cuda()
+    for part in idx.split(128):
+        d = X[None] - X[part][:, None]
+        t = (M * ((d * d).sum(-1) + eps * eps)**-1.5)[..., None] * d
+        err, size = (got[part] - t.sum(1)).abs(), t.abs().sum(1)
+        assert bool((err <= 271 * 2.0**-24 * size).all()), (err / size).max().item() * 2.0**24
