@@ -301,6 +301,7 @@ struct nb_ctx {
   size_t sym_i_cap = 0, sym_j_cap = 0;
   bool sym_off = false;
   bool eq_mass = false;  // every mass is m_eq
+  int small_step = -1;   // one launch per shared step: 1 yes, 0 no, -1 not yet looked at
   double m_eq = 0.0, m_mean = 0.0;
   double *red = nullptr;        // energy scratch
   unsigned char *en_rec = nullptr;  // records of the split-precision energy
@@ -994,6 +995,67 @@ nb_status force_active(nb_ctx *c, int64_t n_idx, bool rows, EndArgs *end = nullp
   return s;
 }
 
+// Whether this step (of every particle, nb_next_block has just found it) is
+// one launch: a small system with shared steps and the built-in force shape.
+bool takes_small_step(nb_ctx *c) {
+  if (!c->uniform || c->sh.p > 1 || c->variant_override >= 0 || c->table_count > 0 ||
+      c->grid_cap > 0)
+    return false;
+  if (c->small_step < 0) {
+    int dev = 0, coop = 0, smem = 0;
+    const int prec = c->cfg.precision;
+    const bool ok =
+        small_step_fits(c->n, c->n_jt, prec, eps_masks(c->cfg.eps), c->num_sms) &&
+        cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+        cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) ==
+            cudaSuccess &&
+        small_step_smem(c->n_jt, prec) + 2048 <= static_cast<size_t>(smem) &&
+        small_step_prepare(c->n_jt, prec) == cudaSuccess;
+    c->small_step = ok ? 1 : 0;
+  }
+  return c->small_step == 1;
+}
+
+nb_status queue_small_step(nb_ctx *c) {
+  Range r("nb_step");
+  SmallStepArgs A;
+  A.n = c->n;
+  A.n_jt = c->n_jt;
+  A.t_next = c->t_block;
+  A.x = c->x;
+  A.v = c->v;
+  A.a = c->a;
+  A.jk = c->jk;
+  A.m = c->m;
+  A.t_tick = c->t_tick;
+  A.lev = c->lev;
+  A.jhi = c->jhi;
+  A.jlo = c->jlo;
+  A.jvel = c->jvel;
+  A.jrel = c->jrel;
+  A.tinfo = c->tinfo;
+  A.eps2 = eps2_f32(c->cfg.eps);
+  A.G = c->cfg.G;
+  A.P = force_grid(choose_variant(c->cfg.precision, 0, c->n, c->n_jt, c->num_sms), c->n, c->n_jt,
+                   c->num_sms, 0);
+  A.err = c->err;
+  A.bar = reinterpret_cast<unsigned long long *>(c->scal + kCtlBar);
+  A.eta = c->cfg.eta;
+  A.lev_min = c->cfg.lev_min;
+  A.lev_max = c->cfg.lev_max;
+  A.n_clamped = c->clamped;
+  A.ext = c->ext;
+  NB_CUDA(launch_small_step(A, c->cfg.precision, c->stream));
+  c->launches += 1;
+  c->interactions += c->n * c->n;
+  c->t_pred = c->t_block;
+  c->force_done = false;
+  c->have_block = false;
+  c->u_tick = c->t_block;
+  return NB_OK;
+}
+
 }  // namespace
 
 extern "C" {
@@ -1119,6 +1181,13 @@ nb_status nb_step(nb_ctx *c, double *t_next, int64_t *n_active) {
   int64_t na;
   nb_status s = nb_next_block(c, &tn, &na);
   if (s != NB_OK) return s;
+  if (takes_small_step(c)) {
+    s = queue_small_step(c);
+    if (s != NB_OK) return s;
+    if (t_next) *t_next = tn;
+    if (n_active) *n_active = na;
+    return NB_OK;
+  }
   s = nb_predict(c, tn);
   if (s != NB_OK) return s;
   const int64_t short_list = static_cast<int64_t>(kEndThreads / 32) * 2 * c->num_sms;

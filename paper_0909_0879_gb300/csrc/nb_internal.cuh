@@ -81,6 +81,7 @@ constexpr int kCtlTicket = 9;   // CTA tickets of the fused block-begin kernel
 constexpr int kCtlBad = 10;     // nonzero: the schedule is not level-structured
 constexpr int kCtlTcur = 11;    // latest particle time (ticks), from the check
 constexpr int kCtlLevCnt = 16;  // kTicksLog2 + 1 slots: particles per level
+constexpr int kCtlBar = 38;     // arrivals at the small step's grid barrier
 constexpr int kCtlSlots = 40;
 
 // Device error-word bit of a timed-out look-back in the fused compaction.
@@ -219,6 +220,30 @@ cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq, int64_t n_jt);
 // with_records false: recs already hold the positions (launch_kick_drift).
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
                              int *launches, bool with_records = true);
+
+// --- one shared step of a small system in one launch (nb_smallstep.cu) ---
+struct SmallStepArgs {
+  int64_t n, n_jt, t_next;
+  double *x, *v, *a, *jk;
+  const double *m;
+  int64_t *t_tick;
+  int32_t *lev;
+  float4 *jhi, *jlo, *jvel, *jrel, *tinfo;
+  float eps2;
+  double G;
+  int P;  // CTAs of the short-list force shape, whose sums these are
+  int *err;
+  unsigned long long *bar;
+  double eta;
+  int lev_min, lev_max;
+  unsigned long long *n_clamped;
+  ExtField ext;
+};
+// Whether n particles run the short-list force shape and fit the SMs.
+bool small_step_fits(int64_t n, int64_t n_jt, int prec, int mask, int num_sms);
+size_t small_step_smem(int64_t n_jt, int prec);
+cudaError_t small_step_prepare(int64_t n_jt, int prec);
+cudaError_t launch_small_step(const SmallStepArgs &A, int prec, cudaStream_t s);
 
 // --- Hermite and bookkeeping kernels (nb_hermite.cu) ---
 // The j-records of every particle at t_next and, with jrel set, per

@@ -575,3 +575,33 @@ def test_shared_steps_without_a_look_at_the_schedule(nb, n):
         for k in sa:
             assert np.array_equal(sa[k], sb[k]), k
         assert a.step()[0] == 6 * 2.0**-9
+
+
+# a particle, a partial and a whole i-block of 16, tile edges, N = 1024, the
+# most i-blocks that fit one per SM, and just past them (separate launches)
+@pytest.mark.parametrize("n", [2, 15, 16, 17, 255, 257, 1024, 2203, 2304, 2500])
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+@pytest.mark.parametrize("field", [False, True])
+def test_small_step_bitwise_equals_separate_launches(nb, n, prec, field):
+    m, x, v = ics.plummer(n, 50 + n, masses=ics.salpeter_masses(n, n))
+    kw = dict(eps=1e-2, precision=prec, block_steps=False, lev_shared=9)
+    keys = ("x", "v", "a", "jerk", "t_tick", "lev")
+    with nb.NBody(m, x, v, **kw) as s, nb.NBody(m, x, v, **kw) as o:
+        if field:
+            s.set_external({})
+            o.set_external({})
+        idx = np.arange(0, n, 3, dtype=np.int32)
+        for _ in range(3):
+            t, na = s.step()
+            t2, na2 = o.next_block()
+            o.predict(t2)
+            o.force_jerk()
+            a2, j2 = o.force_jerk(idx)
+            o.correct(t2)
+            assert (t, na) == (t2, na2)
+            # the prediction stays in place for calls that follow
+            a1, j1 = s.force_jerk(idx)
+            assert np.array_equal(a1, a2) and np.array_equal(j1, j2)
+        p, q = s.get_state(want=keys), o.get_state(want=keys)
+    for k in keys:
+        assert np.array_equal(p[k], q[k]), k
