@@ -1010,8 +1010,8 @@ bool takes_small_step(nb_ctx *c) {
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
         cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) ==
             cudaSuccess &&
-        small_step_smem(c->n_jt, prec) + 2048 <= static_cast<size_t>(smem) &&
-        small_step_prepare(c->n_jt, prec) == cudaSuccess;
+        small_step_smem(c->n_jt, prec) + 16384 <= static_cast<size_t>(smem) &&
+        small_step_prepare(c->n, c->n_jt, prec, c->num_sms) == cudaSuccess;
     c->small_step = ok ? 1 : 0;
   }
   return c->small_step == 1;
@@ -1046,7 +1046,7 @@ nb_status queue_small_step(nb_ctx *c) {
   A.lev_max = c->cfg.lev_max;
   A.n_clamped = c->clamped;
   A.ext = c->ext;
-  NB_CUDA(launch_small_step(A, c->cfg.precision, c->stream));
+  NB_CUDA(launch_small_step(A, c->cfg.precision, c->num_sms, c->stream));
   c->launches += 1;
   c->interactions += c->n * c->n;
   c->t_pred = c->t_block;

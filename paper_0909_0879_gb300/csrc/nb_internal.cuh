@@ -242,8 +242,8 @@ struct SmallStepArgs {
 // Whether n particles run the short-list force shape and fit the SMs.
 bool small_step_fits(int64_t n, int64_t n_jt, int prec, int mask, int num_sms);
 size_t small_step_smem(int64_t n_jt, int prec);
-cudaError_t small_step_prepare(int64_t n_jt, int prec);
-cudaError_t launch_small_step(const SmallStepArgs &A, int prec, cudaStream_t s);
+cudaError_t small_step_prepare(int64_t n, int64_t n_jt, int prec, int num_sms);
+cudaError_t launch_small_step(const SmallStepArgs &A, int prec, int num_sms, cudaStream_t s);
 
 // --- Hermite and bookkeeping kernels (nb_hermite.cu) ---
 // The j-records of every particle at t_next and, with jrel set, per
