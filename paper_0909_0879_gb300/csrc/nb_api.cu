@@ -1199,8 +1199,8 @@ nb_status nb_step(nb_ctx *c, double *t_next, int64_t *n_active) {
   } else {
     // short lists, up to one particle per warp of the block-end kernel: the
     // fix-up of split i-blocks and the corrector in one launch, the arithmetic
-    // of nb_force_jerk_dev and nb_correct (N = 1024 shared steps: 29 -> 20 us
-    // per step; longer lists are 1 % slower that way)
+    // of nb_force_jerk_dev and nb_correct (1,024 particles: 29 -> 20 us per
+    // step; longer lists are 1 % slower that way)
     EndArgs E = end_args(c);
     E.ctl = nullptr;
     E.sp4 = nullptr;  // rebuilt by nb_run_blocks

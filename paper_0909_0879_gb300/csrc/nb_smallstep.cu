@@ -8,7 +8,7 @@
 // records, through global memory and one grid barrier (cooperative launch: all
 // CTAs are resident).  Split precision, per step: N = 256 12.4 us, N = 1,024
 // 14.4 us (18.4 with 16 particles per CTA), N = 2,048 22.6 us; FP32 12.3 / 14.4 /
-// 20.5 us.  Up to 2,280 particles, as many as the SMs hold at 16 each.
+// 20.5 us.  Up to 2,288 particles, as many as the SMs hold at 16 each.
 //
 // The sums are those of the short-list force shape (a warp per i-particle,
 // 8 records per lane and tile), segment by segment of its split over CTAs, and
