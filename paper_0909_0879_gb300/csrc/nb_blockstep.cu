@@ -304,7 +304,7 @@ struct EndStage {
 // One round of block_end over the entries k0 .. k0 + NQ * kEndWarps - 1:
 // the warps add the split partial sums of NQ entries each, then warp 0
 // corrects the round's entries, a lane each.
-template <int NQ>
+template <int NQ, bool HOST>
 __device__ __forceinline__ void end_round(const EndArgs &E, int64_t k0, int64_t n_act,
                                           int64_t t_next, int BI, uint64_t U, int P,
                                           EndStage &sg) {
@@ -383,21 +383,26 @@ __device__ __forceinline__ void end_round(const EndArgs &E, int64_t k0, int64_t 
     const unsigned mask = nv >= 10 ? 0x3fffffffu : ((1u << (3 * nv)) - 1u);
     dev::correct_vals3(cq, mask, lane - cq, ci, st, an, jn, t_next, E.x, E.v, E.a, E.jk,
                        E.t_tick, E.lev, E.eta, E.lev_min, E.lev_max, E.block_steps,
-                       E.n_clamped, E.ctl ? E.ctl + kCtlLevCnt : nullptr, &E.ext, E.sp4, E.sp2);
+                       E.n_clamped, HOST ? nullptr : E.ctl + kCtlLevCnt, &E.ext, E.sp4, E.sp2);
   }
   __syncthreads();
 }
 
+// HOST: a host-driven step, whose time, count and split are arguments (as
+// run-time cases of one kernel they cost the device-driven step 0.4 us, 3 % of
+// a step at N = 3,018); WHOLE: steps of all particles may come from the
+// pair-symmetric kernel.
+template <bool HOST, bool WHOLE>
 __global__ void __launch_bounds__(kEndThreads) block_end_kernel(const EndArgs E) {
   __shared__ EndStage sg;
-  int64_t t_next = E.t_next, n_act = E.n_act;
+  const int64_t t_next = HOST ? E.t_next : E.ctl[kCtlTnext];
+  if (t_next < 0) return;
+  const int64_t n_act = HOST ? E.n_act : E.ctl[kCtlNact];
   int BI = E.h_bi, P = E.h_p;
-  uint64_t U = dev::udiv(static_cast<uint64_t>(n_act + BI - 1), BI) *
-               static_cast<uint64_t>(E.n_jt);
-  if (E.ctl) {
-    t_next = E.ctl[kCtlTnext];
-    if (t_next < 0) return;
-    n_act = E.ctl[kCtlNact];
+  uint64_t U;
+  if (HOST) {
+    U = dev::udiv(static_cast<uint64_t>(n_act + BI - 1), BI) * static_cast<uint64_t>(E.n_jt);
+  } else {
     if (blockIdx.x == 0 && threadIdx.x == 0) {
       // reductions without a return value: the thread does not wait for a
       // round trip before its CTA's corrector work
@@ -409,7 +414,7 @@ __global__ void __launch_bounds__(kEndThreads) block_end_kernel(const EndArgs E)
     int b = -1;
     for (int q = 0; q < E.nbk; ++q)
       if (n_act >= E.lo[q] && n_act < E.hi[q]) b = q;
-    const bool whole = b < 0 && E.sym_all && n_act == E.n;
+    const bool whole = WHOLE && b < 0 && n_act == E.n;
     if (b < 0 && !whole) return;
     // the split the force launch of this bucket derived from the same count;
     // one CTA for everything (no split i-block) where the pair-symmetric
@@ -426,11 +431,11 @@ __global__ void __launch_bounds__(kEndThreads) block_end_kernel(const EndArgs E)
   if (n_act <= static_cast<int64_t>(kEndWarps) * gridDim.x) {
     for (int64_t k0 = static_cast<int64_t>(blockIdx.x) * kEndWarps; k0 < n_act;
          k0 += static_cast<int64_t>(gridDim.x) * kEndWarps)
-      end_round<1>(E, k0, n_act, t_next, BI, U, P, sg);
+      end_round<1, HOST>(E, k0, n_act, t_next, BI, U, P, sg);
   } else {
     for (int64_t k0 = static_cast<int64_t>(blockIdx.x) * 4 * kEndWarps; k0 < n_act;
          k0 += static_cast<int64_t>(gridDim.x) * 4 * kEndWarps)
-      end_round<4>(E, k0, n_act, t_next, BI, U, P, sg);
+      end_round<4, HOST>(E, k0, n_act, t_next, BI, U, P, sg);
   }
 }
 
@@ -543,7 +548,13 @@ cudaError_t launch_block_begin(const BeginArgs &B, cudaStream_t s) {
 }
 
 cudaError_t launch_block_end(const EndArgs &E, int grid, cudaStream_t s) {
-  block_end_kernel<<<static_cast<unsigned>(grid), kEndThreads, 0, s>>>(E);
+  const unsigned g = static_cast<unsigned>(grid);
+  if (!E.ctl)
+    block_end_kernel<true, false><<<g, kEndThreads, 0, s>>>(E);
+  else if (E.sym_all)
+    block_end_kernel<false, true><<<g, kEndThreads, 0, s>>>(E);
+  else
+    block_end_kernel<false, false><<<g, kEndThreads, 0, s>>>(E);
   return cudaGetLastError();
 }
 
