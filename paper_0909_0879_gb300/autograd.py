@@ -14,10 +14,13 @@ import torch
 from . import _lib
 
 
+_SCRATCH_FROM = 16384  # _lib.lf_scratch_bytes(n) is 0 below (spares small systems the call)
+
+
 def _scratch(n, device):
     """Memory for the pair-symmetric force, or None (small n, or no room: the
     one-sided force needs none)."""
-    size = _lib.lf_scratch_bytes(n)
+    size = _lib.lf_scratch_bytes(n) if n >= _SCRATCH_FROM else 0
     if size == 0:
         return None
     try:
