@@ -121,8 +121,9 @@ nb_status nb_force_jerk(nb_ctx *ctx, const int32_t *idx, int64_t n_idx,
  * which case the result is kept only for nb_correct).  Indices are not
  * range-checked on the device: an out-of-range index is undefined behaviour.
  *
- * In a context with shared steps (block_steps == 0) and n >= 16384 a step of
- * all particles whose rows are not handed out (d_idx, d_acc and d_jerk NULL,
+ * In a context with shared steps (block_steps == 0) and enough particles
+ * (n >= 16384, and where its work divides well over the GPU from n = 6.7e3) a
+ * step of all particles whose rows are not handed out (d_idx, d_acc and d_jerk NULL,
  * as nb_step calls it; also nb_init and nb_run_blocks) evaluates each pair
  * once for both particles; rows that are handed out are the one-sided
  * kernel's, the same for any list a particle stands in.  The two differ by
@@ -184,8 +185,8 @@ nb_status nb_last_block_path(nb_ctx *ctx, int32_t *fused);
  * backwards) of the scheme of the given order, on the context's FP64
  * state with forces in its precision (FP32 or split precision, softening
  * eps, no jerk; the built-in force shapes, not a forced variant or an
- * installed tuning table; from n = 16384 on each pair is evaluated once for
- * both particles, see nb_force_jerk_dev).
+ * installed tuning table; with enough particles each pair is evaluated once
+ * for both, see nb_force_jerk_dev).
  *   order 2: kick-drift-kick leapfrog, one force evaluation per step;
  *   order 6: the symmetric composition of seven leapfrog steps of lengths
  *            w_k dt with the sixth-order weights of Kinoshita, Yoshida &

@@ -515,19 +515,31 @@ nb_status ensure_part(nb_ctx *c, size_t bytes) {
   return NB_OK;
 }
 
-// Smallest n of the pair-symmetric force.  Below it the ring has too few
-// tiles per CTA: N = 12,000 0.205 ms against 0.193 one-sided (split
-// precision, jerk), N = 16,384 0.261 against 0.308.
+// From kSymMin the pair-symmetric force is always the faster one.  Below it
+// its time goes with the units (1,024 x 256 pairs) of the fullest CTA, in steps,
+// and the one-sided kernel's with n^2: it is taken where n^2 exceeds 0.56 of
+// the interactions that a CTA per SM would do with that many units (the line of
+// the tightest case, jerk in split precision with eps > 0; N = 7,168 / 8,192 /
+// 9,000 / 10,240 / 12,000 / 15,000: 80 / 80 / 129 / 131 / 177 / 224 us against
+// 83 / 102 / 118 / 146 / 187 / 260 one-sided, acceleration 43 / 45 / 72 / 74 /
+// 103 / 131 against 56 / 68 / 78 / 97 / 124 / 160).
 constexpr int64_t kSymMin = 16384;
+
+bool sym_pays(int64_t n, const SymSplit &S, int bi, int num_sms) {
+  if (n >= kSymMin) return true;
+  const double most = static_cast<double>((S.units + S.ctas - 1) / S.ctas);
+  return static_cast<double>(n) * n >= 0.56 * 2.0 * most * num_sms * bi * kJT;
+}
 
 // The split and scratch of the pair-symmetric force of all particles; false
 // when this context does not take it: too few particles, or no room for
 // its partial sums (at most 1/16 of the device's memory).
 bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
-  if (c->sym_off || c->n < kSymMin) return false;
+  if (c->sym_off) return false;
   const int prec = c->cfg.precision, mask = eps_masks(c->cfg.eps);
   SymSplit S;
-  if (!sym_split(c->n_jt, sym_block_i(prec, mask, jrk, c->n_jt), c->num_sms, &S)) return false;
+  const int bi = sym_block_i(prec, mask, jrk, c->n_jt);
+  if (!sym_split(c->n_jt, bi, c->num_sms, &S) || !sym_pays(c->n, S, bi, c->num_sms)) return false;
   const size_t ib = sym_ipart_bytes(S, jrk), jb = sym_jpart_bytes(S, jrk);
   const size_t rb = sym_record_bytes(c->n_jt, prec);
   if (ib > c->sym_i_cap || jb > c->sym_j_cap) {
@@ -837,10 +849,15 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x,
   c->launches += 1;
   TRY(queue_predict(c, 0));
   SymArgs SA;
-  if (sym_hermite(c, &SA))
+  if (sym_hermite(c, &SA)) {
     TRY(queue_sym(c, SA, c->a, c->jk));
-  else
+  } else {
     TRY(queue_force(c, nullptr, n, c->a, c->jk));
+    // Scratch for symplectic steps of a middle-sized system (at most 40 MB)
+    // now: allocated by the first of them it made that call 0.1 ms longer,
+    // more than the kernel saves in it (N = 7,000: 239 -> 344 us).
+    if (n < kSymMin) sym_ready(c, false, &SA);
+  }
   TRYC(launch_init_levels(n, c->a, c->jk, cfg->eta_start, cfg->lev_min, cfg->lev_max,
                           cfg->block_steps, cfg->lev_shared, c->lev, c->t_tick, st));
   c->launches += 1;

@@ -200,3 +200,26 @@ def test_wide_blocks_against_fp64_sums(nb, n, equal):
         t = (M * ((d * d).sum(-1) + eps * eps)**-1.5)[..., None] * d
         err, size = (got[part] - t.sum(1)).abs(), t.abs().sum(1)
         assert bool((err <= 271 * 2.0**-24 * size).all()), (err / size).max().item() * 2.0**24
+
+
+# below MIN_N the pair-symmetric kernel runs where its units divide well:
+# (7,168 and 8,192: one per CTA; 9,000: two for 180 units on 152 SMs, left to
+# the one-sided kernel; 12,289: a last block of one particle)
+@pytest.mark.parametrize("n,taken", [(6000, False), (7168, True), (8192, True), (9000, False),
+                                     (12289, True), (MIN_N - 1, True)])
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+def test_middle_sizes(nb, oracle_mod, n, taken, prec):
+    m, x, v = _system(nb, n, False)
+    with nb.NBody(m, x, v, eps=1e-3, precision=prec, block_steps=False, lev_shared=10) as s:
+        got = s.get_state(want=("a", "jerk"))
+    with nb.NBody(m, x, v, eps=1e-3, precision=prec) as s:
+        one = s.get_state(want=("a", "jerk"))
+    import torch
+
+    if torch.cuda.get_device_properties(0).multi_processor_count == 152:
+        assert np.array_equal(got["a"], one["a"]) != taken
+    idx = np.arange(0, n, 7, dtype=np.int32)
+    ra, rj = oracle_mod.force_jerk(m, x, v, 1e-3, idx=idx)
+    ta, tj = TOL[prec]
+    assert np.linalg.norm(got["a"][idx] - ra) <= ta * np.linalg.norm(ra)
+    assert np.linalg.norm(got["jerk"][idx] - rj) <= tj * np.linalg.norm(rj)
