@@ -853,10 +853,11 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x,
     TRY(queue_sym(c, SA, c->a, c->jk));
   } else {
     TRY(queue_force(c, nullptr, n, c->a, c->jk));
-    // Scratch for symplectic steps of a middle-sized system (at most 40 MB)
-    // now: allocated by the first of them it made that call 0.1 ms longer,
-    // more than the kernel saves in it (N = 7,000: 239 -> 344 us).
-    if (n < kSymMin) sym_ready(c, false, &SA);
+    // Scratch for symplectic steps of a middle-sized system (at most 80 MB)
+    // now: allocated by the first of them it made that call 0.1 .. 0.2 ms
+    // longer, more than the kernel saves in it (N = 7,000 239 -> 344 us, N =
+    // 20,000 482 -> 521 us; from 40,000 on the call still gains).
+    if (n < 2 * kSymMin) sym_ready(c, false, &SA);
   }
   TRYC(launch_init_levels(n, c->a, c->jk, cfg->eta_start, cfg->lev_min, cfg->lev_max,
                           cfg->block_steps, cfg->lev_shared, c->lev, c->t_tick, st));
