@@ -1892,6 +1892,29 @@ extern "C" nb_status nb_run_blocks(nb_ctx *c, double t_end, int64_t max_blocks,
   if (max_blocks < 0) return fail(NB_ERR_INVALID_ARG, "negative block budget");
   s = relayout_if_due(c);
   if (s != NB_OK) return s;
+  if (c->block_mode == 0 && !c->inject_lookback && takes_small_step(c)) {
+    // a small system's shared steps: one launch each, their times known here
+    // (N = 1,024: 20.7 us per step with the graph below -> 14.4)
+    const int64_t step = int64_t(1) << (kTicksLog2 - c->u_lev);
+    int64_t done = 0;
+    while ((max_blocks == 0 || done < max_blocks) && c->u_tick + step <= tend) {
+      c->t_block = c->u_tick + step;
+      s = queue_small_step(c);
+      if (s != NB_OK) return s;
+      if (++done % 256 == 0 && (s = sync_ctx(c)) != NB_OK) return s;
+    }
+    s = sync_ctx(c);
+    if (s != NB_OK) return s;
+    c->n_blocks += done;
+    if (done > 0) c->fresh = false;
+    c->have_block = false;
+    c->force_done = false;
+    c->t_pred = -1;
+    c->last_fused = 1;
+    if (blocks_done) *blocks_done = done;
+    if (t_last) *t_last = std::ldexp(static_cast<double>(c->u_tick), -kTicksLog2);
+    return NB_OK;
+  }
   // partial-sum scratch for every shape the device-resident steps may run
   size_t pb = 0;
   {

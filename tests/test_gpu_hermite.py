@@ -605,3 +605,20 @@ def test_small_step_bitwise_equals_separate_launches(nb, n, prec, field):
         p, q = s.get_state(want=keys), o.get_state(want=keys)
     for k in keys:
         assert np.array_equal(p[k], q[k]), k
+
+
+@pytest.mark.parametrize("n,prec", [(300, "ds"), (1024, "fp32")])
+def test_small_run_blocks_equals_general_path(nb, n, prec):
+    """Shared steps of a small system in nb_run_blocks: t_end, the block
+    budget, counts and states as the general device-resident path's."""
+    m, x, v = ics.plummer(n, 77)
+    kw = dict(eps=1e-2, precision=prec, block_steps=False, lev_shared=8)
+    dt = 2.0**-8
+    with nb.NBody(m, x, v, **kw) as s, nb.NBody(m, x, v, **kw) as o:
+        o.set_block_mode("general")
+        for t_end, most in ((0.0, 0), (4.5 * dt, 0), (1.0, 3), (7 * dt, 5), (300 * dt, 0)):
+            assert s.run_blocks(t_end, max_blocks=most) == o.run_blocks(t_end, max_blocks=most)
+        p, q = s.get_state(), o.get_state()
+        for k in p:
+            assert np.array_equal(p[k], q[k]), k
+        assert s.step() == o.step()
