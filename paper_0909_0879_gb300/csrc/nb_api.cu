@@ -1028,7 +1028,7 @@ bool takes_small_step(nb_ctx *c) {
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
         cudaDeviceGetAttribute(&smem, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) ==
             cudaSuccess &&
-        small_step_smem(c->n_jt, prec) + 16384 <= static_cast<size_t>(smem) &&
+        small_step_smem(c->n_jt, prec) + 28672 <= static_cast<size_t>(smem) &&
         small_step_prepare(c->n, c->n_jt, prec, c->num_sms) == cudaSuccess;
     c->small_step = ok ? 1 : 0;
   }

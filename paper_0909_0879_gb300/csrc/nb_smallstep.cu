@@ -8,7 +8,9 @@
 // records, through global memory and one grid barrier (cooperative launch: all
 // CTAs are resident).  Split precision, per step: N = 256 12.4 us, N = 1,024
 // 14.4 us (18.4 with 16 particles per CTA), N = 2,048 22.6 us; FP32 12.3 / 14.4 /
-// 20.5 us.  Up to 2,288 particles, as many as the SMs hold at 16 each.
+// 20.5 us.  Up to 2,288 particles the SMs hold them at 16 each, from there to
+// 4,096 (the records' shared memory) at 32, two per warp: N = 2,500 / 3,000 /
+// 4,096 38.9 / 45.1 / 61.3 us with three launches -> 34.8 / 38.9 / 45.1.
 //
 // The sums are those of the short-list force shape (a warp per i-particle,
 // 8 records per lane and tile), segment by segment of its split over CTAs, and
@@ -44,11 +46,12 @@ __device__ __forceinline__ bool grid_barrier(unsigned long long *bar) {
   return s_ok != 0;
 }
 
-// NI i-particles per CTA, 16 / NI warps each: the segments of the split go to
-// the warps in turn.
+// NI i-particles per CTA: 16 / NI warps each, the segments of the split going to
+// the warps in turn, or NI / 16 per warp.
 template <int PREC, int NI>
 __global__ void __launch_bounds__(32 * kWarps, 1) small_step_kernel(const SmallStepArgs A) {
-  constexpr int WPI = kWarps / NI;
+  constexpr int WPI = NI < kWarps ? kWarps / NI : 1, IPW = NI > kWarps ? NI / kWarps : 1;
+  static_assert(NI <= 32, "the prediction is one warp's");
   using O = dev::VOps<float>;
   extern __shared__ __align__(16) float4 rec[];
   __shared__ double s_f[NI][6];
@@ -90,98 +93,125 @@ __global__ void __launch_bounds__(32 * kWarps, 1) small_step_kernel(const SmallS
   }
   __syncthreads();
 
-  // the segments of the i-block's tiles: owners plo .. phi of the split
-  const uint64_t U = static_cast<uint64_t>((n + kBlock - 1) / kBlock) * n_jt;
-  const uint64_t u0 = static_cast<uint64_t>(k0 / kBlock) * n_jt;
+  // the segments of the i-block's tiles: owners plo .. phi of the split (a
+  // warp's particles lie in one i-block of 16)
+  const int blocks = (n + kBlock - 1) / kBlock;
+  const uint64_t U = static_cast<uint64_t>(blocks) * n_jt;
+  const int blk = NI <= kBlock ? k0 / kBlock  // (the last: warps past n)
+                               : min((k0 + wid / WPI * IPW) / kBlock, blocks - 1);
+  const uint64_t u0 = static_cast<uint64_t>(blk) * n_jt;
   const int plo = dev::owner_of(u0, U, A.P), phi = dev::owner_of(u0 + n_jt - 1, U, A.P);
   {
-    const int e = wid / WPI, k = k0 + e;
-    const int i = k < n ? k : 0;
-    const float4 hi = s_hi[i], wi = s_v[i];
-    const float4 li = PREC ? s_lo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
-    const float nx[3] = {-hi.x, -hi.y, -hi.z}, nl[3] = {-li.x, -li.y, -li.z};
-    const float nv[3] = {-wi.x, -wi.y, -wi.z};
+    const int e0 = wid / WPI * IPW;
+    float nx[IPW][3], nl[IPW][3], nv[IPW][3];
+#pragma unroll
+    for (int w = 0; w < IPW; ++w) {
+      const int i = k0 + e0 + w < n ? k0 + e0 + w : 0;
+      const float4 hi = s_hi[i], wi = s_v[i];
+      const float4 li = PREC ? s_lo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+      nx[w][0] = -hi.x, nx[w][1] = -hi.y, nx[w][2] = -hi.z;
+      nl[w][0] = -li.x, nl[w][1] = -li.y, nl[w][2] = -li.z;
+      nv[w][0] = -wi.x, nv[w][1] = -wi.y, nv[w][2] = -wi.z;
+    }
     int t0 = 0;
     for (int p = plo; p <= phi; ++p) {
       const uint64_t ue = dev::udiv(U * static_cast<uint64_t>(p + 1), static_cast<uint64_t>(A.P));
       const int t1 = p == phi ? n_jt : static_cast<int>(ue - u0);
       if ((p - plo) % WPI == wid % WPI) {
-        float sh[6], sl[6];
+        float sh[IPW][6], sl[IPW][6];
 #pragma unroll
-        for (int c = 0; c < 6; ++c) sh[c] = sl[c] = 0.f;
+        for (int w = 0; w < IPW; ++w)
+#pragma unroll
+          for (int c = 0; c < 6; ++c) sh[w][c] = sl[w][c] = 0.f;
         for (int jt = t0; jt < t1; ++jt) {
-          float pa[3] = {0.f, 0.f, 0.f}, p1[3] = {0.f, 0.f, 0.f}, p2[3] = {0.f, 0.f, 0.f};
+          float pa[IPW][3], p1[IPW][3], p2[IPW][3];
+#pragma unroll
+          for (int w = 0; w < IPW; ++w)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) pa[w][c] = p1[w][c] = p2[w][c] = 0.f;
 #pragma unroll
           for (int q = 0; q < kJT / 32; ++q) {
             const int j = jt * kJT + q * 32 + lane;
             const float4 hj = s_hi[j], wj = s_v[j];
-            float dx, dy, dz;
-            if (PREC) {
-              const float4 lj = s_lo[j];
-              dx = O::add(O::add(hj.x, nx[0]), O::add(lj.x, nl[0]));
-              dy = O::add(O::add(hj.y, nx[1]), O::add(lj.y, nl[1]));
-              dz = O::add(O::add(hj.z, nx[2]), O::add(lj.z, nl[2]));
-            } else {
-              dx = O::add(hj.x, nx[0]);
-              dy = O::add(hj.y, nx[1]);
-              dz = O::add(hj.z, nx[2]);
+            const float4 lj = PREC ? s_lo[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+            for (int w = 0; w < IPW; ++w) {
+              float dx, dy, dz;
+              if (PREC) {
+                dx = O::add(O::add(hj.x, nx[w][0]), O::add(lj.x, nl[w][0]));
+                dy = O::add(O::add(hj.y, nx[w][1]), O::add(lj.y, nl[w][1]));
+                dz = O::add(O::add(hj.z, nx[w][2]), O::add(lj.z, nl[w][2]));
+              } else {
+                dx = O::add(hj.x, nx[w][0]);
+                dy = O::add(hj.y, nx[w][1]);
+                dz = O::add(hj.z, nx[w][2]);
+              }
+              const float ux = O::add(wj.x, nv[w][0]), uy = O::add(wj.y, nv[w][1]),
+                          uz = O::add(wj.z, nv[w][2]);
+              const float r2 = O::fma(dx, dx, O::fma(dy, dy, O::fma(dz, dz, A.eps2)));
+              const float rinv = O::rsq<0>(r2);
+              const float rinv2 = O::mul(rinv, rinv);
+              const float mr3 = O::mul(O::mul(hj.w, rinv), rinv2);
+              const float rv = O::fma(dx, ux, O::fma(dy, uy, O::mul(dz, uz)));
+              const float cc = O::mul(O::mul(rv, rinv2), mr3);
+              pa[w][0] = O::fma(mr3, dx, pa[w][0]);
+              pa[w][1] = O::fma(mr3, dy, pa[w][1]);
+              pa[w][2] = O::fma(mr3, dz, pa[w][2]);
+              p1[w][0] = O::fma(mr3, ux, p1[w][0]);
+              p1[w][1] = O::fma(mr3, uy, p1[w][1]);
+              p1[w][2] = O::fma(mr3, uz, p1[w][2]);
+              p2[w][0] = O::fma(cc, dx, p2[w][0]);
+              p2[w][1] = O::fma(cc, dy, p2[w][1]);
+              p2[w][2] = O::fma(cc, dz, p2[w][2]);
             }
-            const float ux = O::add(wj.x, nv[0]), uy = O::add(wj.y, nv[1]), uz = O::add(wj.z, nv[2]);
-            const float r2 = O::fma(dx, dx, O::fma(dy, dy, O::fma(dz, dz, A.eps2)));
-            const float rinv = O::rsq<0>(r2);
-            const float rinv2 = O::mul(rinv, rinv);
-            const float mr3 = O::mul(O::mul(hj.w, rinv), rinv2);
-            const float rv = O::fma(dx, ux, O::fma(dy, uy, O::mul(dz, uz)));
-            const float cc = O::mul(O::mul(rv, rinv2), mr3);
-            pa[0] = O::fma(mr3, dx, pa[0]);
-            pa[1] = O::fma(mr3, dy, pa[1]);
-            pa[2] = O::fma(mr3, dz, pa[2]);
-            p1[0] = O::fma(mr3, ux, p1[0]);
-            p1[1] = O::fma(mr3, uy, p1[1]);
-            p1[2] = O::fma(mr3, uz, p1[2]);
-            p2[0] = O::fma(cc, dx, p2[0]);
-            p2[1] = O::fma(cc, dy, p2[1]);
-            p2[2] = O::fma(cc, dz, p2[2]);
           }
 #pragma unroll
-          for (int c = 0; c < 3; ++c) {
-            const float jt3 = fmaf(-3.f, p2[c], p1[c]);
-            if (PREC) {
-              dev::ds_add(sh[c], sl[c], pa[c]);
-              dev::ds_add(sh[3 + c], sl[3 + c], jt3);
-            } else {
-              sh[c] += pa[c];
-              sh[3 + c] += jt3;
+          for (int w = 0; w < IPW; ++w)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) {
+              const float jt3 = fmaf(-3.f, p2[w][c], p1[w][c]);
+              if (PREC) {
+                dev::ds_add(sh[w][c], sl[w][c], pa[w][c]);
+                dev::ds_add(sh[w][3 + c], sl[w][3 + c], jt3);
+              } else {
+                sh[w][c] += pa[w][c];
+                sh[w][3 + c] += jt3;
+              }
             }
-          }
         }
 #pragma unroll
-        for (int off = 1; off < 32; off <<= 1)
+        for (int w = 0; w < IPW; ++w) {
 #pragma unroll
-          for (int c = 0; c < 6; ++c) {
-            const float oh = __shfl_xor_sync(0xffffffffu, sh[c], off);
-            const float ol = __shfl_xor_sync(0xffffffffu, sl[c], off);
-            dev::ds_add_pair(sh[c], sl[c], oh, ol, sh[c], sl[c]);
-          }
-        if (lane == 0)
+          for (int off = 1; off < 32; off <<= 1)
 #pragma unroll
-          for (int c = 0; c < 6; ++c) s_seg[e][p - plo][c] = make_float2(sh[c], sl[c]);
+            for (int c = 0; c < 6; ++c) {
+              const float oh = __shfl_xor_sync(0xffffffffu, sh[w][c], off);
+              const float ol = __shfl_xor_sync(0xffffffffu, sl[w][c], off);
+              dev::ds_add_pair(sh[w][c], sl[w][c], oh, ol, sh[w][c], sl[w][c]);
+            }
+          if (lane == 0)
+#pragma unroll
+            for (int c = 0; c < 6; ++c) s_seg[e0 + w][p - plo][c] = make_float2(sh[w][c], sl[w][c]);
+        }
       }
       t0 = t1;
     }
   }
   __syncthreads();
-  if (wid < NI) {
+#pragma unroll
+  for (int q = 0; q < IPW; ++q) {
+    const int e = wid * IPW + q;
+    if (e >= NI) break;
     // the fix-up's sum: lane q has segment q
     float h[6], l[6];
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
       h[c] = l[c] = 0.f;
       if (plo == phi) {
-        h[c] = s_seg[wid][0][c].x;
-        l[c] = s_seg[wid][0][c].y;
+        h[c] = s_seg[e][0][c].x;
+        l[c] = s_seg[e][0][c].y;
       } else if (lane <= phi - plo) {
-        const float2 w = s_seg[wid][lane][c];
+        const float2 w = s_seg[e][lane][c];
         dev::ds_add_pair(h[c], l[c], w.x, w.y, h[c], l[c]);
       }
     }
@@ -203,7 +233,7 @@ __global__ void __launch_bounds__(32 * kWarps, 1) small_step_kernel(const SmallS
           hh = h[c];
           ll = l[c];
         }
-      s_f[wid][lane] = dev::ds_to_double(hh, ll, A.G);
+      s_f[e][lane] = dev::ds_to_double(hh, ll, A.G);
     }
   }
   __syncthreads();
@@ -221,9 +251,10 @@ __global__ void __launch_bounds__(32 * kWarps, 1) small_step_kernel(const SmallS
 
 }  // namespace
 
-// 8 particles per CTA where that leaves an SM for each CTA, otherwise 16; 0: too many.
+// 8 particles per CTA where that leaves an SM for each CTA, otherwise 16 or 32; 0:
+// too many.
 static int small_ni(int64_t n, int64_t n_jt, int num_sms) {
-  for (int ni = 8; ni <= 16; ni *= 2)
+  for (int ni = 8; ni <= 32; ni *= 2)
     if ((n + ni - 1) / ni + n_jt <= num_sms) return ni;
   return 0;
 }
@@ -241,7 +272,8 @@ size_t small_step_smem(int64_t n_jt, int prec) {
 using SmallKernel = void (*)(const SmallStepArgs);
 static SmallKernel small_kernel(int prec, int ni) {
   if (ni == 8) return prec ? small_step_kernel<1, 8> : small_step_kernel<0, 8>;
-  return prec ? small_step_kernel<1, 16> : small_step_kernel<0, 16>;
+  if (ni == 16) return prec ? small_step_kernel<1, 16> : small_step_kernel<0, 16>;
+  return prec ? small_step_kernel<1, 32> : small_step_kernel<0, 32>;
 }
 
 cudaError_t small_step_prepare(int64_t n, int64_t n_jt, int prec, int num_sms) {

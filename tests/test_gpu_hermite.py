@@ -578,8 +578,9 @@ def test_shared_steps_without_a_look_at_the_schedule(nb, n):
 
 
 # a particle, a partial and a whole i-block of 16, tile edges, N = 1024, the
-# most i-blocks that fit one per SM, and just past them (separate launches)
-@pytest.mark.parametrize("n", [2, 15, 16, 17, 255, 257, 1024, 2203, 2304, 2500])
+# most that 16 per SM hold and past it (32, with a CTA's second block empty),
+# the most the records' shared memory holds and past it (separate launches)
+@pytest.mark.parametrize("n", [2, 15, 16, 17, 255, 257, 1024, 2203, 2304, 2289, 2500, 4096, 4097])
 @pytest.mark.parametrize("prec", ["ds", "fp32"])
 @pytest.mark.parametrize("field", [False, True])
 def test_small_step_bitwise_equals_separate_launches(nb, n, prec, field):
