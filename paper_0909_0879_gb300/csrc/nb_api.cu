@@ -302,6 +302,7 @@ struct nb_ctx {
   bool sym_off = false;
   bool eq_mass = false;  // every mass is m_eq
   int small_step = -1;   // one launch per shared step: 1 yes, 0 no, -1 not yet looked at
+  int small_symp = -1;   // symplectic runs likewise
   double m_eq = 0.0, m_mean = 0.0;
   double *red = nullptr;        // energy scratch
   unsigned char *en_rec = nullptr;  // records of the split-precision energy
@@ -1518,6 +1519,64 @@ nb_status queue_symplectic_step(nb_ctx *c, const SymArrays &A, const SymArgs *P,
   return P ? NB_OK : queue_kick_drift(c, A, P, s, close, 0.0, false, launches);
 }
 
+// Whether symplectic runs of this context are launches of many stages each.
+bool takes_small_symplectic(nb_ctx *c) {
+  if (c->small_symp < 0) {
+    int dev = 0, coop = 0;
+    const int prec = c->cfg.precision;
+    // the second record buffer is the block steps' stored split, which
+    // nb_run_blocks rebuilds
+    const bool ok =
+        4 * c->n >= 2 * c->n_pad &&
+        small_symp_fits(c->n, c->n_jt, prec, eps_masks(c->cfg.eps), c->num_sms) &&
+        cudaGetDevice(&dev) == cudaSuccess &&
+        cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
+        small_symp_prepare(c->n, c->n_jt, prec, c->num_sms) == cudaSuccess;
+    c->small_symp = ok ? 1 : 0;
+  }
+  return c->small_symp == 1;
+}
+
+// A(x) at the start, then nsteps steps; v, x and the total a in A.
+nb_status queue_small_symplectic(nb_ctx *c, const SymArrays &S, const double *w, int stages,
+                                 double dt, int64_t nsteps, int64_t *launches) {
+  SmallSympArgs A;
+  A.n = c->n;
+  A.n_jt = c->n_jt;
+  A.S = stages;
+  for (int k = 0; k < stages; ++k) {
+    A.h[k] = 0.5 * dt * ((k > 0 ? w[k - 1] : 0.0) + w[k]);
+    A.d[k] = w[k] * dt;
+  }
+  A.close = 0.5 * dt * w[stages - 1];
+  A.x = S.x;
+  A.v = S.v;
+  A.a = S.a;
+  A.m = S.m;
+  A.hi[0] = c->jhi;
+  A.lo[0] = c->jlo;
+  A.hi[1] = c->sp4;
+  A.lo[1] = c->sp4 + c->n_pad;
+  A.eps2 = eps2_f32(c->cfg.eps);
+  A.G = c->cfg.G;
+  A.ext = c->ext;
+  A.P = force_grid(acc_shape(choose_variant(c->cfg.precision, 0, c->n, c->n_jt, c->num_sms)),
+                   c->n, c->n_jt, c->num_sms, 0);
+  A.err = c->err;
+  A.bar = reinterpret_cast<unsigned long long *>(c->scal + kCtlBarSymp);
+  // a run that gave up at a barrier leaves an odd count
+  NB_CUDA(cudaMemsetAsync(A.bar, 0, sizeof(*A.bar), c->stream));
+  // launches of a few milliseconds
+  const int64_t most = 512 / stages;
+  for (int64_t done = 0; done < nsteps; done += most) {
+    A.init = done == 0 ? 1 : 0;
+    A.stages = std::min(most, nsteps - done) * stages;
+    NB_CUDA(launch_small_symplectic(A, c->cfg.precision, c->num_sms, c->stream));
+    *launches += 1;
+  }
+  return NB_OK;
+}
+
 nb_status capture_symplectic(nb_ctx *c, const SymArrays &A, const SymArgs *P, const double *w,
                              int S, double dt) {
   if (c->sym_graph) {
@@ -1821,9 +1880,14 @@ extern "C" nb_status nb_symplectic(nb_ctx *c, int32_t order, double dt, int64_t 
     SA.x = A.x;
     SA.v = A.v;
   }
-  s = queue_kick_drift(c, A, P, c->stream, 0.0, 0.0, true, &nl);
-  if (s == NB_OK)
-    s = P ? queue_acc_sym(c, *P, c->stream, 0.0, &nl) : queue_acc_all(c, A, c->stream, &nl);
+  const bool small = nsteps > 0 && !P && takes_small_symplectic(c);
+  if (small) {
+    s = queue_small_symplectic(c, A, w, S, dt, nsteps, &nl);
+  } else {
+    s = queue_kick_drift(c, A, P, c->stream, 0.0, 0.0, true, &nl);
+    if (s == NB_OK)
+      s = P ? queue_acc_sym(c, *P, c->stream, 0.0, &nl) : queue_acc_all(c, A, c->stream, &nl);
+  }
   if (s != NB_OK) return s;
   c->launches += nl;
   c->interactions += c->n * c->n;
@@ -1832,7 +1896,9 @@ extern "C" nb_status nb_symplectic(nb_ctx *c, int32_t order, double dt, int64_t 
   c->have_block = false;
   c->force_done = false;
   c->t_pred = -1;
-  if (nsteps > 0) {
+  if (small) {
+    c->interactions += nsteps * S * c->n * c->n;
+  } else if (nsteps > 0) {
     if (!c->sym_graph || c->sym_order != order || c->sym_dt != dt ||
         c->sym_graph_part != c->part || c->sym_graph_stale || c->sym_graph_x != A.x) {
       s = capture_symplectic(c, A, P, w, S, dt);
@@ -1848,7 +1914,7 @@ extern "C" nb_status nb_symplectic(nb_ctx *c, int32_t order, double dt, int64_t 
     c->interactions += nsteps * S * c->n * c->n;
   }
   // the acceleration left in the state is the total one at the final x
-  if (c->ext.on && !P) {
+  if (c->ext.on && !P && !small) {
     NB_CUDA(launch_ext_add(c->n, c->ext, A.x, A.a, c->stream));
     c->launches += 1;
   }

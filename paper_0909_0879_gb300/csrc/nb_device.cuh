@@ -729,6 +729,12 @@ __device__ __forceinline__ void load_state(int64_t i, const double *__restrict__
   st.lev = lev[i];
 }
 
+// a += the field's acceleration at x.  Not inlined, so that every kernel
+// rounds it alike.
+static __device__ __noinline__ void ext_acc(const ExtField &E, const double x[3], double a[3]) {
+  ext_field(E, x, nullptr, a, nullptr, nullptr);
+}
+
 // The field's acceleration and jerk at the predictor's position and
 // velocity (the expression of predict_pos_vel) added into an, jn.  Not
 // inlined: the corrector kernels keep their registers when no field is set.

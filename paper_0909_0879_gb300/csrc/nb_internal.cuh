@@ -82,6 +82,7 @@ constexpr int kCtlBad = 10;     // nonzero: the schedule is not level-structured
 constexpr int kCtlTcur = 11;    // latest particle time (ticks), from the check
 constexpr int kCtlLevCnt = 16;  // kTicksLog2 + 1 slots: particles per level
 constexpr int kCtlBar = 38;     // arrivals at the small step's grid barrier
+constexpr int kCtlBarSymp = 39; // ... at a small symplectic run's
 constexpr int kCtlSlots = 40;
 
 // Device error-word bit of a timed-out look-back in the fused compaction.
@@ -244,6 +245,26 @@ bool small_step_fits(int64_t n, int64_t n_jt, int prec, int mask, int num_sms);
 size_t small_step_smem(int64_t n_jt, int prec);
 cudaError_t small_step_prepare(int64_t n, int64_t n_jt, int prec, int num_sms);
 cudaError_t launch_small_step(const SmallStepArgs &A, int prec, int num_sms, cudaStream_t s);
+
+// A run of symplectic stages of a small system: stages = steps * S, kick h and
+// drift d of each stage of a step, the step's closing kick.
+struct SmallSympArgs {
+  int64_t n, n_jt, stages;
+  int S, init, P;
+  double h[7], d[7], close;
+  double *x, *v, *a;
+  const double *m;
+  float4 *hi[2], *lo[2];  // record buffers (lo: split precision)
+  float eps2;
+  double G;
+  ExtField ext;
+  int *err;
+  unsigned long long *bar;
+};
+bool small_symp_fits(int64_t n, int64_t n_jt, int prec, int mask, int num_sms);
+cudaError_t small_symp_prepare(int64_t n, int64_t n_jt, int prec, int num_sms);
+cudaError_t launch_small_symplectic(const SmallSympArgs &A, int prec, int num_sms,
+                                    cudaStream_t s);
 
 // --- Hermite and bookkeeping kernels (nb_hermite.cu) ---
 // The j-records of every particle at t_next and, with jrel set, per

@@ -1,5 +1,6 @@
 // One shared Hermite step of a small system in one launch: prediction of
-// every particle, force + jerk of all of them, correction (paper Sec. 2.2).
+// every particle, force + jerk of all of them, correction (paper Sec. 2.2); and
+// its symplectic runs (below).
 //
 // Bound: latency.  At N = 1,024 the pairs take 1 us of the FP32 pipes, while
 // three launches (predictor, force, fix-up + corrector) cost a launch, a drain
@@ -249,6 +250,219 @@ __global__ void __launch_bounds__(32 * kWarps, 1) small_step_kernel(const SmallS
   }
 }
 
+// Acceleration of the CTA's NI particles (k0 ..) from the records in shared
+// memory, into s_f: the sums of the acceleration-only short-list shape and its
+// fix-up.  Called by the whole CTA.
+template <int PREC, int NI>
+__device__ __forceinline__ void small_acc(int n, int n_jt, int k0, int P, float eps2, double G,
+                                          const float4 *s_hi, const float4 *s_lo,
+                                          float2 (*s_seg)[kSmallMostTiles][3], double (*s_f)[3]) {
+  using O = dev::VOps<float>;
+  constexpr int WPI = NI < kWarps ? kWarps / NI : 1, IPW = NI > kWarps ? NI / kWarps : 1;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int blocks = (n + kBlock - 1) / kBlock;
+  const uint64_t U = static_cast<uint64_t>(blocks) * n_jt;
+  const int blk = NI <= kBlock ? k0 / kBlock
+                               : min((k0 + wid / WPI * IPW) / kBlock, blocks - 1);
+  const uint64_t u0 = static_cast<uint64_t>(blk) * n_jt;
+  const int plo = dev::owner_of(u0, U, P), phi = dev::owner_of(u0 + n_jt - 1, U, P);
+  const int e0 = wid / WPI * IPW;
+  float nx[IPW][3], nl[IPW][3];
+#pragma unroll
+  for (int w = 0; w < IPW; ++w) {
+    const int i = k0 + e0 + w < n ? k0 + e0 + w : 0;
+    const float4 hi = s_hi[i];
+    const float4 li = PREC ? s_lo[i] : make_float4(0.f, 0.f, 0.f, 0.f);
+    nx[w][0] = -hi.x, nx[w][1] = -hi.y, nx[w][2] = -hi.z;
+    nl[w][0] = -li.x, nl[w][1] = -li.y, nl[w][2] = -li.z;
+  }
+  int t0 = 0;
+  for (int p = plo; p <= phi; ++p) {
+    const uint64_t ue = dev::udiv(U * static_cast<uint64_t>(p + 1), static_cast<uint64_t>(P));
+    const int t1 = p == phi ? n_jt : static_cast<int>(ue - u0);
+    if ((p - plo) % WPI == wid % WPI) {
+      float sh[IPW][3], sl[IPW][3];
+#pragma unroll
+      for (int w = 0; w < IPW; ++w)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) sh[w][c] = sl[w][c] = 0.f;
+      for (int jt = t0; jt < t1; ++jt) {
+        float pa[IPW][3];
+#pragma unroll
+        for (int w = 0; w < IPW; ++w)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) pa[w][c] = 0.f;
+#pragma unroll
+        for (int q = 0; q < kJT / 32; ++q) {
+          const int j = jt * kJT + q * 32 + lane;
+          const float4 hj = s_hi[j];
+          const float4 lj = PREC ? s_lo[j] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+          for (int w = 0; w < IPW; ++w) {
+            float dx, dy, dz;
+            if (PREC) {
+              dx = O::add(O::add(hj.x, nx[w][0]), O::add(lj.x, nl[w][0]));
+              dy = O::add(O::add(hj.y, nx[w][1]), O::add(lj.y, nl[w][1]));
+              dz = O::add(O::add(hj.z, nx[w][2]), O::add(lj.z, nl[w][2]));
+            } else {
+              dx = O::add(hj.x, nx[w][0]);
+              dy = O::add(hj.y, nx[w][1]);
+              dz = O::add(hj.z, nx[w][2]);
+            }
+            const float r2 = O::fma(dx, dx, O::fma(dy, dy, O::fma(dz, dz, eps2)));
+            const float rinv = O::rsq<0>(r2);
+            const float mr3 = O::mul(O::mul(hj.w, rinv), O::mul(rinv, rinv));
+            pa[w][0] = O::fma(mr3, dx, pa[w][0]);
+            pa[w][1] = O::fma(mr3, dy, pa[w][1]);
+            pa[w][2] = O::fma(mr3, dz, pa[w][2]);
+          }
+        }
+#pragma unroll
+        for (int w = 0; w < IPW; ++w)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            if (PREC)
+              dev::ds_add(sh[w][c], sl[w][c], pa[w][c]);
+            else
+              sh[w][c] += pa[w][c];
+          }
+      }
+#pragma unroll
+      for (int w = 0; w < IPW; ++w) {
+#pragma unroll
+        for (int off = 1; off < 32; off <<= 1)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) {
+            const float oh = __shfl_xor_sync(0xffffffffu, sh[w][c], off);
+            const float ol = __shfl_xor_sync(0xffffffffu, sl[w][c], off);
+            dev::ds_add_pair(sh[w][c], sl[w][c], oh, ol, sh[w][c], sl[w][c]);
+          }
+        if (lane == 0)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) s_seg[e0 + w][p - plo][c] = make_float2(sh[w][c], sl[w][c]);
+      }
+    }
+    t0 = t1;
+  }
+  __syncthreads();
+#pragma unroll
+  for (int q = 0; q < IPW; ++q) {
+    const int e = wid * IPW + q;
+    if (e >= NI) break;
+    float h[3], l[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      h[c] = l[c] = 0.f;
+      if (plo == phi) {
+        h[c] = s_seg[e][0][c].x;
+        l[c] = s_seg[e][0][c].y;
+      } else if (lane <= phi - plo) {
+        const float2 w = s_seg[e][lane][c];
+        dev::ds_add_pair(h[c], l[c], w.x, w.y, h[c], l[c]);
+      }
+    }
+    if (plo != phi) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const float oh = __shfl_xor_sync(0xffffffffu, h[c], off);
+          const float ol = __shfl_xor_sync(0xffffffffu, l[c], off);
+          dev::ds_add_pair(h[c], l[c], oh, ol, h[c], l[c]);
+        }
+    }
+    if (lane < 3)
+      s_f[e][lane] = dev::ds_to_double(dev::sel3(h, lane), dev::sel3(l, lane), G);
+  }
+  __syncthreads();
+}
+
+// A run of symplectic steps of a small system in one launch: a CTA keeps its
+// particles' x and v in registers (one thread each) from the first step to the
+// last; per stage the records cross one grid barrier, through two buffers in
+// turn (a CTA writes a buffer again only after the barrier that all CTAs enter
+// with their reads of it done).  With init the acceleration at the start is
+// evaluated first, otherwise A.a holds it.  The arithmetic of kick_drift_kernel,
+// the acceleration-only force and its fix-up: the same bits.  Bound: latency (a
+// stage of separate launches is three of them).  Whole calls of one step with
+// read-back, before -> now: leapfrog in the Galactic field N = 1,191 114 -> 66 us,
+// sixth order FP32 N = 1,000 124 -> 82, split precision N = 2,300 200 -> 132, with
+// the field N = 3,500 424 -> 270 (no graph to capture: a first call 192 -> 109 at
+// N = 1,191).
+template <int PREC, int NI>
+__global__ void __launch_bounds__(32 * kWarps, 1) small_symplectic_kernel(const SmallSympArgs A) {
+  extern __shared__ __align__(16) float4 rec[];
+  __shared__ double s_f[NI][3];
+  __shared__ float2 s_seg[NI][kSmallMostTiles][3];
+  const int tid = threadIdx.x;
+  const int n = static_cast<int>(A.n), n_jt = static_cast<int>(A.n_jt), n_pad = n_jt * kJT;
+  const int k0 = blockIdx.x * NI, k = k0 + tid;
+  const bool own = tid < NI && k < n;
+  float4 *s_hi = rec, *s_lo = rec + n_pad;
+  if (blockIdx.x == 0)  // padding of the second buffer: zero mass far away
+    for (int j = n + tid; j < n_pad; j += 32 * kWarps) {
+      A.hi[1][j] = make_float4(1.0e15f, 1.0e15f, 1.0e15f, 0.f);
+      if (PREC) A.lo[1][j] = make_float4(0.f, 0.f, 0.f, 0.f);
+    }
+  double x[3], v[3], a[3], m = 0.0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    x[c] = own ? A.x[3 * k + c] : 0.0;
+    v[c] = own ? A.v[3 * k + c] : 0.0;
+    a[c] = own ? A.a[3 * k + c] : 0.0;
+  }
+  if (own) m = A.m[k];
+  int buf = 0;
+  // stage -1: the acceleration at the start
+  for (int64_t q = A.init ? -1 : 0; q < A.stages; ++q) {
+    const int st = q < 0 ? 0 : static_cast<int>(q % A.S);
+    if (own) {
+      if (q >= 0) {
+        if (A.h[st] != 0.0)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) v[c] = fma(A.h[st], a[c], v[c]);
+        if (A.d[st] != 0.0)
+#pragma unroll
+          for (int c = 0; c < 3; ++c) x[c] = fma(A.d[st], v[c], x[c]);
+      }
+      float hx[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) hx[c] = dev::d2f_rn(x[c]);
+      A.hi[buf][k] = make_float4(hx[0], hx[1], hx[2], dev::d2f_rn(m));
+      if (PREC)
+        A.lo[buf][k] = make_float4(dev::d2f_rn(x[0] - dev::f2d(hx[0])),
+                                   dev::d2f_rn(x[1] - dev::f2d(hx[1])),
+                                   dev::d2f_rn(x[2] - dev::f2d(hx[2])), 0.f);
+    }
+    if (!grid_barrier(A.bar)) {
+      if (tid == 0) atomicOr(A.err, kErrWaitTimeout);
+      return;
+    }
+    for (int j = tid; j < n_pad; j += 32 * kWarps) {
+      s_hi[j] = __ldcg(A.hi[buf] + j);
+      if (PREC) s_lo[j] = __ldcg(A.lo[buf] + j);
+    }
+    __syncthreads();
+    small_acc<PREC, NI>(n, n_jt, k0, A.P, A.eps2, A.G, s_hi, s_lo, s_seg, s_f);
+    if (own) {
+#pragma unroll
+      for (int c = 0; c < 3; ++c) a[c] = s_f[tid][c];
+      if (A.ext.on) dev::ext_acc(A.ext, x, a);
+      if (q >= 0 && st == A.S - 1 && A.close != 0.0)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[c] = fma(A.close, a[c], v[c]);
+    }
+    buf ^= 1;
+  }
+  if (own)
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      A.x[3 * k + c] = x[c];
+      A.v[3 * k + c] = v[c];
+      A.a[3 * k + c] = a[c];
+    }
+}
+
 }  // namespace
 
 // 8 particles per CTA where that leaves an SM for each CTA, otherwise 16 or 32; 0:
@@ -296,6 +510,53 @@ cudaError_t launch_small_step(const SmallStepArgs &A, int prec, int num_sms, cud
   cfg.attrs = &at;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, small_kernel(prec, ni), A);
+}
+
+// ---- symplectic runs
+
+static int small_symp_ni(int64_t n, int num_sms) {
+  for (int ni = 8; ni <= 32; ni *= 2)
+    if ((n + ni - 1) / ni <= num_sms) return ni;
+  return 0;
+}
+
+using SmallSympKernel = void (*)(const SmallSympArgs);
+static SmallSympKernel small_symp_kernel(int prec, int ni) {
+  if (ni == 8) return prec ? small_symplectic_kernel<1, 8> : small_symplectic_kernel<0, 8>;
+  if (ni == 16) return prec ? small_symplectic_kernel<1, 16> : small_symplectic_kernel<0, 16>;
+  return prec ? small_symplectic_kernel<1, 32> : small_symplectic_kernel<0, 32>;
+}
+
+static size_t small_symp_smem(int64_t n_jt, int prec) {
+  return static_cast<size_t>(n_jt) * kJT * (prec ? 2 : 1) * sizeof(float4);
+}
+
+bool small_symp_fits(int64_t n, int64_t n_jt, int prec, int mask, int num_sms) {
+  if (mask || n_jt > kSmallMostTiles || small_symp_ni(n, num_sms) == 0) return false;
+  const Variant &V = variant_at(acc_shape(choose_variant(prec, mask, n, n_jt, num_sms)));
+  return V.ipt == 1 && V.tpi == 32 && V.threads == 32 * kBlock && !V.rel;
+}
+
+cudaError_t small_symp_prepare(int64_t n, int64_t n_jt, int prec, int num_sms) {
+  return cudaFuncSetAttribute(small_symp_kernel(prec, small_symp_ni(n, num_sms)),
+                              cudaFuncAttributeMaxDynamicSharedMemorySize,
+                              static_cast<int>(small_symp_smem(n_jt, prec)));
+}
+
+cudaError_t launch_small_symplectic(const SmallSympArgs &A, int prec, int num_sms,
+                                    cudaStream_t s) {
+  cudaLaunchConfig_t cfg = {};
+  const int ni = small_symp_ni(A.n, num_sms);
+  cfg.gridDim = dim3(static_cast<unsigned>((A.n + ni - 1) / ni));
+  cfg.blockDim = dim3(32 * kWarps);
+  cfg.dynamicSmemBytes = small_symp_smem(A.n_jt, prec);
+  cfg.stream = s;
+  cudaLaunchAttribute at = {};
+  at.id = cudaLaunchAttributeCooperative;
+  at.val.cooperative = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = 1;
+  return cudaLaunchKernelEx(&cfg, small_symp_kernel(prec, ni), A);
 }
 
 }  // namespace nbi

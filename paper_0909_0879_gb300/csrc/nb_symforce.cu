@@ -651,7 +651,7 @@ __global__ void __launch_bounds__(kFixP *NC) sym_fixup_kernel(const SymArgs A) {
     if (c == 0 && real) {
       const double xv[3] = {A.x[3 * i], A.x[3 * i + 1], A.x[3 * i + 2]};
       double at[3] = {s_a[0][pl], s_a[1][pl], s_a[2][pl]};
-      dev::ext_field(A.ext, xv, nullptr, at, nullptr, nullptr);
+      dev::ext_acc(A.ext, xv, at);
 #pragma unroll
       for (int q = 0; q < 3; ++q) s_a[q][pl] = at[q];
     }

@@ -54,7 +54,7 @@ __global__ void __launch_bounds__(kJT)
     }
     if (h != 0.0) {
       double at[3] = {a[3 * j], a[3 * j + 1], a[3 * j + 2]};
-      if (E.on) dev::ext_field(E, xv, nullptr, at, nullptr, nullptr);
+      if (E.on) dev::ext_acc(E, xv, at);
 #pragma unroll
       for (int c = 0; c < 3; ++c) {
         vv[c] = fma(h, at[c], vv[c]);
@@ -93,7 +93,7 @@ __global__ void ext_add_kernel(int64_t n, const ExtField E, const double *__rest
   if (i >= n) return;
   const double xv[3] = {x[3 * i], x[3 * i + 1], x[3 * i + 2]};
   double av[3] = {a[3 * i], a[3 * i + 1], a[3 * i + 2]};
-  dev::ext_field(E, xv, nullptr, av, nullptr, nullptr);
+  dev::ext_acc(E, xv, av);
   for (int c = 0; c < 3; ++c) a[3 * i + c] = av[c];
 }
 

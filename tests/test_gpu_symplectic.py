@@ -324,3 +324,31 @@ def test_automatic_layout_choice(nb):
     with nb.NBody(m, x, v, eps=eps) as s:
         with pytest.raises(KeyError):
             s.set_symplectic_layout("diagonal")
+
+
+# one thread per particle of 8, 16 and 32 per CTA, a ragged last CTA and tile,
+# the most the shared memory holds and past it (separate launches)
+@pytest.mark.parametrize("n", [300, 1024, 1217, 2048, 2433, 4096, 4097])
+@pytest.mark.parametrize("order", [2, 6])
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+@pytest.mark.parametrize("field", [False, True])
+def test_small_runs_in_one_launch(nb, n, order, prec, field):
+    """Three steps in one call, one by one, and more than a launch's worth of
+    stages: the same bits; the acceleration left is the separate kernels' (a
+    call of no steps) at the same positions."""
+    m, x, v = ics.plummer(n, 60 + n, masses=ics.salpeter_masses(n, n))
+    with nb.NBody(m, x, v, eps=1e-2, precision=prec) as s, \
+            nb.NBody(m, x, v, eps=1e-2, precision=prec) as o:
+        if field:
+            s.set_external({})
+            o.set_external({})
+        most = 520 if order == 2 and n == 1024 else 3
+        s.symplectic(order, 2.0**-9, most)
+        for k in (1, 1, most - 2):
+            o.symplectic(order, 2.0**-9, k)
+        p, q = s.get_state(want=("x", "v", "a")), o.get_state(want=("x", "v", "a"))
+        for k in p:
+            assert np.array_equal(p[k], q[k]), k
+        s.symplectic(order, 2.0**-9, 0)
+        assert np.array_equal(s.get_state(want=("a",))["a"], p["a"])
+        assert np.array_equal(s.get_state(want=("x",))["x"], p["x"])
