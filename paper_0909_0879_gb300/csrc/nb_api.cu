@@ -1497,7 +1497,7 @@ nb_status queue_acc_sym(nb_ctx *c, const SymArgs &P, cudaStream_t s, double kick
   SymArgs A = P;
   A.kick = kick;
   int nl = 0;
-  NB_CUDA(launch_sym_force(c->cfg.precision, eps_masks(c->cfg.eps), A, s, &nl, false));
+  NB_CUDA(launch_sym_force(c->cfg.precision, eps_masks(c->cfg.eps), A, s, &nl));
   *launches += nl;
   return NB_OK;
 }

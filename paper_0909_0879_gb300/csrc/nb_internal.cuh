@@ -218,9 +218,9 @@ size_t sym_ipart_bytes(const SymSplit &S, bool jrk);
 size_t sym_jpart_bytes(const SymSplit &S, bool jrk);
 // Shared-memory attribute of the kernel; before its first launch or capture.
 cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq, int64_t n_jt);
-// with_records false: recs already hold the positions (launch_kick_drift).
+// Without jerk, recs already hold the positions (launch_kick_drift and the like).
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A, cudaStream_t s,
-                             int *launches, bool with_records = true);
+                             int *launches);
 
 // --- one shared step of a small system in one launch (nb_smallstep.cu) ---
 struct SmallStepArgs {

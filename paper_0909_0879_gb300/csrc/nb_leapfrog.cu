@@ -664,7 +664,7 @@ cudaError_t lf_sym_eval(LfCtx &C, const float *x_in, float *x_out, const float *
   if (e != cudaSuccess) return e;
   C.S.acc_f = acc;
   int nl = 0;
-  e = launch_sym_force(0, C.mask, C.S, C.s, &nl, false);
+  e = launch_sym_force(0, C.mask, C.S, C.s, &nl);
   C.launches += nl;
   return e;
 }

@@ -129,7 +129,8 @@ __host__ __device__ __forceinline__ uint32_t sym_tile(const SymSplit &S, uint32_
   return b * S.tb + (off - d * S.tb);
 }
 
-// One CTA per tile, one thread per pair.
+// The jerk kernel's records from the predictor's; one CTA per tile, one thread
+// per pair.
 template <int PREC>
 __global__ void __launch_bounds__(kPairs) sym_records_kernel(const SymArgs A) {
   if (A.ctl && A.ctl[kCtlNact] != A.n) return;
@@ -155,7 +156,7 @@ __global__ void __launch_bounds__(kPairs) sym_records_kernel(const SymArgs A) {
     put(A.jlo, rec_lo(), false, A.sc);
     put(A.jrel, rec_rel(), true, A.sc);
   }
-  if (A.jerk) put(A.jvel, rec_vel(PREC), false, 1.f);
+  put(A.jvel, rec_vel(PREC), false, 1.f);
 }
 
 template <int PREC, int MASK, int JRK, int EQ, int IPT, int NT, int ST, int SACC>
@@ -777,7 +778,7 @@ int sym_exponent(double mean_mass, float eps2) {
 }
 
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A0, cudaStream_t s,
-                             int *launches, bool with_records) {
+                             int *launches) {
   SymArgs A = A0;
   const bool jrk = A.jerk != nullptr;
   A.sc = static_cast<float>(std::ldexp(1.0, A.sexp));
@@ -786,7 +787,7 @@ cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A0, cudaStream_t
   A.g_acc = std::ldexp(A.g_jerk, -A.sexp);
   const SymEntry &E = sym_pick(prec, mask, jrk, A.eq != 0, A.n_jt);
   const unsigned tiles = static_cast<unsigned>(A.n_jt);
-  if (with_records) {
+  if (jrk) {  // a drift has written the acceleration's records
     if (prec)
       sym_records_kernel<1><<<tiles, kPairs, 0, s>>>(A);
     else
