@@ -566,10 +566,11 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
       cudaStreamSynchronize(c->stream);
       cudaFree(c->sym_i);
       cudaFree(c->sym_j);
-      if (c->sym_graph) {  // holds the old scratch
-        cudaGraphExecDestroy(c->sym_graph);
-        c->sym_graph = nullptr;
-      }
+      for (cudaGraphExec_t *g : {&c->sym_graph, &c->blk_graph, &c->fus_graph})
+        if (*g) {  // may hold the old scratch
+          cudaGraphExecDestroy(*g);
+          *g = nullptr;
+        }
     }
     c->sym_i = ni;
     c->sym_j = nj;
