@@ -424,7 +424,14 @@ __global__ void __launch_bounds__(NT, 2) batched_team_kernel(const BatchArgs B) 
       team::sync();
       const int item = s_item;
       if (item >= B.n_large) break;  // the whole team
-      batched_cluster<PREC, 1, NT, MASK, 0, 1, IPT>(B, B.order[item], srec);
+      // a CTA's share: one particle per thread while that gives it warps
+      // enough, from 160 on two, packed (20 steps of 1,000 clusters 5.33 -> 4.67
+      // ms; from 100 on 50 / 150 clusters lose, 0.89 / 1.17 -> 1.28 / 2.01)
+      const int c = B.order[item];
+      if (PACK && B.off[c + 1] - B.off[c] > 160 * static_cast<int>(parts))
+        batched_cluster<PREC, IPT, NT, MASK, PACK, 1, IPT>(B, c, srec);
+      else
+        batched_cluster<PREC, 1, NT, MASK, 0, 1, IPT>(B, c, srec);
     }
   }
   for (;;) {
@@ -575,10 +582,10 @@ size_t bsmem(const BEntry &E, int cap) {
 // longest cluster.  Where that has more than twice the mean load of a CTA, sum
 // n^2 / (2 SMs), the clusters above the mean are shared by teams of 4 or 8
 // CTAs (at twice the mean or less a team of two gains nothing: 1,500 clusters
-// 7.38 against 7.36 ms); as many teams as the large clusters' part of the
+// 7.38 against 7.36 ms in the scalar shape); as many teams as the large clusters' part of the
 // work.  Clusters of up to 256 gain nothing from it.  20 steps of clusters of
 // 16 .. 1,024, split precision, 50 / 150 / 400 / 1,000 clusters: 4.23 / 4.23 /
-// 4.32 / 5.93 -> 0.85 / 1.20 / 2.69 / 5.33 ms.
+// 4.32 / 5.93 -> 0.89 / 1.17 / 2.62 / 4.67 ms.
 constexpr int kTeamMin = 256, kTeamMost = 8;
 
 void pick_team(nb_batch *b, const int64_t *offsets) {
