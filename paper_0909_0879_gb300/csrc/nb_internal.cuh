@@ -177,6 +177,10 @@ struct SymSplit {
   uint32_t irows;   // rows a CTA's range can touch
   uint32_t jslots;  // ring tiles from its first row's first tile on
 };
+struct SymScale {
+  float sc, sm, eps2;  // of positions and masses; eps^2 on that scale
+  double g_acc;        // what the sums are taken by
+};
 struct SymArgs {
   const float4 *jhi, *jlo, *jvel, *jrel, *tinfo;
   int64_t n_jt, n;
@@ -204,11 +208,25 @@ struct SymArgs {
   // set by launch_sym_force: 2^sexp, 2^(3 sexp), and what the sums are taken by
   float sc = 1.f, sm = 1.f;
   double g_acc = 0.0, g_jerk = 0.0;
+  // The FP32 acceleration for masses that only the device knows: jhi is on the
+  // kernel's scale like recs, and *dscale has the rest (sexp = 0).
+  const SymScale *dscale = nullptr;
 };
 // The pair kernel works on positions times 2^s and masses times 2^(3 s) (exact),
-// s = sym_exponent: with 2^(-3 s) near the mean mass, 1 / r^3 of the scaled
-// positions has the FP32 range that mass / r^3 has.
-int sym_exponent(double mean_mass, float eps2);
+// s = sym_exponent: with 2^(-3 s) near the mass it is given, 1 / r^3 of the
+// scaled positions has the FP32 range that this mass / r^3 has.
+__host__ __device__ inline int sym_exponent(double mass, float eps2) {
+  if (!(mass > 0.0) || !isfinite(mass)) return 0;
+  int s = static_cast<int>(lround(log2(mass) / -3.0));
+  // positions up to 1e13 keep a finite square, and 2^(3 s) is a float
+  s = s < -40 ? -40 : (s > 20 ? 20 : s);
+  if (eps2 > 0.f) {  // eps^2 stays a normal number
+    const int e = ilogbf(eps2), lo = (-122 - e) / 2, hi = (120 - e) / 2;
+    s = s < lo ? lo : s;
+    s = s > hi ? hi : s;
+  }
+  return s;
+}
 // i-particles per block of the kernel for this precision / masking / output.
 int sym_block_i(int prec, int mask, bool jrk, int64_t n_jt);
 // False when n_jt tiles are too few (or too many) for a ring of such blocks.

@@ -277,7 +277,8 @@ __global__ void __launch_bounds__(NT, 256 / NT)
       nvi[q][0] = -w.x; nvi[q][1] = -w.y; nvi[q][2] = -w.z;
       mi[q] = k < A.n ? h.w * A.sm : 0.f;
     }
-    const V veps2 = O::bc(A.eps2 * A.sc * A.sc);
+    const V veps2 = O::bc(!PREC && !JRK && !EQ && A.dscale ? A.dscale->eps2
+                                                           : A.eps2 * A.sc * A.sc);
     float bc_i[3] = {0.f, 0.f, 0.f}, bh_i[3] = {0.f, 0.f, 0.f};
     if (PREC) {
       // bounding box of the i-block (far test), as in the one-sided kernel
@@ -645,7 +646,8 @@ __global__ void __launch_bounds__(kFixP *NC) sym_fixup_kernel(const SymArgs A) {
   const int64_t i = static_cast<int64_t>(jt) * kJT + t;
   const bool real = i < A.n;
   dev::ds_add_pair(h, l, -gh, -gl, h, l);
-  double val = dev::ds_to_double(h, l, c < 3 ? A.g_acc : A.g_jerk);
+  const double g_acc = NC == 3 && A.dscale ? A.dscale->g_acc : A.g_acc;
+  double val = dev::ds_to_double(h, l, c < 3 ? g_acc : A.g_jerk);
   if (A.ext.on) {
     if (c < 3) s_a[c][pl] = val;
     __syncthreads();
@@ -762,19 +764,6 @@ cudaError_t sym_prepare(int prec, int mask, bool jrk, bool eq, int64_t n_jt) {
   const SymEntry &E = sym_pick(prec, mask, jrk, eq, n_jt);
   return cudaFuncSetAttribute(E.fn, cudaFuncAttributeMaxDynamicSharedMemorySize,
                               static_cast<int>(E.smem));
-}
-
-int sym_exponent(double mean_mass, float eps2) {
-  if (!(mean_mass > 0.0) || !std::isfinite(mean_mass)) return 0;
-  int s = static_cast<int>(std::lround(std::log2(mean_mass) / -3.0));
-  // positions up to 1e13 keep a finite square, and 2^(3 s) is a float
-  s = std::max(-40, std::min(20, s));
-  if (eps2 > 0.f) {  // eps^2 stays a normal number
-    const int e = std::ilogb(eps2);
-    s = std::max(s, (-122 - e) / 2);
-    s = std::min(s, (120 - e) / 2);
-  }
-  return s;
 }
 
 cudaError_t launch_sym_force(int prec, int mask, const SymArgs &A0, cudaStream_t s,

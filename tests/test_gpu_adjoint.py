@@ -254,3 +254,62 @@ def test_lent_scratch_takes_each_pair_once(torch_cuda, n, eps):
     bar = 1e-5 + 12 * dx / np.hypot(gap, eps)
     for a, b in zip(out["pairs"][4:], out["one"][4:]):
         assert ((a - b).norm() <= bar * b.norm()).item()
+
+
+@pytest.mark.parametrize("mass,length", [(2e30, 1e17), (2e33, 3e18), (1.0, 1.0), (1e-30, 1e-8)])
+def test_lent_scratch_in_other_units(torch_cuda, mass, length):
+    """Masses and lengths in SI and cgs units (stars, a parsec), masses of 1 and
+    tiny ones: the pair-symmetric forward steps against FP64 sums of the same
+    FP32 inputs and the run without scratch, with the bars of the test above;
+    masses and lengths on powers of two of N-body units scale every bit."""
+    torch = torch_cuda
+    from paper_0909_0879_gb300 import _lib
+
+    n, u = 16384, 2.0**-24
+    m, x, v = ics.plummer(n, 7, masses=ics.salpeter_masses(n, 7))
+    m = m * n * mass
+    x = x * (length / np.abs(x).max())
+    X, M = [torch.tensor(a, dtype=torch.float32, device="cuda") for a in (x, m)]
+    eps = float(np.float32(1e-3 * length))
+    idx = torch.arange(0, n, 97, device="cuda")
+    d = X.double()[None] - X.double()[idx][:, None]
+    t = (M.double() * ((d * d).sum(-1) + eps * eps)**-1.5)[..., None] * d
+    ref, size_of = t.sum(1), t.abs().sum(1)
+    sc = torch.empty(_lib.lf_scratch_bytes(n), dtype=torch.uint8, device="cuda")
+    # a fourth of the softening in a step of this length from rest
+    dt = float(np.sqrt(0.25 * eps / size_of.max().item()))
+    out = []
+    for lent in (sc, None):
+        acc, xs, vs = torch.empty_like(X), X.clone(), torch.zeros_like(X)
+        _lib.lf_forward(n, M, xs, vs, acc, 0, dt, None, eps=eps, scratch=lent)
+        a0 = acc.clone()
+        _lib.lf_forward(n, M, xs, vs, acc, 2, dt, None, eps=eps, scratch=lent)
+        out.append([a.double() for a in (a0, xs, vs)])
+    err = (out[0][0][idx] - ref).abs()
+    assert bool((err <= 80 * u * size_of).all()), (err / size_of).max().item() / u
+    da = 2 * 80 * u * size_of.max().item()
+    dv = 2 * dt * da + 8 * u * out[1][2].abs().max().item()
+    assert (out[0][2] - out[1][2]).abs().max().item() <= dv
+    dx = 2 * dt * dv + 8 * u * X.abs().max().item()
+    assert (out[0][1] - out[1][1]).abs().max().item() <= dx
+
+
+@pytest.mark.parametrize("n", [16384, 65537])
+def test_lent_scratch_scales_exactly(torch_cuda, n):
+    """Powers of two on masses and lengths change no other bit of the
+    acceleration (four and eight i-particles per thread)."""
+    torch = torch_cuda
+    from paper_0909_0879_gb300 import _lib
+
+    m, x, v = ics.plummer(n, 7, masses=ics.salpeter_masses(n, 7))
+    sc = torch.empty(_lib.lf_scratch_bytes(n), dtype=torch.uint8, device="cuda")
+    res = []
+    for pm, px in ((0, 0), (100, 50), (110, 61), (-40, -20)):
+        X, M = [torch.tensor(a, dtype=torch.float32, device="cuda") for a in (x, m)]
+        X, M = X * 2.0**px, M * 2.0**pm
+        acc = torch.empty_like(X)
+        _lib.lf_forward(n, M, X, torch.zeros_like(X), acc, 0, 0.0, None, eps=2.0**(px - 10),
+                        scratch=sc)
+        res.append(acc.double() * 2.0**(2 * px - pm))
+    for a in res[1:]:
+        assert torch.equal(a, res[0])
