@@ -303,7 +303,7 @@ struct nb_ctx {
   bool eq_mass = false;  // every mass is m_eq
   int small_step = -1;   // one launch per shared step: 1 yes, 0 no, -1 not yet looked at
   int small_symp = -1;   // symplectic runs likewise
-  double m_eq = 0.0, m_mean = 0.0;
+  double m_eq = 0.0, m_top = 0.0;  // m_top: the largest
   double *red = nullptr;        // energy scratch
   unsigned char *en_rec = nullptr;  // records of the split-precision energy
   int *err = nullptr;           // device error word
@@ -588,7 +588,7 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
   A->G = c->cfg.G;
   A->eq = c->eq_mass ? 1 : 0;
   A->m_eq = c->m_eq;
-  A->sexp = sym_exponent(c->m_mean, A->eps2);
+  A->sexp = sym_exponent(c->m_top, A->eps2);
   A->recs = c->sym_rec;
   A->ipart = c->sym_i;
   A->jpart = c->sym_j;
@@ -759,7 +759,7 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x,
   c->cfg = *cfg;
   c->n = n;
   c->m_eq = m[0];
-  c->m_mean = std::accumulate(m, m + n, 0.0) / static_cast<double>(n);
+  c->m_top = *std::max_element(m, m + n);
   c->eq_mass = std::all_of(m, m + n, [&](double q) { return q == m[0]; });
   c->n_jt = (n + kJT - 1) / kJT;
   c->n_pad = c->n_jt * kJT;

@@ -213,8 +213,9 @@ struct SymArgs {
   const SymScale *dscale = nullptr;
 };
 // The pair kernel works on positions times 2^s and masses times 2^(3 s) (exact),
-// s = sym_exponent: with 2^(-3 s) near the mass it is given, 1 / r^3 of the
-// scaled positions has the FP32 range that this mass / r^3 has.
+// s = sym_exponent of the largest mass: with 2^(-3 s) near it, 1 / r^3 of the
+// scaled positions has the FP32 range that this mass / r^3 has (with the mean
+// mass a dominant particle's pull on others went to zero too near to it).
 __host__ __device__ inline int sym_exponent(double mass, float eps2) {
   if (!(mass > 0.0) || !isfinite(mass)) return 0;
   int s = static_cast<int>(lround(log2(mass) / -3.0));

@@ -223,3 +223,28 @@ def test_middle_sizes(nb, oracle_mod, n, taken, prec):
     ta, tj = TOL[prec]
     assert np.linalg.norm(got["a"][idx] - ra) <= ta * np.linalg.norm(ra)
     assert np.linalg.norm(got["jerk"][idx] - rj) <= tj * np.linalg.norm(rj)
+
+
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+def test_one_mass_far_above_the_others(nb, prec):
+    """A black hole among stars in units of a solar mass and a kilometre: its
+    pull at some parsecs is a normal float, the mean mass over the cube of that
+    distance is not."""
+    n = MIN_N
+    m, x, v = ics.plummer(n, 31)
+    m, x, v = np.ones(n), x * 3e13, np.zeros((n, 3))
+    m[0], x[0] = 4e6, 0.0
+    r = np.linalg.norm(x, axis=1)
+    x[r > 2e14] *= 0.05
+    kw = dict(eps=1e9, precision=prec)
+    with nb.NBody(m, x, v, block_steps=False, lev_shared=10, **kw) as s:
+        got = s.get_state(want=("a",))["a"]
+    with nb.NBody(m, x, v, **kw) as s:
+        one = s.get_state(want=("a",))["a"]  # block steps: one-sided
+        s.set_symplectic_layout("as_given")
+        s.symplectic(2, 0.0, 1)
+        acc = s.get_state(want=("a",))["a"]
+    assert (np.linalg.norm(one, axis=1)[1:] > 0).all()
+    for a in (got, acc):
+        d = np.linalg.norm(a - one, axis=1) / np.linalg.norm(one, axis=1)
+        assert d[1:].max() <= 2 * TOL[prec][0]  # the hole's pull is nearly all of it
