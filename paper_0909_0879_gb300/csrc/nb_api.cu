@@ -1532,7 +1532,7 @@ bool takes_small_symplectic(nb_ctx *c) {
         small_symp_fits(c->n, c->n_jt, prec, eps_masks(c->cfg.eps), c->num_sms) &&
         cudaGetDevice(&dev) == cudaSuccess &&
         cudaDeviceGetAttribute(&coop, cudaDevAttrCooperativeLaunch, dev) == cudaSuccess && coop &&
-        small_symp_prepare(c->n, c->n_jt, prec, c->num_sms) == cudaSuccess;
+        small_symp_prepare(c->n, prec, c->num_sms) == cudaSuccess;
     c->small_symp = ok ? 1 : 0;
   }
   return c->small_symp == 1;

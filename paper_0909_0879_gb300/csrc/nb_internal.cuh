@@ -281,7 +281,7 @@ struct SmallSympArgs {
   unsigned long long *bar;
 };
 bool small_symp_fits(int64_t n, int64_t n_jt, int prec, int mask, int num_sms);
-cudaError_t small_symp_prepare(int64_t n, int64_t n_jt, int prec, int num_sms);
+cudaError_t small_symp_prepare(int64_t n, int prec, int num_sms);
 cudaError_t launch_small_symplectic(const SmallSympArgs &A, int prec, int num_sms,
                                     cudaStream_t s);
 

@@ -490,10 +490,12 @@ static SmallKernel small_kernel(int prec, int ni) {
   return prec ? small_step_kernel<1, 32> : small_step_kernel<0, 32>;
 }
 
+// The limit belongs to the kernel, which systems of many sizes share: always the
+// most that any of them takes.
 cudaError_t small_step_prepare(int64_t n, int64_t n_jt, int prec, int num_sms) {
   return cudaFuncSetAttribute(small_kernel(prec, small_ni(n, n_jt, num_sms)),
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(small_step_smem(n_jt, prec)));
+                              static_cast<int>(small_step_smem(kSmallMostTiles, prec)));
 }
 
 cudaError_t launch_small_step(const SmallStepArgs &A, int prec, int num_sms, cudaStream_t s) {
@@ -537,10 +539,10 @@ bool small_symp_fits(int64_t n, int64_t n_jt, int prec, int mask, int num_sms) {
   return V.ipt == 1 && V.tpi == 32 && V.threads == 32 * kBlock && !V.rel;
 }
 
-cudaError_t small_symp_prepare(int64_t n, int64_t n_jt, int prec, int num_sms) {
+cudaError_t small_symp_prepare(int64_t n, int prec, int num_sms) {
   return cudaFuncSetAttribute(small_symp_kernel(prec, small_symp_ni(n, num_sms)),
                               cudaFuncAttributeMaxDynamicSharedMemorySize,
-                              static_cast<int>(small_symp_smem(n_jt, prec)));
+                              static_cast<int>(small_symp_smem(kSmallMostTiles, prec)));
 }
 
 cudaError_t launch_small_symplectic(const SmallSympArgs &A, int prec, int num_sms,

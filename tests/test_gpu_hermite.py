@@ -623,3 +623,38 @@ def test_small_run_blocks_equals_general_path(nb, n, prec):
         for k in p:
             assert np.array_equal(p[k], q[k]), k
         assert s.step() == o.step()
+
+
+@pytest.mark.parametrize("prec", ["ds", "fp32"])
+@pytest.mark.parametrize("how", ["step", "run_blocks", "symplectic"])
+def test_small_systems_of_different_size_in_turn(nb, prec, how):
+    """Contexts whose records take different amounts of shared memory in the same
+    kernel, each stepped after the other: as each of them alone."""
+    def go(s, k):
+        if how == "step":
+            s.step()
+        elif how == "run_blocks":
+            s.run_blocks((k + 1) * 2.0**-9)
+        else:
+            s.symplectic(2, 2.0**-9, 1)
+
+    sizes = (4096, 2500, 900, 300)
+    ics_of = {n: ics.plummer(n, n) for n in sizes}
+    kw = dict(eps=1e-2, precision=prec, block_steps=False, lev_shared=9)
+    alone = {}
+    for n in sizes:
+        with nb.NBody(*ics_of[n], **kw) as s:
+            for k in range(3):
+                go(s, k)
+            alone[n] = s.get_state(want=("x", "v"))
+    ctx = {n: nb.NBody(*ics_of[n], **kw) for n in sizes}
+    try:
+        for k in range(3):
+            for n in sizes:
+                go(ctx[n], k)
+        for n in sizes:
+            st = ctx[n].get_state(want=("x", "v"))
+            assert np.array_equal(st["x"], alone[n]["x"]) and np.array_equal(st["v"], alone[n]["v"])
+    finally:
+        for s in ctx.values():
+            s.close()
