@@ -67,7 +67,9 @@ typedef struct {
   int32_t precision; /* nb_precision: pair arithmetic and accumulation */
   int32_t block_steps; /* 1: Aarseth block steps; 0: shared dt = 2^-lev_shared */
   int32_t lev_shared;  /* shared step level when block_steps == 0 */
-  int32_t sync_timeout_ms; /* host watchdog per synchronisation; <= 0: 600 s */
+  int32_t sync_timeout_ms; /* host watchdog per synchronisation, which may have
+                              several queued shared steps in front of it (see
+                              nb_next_block); <= 0: 600 s */
   void *stream;      /* cudaStream_t to queue work on; NULL = default stream */
 } nb_config;
 
@@ -93,9 +95,11 @@ void nb_destroy(nb_ctx *ctx);
  * units) and the number of active particles.  Synchronises the stream, except
  * in a context with shared steps (block_steps == 0) whose particles are all at
  * one time and level, as nb_init, the steps of this library and an nb_set_state
- * with such values leave them: there the answer is known on the host, the
- * call (and nb_step) waits for nothing, and a device-side error of earlier work
- * is reported by the next call that does. */
+ * with such values leave them: there the answer is known on the host, and the
+ * call (and nb_step) waits only where the steps queued since the last wait are
+ * 256 or may take more than a tenth of a second or a quarter of
+ * sync_timeout_ms; a device-side error of earlier work is reported by the next
+ * call that waits. */
 nb_status nb_next_block(nb_ctx *ctx, double *t_next, int64_t *n_active);
 
 /* Predict every particle to time t (Hermite predictor, FP64):

@@ -361,6 +361,8 @@ struct nb_ctx {
   int64_t u_tick = 0;
   int32_t u_lev = 0;
   bool act_all = false;
+  // since the last wait for the stream: steps queued, and `interactions` then
+  int64_t queued_steps = 0, waited_inter = 0;
   // nb_symplectic moved x and v: the Hermite fields (jerk, times, levels)
   // no longer belong to them until nb_set_state
   bool sym_moved = false;
@@ -434,6 +436,8 @@ bool scratch_alloc(void **p, size_t bytes) {
 // Wait for the stream with a host watchdog, then read the device error word
 // and the small scalars into pinned memory.
 nb_status sync_ctx(nb_ctx *c) {
+  c->queued_steps = 0;
+  c->waited_inter = c->interactions;
   // the control slots (t_next, n_act, error word, clamps, device counters)
   // are contiguous: one copy back
   NB_CUDA(cudaMemcpyAsync(c->h_scal, c->scal, kCtlSlots * sizeof(int64_t),
@@ -468,6 +472,23 @@ nb_status sync_ctx(nb_ctx *c) {
                 (err & kErrWaitTimeout) ? "force kernel shared-memory tile; " : "",
                 (err & kErrScanTimeout) ? "active-list look-back; " : "", err);
   }
+  return NB_OK;
+}
+
+// Counts a step that is queued without a wait of its own, and waits first where
+// the steps queued so far make up 256 or (20 us each and 1e12 interactions per
+// second) more than a tenth of a second or a quarter of the watchdog's time: the
+// watchdog then never has a backlog in front of it, and a device-side error is
+// not far behind.
+nb_status bound_queue(nb_ctx *c) {
+  const double limit_ms = c->cfg.sync_timeout_ms > 0 ? 0.25 * c->cfg.sync_timeout_ms : 100.0;
+  const double queued_ms = 0.02 * static_cast<double>(c->queued_steps) +
+                           1.0e-9 * static_cast<double>(c->interactions - c->waited_inter);
+  if (c->queued_steps >= 256 || queued_ms > std::min(limit_ms, 100.0)) {
+    nb_status s = sync_ctx(c);
+    if (s != NB_OK) return s;
+  }
+  c->queued_steps += 1;
   return NB_OK;
 }
 
@@ -899,7 +920,9 @@ nb_status nb_next_block(nb_ctx *c, double *t_next, int64_t *n_active) {
   s = relayout_if_due(c);
   if (s != NB_OK) return s;
   if (c->uniform) {
-    // nothing to look up and nothing to wait for
+    // nothing to look up
+    s = bound_queue(c);
+    if (s != NB_OK) return s;
     if (!c->act_all) {
       NB_CUDA(launch_iota(c->n, c->act, c->stream));
       c->launches += 1;
@@ -1965,10 +1988,12 @@ extern "C" nb_status nb_run_blocks(nb_ctx *c, double t_end, int64_t max_blocks,
     const int64_t step = int64_t(1) << (kTicksLog2 - c->u_lev);
     int64_t done = 0;
     while ((max_blocks == 0 || done < max_blocks) && c->u_tick + step <= tend) {
+      s = bound_queue(c);
+      if (s != NB_OK) return s;
       c->t_block = c->u_tick + step;
       s = queue_small_step(c);
       if (s != NB_OK) return s;
-      if (++done % 256 == 0 && (s = sync_ctx(c)) != NB_OK) return s;
+      ++done;
     }
     s = sync_ctx(c);
     if (s != NB_OK) return s;

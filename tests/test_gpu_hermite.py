@@ -658,3 +658,16 @@ def test_small_systems_of_different_size_in_turn(nb, prec, how):
     finally:
         for s in ctx.values():
             s.close()
+
+
+def test_watchdog_covers_a_bounded_queue(nb):
+    """A loop of shared steps far longer than the watchdog, each step far
+    shorter: the library waits for the queue in between (120 steps of 65,536
+    particles take some 260 ms)."""
+    n = 65536
+    m, x, v = ics.plummer(n, 5)
+    with nb.NBody(m, x, v, eps=1e-2, block_steps=False, lev_shared=10, sync_timeout_ms=100) as s:
+        for k in range(120):
+            assert s.step() == ((k + 1) * 2.0**-10, n)
+        s.sync()  # the wait with the watchdog
+        assert (s.get_state(want=("t_tick",))["t_tick"] == 120 * 2**10).all()
