@@ -6,7 +6,7 @@
 // part (one warp instruction per ~64 cycles per scheduler, ~18 of them per
 // pair, and one CTA per 256 rows of a triangle: 84.1 ms at N = 65,536, 18.3 at
 // 20,000, 0.90 at 1,024).  From kSplitMin particles on the pair terms are
-// evaluated on the FP32 pipe in split precision, about 88 packed operations
+// evaluated on the FP32 pipe in split precision, about 89 packed operations
 // for two pairs, every term to about 2^-46 of itself with unbiased rounding,
 // and summed in split precision and, every 64 records, FP64; the triangle is
 // cut into equal ranges over 2 CTAs per SM: 6.18 / 0.65 / 0.060 ms, bound by
@@ -33,7 +33,11 @@
 //    matters: squares of full 24-bit values have structured last bits, and
 //    rounding those biases the total by 5e-16.  1/r = y0 (1 + e/2 + 3 e^2/8) is
 //    a Newton step with its second-order term.
-//  * m_j / r as a pair, added by an error-free two-sum.
+//  * m_j / r as a pair, added by an error-free two-sum.  m_j is three words: what
+//    two leave out (2^-49) is the same for all particles of one mass and would
+//    not average out (up to 1.8e-15 of the total).  The third costs 2 % of the time
+//    at N = 65,536; taken into the product with e / 2 instead of a product of its
+//    own it leaves a bias of 1e-15.
 // A pair whose |D|^2 + eps^2 would leave the FP32 range, or whose term is a
 // visible part of the total (hard binaries), takes FP64.
 #include "nb_device.cuh"
@@ -208,17 +212,18 @@ __device__ __forceinline__ int length_exp(const unsigned long long *top, double 
 }
 
 // Records of a tile of kJT particles in pairs: planes of 128 float4
-// (h x, y), (h z, m), (l x, y), (l z, m's low word), (rest x, y) and one of
-// float2 (rest z), each value of both particles side by side.
+// (h x, y), (h z, m), (l x, y), (l z, m's low word), (rest x, y), (rest z, m's
+// rest), each value of both particles side by side.
 constexpr int kEnPairs = kJT / 2;
 constexpr int kEnPlane = kEnPairs;  // float4 per plane
-constexpr size_t kEnTileBytes = 5 * kEnPlane * sizeof(float4) + kEnPairs * sizeof(float2);
+constexpr int kEnPlanes = 6;
+constexpr size_t kEnTileBytes = kEnPlanes * kEnPlane * sizeof(float4);
 // j-records of a unit of work: 32 pairs, a quarter of a tile
 constexpr int kEnSub = 32;
 constexpr int kEnSubs = kEnPairs / kEnSub;
 
 struct EnWord {
-  float h[3], l[3], r[3], mh, ml;
+  float h[3], l[3], r[3], mh, ml, mr;
 };
 
 __device__ __forceinline__ EnWord energy_words(const double *__restrict__ m,
@@ -237,7 +242,9 @@ __device__ __forceinline__ EnWord energy_words(const double *__restrict__ m,
   }
   const double ms = m[i] * sm;
   w.mh = static_cast<float>(ms);
-  w.ml = static_cast<float>(ms - static_cast<double>(w.mh));
+  const double mt = ms - static_cast<double>(w.mh);
+  w.ml = static_cast<float>(mt);
+  w.mr = static_cast<float>(mt - static_cast<double>(w.ml));
   return w;
 }
 
@@ -254,7 +261,7 @@ __global__ void __launch_bounds__(kEnPairs)
     if (j < n) {
       w[q] = energy_words(m, x, j, sx, sm);
     } else {  // no mass, outside the box
-      w[q] = EnWord{{2.f, 2.f, 2.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, 0.f, 0.f};
+      w[q] = EnWord{{2.f, 2.f, 2.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, 0.f, 0.f, 0.f};
     }
   }
   const EnWord &a = w[0], &b = w[1];
@@ -263,7 +270,7 @@ __global__ void __launch_bounds__(kEnPairs)
   p[2 * kEnPlane + k] = make_float4(a.l[0], b.l[0], a.l[1], b.l[1]);
   p[3 * kEnPlane + k] = make_float4(a.l[2], b.l[2], a.ml, b.ml);
   p[4 * kEnPlane + k] = make_float4(a.r[0], b.r[0], a.r[1], b.r[1]);
-  reinterpret_cast<float2 *>(p + 5 * kEnPlane)[k] = make_float2(a.r[2], b.r[2]);
+  p[5 * kEnPlane + k] = make_float4(a.r[2], b.r[2], a.mr, b.mr);
 }
 
 // Sum of the blocks' mass sums, by the whole CTA in a fixed order.
@@ -291,8 +298,7 @@ __global__ void __launch_bounds__(kEnThreads, 2)
                         const double *__restrict__ mpart, double *__restrict__ part) {
   using V = float2;
   using O = dev::VOps<V>;
-  __shared__ float4 sj[5][kEnSub];
-  __shared__ float2 sz[kEnSub];
+  __shared__ float4 sj[kEnPlanes][kEnSub];
   __shared__ double sh[kEnThreads];
   const int tid = threadIdx.x;
   const int ex = length_exp(top, eps), em = down_exp(top[1]);
@@ -318,7 +324,7 @@ __global__ void __launch_bounds__(kEnThreads, 2)
     for (int64_t u = u0; u < u1; ++ib, sub = kEnSubs * ib) {
       const int64_t i = ib * kJT + tid;
       const bool real = i < n;
-      EnWord w = EnWord{{3.f, 3.f, 3.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, 0.f, 0.f};
+      EnWord w = EnWord{{3.f, 3.f, 3.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, 0.f, 0.f, 0.f};
       if (real) w = energy_words(m, x, i, sx, sm);
       // m_j / r of a pair that is 1e-3 of the least |W| can be, (M / L)^2 / 7
       const float p_max = real ? static_cast<float>(1.4e-4 * msum * msum / (m[i] * sm)) : 3e38f;
@@ -345,22 +351,21 @@ __global__ void __launch_bounds__(kEnThreads, 2)
         const float4 *src =
             reinterpret_cast<const float4 *>(recs + static_cast<size_t>(jt) * kEnTileBytes);
         __syncthreads();
-        if (tid < 5 * kEnSub)
+        if (tid < kEnPlanes * kEnSub)
           sj[tid / kEnSub][tid % kEnSub] = src[(tid / kEnSub) * kEnPlane + k0 + tid % kEnSub];
-        else if (tid < 6 * kEnSub)
-          sz[tid - 5 * kEnSub] =
-              reinterpret_cast<const float2 *>(src + 5 * kEnPlane)[k0 + tid - 5 * kEnSub];
         __syncthreads();
         const bool own = jt == ib;
 #pragma unroll 2
         for (int k = 0; k < kEnSub; ++k) {
           const float4 a = sj[0][k], b = sj[1][k], c4 = sj[2][k], d4 = sj[3][k], e4 = sj[4][k];
-          const float2 f2 = sz[k];
+          const float4 f4 = sj[5][k];
           const V hj[3] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y)};
           const V lj[3] = {make_float2(c4.x, c4.y), make_float2(c4.z, c4.w),
                            make_float2(d4.x, d4.y)};
-          const V rj[3] = {make_float2(e4.x, e4.y), make_float2(e4.z, e4.w), f2};
+          const V rj[3] = {make_float2(e4.x, e4.y), make_float2(e4.z, e4.w),
+                           make_float2(f4.x, f4.y)};
           V mh = make_float2(b.z, b.w), ml = make_float2(d4.z, d4.w);
+          V mr = make_float2(f4.z, f4.w);
           V D[3], E[3];
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
@@ -373,8 +378,8 @@ __global__ void __launch_bounds__(kEnThreads, 2)
           R = O::fma(D[0], D[0], O::fma(D[1], D[1], R));
           if (own) {  // only j > i counts; the others get a harmless distance
             const int j = 2 * (k0 + k);
-            if (j <= tid) mh.x = ml.x = 0.f, R.x = 1.f;
-            if (j + 1 <= tid) mh.y = ml.y = 0.f, R.y = 1.f;
+            if (j <= tid) mh.x = ml.x = mr.x = 0.f, R.x = 1.f;
+            if (j + 1 <= tid) mh.y = ml.y = mr.y = 0.f, R.y = 1.f;
           }
           // pairs in FP64: squares outside the FP32 range, and terms so large
           // that their own rounding would show in the total
@@ -391,8 +396,8 @@ __global__ void __launch_bounds__(kEnThreads, 2)
                 wi += m[j] * sm * rsqrt(dx * dx + dy * dy + dz * dz + eps_s * eps_s);
               }
             }
-            if (bx) mh.x = ml.x = p.x = 0.f, y.x = 1.f;
-            if (by) mh.y = ml.y = p.y = 0.f, y.y = 1.f;
+            if (bx) mh.x = ml.x = mr.x = p.x = 0.f, y.x = 1.f;
+            if (by) mh.y = ml.y = mr.y = p.y = 0.f, y.y = 1.f;
           }
           const V ny = O::mul(y, mone);
           V s = one, qe = O::bc(0.f), zz = O::bc(0.f);
@@ -421,7 +426,7 @@ __global__ void __launch_bounds__(kEnThreads, 2)
           const V e = O::fma(two, cr, sub2(s, qe));
           // m / r = m y (1 + e / 2 + 3 e^2 / 8) = p - np
           const V w2 = O::mul(e, O::mul(e, O::bc(-0.375f)));
-          V np = O::fma(p, w2, O::fma(mh, ny, p));
+          V np = O::fma(p, w2, O::fma(mr, ny, O::fma(mh, ny, p)));
           np = O::fma(mh, O::mul(ny, O::mul(e, O::bc(0.5f))), O::fma(ml, ny, np));
           const V t = O::add(ah, p);
           const V bb = sub2(t, ah);
