@@ -23,9 +23,9 @@
 //  * Positions, scaled by a power of two to |x| <= 1, are three words: h a
 //    multiple of 2^-23, l a multiple of 2^-46 (|l| <= 2^-24) and the rest.  The
 //    differences of h and of l are then exact in FP32, a fast two-sum makes
-//    them a pair D + E, and the rest's difference joins E: D + E is the
-//    difference of the FP64 positions to 2^-48 of itself, however close the
-//    particles are.
+//    them a pair D + E, and the rest's difference joins E: |E| < 2^-46 beside the
+//    rounding of D, good to 2^-70.  From a softened distance of 2^-24 on (kEnNear)
+//    that is 2^-46 of the distance, and D alone is good enough to start from.
 //  * y0 = rsqrt(|D|^2 + eps^2) from the MUFU (2^-22).  Each component u of y0
 //    (d, eps) is g + its error term, g rounded to the grid 2^-21 (adding 6 and
 //    subtracting it again); g^2 is split at 2^-23 (adding 1), so that 1 - sum
@@ -38,8 +38,9 @@
 //    not average out (up to 1.8e-15 of the total).  The third costs 2 % of the time
 //    at N = 65,536; taken into the product with e / 2 instead of a product of its
 //    own it leaves a bias of 1e-15.
-// A pair whose |D|^2 + eps^2 would leave the FP32 range, or whose term is a
-// visible part of the total (hard binaries), takes FP64.
+// A closer pair, or one whose term is a visible part of the total (hard
+// binaries), takes FP64.  (With every softened distance from 2^-46 on in split
+// precision a close pair of light particles was off by up to 1e-1 of its term.)
 #include "nb_device.cuh"
 
 #include <algorithm>
@@ -216,6 +217,7 @@ __device__ __forceinline__ int length_exp(const unsigned long long *top, double 
 // rest), each value of both particles side by side.
 constexpr int kEnPairs = kJT / 2;
 constexpr int kEnPlane = kEnPairs;  // float4 per plane
+constexpr float kEnNear = 0x1p-48f;  // square of the least softened distance
 constexpr int kEnPlanes = 6;
 constexpr size_t kEnTileBytes = kEnPlanes * kEnPlane * sizeof(float4);
 // j-records of a unit of work: 32 pairs, a quarter of a tile
@@ -381,10 +383,10 @@ __global__ void __launch_bounds__(kEnThreads, 2)
             if (j <= tid) mh.x = ml.x = mr.x = 0.f, R.x = 1.f;
             if (j + 1 <= tid) mh.y = ml.y = mr.y = 0.f, R.y = 1.f;
           }
-          // pairs in FP64: squares outside the FP32 range, and terms so large
+          // pairs in FP64: distances too short for the words, and terms so large
           // that their own rounding would show in the total
           V y = O::rsq<0>(R), p = O::mul(mh, y);
-          const bool bx = R.x < 1e-28f || p.x > p_max, by = R.y < 1e-28f || p.y > p_max;
+          const bool bx = R.x < kEnNear || p.x > p_max, by = R.y < kEnNear || p.y > p_max;
           if (__any_sync(0xffffffffu, bx || by)) {
             for (int q = 0; q < 2; ++q) {
               if (!(q ? by : bx)) continue;

@@ -118,3 +118,20 @@ def test_energy_of_equal_masses(nb, n, mass):
     _, w_ref = _reference(m, x, v, 1e-3)
     with nb.NBody(m, x, v, eps=1e-3) as s:
         assert abs(s.energy()[1] / w_ref - 1.0) <= 8e-16
+
+
+@pytest.mark.parametrize("sep", [1e-13, 1e-12, 1e-10, 1e-8])
+def test_energy_of_close_light_pairs(nb, sep):
+    """Close pairs of light particles, each 1e-5 of the pair energy, at
+    separations near the last bits of the coordinates."""
+    n = 1100
+    for seed in range(4):
+        m, x, v = ics.plummer(n, 71 + seed)
+        r = np.random.default_rng(seed)
+        for k in range(10, 20, 2):
+            m[k] = m[k + 1] = np.sqrt(1e-5 * sep)
+            d = r.normal(size=3)
+            x[k + 1] = x[k] + sep / np.linalg.norm(d) * d
+        _, w_ref = _reference(m, x, v, 0.0)
+        with nb.NBody(m, x, v, eps=0.0) as s:
+            assert abs(s.energy()[1] / w_ref - 1.0) <= BAR
