@@ -2110,18 +2110,22 @@ nb_status nb_energy(nb_ctx *c, double *kin, double *pot, double *tot) {
   Range r("nb_energy");
   nb_status s = check_ctx(c);
   if (s != NB_OK) return s;
-  int nl = 0;
-  double *d_out = c->red + energy_scratch_doubles(c->n) - 3;
+  double *d_out = c->red + energy_scratch_doubles(c->n) - 4;
   const size_t rb = energy_record_bytes(c->n);
-  // without room for the records: the FP64 pair sum
+  // without room for the records, or where the kernels ask for it: the FP64
+  // pair sum
   if (rb && !c->en_rec) scratch_alloc(reinterpret_cast<void **>(&c->en_rec), rb);
-  NB_CUDA(launch_energy(c->n, c->m, c->x, c->v, c->cfg.G, c->cfg.eps, c->ext, c->red,
-                        rb ? c->en_rec : nullptr, c->num_sms, d_out, c->stream, &nl));
-  c->launches += nl;
-  NB_CUDA(cudaMemcpyAsync(c->h_energy, d_out, 3 * sizeof(double), cudaMemcpyDeviceToHost,
-                          c->stream));
-  s = sync_ctx(c);
-  if (s != NB_OK) return s;
+  for (unsigned char *recs = rb ? c->en_rec : nullptr;; recs = nullptr) {
+    int nl = 0;
+    NB_CUDA(launch_energy(c->n, c->m, c->x, c->v, c->cfg.G, c->cfg.eps, c->ext, c->red, recs,
+                          c->num_sms, d_out, c->stream, &nl));
+    c->launches += nl;
+    NB_CUDA(cudaMemcpyAsync(c->h_energy, d_out, 4 * sizeof(double), cudaMemcpyDeviceToHost,
+                            c->stream));
+    s = sync_ctx(c);
+    if (s != NB_OK) return s;
+    if (c->h_energy[3] == 0.0) break;
+  }
   const double w = c->h_energy[1] + c->h_energy[2];
   if (kin) *kin = c->h_energy[0];
   if (pot) *pot = w;

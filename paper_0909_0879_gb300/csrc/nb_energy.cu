@@ -136,22 +136,6 @@ __global__ void ext_potential_kernel(int64_t n, const ExtField E, const double *
   if (threadIdx.x == 0) part[blockIdx.x] = s;
 }
 
-// Sums in a fixed order: out = {sum kin, -G sum pot, sum ext}.
-__global__ void energy_final_kernel(int64_t n_kin, const double *__restrict__ kin, int64_t n_pot,
-                                    const double *__restrict__ pot, int64_t n_ext,
-                                    const double *__restrict__ ext, double G,
-                                    double *__restrict__ out) {
-  __shared__ double sh[kEnThreads];
-  const double *const src[3] = {kin, pot, ext};
-  const int64_t cnt[3] = {n_kin, n_pot, n_ext};
-  for (int k = 0; k < 3; ++k) {
-    double s = 0.0;
-    for (int64_t b = threadIdx.x; b < cnt[k]; b += blockDim.x) s += src[k][b];
-    s = block_sum(s, sh);
-    if (threadIdx.x == 0) out[k] = k == 1 ? -G * s : s;
-  }
-}
-
 // ---- split-precision pair sum
 
 // Kinetic energy and mass of the block's particles into part[blockIdx.x]
@@ -250,9 +234,14 @@ __device__ __forceinline__ EnWord energy_words(const double *__restrict__ m,
   return w;
 }
 
+// The records of a tile, and the sum of its squared (scaled) masses into
+// m2part[blockIdx.x].
 __global__ void __launch_bounds__(kEnPairs)
     energy_records_kernel(int64_t n, const double *__restrict__ m, const double *__restrict__ x,
-                          double eps, const unsigned long long *top, unsigned char *recs) {
+                          double eps, const unsigned long long *top, unsigned char *recs,
+                          double *__restrict__ m2part) {
+  __shared__ double sh[kEnPairs];
+  double m2 = 0.0;
   const double sx = pow2d(-length_exp(top, eps)), sm = pow2d(-down_exp(top[1]));
   const int k = threadIdx.x;
   float4 *p = reinterpret_cast<float4 *>(recs + static_cast<size_t>(blockIdx.x) * kEnTileBytes);
@@ -262,6 +251,7 @@ __global__ void __launch_bounds__(kEnPairs)
     const int64_t j = static_cast<int64_t>(blockIdx.x) * kJT + 2 * k + q;
     if (j < n) {
       w[q] = energy_words(m, x, j, sx, sm);
+      m2 += (m[j] * sm) * (m[j] * sm);
     } else {  // no mass, outside the box
       w[q] = EnWord{{2.f, 2.f, 2.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, 0.f, 0.f, 0.f};
     }
@@ -273,6 +263,8 @@ __global__ void __launch_bounds__(kEnPairs)
   p[3 * kEnPlane + k] = make_float4(a.l[2], b.l[2], a.ml, b.ml);
   p[4 * kEnPlane + k] = make_float4(a.r[0], b.r[0], a.r[1], b.r[1]);
   p[5 * kEnPlane + k] = make_float4(a.r[2], b.r[2], a.mr, b.mr);
+  m2 = block_sum(m2, sh);
+  if (k == 0) m2part[blockIdx.x] = m2;
 }
 
 // Sum of the blocks' mass sums, by the whole CTA in a fixed order.
@@ -328,7 +320,8 @@ __global__ void __launch_bounds__(kEnThreads, 2)
       const bool real = i < n;
       EnWord w = EnWord{{3.f, 3.f, 3.f}, {0.f, 0.f, 0.f}, {0.f, 0.f, 0.f}, 0.f, 0.f, 0.f};
       if (real) w = energy_words(m, x, i, sx, sm);
-      // m_j / r of a pair that is 1e-3 of the least |W| can be, (M / L)^2 / 7
+      // m_j / r of a pair that is 1.4e-3 of the least |W| can be, M^2 / (10 L) where
+      // no particle dominates (see energy_final_kernel)
       const float p_max = real ? static_cast<float>(1.4e-4 * msum * msum / (m[i] * sm)) : 3e38f;
       V nh[3], nl[3], nr[3];
 #pragma unroll
@@ -448,11 +441,46 @@ __global__ void __launch_bounds__(kEnThreads, 2)
   if (tid == 0) part[blockIdx.x] = t * pow2d(-ex) * pow2d(em);
 }
 
+// Sums in a fixed order: out = {sum kin, -G sum pot, sum ext}; out[3] says whether
+// the split-precision pair sum is to be thrown away for the FP64 one, because one
+// particle dominates: the squares of the masses add up to more than a fourth of
+// the square of their sum.  The pair energy is then the terms of that particle,
+// too few for their roundings to average out (1,100 particles around a heavy one:
+// 1.5e-15 against 6e-16 in FP64), and with light particles below 2^-64 of the
+// heavy one the correction of a term leaves the FP32 range (5e-31: 2e-8, below
+// 1e-38 the whole term).
+__global__ void energy_final_kernel(int64_t nb, const double *__restrict__ kin, int64_t n_pot,
+                                    const double *__restrict__ pot, int64_t n_ext,
+                                    const double *__restrict__ ext, double G,
+                                    const unsigned long long *top,
+                                    const double *__restrict__ mpart,
+                                    const double *__restrict__ m2part,
+                                    double *__restrict__ out) {
+  __shared__ double sh[kEnThreads];
+  auto sum = [&](int64_t cnt, const double *src) {
+    double s = 0.0;
+    for (int64_t b = threadIdx.x; b < cnt; b += blockDim.x) s += src[b];
+    return block_sum(s, sh);
+  };
+  const double k = sum(nb, kin), w = sum(n_pot, pot), e = sum(n_ext, ext);
+  bool redo = false;
+  if (mpart) {
+    const double mass = sum(nb, mpart) * pow2d(-down_exp(top[1])), m2 = sum(nb, m2part);
+    redo = !(m2 <= 0.25 * mass * mass) || !isfinite(w);
+  }
+  if (threadIdx.x == 0) {
+    out[0] = k;
+    out[1] = -G * w;
+    out[2] = e;
+    out[3] = redo ? 1.0 : 0.0;
+  }
+}
+
 }  // namespace
 
 int64_t energy_scratch_doubles(int64_t n) {
   const int64_t nb = (n + kEnThreads - 1) / kEnThreads;
-  return 3 * nb + std::max<int64_t>(nb, kEnMaxCtas) + 5;
+  return 4 * nb + std::max<int64_t>(nb, kEnMaxCtas) + 6;
 }
 
 size_t energy_record_bytes(int64_t n) {
@@ -469,14 +497,15 @@ cudaError_t launch_energy(int64_t n, const double *m, const double *x, const dou
   double *pe = pk + nb;
   double *pw = pe + nb;
   unsigned long long *top =
-      reinterpret_cast<unsigned long long *>(red + energy_scratch_doubles(n) - 5);
+      reinterpret_cast<unsigned long long *>(red + energy_scratch_doubles(n) - 6);
+  double *pm = pw + std::max<int64_t>(nb, kEnMaxCtas);
+  double *pm2 = pm + nb;
   int64_t np = nb;
   if (recs) {
     cudaError_t e = cudaMemsetAsync(top, 0, 2 * sizeof(*top), s);
     if (e != cudaSuccess) return e;
-    double *pm = pw + std::max<int64_t>(nb, kEnMaxCtas);
     energy_scan_kernel<<<g, kEnThreads, 0, s>>>(n, m, x, v, pk, pm, top);
-    energy_records_kernel<<<g, kEnPairs, 0, s>>>(n, m, x, eps, top, recs);
+    energy_records_kernel<<<g, kEnPairs, 0, s>>>(n, m, x, eps, top, recs, pm2);
     np = std::min<int64_t>(std::min<int64_t>(2 * num_sms, kEnMaxCtas), tri_start(nb, nb));
     const unsigned gp = static_cast<unsigned>(np);
     if (eps > 0.0)
@@ -490,7 +519,8 @@ cudaError_t launch_energy(int64_t n, const double *m, const double *x, const dou
     if (launches) *launches += 2;
   }
   if (E.on) ext_potential_kernel<<<g, kEnThreads, 0, s>>>(n, E, m, x, pe);
-  energy_final_kernel<<<1, kEnThreads, 0, s>>>(nb, pk, np, pw, E.on ? nb : 0, pe, G, d_out);
+  energy_final_kernel<<<1, kEnThreads, 0, s>>>(nb, pk, np, pw, E.on ? nb : 0, pe, G, top,
+                                               recs ? pm : nullptr, pm2, d_out);
   if (launches) *launches += E.on ? 2 : 1;
   return cudaGetLastError();
 }

@@ -332,7 +332,7 @@ constexpr int64_t kEnMaxCtas = 1024;
 // Kinetic and softened potential energy into d_out[0..1], and the external
 // field's potential energy sum_i m_i Phi(x_i) into d_out[2] (0 when E.on
 // is 0).  recs: energy_record_bytes(n) of scratch, or null for the FP64
-// pair sum.
+// pair sum.  d_out[3] is not 0 where this system needs the latter.
 cudaError_t launch_energy(int64_t n, const double *m, const double *x,
                           const double *v, double G, double eps, const ExtField &E,
                           double *red, unsigned char *recs, int num_sms, double *d_out,

@@ -135,3 +135,46 @@ def test_energy_of_close_light_pairs(nb, sep):
         _, w_ref = _reference(m, x, v, 0.0)
         with nb.NBody(m, x, v, eps=0.0) as s:
             assert abs(s.energy()[1] / w_ref - 1.0) <= BAR
+
+
+def _without_scratch(s):
+    os.environ["NB_TEST_MAX_BYTES"] = "1000"
+    try:
+        return s.energy()  # the FP64 sum
+    finally:
+        del os.environ["NB_TEST_MAX_BYTES"]
+
+
+@pytest.mark.parametrize("ratio", [1e-6, 1e-18, 5e-31, 1e-37, 1e-45, 0.0])
+@pytest.mark.parametrize("first", [True, False])
+def test_energy_around_a_dominant_particle(nb, ratio, first):
+    """Far lighter particles before or after a heavy one: the FP64 sum, whose
+    chain of n additions is good to n / 2 ulps."""
+    n = 1100
+    m, x, v = ics.plummer(n, 71, masses=ics.salpeter_masses(n, 72))
+    m *= ratio * n
+    m[0 if first else n - 1] = 1.0
+    m[1 if first else 0] = 0.0
+    _, w_ref = _reference(m, x, v, 1e-4)
+    with nb.NBody(m, x, v, eps=1e-4) as s, nb.NBody(m, x, v, eps=1e-4) as o:
+        w, w64 = s.energy()[1], _without_scratch(o)[1]
+    assert w == w64
+    assert abs(w - w_ref) <= n * 2.0**-53 * abs(w_ref)
+
+
+def test_energy_of_two_light_particles_around_a_heavy_one(nb):
+    """Their own term is most of the pair energy, and small beside the square of
+    the total mass."""
+    n = 1024
+    for seed in range(16):
+        r = np.random.default_rng(seed)
+        m, x, v = np.full(n, 1e-13), r.uniform(-1, 1, (n, 3)), np.zeros((n, 3))
+        m[0] = 1.0
+        m[5], m[700] = 2.9e-6, 2.9e-6
+        d = r.normal(size=3)
+        x[700] = x[5] + 6.3e-8 * d / np.linalg.norm(d)
+        _, w_ref = _reference(m, x, v, 0.0)
+        with nb.NBody(m, x, v, eps=0.0) as s, nb.NBody(m, x, v, eps=0.0) as o:
+            w, w64 = s.energy()[1], _without_scratch(o)[1]
+        assert w == w64
+        assert abs(w - w_ref) <= n * 2.0**-53 * abs(w_ref)
