@@ -9,15 +9,14 @@
 // evaluated on the FP32 pipe in split precision, about 89 packed operations
 // for two pairs, every term to about 2^-46 of itself with unbiased rounding,
 // and summed in split precision and, every 64 records, FP64; the triangle is
-// cut into equal ranges over 2 CTAs per SM: 6.18 / 0.65 / 0.060 ms, bound by
+// cut into equal ranges over 2 CTAs per SM: 6.32 / 0.67 / 0.062 ms, bound by
 // the FP32 pipe (0.76 of its rate).  The total is as exact as the FP64 sum,
 // whose own rounding it replaces, because the term errors are independent
 // and average over the N^2 / 2 pairs: relative error against extended
 // precision, rms over 36 systems of N = 1,024 to 40,000 (Salpeter masses,
 // softening 0 to 1e-2, with and without hard binaries), 1.2e-16 against
-// 1.6e-16.  (Where the softening is as long as the separations, so that the
-// softened distances hardly differ, the rounding is not independent: 4e-16
-// to 6e-16.)
+// 1.6e-16.  Systems whose term errors are not independent, or too few, take the
+// FP64 sum after all (see energy_final_kernel).
 //
 // Pair term:
 //  * Positions, scaled by a power of two to |x| <= 1, are three words: h a
@@ -442,16 +441,21 @@ __global__ void __launch_bounds__(kEnThreads, 2)
 }
 
 // Sums in a fixed order: out = {sum kin, -G sum pot, sum ext}; out[3] says whether
-// the split-precision pair sum is to be thrown away for the FP64 one, because one
-// particle dominates: the squares of the masses add up to more than a fourth of
-// the square of their sum.  The pair energy is then the terms of that particle,
-// too few for their roundings to average out (1,100 particles around a heavy one:
-// 1.5e-15 against 6e-16 in FP64), and with light particles below 2^-64 of the
-// heavy one the correction of a term leaves the FP32 range (5e-31: 2e-8, below
-// 1e-38 the whole term).
+// the split-precision pair sum is to be thrown away for the FP64 one, because its
+// terms' roundings would not average out:
+//  * One particle dominates: the squares of the masses add up to more than a
+//    fourth of the square of their sum.  The pair energy is then the terms of that
+//    particle, too few of them (1,100 particles around a heavy one: 1.5e-15 against
+//    6e-16 in FP64), and with light particles below 2^-64 of the heavy one the
+//    correction of a term leaves the FP32 range (5e-31: 2e-8, below 1e-38 the
+//    whole term).
+//  * The softening is more than a fourth of the harmonic mean softened distance:
+//    the distances hardly differ, and neither do the roundings (Plummer spheres of
+//    1,024 and 1,500, softening over that distance 0.1 / 0.26 / 0.49 / 0.99: mean
+//    error 6e-17 / 1.1e-16 / 2.5e-16 / 3e-16, FP64 1e-16 throughout).
 __global__ void energy_final_kernel(int64_t nb, const double *__restrict__ kin, int64_t n_pot,
                                     const double *__restrict__ pot, int64_t n_ext,
-                                    const double *__restrict__ ext, double G,
+                                    const double *__restrict__ ext, double G, double eps,
                                     const unsigned long long *top,
                                     const double *__restrict__ mpart,
                                     const double *__restrict__ m2part,
@@ -465,8 +469,9 @@ __global__ void energy_final_kernel(int64_t nb, const double *__restrict__ kin, 
   const double k = sum(nb, kin), w = sum(n_pot, pot), e = sum(n_ext, ext);
   bool redo = false;
   if (mpart) {
-    const double mass = sum(nb, mpart) * pow2d(-down_exp(top[1])), m2 = sum(nb, m2part);
-    redo = !(m2 <= 0.25 * mass * mass) || !isfinite(w);
+    const double sm = pow2d(-down_exp(top[1]));
+    const double mass = sum(nb, mpart) * sm, m2 = sum(nb, m2part), most = 0.25 * mass * mass;
+    redo = !(m2 <= most) || !(2.0 * eps * (w * sm * sm) <= most);
   }
   if (threadIdx.x == 0) {
     out[0] = k;
@@ -519,7 +524,7 @@ cudaError_t launch_energy(int64_t n, const double *m, const double *x, const dou
     if (launches) *launches += 2;
   }
   if (E.on) ext_potential_kernel<<<g, kEnThreads, 0, s>>>(n, E, m, x, pe);
-  energy_final_kernel<<<1, kEnThreads, 0, s>>>(nb, pk, np, pw, E.on ? nb : 0, pe, G, top,
+  energy_final_kernel<<<1, kEnThreads, 0, s>>>(nb, pk, np, pw, E.on ? nb : 0, pe, G, eps, top,
                                                recs ? pm : nullptr, pm2, d_out);
   if (launches) *launches += E.on ? 2 : 1;
   return cudaGetLastError();

@@ -178,3 +178,21 @@ def test_energy_of_two_light_particles_around_a_heavy_one(nb):
             w, w64 = s.energy()[1], _without_scratch(o)[1]
         assert w == w64
         assert abs(w - w_ref) <= n * 2.0**-53 * abs(w_ref)
+
+
+# a twentieth of the harmonic mean distance, more than half of it, and far more
+@pytest.mark.parametrize("eps,fp64", [(0.05, False), (1.0, True), (4.0, True), (1e4, True)])
+@pytest.mark.parametrize("n", [1024, 1300])
+def test_energy_where_softening_dominates(nb, eps, fp64, n):
+    """Softening as long as the separations and longer: hardly any of the
+    roundings are independent, and the FP64 sum is taken."""
+    same = []
+    for seed in range(3):
+        m, x, v = ics.plummer(n, 71 + seed, masses=ics.salpeter_masses(n, 72))
+        x = x + np.array([30.0, 0.0, 0.0])
+        _, w_ref = _reference(m, x, v, eps)
+        with nb.NBody(m, x, v, eps=eps) as s, nb.NBody(m, x, v, eps=eps) as o:
+            w, w64 = s.energy()[1], _without_scratch(o)[1]
+        assert abs(w / w_ref - 1.0) <= BAR
+        same.append(w == w64)
+    assert all(same) or not fp64
