@@ -132,9 +132,9 @@ nb_status nb_force_jerk(nb_ctx *ctx, const int32_t *idx, int64_t n_idx,
  * once for both particles; rows that are handed out are the one-sided
  * kernel's, the same for any list a particle stands in.  The two differ by
  * rounding only.  The partial sums of the pair-symmetric form take device
- * memory of the context (3.9 GB at n = 2^20, growing as n; nothing above
- * 1/16 of the device's memory or half of what is free: then, and with a
- * forced shape, table or grid, the one-sided kernel runs). */
+ * memory of the context (3.9 GB at n = 2^20, growing as n).  Where they would
+ * be above 1/16 of the device's memory or cannot be allocated, and with a
+ * forced shape, table or grid, the one-sided kernel runs. */
 nb_status nb_force_jerk_dev(nb_ctx *ctx, const int32_t *d_idx, int64_t n_idx,
                             double *d_acc, double *d_jerk);
 
@@ -290,7 +290,9 @@ nb_status nb_energy(nb_ctx *ctx, double *kin, double *pot, double *tot);
 /* Copy the integrator state to host arrays (any may be NULL):
  * x, v, a, jerk (n,3); t_tick (n) int64 ticks of 2^-20; lev (n) int32.
  * Synchronises.  Together with nb_set_state this is checkpoint/resume:
- * a run continued from a copied state is bitwise identical. */
+ * a run continued from a copied state is bitwise identical (where either of two
+ * contexts had no room for the partial sums of the pair-symmetric force, see
+ * nb_force_jerk_dev: identical up to rounding). */
 nb_status nb_get_state(nb_ctx *ctx, double *x, double *v, double *a,
                        double *jerk, int64_t *t_tick, int32_t *lev);
 

@@ -248,3 +248,28 @@ def test_one_mass_far_above_the_others(nb, prec):
     for a in (got, acc):
         d = np.linalg.norm(a - one, axis=1) / np.linalg.norm(one, axis=1)
         assert d[1:].max() <= 2 * TOL[prec][0]  # the hole's pull is nearly all of it
+
+
+def test_path_does_not_follow_free_memory(nb):
+    """A context made while most of the device is in use takes the same kernel,
+    and so gives the same bits, as one made on an empty device."""
+    import torch
+
+    n = 262144
+    m, x, v = ics.plummer(n, 31)
+    p = nb.spatial_order(x, 256)
+    m, x, v = m[p], x[p], v[p]
+    kw = dict(eps=1e-3, block_steps=False, lev_shared=10)
+    with nb.NBody(m, x, v, **kw) as s:
+        want = s.get_state(want=("a",))["a"]
+    torch.cuda.empty_cache()
+    free, _ = torch.cuda.mem_get_info()
+    # the partial sums take 1 GB at this n, the context 0.2 GB
+    hold = torch.empty(max(0, free - (7 << 28)), dtype=torch.uint8, device="cuda")
+    try:
+        with nb.NBody(m, x, v, **kw) as s:
+            got = s.get_state(want=("a",))["a"]
+    finally:
+        del hold
+        torch.cuda.empty_cache()
+    assert np.array_equal(got, want)
