@@ -294,11 +294,10 @@ struct nb_ctx {
   int64_t *scal = nullptr;      // [0] t_next ticks, [1] n_act
   double *part = nullptr;       // force partial sums
   size_t part_cap = 0;
-  // partial sums of the pair-symmetric force of all particles (allocated at
-  // its first use; sym_off: no room for them, the one-sided kernel runs)
-  float2 *sym_i = nullptr, *sym_j = nullptr;
-  unsigned char *sym_rec = nullptr;
-  size_t sym_i_cap = 0, sym_j_cap = 0;
+  // records and partial sums of the pair-symmetric force of all particles
+  // (allocated at its first use; sym_off: no room, the one-sided kernel runs)
+  unsigned char *sym_buf = nullptr;
+  size_t sym_cap = 0;
   bool sym_off = false;
   bool eq_mass = false;  // every mass is m_eq
   int small_step = -1;   // one launch per shared step: 1 yes, 0 no, -1 not yet looked at
@@ -562,43 +561,28 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
   SymSplit S;
   const int bi = sym_block_i(prec, mask, jrk, c->n_jt);
   if (!sym_split(c->n_jt, bi, c->num_sms, &S) || !sym_pays(c->n, S, bi, c->num_sms)) return false;
-  const size_t ib = sym_ipart_bytes(S, jrk), jb = sym_jpart_bytes(S, jrk);
-  const size_t rb = sym_record_bytes(c->n_jt, prec);
-  if (ib > c->sym_i_cap || jb > c->sym_j_cap) {
+  auto up = [](size_t b) { return (b + 255) / 256 * 256; };
+  const size_t at_i = up(sym_record_bytes(c->n_jt, prec));
+  const size_t at_j = at_i + up(sym_ipart_bytes(S, jrk));
+  const size_t need = at_j + up(sym_jpart_bytes(S, jrk));
+  // one allocation, and no other: a context with shared steps asks for the
+  // jerk's sums first (nb_init), one with block steps for the acceleration's only
+  if (!c->sym_buf) {
     // the device's memory, not what is free of it: a context made on a fuller
     // device takes the same kernel, and gives the same bits, while it has room
     size_t avail = 0, total = 0;
-    bool ok = cudaMemGetInfo(&avail, &total) == cudaSuccess && ib + jb + rb <= total / 16;
-    // grows once: from the acceleration's sums to the jerk's
-    float2 *ni = nullptr, *nj = nullptr;
-    if (ok && !c->sym_rec) ok = scratch_alloc(reinterpret_cast<void **>(&c->sym_rec), rb);
-    if (ok) ok = scratch_alloc(reinterpret_cast<void **>(&ni), ib) &&
-                 scratch_alloc(reinterpret_cast<void **>(&nj), jb);
-    if (ok) ok = sym_prepare(prec, mask, true, c->eq_mass, c->n_jt) == cudaSuccess &&
-                 sym_prepare(prec, mask, false, c->eq_mass, c->n_jt) == cudaSuccess;
+    const bool ok = cudaMemGetInfo(&avail, &total) == cudaSuccess && need <= total / 16 &&
+                    sym_prepare(prec, mask, true, c->eq_mass, c->n_jt) == cudaSuccess &&
+                    sym_prepare(prec, mask, false, c->eq_mass, c->n_jt) == cudaSuccess &&
+                    scratch_alloc(reinterpret_cast<void **>(&c->sym_buf), need);
     if (!ok) {
       cudaGetLastError();  // a refused query is not this call's error
-      if (ni) cudaFree(ni);
-      if (nj) cudaFree(nj);
-      // scratch that is there still serves the acceleration
-      if (!c->sym_j) c->sym_off = true;
+      c->sym_off = true;
       return false;
     }
-    if (c->sym_j) {
-      cudaStreamSynchronize(c->stream);
-      cudaFree(c->sym_i);
-      cudaFree(c->sym_j);
-      for (cudaGraphExec_t *g : {&c->sym_graph, &c->blk_graph, &c->fus_graph})
-        if (*g) {  // may hold the old scratch
-          cudaGraphExecDestroy(*g);
-          *g = nullptr;
-        }
-    }
-    c->sym_i = ni;
-    c->sym_j = nj;
-    c->sym_i_cap = ib;
-    c->sym_j_cap = jb;
+    c->sym_cap = need;
   }
+  if (need > c->sym_cap) return false;
   A->jhi = c->jhi;
   A->jlo = c->jlo;
   A->jvel = c->jvel;
@@ -611,9 +595,9 @@ bool sym_ready(nb_ctx *c, bool jrk, SymArgs *A) {
   A->eq = c->eq_mass ? 1 : 0;
   A->m_eq = c->m_eq;
   A->sexp = sym_exponent(c->m_top, A->eps2);
-  A->recs = c->sym_rec;
-  A->ipart = c->sym_i;
-  A->jpart = c->sym_j;
+  A->recs = c->sym_buf;
+  A->ipart = reinterpret_cast<float2 *>(c->sym_buf + at_i);
+  A->jpart = reinterpret_cast<float2 *>(c->sym_buf + at_j);
   A->err = c->err;
   A->split = S;
   return true;
@@ -749,9 +733,7 @@ void nb_destroy(nb_ctx *c) {
   for (void *p : c->allocs)
     if (p) cudaFree(p);
   if (c->en_rec) cudaFree(c->en_rec);
-  if (c->sym_rec) cudaFree(c->sym_rec);
-  if (c->sym_i) cudaFree(c->sym_i);
-  if (c->sym_j) cudaFree(c->sym_j);
+  if (c->sym_buf) cudaFree(c->sym_buf);
   if (c->h_scal) cudaFreeHost(c->h_scal);
   if (c->h_energy) cudaFreeHost(c->h_energy);
   if (c->h_sh_off) cudaFreeHost(c->h_sh_off);

@@ -433,14 +433,11 @@ __global__ void __launch_bounds__(kLfVjpMaxThreads)
   }
 }
 
-// v += a h; then, if drift, x += v dt.
-__global__ void lf_kick_drift_kernel(int64_t n3, float *__restrict__ x, float *__restrict__ v,
-                                     const float *__restrict__ a, float h, float dt, int drift) {
+// v += a h.
+__global__ void lf_kick_kernel(int64_t n3, float *__restrict__ v, const float *__restrict__ a,
+                               float h) {
   const int64_t q = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (q >= n3) return;
-  const float vn = fmaf(a[q], h, v[q]);
-  v[q] = vn;
-  if (drift) x[q] = fmaf(vn, dt, x[q]);
+  if (q < n3) v[q] = fmaf(a[q], h, v[q]);
 }
 
 // One drift of a run of KDK steps with the kicks around it merged: with
@@ -735,10 +732,9 @@ cudaError_t lf_vjp(LfCtx &C, const float *x, const float *lv, float h, float *lx
                 : launch_lf_vjp<0, 2>(C, x, lv, h, lx, lm, lv_out, dlv);
 }
 
-cudaError_t lf_kick(LfCtx &C, float *x, float *v, const float *a, float h, float dt, int drift) {
+cudaError_t lf_kick(LfCtx &C, float *v, const float *a, float h) {
   const int64_t n3 = 3 * C.n;
-  lf_kick_drift_kernel<<<static_cast<unsigned>((n3 + 255) / 256), 256, 0, C.s>>>(n3, x, v, a, h,
-                                                                                  dt, drift);
+  lf_kick_kernel<<<static_cast<unsigned>((n3 + 255) / 256), 256, 0, C.s>>>(n3, v, a, h);
   ++C.launches;
   return cudaGetLastError();
 }
@@ -902,7 +898,7 @@ nb_status nb_lf_forward_lent(int64_t n, const float *d_m, float *d_x, float *d_v
   if (e == cudaSuccess) e = lf_acc(C, d_x, d_acc);
   for (int64_t st = 0; st < nsteps && e == cudaSuccess; ++st)
     e = lf_half_step(C, d_x, d_x, d_v, d_v, d_acc, dt, st > 0, ck(st));
-  if (e == cudaSuccess && nsteps > 0) e = lf_kick(C, d_x, d_v, d_acc, 0.5f * dt, dt, 0);
+  if (e == cudaSuccess && nsteps > 0) e = lf_kick(C, d_v, d_acc, 0.5f * dt);
   return e == cudaSuccess ? NB_OK : lf_err(e);
 }
 
