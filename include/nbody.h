@@ -134,7 +134,10 @@ nb_status nb_force_jerk(nb_ctx *ctx, const int32_t *idx, int64_t n_idx,
  * rounding only.  The partial sums of the pair-symmetric form take device
  * memory of the context (3.9 GB at n = 2^20, growing as n).  Where they would
  * be above 1/16 of the device's memory or cannot be allocated, and with a
- * forced shape, table or grid, the one-sided kernel runs. */
+ * forced shape, table or grid, the one-sided kernel runs.  nb_init allocates
+ * them where its own steps take this form, and, for nb_symplectic, in every
+ * context of fewer than 32768 particles that has enough for it (30 to 80 MB);
+ * otherwise the first nb_symplectic call does. */
 nb_status nb_force_jerk_dev(nb_ctx *ctx, const int32_t *d_idx, int64_t n_idx,
                             double *d_acc, double *d_jerk);
 

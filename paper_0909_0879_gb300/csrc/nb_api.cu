@@ -859,10 +859,11 @@ nb_status nb_init(nb_ctx **out, int64_t n, const double *m, const double *x,
     TRY(queue_sym(c, SA, c->a, c->jk));
   } else {
     TRY(queue_force(c, nullptr, n, c->a, c->jk));
-    // Scratch for symplectic steps of a middle-sized system (at most 80 MB)
-    // now: allocated by the first of them it made that call 0.1 .. 0.2 ms
-    // longer, more than the kernel saves in it (N = 7,000 239 -> 344 us, N =
-    // 20,000 482 -> 521 us; from 40,000 on the call still gains).
+    // Scratch for symplectic steps of a middle-sized system (30 to 80 MB) now,
+    // behind the queued force, where it takes 20 us: allocated by the first
+    // nb_symplectic it makes that call 90 us longer, more than the kernel saves in
+    // one step (leapfrog, N = 7,168 / 12,000 / 16,384 / 20,000: 207 / 333 / 390 / 508
+    // against 118 / 241 / 299 / 414 us, one-sided 136 / 264 / 383 / 560).
     if (n < 2 * kSymMin) sym_ready(c, false, &SA);
   }
   TRYC(launch_init_levels(n, c->a, c->jk, cfg->eta_start, cfg->lev_min, cfg->lev_max,
