@@ -14,13 +14,10 @@ import torch
 from . import _lib
 
 
-_SCRATCH_FROM = 16384  # _lib.lf_scratch_bytes(n) is 0 below (spares small systems the call)
-
-
 def _scratch(n, device):
     """Memory for the pair-symmetric force, or None (small n, or no room: the
     one-sided force needs none)."""
-    size = _lib.lf_scratch_bytes(n) if n >= _SCRATCH_FROM else 0
+    size = _lib.lf_scratch_bytes(n)
     if size == 0:
         return None
     try:
@@ -43,9 +40,13 @@ class LeapfrogFunction(torch.autograd.Function):
         acc = torch.empty_like(x)
         ckpt = torch.empty(_lib.lf_ckpt_floats(n, nsteps, ckpt_every), dtype=torch.float32,
                            device=x.device)
+        scratch = _scratch(n, x.device)
         _lib.lf_forward(n, mm, x, v, acc, nsteps, dt, ckpt, eps=eps, G=G, ckpt_every=ckpt_every,
-                        stream=stream, scratch=_scratch(n, x.device))
+                        stream=stream, scratch=scratch)
         ctx.save_for_backward(mm, ckpt)
+        # the backward pass re-runs these steps: with the same force (should there
+        # be no room for its scratch then, up to FP32 rounding)
+        ctx.lent = scratch is not None
         ctx.cfg = (n, nsteps, dt, eps, G, ckpt_every)
         return x, v
 
@@ -62,7 +63,7 @@ class LeapfrogFunction(torch.autograd.Function):
         work = torch.empty(_lib.lf_work_floats(n, ckpt_every), dtype=torch.float32, device=dev)
         _lib.lf_backward(n, mm, ckpt, nsteps, dt, lx, lv, lm, work, eps=eps, G=G,
                          ckpt_every=ckpt_every, stream=torch.cuda.current_stream(dev),
-                         scratch=_scratch(n, dev))
+                         scratch=_scratch(n, dev) if ctx.lent else None)
         return lx, lv, lm, None, None, None, None, None
 
 

@@ -313,3 +313,26 @@ def test_lent_scratch_scales_exactly(torch_cuda, n):
         res.append(acc.double() * 2.0**(2 * px - pm))
     for a in res[1:]:
         assert torch.equal(a, res[0])
+
+
+def test_backward_lends_only_what_forward_had(torch_cuda, monkeypatch):
+    """The forward pass found no room for scratch and the backward pass does: the
+    segments are re-run without it, so the gradients are those of a run that never
+    had any."""
+    torch = torch_cuda
+    from paper_0909_0879_gb300 import autograd
+
+    n = 16384
+    m, x, v = ics.plummer(n, 7)
+    real, grads = autograd._scratch, []
+    for room in ((False, False), (False, True), (True, True)):
+        asked = iter(room)
+        monkeypatch.setattr(autograd, "_scratch",
+                            lambda *a: real(*a) if next(asked, False) else None)
+        leaves = [torch.tensor(a, dtype=torch.float32, device="cuda", requires_grad=True)
+                  for a in (x, v, m)]
+        xT, vT = autograd.leapfrog(*leaves, 6, 2.0**-9, 1e-2, ckpt_every=3)
+        (xT.square().sum() + 0.5 * vT.square().sum()).backward()
+        grads.append([t.grad for t in leaves])
+    assert all(torch.equal(a, b) for a, b in zip(grads[0], grads[1]))
+    assert not all(torch.equal(a, b) for a, b in zip(grads[0], grads[2]))
