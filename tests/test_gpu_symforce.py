@@ -273,3 +273,27 @@ def test_path_does_not_follow_free_memory(nb):
         del hold
         torch.cuda.empty_cache()
     assert np.array_equal(got, want)
+
+
+# a shape, a cap of the grid (below the built-in grid of either size), both, a table
+@pytest.mark.parametrize("force", [lambda s: s.set_force_variant(26),
+                                   lambda s: s.set_force_variant(-1, 7),
+                                   lambda s: s.set_force_variant(1, 7),
+                                   lambda s: s.set_force_table([(4096, 0), (0, 3)])])
+@pytest.mark.parametrize("n", [1000, MIN_N])
+def test_a_forced_shape_is_the_shape_that_steps(nb, n, force):
+    """nb_step under a forced shape, grid or table takes the rows that the same
+    setting hands out, bit for bit, and not the sums of the built-in path."""
+    m, x, v = _system(nb, n, False)
+    kw = dict(eps=1e-3, block_steps=False, lev_shared=10)
+    with nb.NBody(m, x, v, **kw) as s, nb.NBody(m, x, v, **kw) as o, nb.NBody(m, x, v, **kw) as d:
+        force(s)
+        force(o)
+        s.step()
+        d.step()
+        t, na = o.next_block()
+        o.predict(t)
+        a, j = o.force_jerk()
+        got, built_in = s.get_state(want=("a", "jerk")), d.get_state(want=("a", "jerk"))
+    assert np.array_equal(got["a"], a) and np.array_equal(got["jerk"], j)
+    assert not np.array_equal(built_in["jerk"], j)
