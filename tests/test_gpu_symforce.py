@@ -283,7 +283,8 @@ def test_path_does_not_follow_free_memory(nb):
 @pytest.mark.parametrize("n", [1000, MIN_N])
 def test_a_forced_shape_is_the_shape_that_steps(nb, n, force):
     """nb_step under a forced shape, grid or table takes the rows that the same
-    setting hands out, bit for bit, and not the sums of the built-in path."""
+    setting hands out, bit for bit, and not the pair-symmetric sums (the one launch
+    of a small step has the separate kernels' bits)."""
     m, x, v = _system(nb, n, False)
     kw = dict(eps=1e-3, block_steps=False, lev_shared=10)
     with nb.NBody(m, x, v, **kw) as s, nb.NBody(m, x, v, **kw) as o, nb.NBody(m, x, v, **kw) as d:
@@ -296,4 +297,4 @@ def test_a_forced_shape_is_the_shape_that_steps(nb, n, force):
         a, j = o.force_jerk()
         got, built_in = s.get_state(want=("a", "jerk")), d.get_state(want=("a", "jerk"))
     assert np.array_equal(got["a"], a) and np.array_equal(got["jerk"], j)
-    assert not np.array_equal(built_in["jerk"], j)
+    assert n < MIN_N or not np.array_equal(built_in["a"], a)
