@@ -8,8 +8,9 @@ dt = 2^-10 so that every particle is active in every step.  One timed step
 is one pass of the whole path: block scheduling, predictor (split
 precision on the FP32 pipe from the FP64 state, writing the j-records),
 force + jerk of all N active particles against all N, corrector (FP64
-position and velocity update).  An interaction is one (i, j) pair
-evaluation; a step evaluates N^2 of them.
+position and velocity update).  An interaction is the force of one particle j
+on one particle i; a step has N^2 of them, each pair of particles evaluated once
+for both.
 
 Output: one JSON line (rank 0).  `value` is whole-job interactions/s from
 CUDA events on the library's stream with inputs resident in HBM; `e2e` is
@@ -45,6 +46,7 @@ N_DEFAULT = 1 << 20
 EPS = 1e-4
 W0 = 7.0
 LEV_SHARED = 10
+SYM_MIN = 16384  # from here on steps of all particles evaluate each pair once
 METRIC = "G pair-interactions/s (acc+jerk, N=1M)"
 UNIT = "Ginteractions/s"
 
@@ -57,7 +59,7 @@ def parse():
     p.add_argument("--impl", default="ours", choices=["ours", "reference"])
     p.add_argument("--precision", default="ds", choices=["ds", "fp32"])
     p.add_argument("--n", type=int, default=N_DEFAULT)
-    p.add_argument("--no-energy", action="store_true", help="skip the FP64 energy check")
+    p.add_argument("--no-energy", action="store_true", help="skip the energy check")
     p.add_argument("--no-cpu", action="store_true", help="skip the CPU-baseline leg")
     p.add_argument("--cpu-seconds", type=float, default=12.0)
     p.add_argument("--e2e-steps", type=int, default=0,
@@ -161,12 +163,13 @@ class ClockSampler:
 # --------------------------------------------------------------- roofline
 
 
-def force_traffic_from_profile(n):
-    """DRAM bytes per force launch from the committed ncu record
-    (profiles/force_jerk_ds_traffic.json), if it was taken on the current source
-    of the timed steps' kernel at this N; otherwise None."""
-    path = os.path.join(ROOT, "profiles", "force_jerk_ds_traffic.json")
-    src = os.path.join(ROOT, "paper_0909_0879_gb300", "csrc", "nb_symforce.cu")
+def force_traffic_from_profile(n, record="force_jerk_ds_traffic.json", source="nb_force.cu"):
+    """DRAM bytes per force evaluation from a committed ncu record in profiles/
+    (the one-sided kernel's; the pair-symmetric one's is pair_force_ds_traffic.json
+    with nb_symforce.cu), if it was taken on the kernel's current source at this
+    N; otherwise None."""
+    path = os.path.join(ROOT, "profiles", record)
+    src = os.path.join(ROOT, "paper_0909_0879_gb300", "csrc", source)
     try:
         rec = json.load(open(path))
     except (OSError, ValueError):
@@ -438,9 +441,17 @@ def run_ours(args, rank, world, local_rank):
     s.set_state(st0)
     s.predict(0.0)
     force_s = float(np.mean(force_ms)) / 1e3
-    achieved = metrics.FLOPS_PER_INTERACTION * n * n / force_s / 1e12
+    # flops of what the timed kernel evaluates: unordered pairs, or (a forced shape
+    # or grid, fewer particles) every ordered interaction
+    one_sided = args.variant >= 0 or args.grid > 0 or n < SYM_MIN
+    flops = (metrics.FLOPS_PER_INTERACTION * n * n if one_sided
+             else metrics.FLOPS_PER_PAIR * metrics.pair_count(n))
+    achieved = flops / force_s / 1e12
     peak, sm_max, peak_src = peak_info(num_sms)
-    traffic = force_traffic_from_profile(n) if args.precision == "ds" else None
+    traffic = None
+    if args.precision == "ds":
+        traffic = force_traffic_from_profile(
+            n, *(() if one_sided else ("pair_force_ds_traffic.json", "nb_symforce.cu")))
     clk_mhz = clocks.get("sm_mhz") if clocks else None
     cpu = None
     ferr = None
@@ -500,8 +511,9 @@ def run_ours(args, rank, world, local_rank):
             "relayouts_timed": relayouts,
         },
         "dE_over_E": dE,
-        "dE_note": f"FP64 GPU energy before warm-up and after {args.warmup + args.steps} steps "
-                   f"of dt 2^-{LEV_SHARED}" if dE is not None else None,
+        "dE_note": f"nb_energy (pair terms to 2^-46, summed in FP64; as exact as an FP64 sum) "
+                   f"before warm-up and after {args.warmup + args.steps} steps of dt "
+                   f"2^-{LEV_SHARED}" if dE is not None else None,
         "roofline": {
             "bound": "alu",
             "achieved": achieved,
@@ -509,16 +521,21 @@ def run_ours(args, rank, world, local_rank):
             "unit": "TFLOP/s",
             "frac": achieved / peak,
             "traffic": traffic,
-            "kernel": "pair-symmetric force (records, pairs, fix-up) per force evaluation, CUDA "
-                      "events on the library stream; achieved counts the flops of each ordered "
-                      "interaction, the kernel evaluates a pair once for both particles, so "
-                      "that frac may exceed 1",
-            "flops_per_interaction": metrics.FLOPS_PER_INTERACTION,
+            "kernel": ("one-sided force (pairs, fix-up)" if one_sided else
+                       "pair-symmetric force (records, pairs, fix-up)")
+                      + " per force evaluation, CUDA events on the library stream",
+            "flops_per_unit": (f"{metrics.FLOPS_PER_INTERACTION} per ordered interaction"
+                               if one_sided else
+                               f"{metrics.FLOPS_PER_PAIR} per unordered pair (both particles)"),
             "peak_def": f"{num_sms} SMs x 128 FP32 lanes x 2 x {sm_max:.0f} MHz ({peak_src})",
             "frac_at_measured_clock": (achieved / metrics.fp32_peak_tflops(num_sms, clk_mhz)
                                        if clk_mhz else None),
-            "frac_60flop_convention": achieved / metrics.FLOPS_PER_INTERACTION
-            * metrics.FLOPS_PER_INTERACTION_CONVENTION / peak,
+            # as if every ordered interaction were evaluated by itself (it is not: no
+            # fraction of what the hardware does, and may exceed 1)
+            "ordered_44flop_over_peak": (metrics.FLOPS_PER_INTERACTION * n * n / force_s / 1e12
+                                         / peak),
+            "ordered_60flop_over_peak": (metrics.FLOPS_PER_INTERACTION_CONVENTION * n * n
+                                         / force_s / 1e12 / peak),
         },
         "force_ms": float(np.mean(force_ms)),
         "e2e": {"value": e2e_val, "unit": UNIT, "h2d_bytes_per_step": int(h2d),
@@ -1003,6 +1020,8 @@ def run_symplectic(args):
     props = torch.cuda.get_device_properties(0)
     peak = metrics.fp32_peak_tflops(props.multi_processor_count, 2070.0) * 1e12
     speed = []
+    flops = (metrics.FLOPS_PER_ACC_PAIR * metrics.pair_count(n) if n >= SYM_MIN
+             else metrics.FLOPS_PER_ACC_INTERACTION * n * n)
     # input order x the library's layout setting: generation order stepped as
     # given, with the automatic layout (the default), and with the spatial
     # layout forced; and input presorted with nb_spatial_order stepped as given
@@ -1023,7 +1042,7 @@ def run_symplectic(args):
                               "s_per_step": per_step,
                               "ms_per_force_evaluation": per_step / stages * 1e3,
                               "interactions_per_s": ips,
-                              "frac_of_fp32_peak": ips * metrics.FLOPS_PER_ACC_INTERACTION / peak})
+                              "frac_of_fp32_peak": stages * flops / per_step / peak})
                 print(json.dumps(speed[-1]), file=sys.stderr, flush=True)
     accuracy = []
     for k in (7, 8, 9, 10):
@@ -1087,7 +1106,7 @@ def run_symplectic(args):
         print(json.dumps(row), file=sys.stderr, flush=True)
     out = {"metric": "interactions/s and energy error of the symplectic integrators",
            "unit": "interactions/s", "workload": f"uniform_sphere_salpeter_q1_n{n}_eps0.1d",
-           "flops_per_interaction": metrics.FLOPS_PER_ACC_INTERACTION,
+           "flops_per_force_evaluation": flops,
            "peak_basis": "FP32 lanes x 2 x 2070 MHz", "speed": speed,
            "energy_at_t_1/8": accuracy,
            "galactic_cluster": {"workload": f"plummer_n{n}_1e5msun_rv10pc_at_8.5kpc_allen_santillan",

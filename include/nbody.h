@@ -283,11 +283,19 @@ void nb_external_allen_santillan(nb_external *e);
  * gamma_halo <= 1. */
 nb_status nb_set_external(nb_ctx *ctx, const nb_external *e);
 
-/* Energy of the current (synchronised) state in FP64 on the GPU:
+/* Energy of the current (synchronised) state:
  * K = 1/2 sum m v^2, W = -G sum_{i<j} m_i m_j / sqrt(r_ij^2 + eps^2)
  * (the softened pair potential consistent with the force), plus
  * sum_i m_i Phi_ext(x_i) when an external field is set.  Uses the
- * particles' own stored x, v (not predicted).  Synchronises. */
+ * particles' own stored x, v (not predicted).  K and the field in FP64.  W in
+ * FP64 below 1,024 particles; from there on the terms are evaluated in split
+ * precision on the FP32 pipe, each to about 2^-46, and summed in FP64, which is
+ * as exact as the FP64 sum because their errors average out.  Where they would
+ * not, W is summed in FP64 all the same, more than ten times as long at 65,536
+ * particles: one particle dominates (sum m^2 above a fourth of (sum m)^2), or eps
+ * is more than a fourth of the harmonic mean softened distance; and where
+ * there is no device memory for the records (96 bytes per particle), up to the
+ * last bits.  Synchronises. */
 nb_status nb_energy(nb_ctx *ctx, double *kin, double *pot, double *tot);
 
 /* Copy the integrator state to host arrays (any may be NULL):

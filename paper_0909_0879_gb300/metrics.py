@@ -14,6 +14,12 @@ reciprocal square root as 1.  The split-precision variant executes extra
 additions for the position differences and the per-tile folds; those are
 overhead, not algorithmic work, and are not counted.
 
+FLOPS_PER_PAIR = 54 is the count of the pair-symmetric kernel, which evaluates
+an unordered pair once for both particles: 6 FADD, 3 FFMA (s^2), 1 reciprocal
+square root, 2 FMUL (1/s^2, 1/s^3), 2 FMUL (a mass each), 1 FMUL and 2 FFMA
+(d.w), 2 FMUL and 3 FFMA (w - 3 (d.w) d / s^2), and 3 FFMA per sum for the
+acceleration and the jerk of either particle (12 FFMA).
+
 The paper's own cost model (Sec. 2, Table 1) is about 30 flops per
 symmetric acceleration-only pair, n_f = 30 N (N - 1) / 2.
 """
@@ -24,7 +30,9 @@ FLOPS_PER_INTERACTION = 44
 # 3 FFMA (s^2), 1 reciprocal square root, 3 FMUL (1/s^2, m/s, m/s^3) and
 # 3 FFMA (acceleration), a fused multiply-add counted as 2 flops.
 FLOPS_PER_ACC_INTERACTION = 19
+FLOPS_PER_ACC_PAIR = 26  # both particles of a pair: 19 - 6 + 1 + 2 x 6
 FLOPS_PER_INTERACTION_CONVENTION = 60  # common acc+jerk convention in the literature
+FLOPS_PER_PAIR = 54
 PAPER_FLOPS_PER_PAIR = 30
 FP32_LANES_PER_SM = 128
 
