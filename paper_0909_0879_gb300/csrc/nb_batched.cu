@@ -185,15 +185,16 @@ __device__ __forceinline__ void batched_cluster(const BatchArgs &B, int c, float
   while (tpi < 32 && (NT / (tpi * 2)) * TPI_IPT >= n) tpi *= 2;
   const int g = tid / tpi;
   const int r = tid % tpi;
-  // the i-particles in equal passes, each packed onto as few warps as hold it:
-  // the idle warps cost no issue slots (600 particles in two passes of 512
-  // slots: 41 % of them padding; 4,096 clusters 19.7 -> 18.9 ms)
+  // the i-particles in full passes and a last one, packed onto as few warps as
+  // hold it: the idle warps cost no issue slots (600 particles in two passes of 512
+  // slots: 41 % of them padding).  In equal passes the last warps of every CTA, and
+  // so the same scheduler of every SM, would idle in each: 4,096 clusters, 300
+  // steps, shapes 10 / 11 / 13 / 14 766 / 678 / 901 / 820 against 781 / 732 / 922 /
+  // 873 G interactions/s, without either 750 / 665 / 928 / 810
   const int parts = TEAM ? static_cast<int>(team::size()) : 1;
   const int part = TEAM ? static_cast<int>(team::rank()) : 0;
   const int lo = n * part / parts, hi = n * (part + 1) / parts;  // this CTA's i-particles
-  const int most = NT / tpi * IPT;
-  const int passes = max(1, (hi - lo + most - 1) / most);
-  const int per = max(1, (hi - lo + passes - 1) / passes);
+  const int per = NT / tpi * IPT;
   float4 *s_hi = srec;
   float4 *s_lo = srec + B.cap;
   float4 *s_v = srec + (NARR - 1) * B.cap;
