@@ -9,7 +9,7 @@
 // evaluated on the FP32 pipe in split precision, about 89 packed operations
 // for two pairs, every term to about 2^-46 of itself with unbiased rounding,
 // and summed in split precision and, every 64 records, FP64; the triangle is
-// cut into equal ranges over 2 CTAs per SM: 6.32 / 0.67 / 0.062 ms, bound by
+// cut into equal ranges over 2 CTAs per SM: 6.06 / 0.64 / 0.094 ms, bound by
 // the FP32 pipe (0.76 of its rate).  The total is as exact as the FP64 sum,
 // whose own rounding it replaces, because the term errors are independent
 // and average over the N^2 / 2 pairs: relative error against extended
@@ -34,9 +34,8 @@
 //    a Newton step with its second-order term.
 //  * m_j / r as a pair, added by an error-free two-sum.  m_j is three words: what
 //    two leave out (2^-49) is the same for all particles of one mass and would
-//    not average out (up to 1.8e-15 of the total).  The third costs 2 % of the time
-//    at N = 65,536; taken into the product with e / 2 instead of a product of its
-//    own it leaves a bias of 1e-15.
+//    not average out (up to 1.8e-15 of the total).  The third is a product of its
+//    own: taken into the one with e / 2 it leaves a bias of 1e-15.
 // A closer pair, or one whose term is a visible part of the total (hard
 // binaries), takes FP64.  (With every softened distance from 2^-46 on in split
 // precision a close pair of light particles was off by up to 1e-1 of its term.)
@@ -200,6 +199,8 @@ __device__ __forceinline__ int length_exp(const unsigned long long *top, double 
 // rest), each value of both particles side by side.
 constexpr int kEnPairs = kJT / 2;
 constexpr int kEnPlane = kEnPairs;  // float4 per plane
+// distance of what does not count: its reciprocal root, and so every product, is 0
+constexpr float kEnInf = __builtin_huge_valf();
 constexpr float kEnNear = 0x1p-48f;  // square of the least softened distance
 constexpr int kEnPlanes = 6;
 constexpr size_t kEnTileBytes = kEnPlanes * kEnPlane * sizeof(float4);
@@ -352,14 +353,13 @@ __global__ void __launch_bounds__(kEnThreads, 2)
 #pragma unroll 2
         for (int k = 0; k < kEnSub; ++k) {
           const float4 a = sj[0][k], b = sj[1][k], c4 = sj[2][k], d4 = sj[3][k], e4 = sj[4][k];
-          const float4 f4 = sj[5][k];
+          const float2 f2 = reinterpret_cast<const float2 *>(&sj[5][k])[0];
           const V hj[3] = {make_float2(a.x, a.y), make_float2(a.z, a.w), make_float2(b.x, b.y)};
           const V lj[3] = {make_float2(c4.x, c4.y), make_float2(c4.z, c4.w),
                            make_float2(d4.x, d4.y)};
           const V rj[3] = {make_float2(e4.x, e4.y), make_float2(e4.z, e4.w),
-                           make_float2(f4.x, f4.y)};
+                           f2};
           V mh = make_float2(b.z, b.w), ml = make_float2(d4.z, d4.w);
-          V mr = make_float2(f4.z, f4.w);
           V D[3], E[3];
 #pragma unroll
           for (int c = 0; c < 3; ++c) {
@@ -370,10 +370,10 @@ __global__ void __launch_bounds__(kEnThreads, 2)
           V R = O::mul(D[2], D[2]);
           if (SOFT) R = O::fma(D[2], D[2], ve2);
           R = O::fma(D[0], D[0], O::fma(D[1], D[1], R));
-          if (own) {  // only j > i counts; the others get a harmless distance
+          if (own) {  // only j > i counts
             const int j = 2 * (k0 + k);
-            if (j <= tid) mh.x = ml.x = mr.x = 0.f, R.x = 1.f;
-            if (j + 1 <= tid) mh.y = ml.y = mr.y = 0.f, R.y = 1.f;
+            if (j <= tid) R.x = kEnInf;
+            if (j + 1 <= tid) R.y = kEnInf;
           }
           // pairs in FP64: distances too short for the words, and terms so large
           // that their own rounding would show in the total
@@ -390,8 +390,8 @@ __global__ void __launch_bounds__(kEnThreads, 2)
                 wi += m[j] * sm * rsqrt(dx * dx + dy * dy + dz * dz + eps_s * eps_s);
               }
             }
-            if (bx) mh.x = ml.x = mr.x = p.x = 0.f, y.x = 1.f;
-            if (by) mh.y = ml.y = mr.y = p.y = 0.f, y.y = 1.f;
+            if (bx) p.x = y.x = 0.f;
+            if (by) p.y = y.y = 0.f;
           }
           const V ny = O::mul(y, mone);
           V s = one, qe = O::bc(0.f), zz = O::bc(0.f);
@@ -420,6 +420,8 @@ __global__ void __launch_bounds__(kEnThreads, 2)
           const V e = O::fma(two, cr, sub2(s, qe));
           // m / r = m y (1 + e / 2 + 3 e^2 / 8) = p - np
           const V w2 = O::mul(e, O::mul(e, O::bc(-0.375f)));
+          // read here, where it is needed: 3 % of the time
+          const V mr = reinterpret_cast<const float2 *>(&sj[5][k])[1];
           V np = O::fma(p, w2, O::fma(mr, ny, O::fma(mh, ny, p)));
           np = O::fma(mh, O::mul(ny, O::mul(e, O::bc(0.5f))), O::fma(ml, ny, np));
           const V t = O::add(ah, p);
@@ -460,25 +462,35 @@ __global__ void energy_final_kernel(int64_t nb, const double *__restrict__ kin, 
                                     const double *__restrict__ mpart,
                                     const double *__restrict__ m2part,
                                     double *__restrict__ out) {
-  __shared__ double sh[kEnThreads];
-  auto sum = [&](int64_t cnt, const double *src) {
+  // the five sums side by side
+  __shared__ double sh[5][kEnThreads];
+  const double *const src[5] = {kin, pot, ext, mpart, m2part};
+  const int64_t cnt[5] = {nb, n_pot, n_ext, mpart ? nb : 0, mpart ? nb : 0};
+#pragma unroll
+  for (int k = 0; k < 5; ++k) {
     double s = 0.0;
-    for (int64_t b = threadIdx.x; b < cnt; b += blockDim.x) s += src[b];
-    return block_sum(s, sh);
-  };
-  const double k = sum(nb, kin), w = sum(n_pot, pot), e = sum(n_ext, ext);
+    for (int64_t b = threadIdx.x; b < cnt[k]; b += blockDim.x) s += src[k][b];
+    sh[k][threadIdx.x] = s;
+  }
+  __syncthreads();
+  for (int o = blockDim.x / 2; o > 0; o >>= 1) {
+    if (threadIdx.x < o)
+#pragma unroll
+      for (int k = 0; k < 5; ++k) sh[k][threadIdx.x] += sh[k][threadIdx.x + o];
+    __syncthreads();
+  }
+  if (threadIdx.x != 0) return;
+  const double w = sh[1][0];
   bool redo = false;
   if (mpart) {
     const double sm = pow2d(-down_exp(top[1]));
-    const double mass = sum(nb, mpart) * sm, m2 = sum(nb, m2part), most = 0.25 * mass * mass;
+    const double mass = sh[3][0] * sm, m2 = sh[4][0], most = 0.25 * mass * mass;
     redo = !(m2 <= most) || !(2.0 * eps * (w * sm * sm) <= most);
   }
-  if (threadIdx.x == 0) {
-    out[0] = k;
-    out[1] = -G * w;
-    out[2] = e;
-    out[3] = redo ? 1.0 : 0.0;
-  }
+  out[0] = sh[0][0];
+  out[1] = -G * w;
+  out[2] = sh[2][0];
+  out[3] = redo ? 1.0 : 0.0;
 }
 
 }  // namespace
