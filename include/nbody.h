@@ -294,7 +294,7 @@ nb_status nb_set_external(nb_ctx *ctx, const nb_external *e);
  * not, W is summed in FP64 all the same, more than ten times as long at 65,536
  * particles: one particle dominates (sum m^2 above a fourth of (sum m)^2), or eps
  * is more than a fourth of the harmonic mean softened distance; and where
- * there is no device memory for the records (96 bytes per particle), up to the
+ * there is no device memory for the records (48 bytes per particle), up to the
  * last bits.  Synchronises. */
 nb_status nb_energy(nb_ctx *ctx, double *kin, double *pot, double *tot);
 
